@@ -377,14 +377,10 @@ int tf_lbm_pressure_force(tf_lbm_handle* H, void* p, void* fx, void* fy, void* s
         (rc = check_dev_ptr(H, fy, "fy", true)))
         return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    const long long n = (long long)H->G.nx * H->G.ny;
-    if (!H->diag) CK(H, cudaMalloc(&H->diag, 2 * n * H->esize), "cudaMalloc diagnostics");
     const Consts<float> c32 = make_consts<float>(H);
     const Consts<double> c64 = make_consts<double>(H);
-    char* sc = (char*)H->diag;
-    cudaError_t e = aux_pressure_force(H->desc, H->buf[H->cur], H->kappa, p, fx, fy, sc, sc + n * H->esize,
-                                       H->G, &c32, &c64, st);
-    CK(H, e, "pressure/force kernels");
+    cudaError_t e = aux_pressure_force(H->desc, H->buf[H->cur], H->kappa, p, fx, fy, H->G, &c32, &c64, st);
+    CK(H, e, "pressure/force kernel");
     return TF_LBM_OK;
 }
 
@@ -499,7 +495,6 @@ void tf_lbm_destroy(tf_lbm_handle* H)
     if (H->kappa) cudaFree(H->kappa);
     if (H->partials) cudaFree(H->partials);
     if (H->flag) cudaFree(H->flag);
-    if (H->diag) cudaFree(H->diag);
     if (H->adj) cudaFree(H->adj);
     if (H->dscr) cudaFree(H->dscr);
     if (H->tscr) cudaFree(H->tscr);

@@ -18,14 +18,33 @@
 namespace tflbm {
 namespace {
 
-__device__ __constant__ int kCx[9] = {0, 1, 1, 0, -1, -1, -1, 0, 1};
-__device__ __constant__ int kCy[9] = {0, 0, 1, 1, 1, 0, -1, -1, -1};
+// Velocities of Eq. (speeds).  Functions of an unrolled index rather than
+// __constant__ arrays: they fold to literals, so a pull needs three wrapped
+// rows and three wrapped columns instead of eighteen runtime ones.
+__host__ __device__ constexpr int cx_of(int l) { return l == 1 || l == 2 || l == 8 ? 1 : (l >= 4 && l <= 6 ? -1 : 0); }
+__host__ __device__ constexpr int cy_of(int l) { return l >= 2 && l <= 4 ? 1 : (l >= 6 ? -1 : 0); }
 
-__device__ __forceinline__ int wrapi(int i, int n)
-{
-    i %= n;
-    return i < 0 ? i + n : i;
-}
+// i in [-1, n] on a ring of n (a compare each way; the integer modulo this
+// replaces cost more than the loads it indexed: plot-file read-out of 2048^2,
+// moments + pressure and force, 250 -> 93 us together with the fused k_pf).
+__device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? n - 1 : (i >= n ? 0 : i); }
+
+// Wrapped columns x-1, x, x+1 and row offsets of y-1, y, y+1 (rows of `pitch`
+// elements).
+struct Around {
+    int x[3], r[3];  // 32-bit: 9 planes stay below 2^31 elements
+    __device__ __forceinline__ Around(int x_, int y_, int nx, int ny, int pitch)
+    {
+        x[0] = wrapi(x_ - 1, nx);
+        x[1] = x_;
+        x[2] = wrapi(x_ + 1, nx);
+        r[0] = wrapi(y_ - 1, ny) * pitch;
+        r[1] = y_ * pitch;
+        r[2] = wrapi(y_ + 1, ny) * pitch;
+    }
+    // element of the node (dx, dy) away, dx, dy in {-1, 0, 1}
+    __device__ __forceinline__ int at(int dx, int dy) const { return r[dy + 1] + x[dx + 1]; }
+};
 
 __device__ __forceinline__ float cvt(float q) { return q; }
 __device__ __forceinline__ double cvt(double q) { return q; }
@@ -40,22 +59,21 @@ template <typename T, typename SM>
 struct Pops {
     T* f0;       // plane 0: f_0 - href
     SM* fm;      // moving planes 1..8
-    long long plane;
-    int pitch;
+    int plane, pitch;
     T href, mscale, minv, r_axis, r_diag;
 
-    __device__ __forceinline__ long long at(int y, int x) const { return (long long)y * pitch + x; }
+    __device__ __forceinline__ int at(int y, int x) const { return y * pitch + x; }
     // the stored value of plane l at element i, decoded (plane 0: f_0 - href)
-    __device__ __forceinline__ T raw(int l, long long i) const
+    __device__ __forceinline__ T raw(int l, int i) const
     {
         if (l == 0) return f0[i];
         const SM q = fm[(l - 1) * plane + i];
         if constexpr (std::is_same<SM, T>::value) return q;
         else return fmaf(cvt(q), minv, (l & 1) ? r_axis : r_diag);
     }
-    __device__ __forceinline__ T full(int l, long long i) const { return l == 0 ? raw(0, i) + href : raw(l, i); }
+    __device__ __forceinline__ T full(int l, int i) const { return l == 0 ? raw(0, i) + href : raw(l, i); }
     // store the population value v (plane 0: v is f_0 - href)
-    __device__ __forceinline__ void put(int l, long long i, T v) const
+    __device__ __forceinline__ void put(int l, int i, T v) const
     {
         if (l == 0) f0[i] = v;
         else if constexpr (std::is_same<SM, T>::value) fm[(l - 1) * plane + i] = v;
@@ -69,7 +87,7 @@ Pops<T, SM> make_pops(const void* buf, const Geom& G, const StoreDesc& D)
     Pops<T, SM> P;
     P.f0 = (T*)buf;
     P.fm = (SM*)((char*)buf + G.plane * sizeof(T));
-    P.plane = G.plane;
+    P.plane = (int)G.plane;
     P.pitch = G.pitch;
     P.href = T(D.href);
     P.mscale = T(D.mscale);
@@ -83,9 +101,9 @@ Pops<T, SM> make_pops(const void* buf, const Geom& G, const StoreDesc& D)
 template <typename T, typename SM>
 __device__ __forceinline__ void pull_at(const Pops<T, SM>& P, const Geom& G, int x, int y, T (&v)[9])
 {
+    const Around N(x, y, G.nx, G.ny, P.pitch);
 #pragma unroll
-    for (int l = 0; l < 9; ++l)
-        v[l] = P.full(l, P.at(wrapi(y - kCy[l], G.ny), wrapi(x - kCx[l], G.nx)));
+    for (int l = 0; l < 9; ++l) v[l] = P.full(l, N.at(-cx_of(l), -cy_of(l)));
 }
 
 template <typename T>
@@ -113,9 +131,10 @@ __global__ void k_init(Pops<T, SM> P, const T* __restrict__ h0, Geom G, T g)
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y;
     if (x >= G.nx) return;
+    const Around N(x, y, G.nx, G.ny, G.nx);
 #pragma unroll
     for (int l = 0; l < 9; ++l) {
-        const T h = h0[(long long)wrapi(y + kCy[l], G.ny) * G.nx + wrapi(x + kCx[l], G.nx)];
+        const T h = h0[N.at(cx_of(l), cy_of(l))];
         const T gh2 = g * h * h;
         T v;
         if (l == 0) v = (h - P.href) - T(5.0 / 6.0) * gh2;
@@ -138,19 +157,6 @@ __global__ void k_moments(Pops<T, SM> P, T* h, T* ux, T* uy, Geom G)
     if (h) h[i] = hh;
     if (ux) ux[i] = jx / hh;
     if (uy) uy[i] = jy / hh;
-}
-
-// Diagnostic film pressure and force, in three plain passes.
-template <typename T, typename SM>
-__global__ void k_pf_h(Pops<T, SM> P, T* hbuf, Geom G)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= G.nx) return;
-    T v[9], hh, jx, jy;
-    pull_at(P, G, x, y, v);
-    moments9(v, hh, jx, jy);
-    hbuf[(long long)y * G.nx + x] = hh;
 }
 
 template <typename T>
@@ -181,36 +187,124 @@ __global__ void k_pf_p(const T* __restrict__ hbuf, const T* __restrict__ kappa, 
     pbuf[(long long)y * G.nx + x] = -C.gamma * lap;
 }
 
-template <typename T, typename SM>
-__global__ void k_pf_f(Pops<T, SM> P, const T* __restrict__ pbuf, T* p, T* fx, T* fy, Geom G,
-                       Consts<T> C)
+// i on a ring of n, for the halo of a tile (any i; the modulo runs only
+// outside the lattice)
+__device__ __forceinline__ int ringi(int i, int n)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= G.nx) return;
-    const int xm = wrapi(x - 1, G.nx), xp = wrapi(x + 1, G.nx);
-    const int ym = wrapi(y - 1, G.ny), yp = wrapi(y + 1, G.ny);
-    auto Pp = [&](int yy, int xx) { return pbuf[(long long)yy * G.nx + xx]; };
-    const T gpx = (Pp(y, xp) - Pp(y, xm)) / T(3) + (Pp(yp, xp) - Pp(yp, xm) + Pp(ym, xp) - Pp(ym, xm)) / T(12);
-    const T gpy = (Pp(yp, x) - Pp(ym, x)) / T(3) + (Pp(yp, xp) - Pp(ym, xp) + Pp(yp, xm) - Pp(ym, xm)) / T(12);
-    T v[9], hh, jx, jy;
-    pull_at(P, G, x, y, v);
-    moments9(v, hh, jx, jy);
-    const T fr = C.nu6 / (T(2) * hh * hh + T(6) * C.delta * hh + T(3) * C.delta * C.delta);
-    const long long i = (long long)y * G.nx + x;
-    if (p) p[i] = Pp(y, x);
-    T Fx = -hh * gpx - fr * jx + hh * C.gx;
-    T Fy = -hh * gpy - fr * jy + hh * C.gy;
-    if (C.forcing) {
-        // second-order forcing: friction at u = (j + F/2)/h, i.e.
-        // h u (1 + fr/2) = j + F'/2 with F' the force without friction
-        const T fpx = hh * (C.gx - gpx), fpy = hh * (C.gy - gpy);
-        const T q = T(1) / (T(1) + T(0.5) * fr);
-        Fx = fpx - fr * (jx + T(0.5) * fpx) * q;
-        Fy = fpy - fr * (jy + T(0.5) * fpy) * q;
+    if ((unsigned)i < (unsigned)n) return i;
+    i %= n;
+    return i < 0 ? i + n : i;
+}
+
+// Film pressure and force of the current state in one pass.  Bound by HBM (36
+// B of populations in, 12 B out a node in FP32) plus the halo's second reads
+// from L1/L2; before, three kernels read the populations twice and moved h
+// and p through memory.  A CTA owns a tile of kPfX x kPfY nodes: h - href of
+// the tile and a halo of 2, the pressure of the tile and a halo of 1, then the
+// force; each thread keeps the momenta of its own four nodes.  64 x 16: rows
+// long enough for coalesced pulls, 1.33 pulls a node.  2048^2 FP32 read-out
+// (k_moments and this): 250 -> 93 us.
+constexpr int kPfX = 64, kPfY = 16, kPfThreads = 256, kPfOwn = kPfX * kPfY / kPfThreads;
+template <typename T, typename SM>
+__global__ void __launch_bounds__(kPfThreads) k_pf(Pops<T, SM> P, const T* __restrict__ kappa, T* p, T* fx, T* fy,
+                                                   Geom G, Consts<T> C)
+{
+    __shared__ T hs[kPfY + 4][kPfX + 4];
+    __shared__ T ps[kPfY + 2][kPfX + 2];
+    const int x0 = blockIdx.x * kPfX, y0 = blockIdx.y * kPfY;
+    const int w = min(kPfX, G.nx - x0), hgt = min(kPfY, G.ny - y0);
+    const int tx = threadIdx.x % kPfX, ty = threadIdx.x / kPfX;
+    // h - href of the node at tile position (c, r), and its momentum
+    auto pull = [&](int c, int r, T& jx, T& jy) {
+        const Around N(ringi(x0 + c, G.nx), ringi(y0 + r, G.ny), G.nx, G.ny, P.pitch);
+        T v[9];
+#pragma unroll
+        for (int l = 0; l < 9; ++l) v[l] = P.raw(l, N.at(-cx_of(l), -cy_of(l)));
+        T dh;
+        moments9(v, dh, jx, jy);
+        return dh;
+    };
+    auto pressure = [&](int c, int r) {
+        const T(&H)[kPfY + 4][kPfX + 4] = hs;
+        const int i = r + 2, j = c + 2;
+        const T axis = (H[i][j - 1] + H[i][j + 1]) + (H[i - 1][j] + H[i + 1][j]);
+        const T diag = (H[i - 1][j - 1] + H[i - 1][j + 1]) + (H[i + 1][j - 1] + H[i + 1][j + 1]);
+        T lap = (T(4) * axis + diag - T(20) * H[i][j]) * T(1.0 / 6.0);
+        const T kap = kappa ? kappa[ringi(y0 + r, G.ny) * G.nx + ringi(x0 + c, G.nx)] : C.kappa_u;
+        const T q = C.hstar / (H[i][j] + P.href);
+        const T fd = C.n_exp == 3 && C.m_exp == 2 ? q * q * (q - T(1)) : ipow_(q, C.n_exp) - ipow_(q, C.m_exp);
+        lap += C.pi_sgn * kap * fd;
+        return -C.gamma * lap;
+    };
+    T jx[kPfOwn], jy[kPfOwn];
+    bool own[kPfOwn];
+#pragma unroll
+    for (int k = 0; k < kPfOwn; ++k) {
+        const int r = ty + k * (kPfThreads / kPfX);
+        own[k] = tx < w && r < hgt;
+        jx[k] = jy[k] = T(0);
+        if (own[k]) hs[r + 2][tx + 2] = pull(tx, r, jx[k], jy[k]);
     }
-    if (fx) fx[i] = Fx;
-    if (fy) fy[i] = Fy;
+    // halo of 2: two rows below and above, two columns left and right
+    constexpr int HR = 4 * (kPfX + 4);
+    for (int i = threadIdx.x; i < HR + 4 * kPfY; i += kPfThreads) {
+        int c, r;
+        if (i < HR) {
+            const int k = i / (kPfX + 4);
+            c = i % (kPfX + 4) - 2;
+            r = k < 2 ? k - 2 : hgt + k - 2;
+        } else {
+            const int k = (i - HR) % 4;
+            r = (i - HR) / 4;
+            c = k < 2 ? k - 2 : w + k - 2;
+        }
+        T a, b;
+        if (c < w + 2 && r < hgt + 2) hs[r + 2][c + 2] = pull(c, r, a, b);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPfOwn; ++k) {
+        const int r = ty + k * (kPfThreads / kPfX);
+        if (own[k]) ps[r + 1][tx + 1] = pressure(tx, r);
+    }
+    constexpr int PR = 2 * (kPfX + 2);
+    for (int i = threadIdx.x; i < PR + 2 * kPfY; i += kPfThreads) {
+        int c, r;
+        if (i < PR) {
+            c = i % (kPfX + 2) - 1;
+            r = i / (kPfX + 2) == 0 ? -1 : hgt;
+        } else {
+            r = (i - PR) / 2;
+            c = (i - PR) % 2 == 0 ? -1 : w;
+        }
+        if (c < w + 1 && r < hgt + 1) ps[r + 1][c + 1] = pressure(c, r);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPfOwn; ++k) {
+        const int r = ty + k * (kPfThreads / kPfX);
+        if (!own[k]) continue;
+        auto Pp = [&](int dy, int dx) { return ps[r + 1 + dy][tx + 1 + dx]; };
+        const T third = T(1.0 / 3.0), twelfth = T(1.0 / 12.0);
+        const T gpx = (Pp(0, 1) - Pp(0, -1)) * third + (Pp(1, 1) - Pp(1, -1) + Pp(-1, 1) - Pp(-1, -1)) * twelfth;
+        const T gpy = (Pp(1, 0) - Pp(-1, 0)) * third + (Pp(1, 1) - Pp(-1, 1) + Pp(1, -1) - Pp(-1, -1)) * twelfth;
+        const T hh = hs[r + 2][tx + 2] + P.href;
+        const T fr = C.nu6 / (T(2) * hh * hh + T(6) * C.delta * hh + T(3) * C.delta * C.delta);
+        const long long i = (long long)(y0 + r) * G.nx + x0 + tx;
+        if (p) p[i] = Pp(0, 0);
+        T Fx = -hh * gpx - fr * jx[k] + hh * C.gx;
+        T Fy = -hh * gpy - fr * jy[k] + hh * C.gy;
+        if (C.forcing) {
+            // second-order forcing: friction at u = (j + F/2)/h, i.e.
+            // h u (1 + fr/2) = j + F'/2 with F' the force without friction
+            const T fpx = hh * (C.gx - gpx), fpy = hh * (C.gy - gpy);
+            const T q = T(1) / (T(1) + T(0.5) * fr);
+            Fx = fpx - fr * (jx[k] + T(0.5) * fpx) * q;
+            Fy = fpy - fr * (jy[k] + T(0.5) * fpy) * q;
+        }
+        if (fx) fx[i] = Fx;
+        if (fy) fy[i] = Fy;
+    }
 }
 
 // Neumaier pair (s, c): value s + c.
@@ -337,7 +431,7 @@ __device__ __forceinline__ Pops<T, SM> pops_of(const BatchDomain<T>& D, int pari
     Pops<T, SM> P;
     P.f0 = (T*)D.buf[parity];
     P.fm = (SM*)((char*)D.buf[parity] + D.G.plane * sizeof(T));
-    P.plane = D.G.plane;
+    P.plane = (int)D.G.plane;
     P.pitch = D.G.pitch;
     P.href = D.C.href;
     P.mscale = D.C.mscale;
@@ -347,90 +441,287 @@ __device__ __forceinline__ Pops<T, SM> pops_of(const BatchDomain<T>& D, int pari
     return P;
 }
 
-// Film diagnostics of domain blockIdx.y of a table (compensated sums in
-// double): [0] h over the lattice; over the wetted nodes (h > h_wet) [1] h,
+// Running sums of the diagnostics, two at a time.  With an FP32 compute type a
+// sum is an error-free FP32 pair (Knuth's TwoSum per addend, products split by
+// fma), which resolves it to about 2^-48, and both sums share Blackwell's
+// paired FP32 instructions; FP64 state sums in compensated doubles.  GB300
+// retires 2 FP64 operations a clock and SM: the same sums in doubles, with a
+// double sincospi per node, were what bounded this pass (32 domains: 2130 us),
+// and per-unit merges in doubles still took half of it (155 us).
+// a - b in one instruction (the paired add takes no negated operand)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+template <typename T> struct Acc2;
+template <> struct Acc2<float> {
+    using V = float2;
+    V s = {0.0f, 0.0f}, c = {0.0f, 0.0f};
+    __device__ __forceinline__ void add(V v)
+    {
+        const V t = __fadd2_rn(s, v), b = sub2(t, s);
+        c = __fadd2_rn(c, __fadd2_rn(sub2(s, sub2(t, b)), sub2(v, b)));
+        s = t;
+    }
+    // += v * (hi + lo)
+    __device__ __forceinline__ void add_product(V v, V hi, V lo)
+    {
+        const V q = __fmul2_rn(v, hi);
+        // the product's rounding error v hi - q is exact in one fma
+        c = __fadd2_rn(c, __ffma2_rn(v, lo, __ffma2_rn(v, hi, V{-q.x, -q.y})));
+        add(q);
+    }
+    // += (s_ + c_) * (hi + lo)
+    __device__ __forceinline__ void add_product(float s_, float c_, V hi, V lo)
+    {
+        add_product(V{s_, s_}, hi, lo);
+        c = __ffma2_rn(V{c_, c_}, hi, c);
+    }
+    __device__ __forceinline__ void merge(const Acc2& a)
+    {
+        add(a.s);
+        c = __fadd2_rn(c, a.c);
+    }
+};
+template <> struct Acc2<double> {
+    using V = double2;
+    V s = {0.0, 0.0}, c = {0.0, 0.0};
+    __device__ __forceinline__ void add(V v)
+    {
+        Comp a{s.x, c.x}, b{s.y, c.y};
+        comp_add(a, v.x);
+        comp_add(b, v.y);
+        s = V{a.s, b.s};
+        c = V{a.c, b.c};
+    }
+    __device__ __forceinline__ void add_product(V v, V hi, V) { add(V{v.x * hi.x, v.y * hi.y}); }
+    __device__ __forceinline__ void add_product(double s_, double c_, V hi, V)
+    {
+        add(V{s_ * hi.x, s_ * hi.y});
+        c.x += c_ * hi.x;
+        c.y += c_ * hi.y;
+    }
+    __device__ __forceinline__ void merge(const Acc2& a)
+    {
+        add(a.s);
+        c.x += a.c.x;
+        c.y += a.c.y;
+    }
+};
+template <typename T>
+__device__ __forceinline__ Acc2<T> warp_total(Acc2<T> a)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Acc2<T> b;
+        b.s.x = __shfl_down_sync(0xffffffffu, a.s.x, o);
+        b.s.y = __shfl_down_sync(0xffffffffu, a.s.y, o);
+        b.c.x = __shfl_down_sync(0xffffffffu, a.c.x, o);
+        b.c.y = __shfl_down_sync(0xffffffffu, a.c.y, o);
+        a.merge(b);
+    }
+    return a;
+}
+
+// One entry of a domain's trigonometric table: cos and sin of 2 pi i / n as
+// hi + lo (FP64 state: lo = 0).  Entries 0 .. nx-1 are the columns, nx ..
+// nx+ny-1 the rows.  A Fourier phase 2 pi m x / n is entry m x mod n, so the
+// table does not depend on the mode and is written once.
+template <typename T> struct Trig;
+template <> struct __align__(16) Trig<float> {
+    float2 hi, lo;  // (cos, sin)
+    __device__ __forceinline__ void set(double c, double s)
+    {
+        hi = make_float2((float)c, (float)s);
+        lo = make_float2((float)(c - (double)hi.x), (float)(s - (double)hi.y));
+    }
+};
+template <> struct __align__(16) Trig<double> {
+    double2 hi;
+    static constexpr double2 lo{0.0, 0.0};
+    __device__ __forceinline__ void set(double c, double s) { hi = make_double2(c, s); }
+};
+static_assert(sizeof(Trig<float>) == kDiagTrigBytes && sizeof(Trig<double>) == kDiagTrigBytes, "table entry size");
+
+template <typename T>
+__global__ void k_diag_table(const BatchDomain<T>* __restrict__ doms, Trig<T>* table, int stride)
+{
+    const Geom G = doms[blockIdx.y].G;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= G.nx + G.ny) return;
+    double s, c;
+    sincospi(i < G.nx ? 2.0 * i / G.nx : 2.0 * (i - G.nx) / G.ny, &s, &c);
+    Trig<T> e;
+    e.set(c, s);
+    table[(long long)blockIdx.y * stride + i] = e;
+}
+
+// Film diagnostics of domain blockIdx.y of a table (compensated sums):
+// [0] h over the lattice; over the wetted nodes (h > h_wet) [1] h,
 // [2] j_x, [3] j_y, [4] 1, [5] h cos(2 pi x / nx), [6] h sin(2 pi x / nx),
 // [7] h cos(2 pi y / ny), [8] h sin(2 pi y / ny); over the lattice
 // [9] h cos(phi), [10] h sin(phi) with phi = 2 pi (mx x / nx + my y / ny);
 // and the largest h.  Block b writes kDiagPartial doubles at
 // partials[(domain * gridDim.x + b) * kDiagPartial].
+//
+// A warp takes units of 32 columns x `rows` rows; a lane sums its own column
+// down the rows, so the column's trigonometric factors multiply one sum per
+// unit and the mode's phase splits into a row factor per node and a column
+// factor per unit (cos(a + b) from the two angles).  The unit height gives
+// every warp of the launch one unit where it can, but at least kDiagRows rows
+// (a unit's products and its reduction over the warp cost about five rows),
+// and the sums of a unit leave the registers at its end, which are then eight
+// sums and two rows of loads.
+// Bound by HBM: 36 B a node in FP32.  32 domains, 7.6 M nodes: 2150 -> 90 us
+// with the final kernel.
 constexpr int kDiagPartial = 2 * kDiagSums + 1;
+constexpr int kDiagRows = 16;
 template <typename T, typename SM>
-__global__ void __launch_bounds__(kMassThreads) k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity,
-                                                               double h_wet, int mx, int my, double* partials)
+__global__ void __launch_bounds__(kMassThreads, sizeof(T) == 4 ? 4 : 1)
+k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T>* __restrict__ table, int stride,
+               double h_wet, int mx, int my, double* partials)
 {
+    constexpr int NW = kMassThreads / 32;
     const BatchDomain<T>& D = doms[blockIdx.y];
     const Pops<T, SM> P = pops_of<T, SM>(D, parity);
     const Geom G = D.G;
-    Comp a[kDiagSums];
-#pragma unroll
-    for (int k = 0; k < kDiagSums; ++k) a[k] = Comp{0.0, 0.0};
-    double hmax = -INFINITY;
-    const long long n = (long long)G.nx * G.ny;
+    const Trig<T>* tx = table + (long long)blockIdx.y * stride;
+    const Trig<T>* ty = tx + G.nx;
+    using V = typename Acc2<T>::V;
+    // per warp: (h, wetted h), (j_x, j_y), wetted h (cos, sin) of the column
+    // and of the row angle, h (cos, sin) of the mode; wetted nodes; largest h
+    __shared__ Acc2<T> sm[5][NW];
+    __shared__ long long scount[NW];
+    __shared__ T smax[NW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (lane < 5) sm[lane][wid] = Acc2<T>();
+    if (lane == 5) scount[wid] = 0;
+    if (lane == 6) smax[wid] = -INFINITY;
+    __syncwarp();
     // integer wave numbers reduced modulo the lattice, so phases stay exact
-    const long long kx = ((mx % G.nx) + G.nx) % G.nx, ky = ((my % G.ny) + G.ny) % G.ny;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % G.nx), y = (int)(i / G.nx);
-        T v[9], hh, jx, jy;
-        pull_at(P, G, x, y, v);
-        moments9(v, hh, jx, jy);
-        const double h = (double)hh;
-        comp_add(a[0], h);
-        const double q = (double)((kx * x) % G.nx) / G.nx + (double)((ky * y) % G.ny) / G.ny;
-        double sp, cp;
-        sincospi(2.0 * q, &sp, &cp);
-        comp_add(a[9], h * cp);
-        comp_add(a[10], h * sp);
-        if (h > h_wet) {
-            comp_add(a[1], h);
-            comp_add(a[2], (double)jx);
-            comp_add(a[3], (double)jy);
-            a[4].s += 1.0;  // exact below 2^53
-            double sx, cx, sy, cy;
-            sincospi(2.0 * x / G.nx, &sx, &cx);
-            sincospi(2.0 * y / G.ny, &sy, &cy);
-            comp_add(a[5], h * cx);
-            comp_add(a[6], h * sx);
-            comp_add(a[7], h * cy);
-            comp_add(a[8], h * sy);
-        }
-        hmax = fmax(hmax, h);
-    }
-    double* out = partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kDiagPartial;
+    const int kx = ((mx % G.nx) + G.nx) % G.nx, ky = ((my % G.ny) + G.ny) % G.ny;
+    // hh > h_wet in the compute type: the nearest float at or below h_wet
+    // separates the same heights
+    T wet_above;
+    if constexpr (std::is_same<T, float>::value) wet_above = __double2float_rd(h_wet);
+    else wet_above = h_wet;
+    const int warps = gridDim.x * NW;
+    const int ux = (G.nx + 31) / 32, most = max(1, warps / ux);
+    const int rows = max(kDiagRows, (G.ny + most - 1) / most), uy = (G.ny + rows - 1) / rows;
+    for (int u = blockIdx.x * NW + wid; u < ux * uy; u += warps) {
+        const int x = (u % ux) * 32 + lane, y0 = (u / ux) * rows, y1 = min(y0 + rows, G.ny);
+        // over this column: (h, wetted h), wetted (j_x, j_y), wetted h (cos,
+        // sin) of the row angle, h (cos, sin) of the row's mode phase
+        Acc2<T> ah, aj, ar, am;
+        int iy = (int)((long long)ky * y0 % G.ny), count = 0;
+        T top = -INFINITY;
+        if (x < G.nx) {
+            const int xm = wrapi(x - 1, G.nx), xp = wrapi(x + 1, G.nx);
+            int ra = wrapi(y0 - 1, G.ny) * P.pitch, r0 = y0 * P.pitch;  // rows y - 1, y
+            auto pull = [&](int y, T(&v)[9]) {  // row y, whose neighbours are ra and the one after r0
+                const int rb = y + 1 == G.ny ? 0 : r0 + P.pitch;
+                v[0] = P.full(0, r0 + x);
+                v[1] = P.full(1, r0 + xm);
+                v[2] = P.full(2, ra + xm);
+                v[3] = P.full(3, ra + x);
+                v[4] = P.full(4, ra + xp);
+                v[5] = P.full(5, r0 + xp);
+                v[6] = P.full(6, rb + xp);
+                v[7] = P.full(7, rb + x);
+                v[8] = P.full(8, rb + xm);
+                ra = r0;
+                r0 = rb;
+            };
+            T v[9], n[9];
+            pull(y0, n);
+            for (int y = y0; y < y1; ++y) {
 #pragma unroll
-    for (int k = 0; k < kDiagSums; ++k) {
-        const Comp b = block_sum(a[k]);
-        if (threadIdx.x == 0) {
-            out[2 * k] = b.s;
-            out[2 * k + 1] = b.c;
+                for (int l = 0; l < 9; ++l) v[l] = n[l];
+                if (y + 1 < y1) pull(y + 1, n);
+                T hh, jx, jy;
+                moments9(v, hh, jx, jy);
+                const bool wet = hh > wet_above;
+                const T hw = wet ? hh : T(0);
+                const Trig<T> m = ty[iy], w = ty[y];
+                ah.add(V{hh, hw});
+                aj.add(V{wet ? jx : T(0), wet ? jy : T(0)});
+                ar.add_product(V{hw, hw}, w.hi, w.lo);
+                am.add_product(V{hh, hh}, m.hi, m.lo);
+                count += wet;
+                iy += ky;
+                if (iy >= G.ny) iy -= G.ny;
+                top = fmax(top, hh);
+            }
+        }
+        const int xc = min(x, G.nx - 1);  // a lane past the lattice holds zeros
+        const Trig<T> w = tx[xc], m = tx[(long long)kx * xc % G.nx];
+        Acc2<T> ac, ap;  // the column angle; the mode: cos(a + b), sin(a + b)
+        ac.add_product(ah.s.y, ah.c.y, w.hi, w.lo);
+        ap.add_product(am.s.x, am.c.x, m.hi, m.lo);
+        ap.add_product(am.s.y, am.c.y, V{-m.hi.y, m.hi.x}, V{-m.lo.y, m.lo.x});
+        auto total = [&](int k, const Acc2<T>& a) {
+            const Acc2<T> q = warp_total(a);
+            if (lane == 0) sm[k][wid].merge(q);
+        };
+        total(0, ah);
+        total(1, aj);
+        total(2, ac);
+        total(3, ar);
+        total(4, ap);
+        count = __reduce_add_sync(0xffffffffu, count);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_down_sync(0xffffffffu, top, o));
+        if (lane == 0) {
+            scount[wid] += count;
+            smax[wid] = fmax(smax[wid], top);
         }
     }
-    const double m = block_max(hmax);
-    if (threadIdx.x == 0) out[2 * kDiagSums] = m;
+    __syncthreads();
+    double* out = partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kDiagPartial;
+    const int k = threadIdx.x;
+    if (k < 5) {
+        Acc2<T> b = sm[k][0];
+        for (int w = 1; w < NW; ++w) b.merge(sm[k][w]);
+        const int q = 2 * (k < 2 ? 2 * k : 2 * k + 1);  // sums (0, 1), (2, 3), (5, 6), (7, 8), (9, 10)
+        out[q] = b.s.x;
+        out[q + 1] = b.c.x;
+        out[q + 2] = b.s.y;
+        out[q + 3] = b.c.y;
+    } else if (k == 5) {
+        long long b = 0;
+        for (int w = 0; w < NW; ++w) b += scount[w];
+        out[8] = (double)b;  // exact below 2^53
+        out[9] = 0.0;
+    } else if (k == 6) {
+        T b = smax[0];
+        for (int w = 1; w < NW; ++w) b = fmax(b, smax[w]);
+        out[2 * kDiagSums] = b;
+    }
 }
 
-// One block per domain: reduce the partials of its nb blocks into
-// out[domain * kDiagOut ..] in the order of tf_lbm_diag: sums 0..4, the
-// maximum, sums 5..10.
-__global__ void __launch_bounds__(kMassThreads) k_diag_final(const double* __restrict__ partials, int nb,
-                                                             double* out)
+// One warp per value: block (k, domain) reduces the partials of the domain's
+// nb blocks into field k of out[domain * kDiagOut ..], the fields of
+// tf_lbm_diag (sums 0..4, the maximum, sums 5..10).  A warp each, not a block
+// per domain, so that the FP64 adds of the twelve values spread over SMs.
+__global__ void __launch_bounds__(32) k_diag_final(const double* __restrict__ partials, int nb, double* out)
 {
-    const double* p = partials + (long long)blockIdx.x * nb * kDiagPartial;
-    double* o = out + (long long)blockIdx.x * kDiagOut;
-    for (int k = 0; k < kDiagSums; ++k) {
+    const double* p = partials + (long long)blockIdx.y * nb * kDiagPartial;
+    const int k = blockIdx.x;
+    double r;
+    if (k == 5) {
+        double m = -INFINITY;
+        for (int i = threadIdx.x; i < nb; i += 32) m = fmax(m, p[(long long)i * kDiagPartial + 2 * kDiagSums]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        r = m;
+    } else {
+        const int q = 2 * (k < 5 ? k : k - 1);
         Comp a{0.0, 0.0};
-        for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-            comp_add(a, p[i * kDiagPartial + 2 * k]);
-            a.c += p[i * kDiagPartial + 2 * k + 1];
+        for (int i = threadIdx.x; i < nb; i += 32) {
+            comp_add(a, p[(long long)i * kDiagPartial + q]);
+            a.c += p[(long long)i * kDiagPartial + q + 1];
         }
-        const Comp b = block_sum(a);
-        if (threadIdx.x == 0) o[k < 5 ? k : k + 1] = b.s + b.c;
+        a = warp_reduce(a);
+        r = a.s + a.c;
     }
-    double m = -INFINITY;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) m = fmax(m, p[i * kDiagPartial + 2 * kDiagSums]);
-    m = block_max(m);
-    if (threadIdx.x == 0) o[5] = m;
+    if (threadIdx.x == 0) out[(long long)blockIdx.y * kDiagOut + k] = r;
 }
 
 // ---- term balance of the appendix (Eq. magnitude): fields h, j, p, div j
@@ -593,6 +884,35 @@ __global__ void k_check(Pops<T, SM> P, Geom G, int* flag)
     if (bad && (threadIdx.x & 31) == 0) atomicOr(flag, bad);
 }
 
+// float to double and back, with the bits FP64 conversions give.  The FP64
+// pipe takes 16 clocks a warp instruction; nine conversions a node bounded the
+// state import and export (2^20 nodes: 24 and 27 us a pass, 16 us now), so the
+// exponent is moved by integer instructions where a node's nine values are
+// normal or zero; other nodes take the conversions.
+__device__ __forceinline__ bool widens(float v)  // normal or zero
+{
+    const uint32_t m = __float_as_uint(v) & 0x7fffffffu;
+    return m - 0x00800000u < 0x7f000000u || m == 0;
+}
+__device__ __forceinline__ double widen(float v)
+{
+    const uint32_t u = __float_as_uint(v), m = u & 0x7fffffffu;
+    return __hiloint2double((int)((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(u << 29));
+}
+__device__ __forceinline__ bool narrows(double v)  // [2^-126, 2^127): the rounding cannot overflow; or zero
+{
+    const uint32_t m = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+    return m - 0x38100000u < 0x0fd00000u || (m | (uint32_t)__double2loint(v)) == 0;
+}
+__device__ __forceinline__ float narrow(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), m = hi & 0x7fffffffu;
+    uint32_t r = ((m - 0x38000000u) << 3) | (lo >> 29);
+    const uint32_t rest = lo & 0x1fffffffu;
+    r += rest > 0x10000000u || (rest == 0x10000000u && (r & 1u));  // to nearest, ties to even
+    return __uint_as_float((hi & 0x80000000u) | ((m | lo) == 0 ? 0u : r));
+}
+
 // State export in double: decoded values plus href in double are exact for
 // float and 16-bit storage, so an export / import round trip reproduces the
 // stored bits.
@@ -603,11 +923,29 @@ __global__ void k_get_state(Pops<T, SM> P, double* out, Geom G)
     const int y = blockIdx.y;
     if (x >= G.nx) return;
     const long long n = (long long)G.nx * G.ny, i = (long long)y * G.nx + x;
+    const Around N(x, y, G.nx, G.ny, P.pitch);
+    T v[9];
 #pragma unroll
-    for (int l = 0; l < 9; ++l) {
-        const double v = (double)P.raw(l, P.at(wrapi(y - kCy[l], G.ny), wrapi(x - kCx[l], G.nx)));
-        out[l * n + i] = l == 0 ? v + (double)P.href : v;
+    for (int l = 0; l < 9; ++l) v[l] = P.raw(l, N.at(-cx_of(l), -cy_of(l)));
+    double d[9];
+    if constexpr (std::is_same<T, float>::value) {
+        bool plain = true;
+#pragma unroll
+        for (int l = 0; l < 9; ++l) plain = plain && widens(v[l]);
+        if (plain) {
+#pragma unroll
+            for (int l = 0; l < 9; ++l) d[l] = widen(v[l]);
+        } else {
+#pragma unroll
+            for (int l = 0; l < 9; ++l) d[l] = (double)v[l];
+        }
+    } else {
+#pragma unroll
+        for (int l = 0; l < 9; ++l) d[l] = v[l];
     }
+    d[0] += (double)P.href;
+#pragma unroll
+    for (int l = 0; l < 9; ++l) out[l * n + i] = d[l];
 }
 
 // Post-streaming populations in the compute type, [9][ny][nx] (adjoint input).
@@ -631,12 +969,30 @@ __global__ void k_set_state(Pops<T, SM> P, const double* __restrict__ in, Geom G
     const int y = blockIdx.y;
     if (x >= G.nx) return;
     const long long n = (long long)G.nx * G.ny;
+    const Around N(x, y, G.nx, G.ny, G.nx);
+    double d[9];
 #pragma unroll
-    for (int l = 0; l < 9; ++l) {
-        const long long src = (long long)wrapi(y + kCy[l], G.ny) * G.nx + wrapi(x + kCx[l], G.nx);
-        const double v = in[l * n + src];
-        P.put(l, P.at(y, x), T(l == 0 ? v - (double)P.href : v));
+    for (int l = 0; l < 9; ++l) d[l] = in[l * n + N.at(cx_of(l), cy_of(l))];
+    d[0] -= (double)P.href;
+    T v[9];
+    if constexpr (std::is_same<T, float>::value) {
+        bool plain = true;
+#pragma unroll
+        for (int l = 0; l < 9; ++l) plain = plain && narrows(d[l]);
+        if (plain) {
+#pragma unroll
+            for (int l = 0; l < 9; ++l) v[l] = narrow(d[l]);
+        } else {
+#pragma unroll
+            for (int l = 0; l < 9; ++l) v[l] = (float)d[l];
+        }
+    } else {
+#pragma unroll
+        for (int l = 0; l < 9; ++l) v[l] = d[l];
     }
+    const int o = P.at(y, x);
+#pragma unroll
+    for (int l = 0; l < 9; ++l) P.put(l, o, v[l]);
 }
 
 inline dim3 grid2d(const Geom& G, int bx) { return dim3((G.nx + bx - 1) / bx, G.ny); }
@@ -658,12 +1014,10 @@ cudaError_t moments_t(const StoreDesc& D, const void* f, void* h, void* ux, void
 
 template <typename T, typename SM>
 cudaError_t pf_t(const StoreDesc& D, const void* f, const void* kappa, void* p, void* fx, void* fy,
-                 void* sh, void* sp, const Geom& G, const Consts<T>& C, cudaStream_t st)
+                 const Geom& G, const Consts<T>& C, cudaStream_t st)
 {
-    const auto P = make_pops<T, SM>(f, G, D);
-    k_pf_h<T, SM><<<grid2d(G, 128), 128, 0, st>>>(P, (T*)sh, G);
-    k_pf_p<T><<<grid2d(G, 128), 128, 0, st>>>((const T*)sh, (const T*)kappa, (T*)sp, G, C);
-    k_pf_f<T, SM><<<grid2d(G, 128), 128, 0, st>>>(P, (const T*)sp, (T*)p, (T*)fx, (T*)fy, G, C);
+    const dim3 grid((G.nx + kPfX - 1) / kPfX, (G.ny + kPfY - 1) / kPfY);
+    k_pf<T, SM><<<grid, kPfThreads, 0, st>>>(make_pops<T, SM>(f, G, D), (const T*)kappa, (T*)p, (T*)fx, (T*)fy, G, C);
     return cudaGetLastError();
 }
 
@@ -677,12 +1031,12 @@ cudaError_t mass_t(const StoreDesc& D, const void* f, const Geom& G, double* par
 }
 
 template <typename T, typename SM>
-cudaError_t diag_t(const void* doms, int ndom, int parity, double h_wet, int mx, int my, double* partials, int nb,
-                   double* out, cudaStream_t st)
+cudaError_t diag_t(const void* doms, int ndom, int parity, const void* table, int stride, double h_wet, int mx,
+                   int my, double* partials, int nb, double* out, cudaStream_t st)
 {
-    k_diag_partial<T, SM><<<dim3(nb, ndom), kMassThreads, 0, st>>>((const BatchDomain<T>*)doms, parity, h_wet,
-                                                                  mx, my, partials);
-    k_diag_final<<<ndom, kMassThreads, 0, st>>>(partials, nb, out);
+    k_diag_partial<T, SM><<<dim3(nb, ndom), kMassThreads, 0, st>>>((const BatchDomain<T>*)doms, parity,
+                                                                  (const Trig<T>*)table, stride, h_wet, mx, my, partials);
+    k_diag_final<<<dim3(kDiagOut, ndom), 32, 0, st>>>(partials, nb, out);
     return cudaGetLastError();
 }
 
@@ -763,14 +1117,14 @@ cudaError_t aux_moments(const StoreDesc& D, const void* f, void* h, void* ux, vo
 }
 
 cudaError_t aux_pressure_force(const StoreDesc& D, const void* f, const void* kappa, void* p, void* fx,
-                               void* fy, void* sh, void* sp, const Geom& G, const Consts<float>* C32,
-                               const Consts<double>* C64, cudaStream_t st)
+                               void* fy, const Geom& G, const Consts<float>* C32, const Consts<double>* C64,
+                               cudaStream_t st)
 {
     switch (D.store) {
-        case kStoreF32: return pf_t<float, float>(D, f, kappa, p, fx, fy, sh, sp, G, *C32, st);
-        case kStoreF64: return pf_t<double, double>(D, f, kappa, p, fx, fy, sh, sp, G, *C64, st);
-        case kStoreF16: return pf_t<float, __half>(D, f, kappa, p, fx, fy, sh, sp, G, *C32, st);
-        case kStoreBF16: return pf_t<float, __nv_bfloat16>(D, f, kappa, p, fx, fy, sh, sp, G, *C32, st);
+        case kStoreF32: return pf_t<float, float>(D, f, kappa, p, fx, fy, G, *C32, st);
+        case kStoreF64: return pf_t<double, double>(D, f, kappa, p, fx, fy, G, *C64, st);
+        case kStoreF16: return pf_t<float, __half>(D, f, kappa, p, fx, fy, G, *C32, st);
+        case kStoreBF16: return pf_t<float, __nv_bfloat16>(D, f, kappa, p, fx, fy, G, *C32, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -781,15 +1135,23 @@ cudaError_t aux_mass(const StoreDesc& D, const void* f, const Geom& G, double* p
     TFLBM_DISPATCH(D, (mass_t<T, SM>(D, f, G, partials, nblocks, result, st)))
 }
 
-cudaError_t aux_diag(int store, const void* doms, int ndom, int parity, double h_wet, int mx, int my,
-                     double* partials, int nb, double* out, cudaStream_t st)
+cudaError_t aux_diag_table(bool dbl, const void* doms, int ndom, int stride, void* table, cudaStream_t st)
+{
+    const dim3 grid((stride + 255) / 256, ndom);
+    if (dbl) k_diag_table<double><<<grid, 256, 0, st>>>((const BatchDomain<double>*)doms, (Trig<double>*)table, stride);
+    else k_diag_table<float><<<grid, 256, 0, st>>>((const BatchDomain<float>*)doms, (Trig<float>*)table, stride);
+    return cudaGetLastError();
+}
+
+cudaError_t aux_diag(int store, const void* doms, int ndom, int parity, const void* table, int stride, double h_wet,
+                     int mx, int my, double* partials, int nb, double* out, cudaStream_t st)
 {
     switch (store) {
-        case kStoreF32: return diag_t<float, float>(doms, ndom, parity, h_wet, mx, my, partials, nb, out, st);
-        case kStoreF64: return diag_t<double, double>(doms, ndom, parity, h_wet, mx, my, partials, nb, out, st);
-        case kStoreF16: return diag_t<float, __half>(doms, ndom, parity, h_wet, mx, my, partials, nb, out, st);
+        case kStoreF32: return diag_t<float, float>(doms, ndom, parity, table, stride, h_wet, mx, my, partials, nb, out, st);
+        case kStoreF64: return diag_t<double, double>(doms, ndom, parity, table, stride, h_wet, mx, my, partials, nb, out, st);
+        case kStoreF16: return diag_t<float, __half>(doms, ndom, parity, table, stride, h_wet, mx, my, partials, nb, out, st);
         case kStoreBF16:
-            return diag_t<float, __nv_bfloat16>(doms, ndom, parity, h_wet, mx, my, partials, nb, out, st);
+            return diag_t<float, __nv_bfloat16>(doms, ndom, parity, table, stride, h_wet, mx, my, partials, nb, out, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -49,6 +49,8 @@ struct tf_lbm_batch {
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     double* dpart = nullptr;  // diagnostics partials
+    void* dtrig = nullptr;    // trigonometric tables of the domains, dstride entries each
+    int dstride = 0;
     std::string err;
 };
 
@@ -405,8 +407,11 @@ int tf_lbm_diagnostics(tf_lbm_handle* H, double h_wet, int32_t mode_x, int32_t m
     const int nb = (int)std::min<long long>(kSumBlocks, std::max<long long>(1, n / (256LL * 16)));
     const size_t tab = 256;  // one BatchDomain record, padded
     static_assert(sizeof(BatchDomain<double>) <= 256, "diagnostics record too large");
-    if (!H->dscr) {
-        cudaError_t e = cudaMalloc(&H->dscr, tab + sizeof(double) * diag_partials(1, kSumBlocks));
+    const size_t trig = (tab + sizeof(double) * diag_partials(1, kSumBlocks) + 255) / 256 * 256;
+    const int stride = H->G.nx + H->G.ny;
+    const bool first = !H->dscr;
+    if (first) {
+        cudaError_t e = cudaMalloc(&H->dscr, trig + kDiagTrigBytes * stride);
         if (e != cudaSuccess) {
             H->dscr = nullptr;
             return handle_cuda_fail(H, e, "cudaMalloc diagnostics scratch");
@@ -419,8 +424,11 @@ int tf_lbm_diagnostics(tf_lbm_handle* H, double h_wet, int32_t mode_x, int32_t m
     else d32 = domain_of<float>(H, H->cur, H->kappa);
     cudaError_t e = cudaMemcpyAsync(H->dscr, rec, domain_bytes(H->dbl), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return handle_cuda_fail(H, e, "cudaMemcpyAsync diagnostics record");
-    e = aux_diag(H->desc.store, H->dscr, 1, 0, h_wet, mode_x, mode_y, (double*)((char*)H->dscr + tab), nb,
-                 (double*)out, st);
+    char* table = (char*)H->dscr + trig;
+    if (first && (e = aux_diag_table(H->dbl, H->dscr, 1, stride, table, st)) != cudaSuccess)
+        return handle_cuda_fail(H, e, "diagnostics table kernel");
+    e = aux_diag(H->desc.store, H->dscr, 1, 0, table, stride, h_wet, mode_x, mode_y,
+                 (double*)((char*)H->dscr + tab), nb, (double*)out, st);
     if (e != cudaSuccess) return handle_cuda_fail(H, e, "diagnostics kernels");
     return TF_LBM_OK;
 }
@@ -471,6 +479,7 @@ void tf_lbm_batch_destroy(tf_lbm_batch* B)
     if (B->items) cudaFree(B->items);
     if (B->queue) cudaFree(B->queue);
     if (B->dpart) cudaFree(B->dpart);
+    if (B->dtrig) cudaFree(B->dtrig);
     delete B;
 }
 
@@ -525,8 +534,13 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     if ((e = cudaMemsetAsync(B->queue, 0, 2 * sizeof(int), st)) != cudaSuccess) return bail(bcuda(B, e, "cudaMemsetAsync"));
     const size_t dp = diag_partials(count, kDiagBlocksPerDomain);
     if ((e = cudaMalloc(&B->dpart, dp * sizeof(double))) != cudaSuccess) return bail(bcuda(B, e, "cudaMalloc diagnostics"));
+    for (auto* H : B->hs) B->dstride = std::max(B->dstride, H->G.nx + H->G.ny);
+    if ((e = cudaMalloc(&B->dtrig, kDiagTrigBytes * B->dstride * count)) != cudaSuccess)
+        return bail(bcuda(B, e, "cudaMalloc diagnostics table"));
     int rc = write_table(B, st);
     if (rc) return bail(rc);
+    if ((e = aux_diag_table(B->dbl, B->doms, count, B->dstride, B->dtrig, st)) != cudaSuccess)
+        return bail(bcuda(B, e, "diagnostics table kernel"));
 
     // default shape: the two-column kernel where it applies and every tau is
     // 1 (as for a single handle), 64 columns per CTA for 16-bit storage and
@@ -710,8 +724,8 @@ int tf_lbm_batch_diagnostics(tf_lbm_batch* B, double h_wet, int32_t mode_x, int3
     cudaStream_t st = (cudaStream_t)stream;
     int rc = sync_table(B, st);
     if (rc) return rc;
-    BCK(B, aux_diag(B->store, B->doms, (int)B->hs.size(), B->phase, h_wet, mode_x, mode_y, B->dpart,
-                    kDiagBlocksPerDomain, (double*)out, st),
+    BCK(B, aux_diag(B->store, B->doms, (int)B->hs.size(), B->phase, B->dtrig, B->dstride, h_wet, mode_x, mode_y,
+                    B->dpart, kDiagBlocksPerDomain, (double*)out, st),
         "diagnostics kernels");
     return TF_LBM_OK;
 }

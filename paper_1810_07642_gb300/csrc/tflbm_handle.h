@@ -30,7 +30,6 @@ struct tf_lbm_handle {
     int* flag = nullptr;
     int* status = nullptr;     // device word kernels set (kStatusTimeout)
     int wait_limit = kWaitLimit;  // polls of one mbarrier before a bulk-copy kernel gives up
-    void* diag = nullptr;      // 2 * ny * nx scratch for tf_lbm_pressure_force (lazy)
     int64_t time = 0;
     Shape shape{128, 64, kPipeLdg};  // replaced by the occupancy-derived default in tf_lbm_init
     int graph_chunk = 0;
@@ -38,7 +37,7 @@ struct tf_lbm_handle {
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     std::string err;
     void* adj = nullptr;       // adjoint scratch (lazy): 10 fields of the compute type
-    void* dscr = nullptr;      // diagnostics scratch (lazy): one BatchDomain entry + partial sums
+    void* dscr = nullptr;      // diagnostics scratch (lazy): one BatchDomain entry + partial sums + trig table
     void* tscr = nullptr;      // term-norm scratch (lazy): 5 fields + partial sums
 };
 

@@ -178,8 +178,8 @@ cudaError_t aux_init(const StoreDesc& D, void* f, const void* h0, const Geom& G,
 cudaError_t aux_moments(const StoreDesc& D, const void* f, void* h, void* ux, void* uy, const Geom& G,
                         cudaStream_t st);
 cudaError_t aux_pressure_force(const StoreDesc& D, const void* f, const void* kappa, void* p, void* fx,
-                               void* fy, void* sh, void* sp, const Geom& G, const Consts<float>* C32,
-                               const Consts<double>* C64, cudaStream_t st);
+                               void* fy, const Geom& G, const Consts<float>* C32, const Consts<double>* C64,
+                               cudaStream_t st);
 cudaError_t aux_mass(const StoreDesc& D, const void* f, const Geom& G, double* partials, int nblocks,
                      double* result, cudaStream_t st);
 cudaError_t aux_check(const StoreDesc& D, const void* f, const Geom& G, int* flag, cudaStream_t st);
@@ -189,12 +189,15 @@ cudaError_t aux_set_state(const StoreDesc& D, void* f, const double* in, const G
 // Film diagnostics of each domain of a BatchDomain table (buffer `parity`):
 // out[d * kDiagOut ..] = the fields of tf_lbm_diag (wetted nodes: h > h_wet;
 // Fourier sums at the integer modes (mx, my)).  partials holds
-// diag_partials(ndom, nb) doubles.
+// diag_partials(ndom, nb) doubles; table is what aux_diag_table wrote for the
+// same domains: stride entries a domain, stride >= its nx + ny.
 constexpr int kDiagSums = 11;
 constexpr int kDiagOut = kDiagSums + 1;
 inline size_t diag_partials(int ndom, int nb) { return (size_t)ndom * nb * (2 * kDiagSums + 1); }
-cudaError_t aux_diag(int store, const void* doms, int ndom, int parity, double h_wet, int mx, int my,
-                     double* partials, int nb, double* out, cudaStream_t st);
+constexpr size_t kDiagTrigBytes = 16;  // one table entry
+cudaError_t aux_diag_table(bool dbl, const void* doms, int ndom, int stride, void* table, cudaStream_t st);
+cudaError_t aux_diag(int store, const void* doms, int ndom, int parity, const void* table, int stride, double h_wet,
+                     int mx, int my, double* partials, int nb, double* out, cudaStream_t st);
 // L2 norms (appendix, Eq. magnitude) of the x-components of the pressure,
 // friction and dissipation terms into out[0..2]; scratch holds 5 fields of
 // the compute type, partials 6 * nb doubles.

@@ -130,7 +130,10 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            tf_lbm_set_launch gives ceil(ny / rows) bands;
  *   graph_chunk: steps per captured CUDA graph in tf_lbm_step (0 = none,
  *            otherwise an even number >= 2);
- *   pipeline: 3 = every thread owns two adjacent columns, loads aligned
+ *   pipeline: 4 = every CTA owns one tile (16 x 8 nodes for block_x 64, 16 x
+ *            16 for 128, 32 x 16 for 256; rows is not used) and runs the
+ *            step's phases over all of it (any nx, ny and dtype);
+ *            3 = every thread owns two adjacent columns, loads aligned
  *            pairs one (FP32) or two (16-bit) rows ahead, takes the values
  *            that cross a pair boundary from the neighbouring lane and
  *            computes both nodes with paired FP32 instructions (nx even, not
@@ -142,6 +145,10 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            asynchronous copies, two rows ahead (TF_LBM_F32 and TF_LBM_F64
  *            only); 0 = row segments streamed into shared memory by bulk
  *            copies four rows ahead (needs nx a multiple of 8, >= 16).
+ * On lattices of up to 1.5 x 2^20 nodes, and for TF_LBM_F64 on all, the shape
+ * chosen by tf_lbm_init runs tiles in place of the bands that its fields
+ * describe, and so does the one chosen by tf_lbm_tune where tiles were the
+ * fastest; passing the fields to tf_lbm_set_launch gives the bands.
  * Results do not depend on rows or graph_chunk; the pipelines agree to
  * rounding. */
 typedef struct tf_lbm_launch {
@@ -252,11 +259,12 @@ void tf_lbm_tape_destroy(tf_lbm_tape* tape);
  * `stream`.  Candidates: block_x in {64, 128, 256}, every pipeline that
  * applies, and band counts of one, two and three waves of resident CTAs
  * (both balanced bands filling the waves exactly and their rounded-up band
- * heights) and band heights of 2 to 256 rows.  The state is copied aside first (one population
+ * heights) and band heights of 2 to 256 rows, then tiles of every block_x in
+ * place of the fastest of these.  The state is copied aside first (one population
  * buffer of device memory, freed before return) and put back after, so f
  * and tf_lbm_time are as before the call.  The graph chunk is kept.
  * Synchronises `stream`.  best (host, may be NULL) receives the shape now in
- * use. */
+ * use as tf_lbm_get_launch reports it (see tf_lbm_launch on tiles). */
 int tf_lbm_tune(tf_lbm_handle* H, int32_t trial_steps, tf_lbm_launch* best, void* stream);
 
 /* -------------------------------------------------------- diagnostics

@@ -14,6 +14,15 @@
 
 using namespace tflbm;
 
+namespace tflbm {
+int sm_count()
+{
+    int sms = 152, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+}  // namespace tflbm
+
 namespace {
 
 thread_local std::string g_init_err;
@@ -106,7 +115,46 @@ int store_of(int dtype)
     }
 }
 
-// Default launch shape: the two-column kernel at tau = 1 where it applies
+// The tile kernel's block_x for a lattice (tile_of): the shape with the least
+// work on the busiest SM, counting a node's pull as a third of its cost and its
+// pressure as a fifth (the halos repeat those) and 40 nodes' worth of fixed
+// latency a tile.  In FP64 the arithmetic units are the bound and halo work
+// counts in full, so tiles are as large as keeps every SM busy.  Measured, one
+// box, us a step with block_x 64 / 128 / 256: FP32 128^2 3.0 / 3.1 / 3.5, 384^2
+// 5.2 / 5.1 / 4.4, 1024^2 19.4 / 19.3 / 16.3; FP64 64^2 7.5 / 11.5 / 20.2, 250 x
+// 190 38 / 20.7 / 38, 768^2 158 / 156 / 151.
+int tile_block_x(int store, int nx, int ny, int sms)
+{
+    auto tiles = [&](int bx) {
+        const TileShape t = tile_of(bx);
+        return (long long)((nx + t.tx - 1) / t.tx) * ((ny + t.ty - 1) / t.ty);
+    };
+    if (store == kStoreF64) return tiles(64) <= sms ? 64 : (tiles(256) >= 7LL * sms ? 256 : 128);
+    int best = 64;
+    double least = 0;
+    for (int bx : {64, 128, 256}) {
+        const TileShape t = tile_of(bx);
+        const double work = 40 + 0.45 * t.tx * t.ty + 0.35 * (t.tx + 4) * (t.ty + 4) + 0.2 * (t.tx + 2) * (t.ty + 2);
+        const double cost = (double)((tiles(bx) + sms - 1) / sms) * work;
+        if (bx == 64 || cost < least) {
+            best = bx;
+            least = cost;
+        }
+    }
+    return best;
+}
+
+// Lattices up to this many nodes run the tile kernel with an FP32 compute type
+// (FP64: all).  Above it the marches win: they pull a node 1.3 times, not 1.4,
+// and prefetch from HBM.  One box, us a step, tile against march: 1024^2 FP32
+// 16.3 / 34.1 (18.5 with 4-row bands), FP16 18.4 / 32.2; 1448^2 FP32 36.7 /
+// 38.7, FP16 40.0 / 36.1, FP32 at tau = 0.8 39.8 / 37.1; 2048^2 FP32 65 / 52.7;
+// FP64 2048^2 1014 / 1101.
+constexpr long long kTileNodes = 3LL << 19;
+
+// Default launch shape: tiles on lattices that L2 holds.  The other fields
+// describe the march that a larger lattice would run, and that the caller gets
+// back by setting them: the two-column kernel at tau = 1 where it applies
 // (CTAs 64 columns wide for 16-bit storage, 128 for FP32), else the one-column kernel
 // with CTAs 128 columns wide (64 on lattices narrower than 1024), and
 // a band height that makes the grid one full wave of
@@ -122,14 +170,12 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     // (the two-column kernel's pulled-population ring costs resident warps)
     const int store = store_of(p.dtype);
     const bool om1 = p.tau == 1.0;
+    if (store == kStoreF64 || (long long)G.nx * G.ny <= kTileNodes) s.tile = tile_block_x(store, G.nx, G.ny, sm_count());
     const bool narrow = store == kStoreF16 || store == kStoreBF16;
     const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     s.block_x = pair ? (narrow ? 64 : 128) : (G.nx >= 1024 ? 128 : 64);
     const int strips = (G.nx + s.block_x - 5) / (s.block_x - 4);  // CTAs overlap by 4 columns
-    int sms = 152;
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     // otherwise per-thread loads: measured faster than the bulk-copy pipeline
     // on GB300 once loads are prefetched a row ahead
     s.pipeline = pair ? kPipePair : kPipeLdg;
@@ -158,12 +204,6 @@ int handle_check_dev_ptr(tf_lbm_handle* H, const void* ptr, const char* name, bo
     return check_dev_ptr(H, ptr, name, allow_null);
 }
 void handle_drop_graphs(tf_lbm_handle* H) { drop_graphs(H); }
-int sm_count()
-{
-    int sms = 152, dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
-}
 int handle_cuda_fail(tf_lbm_handle* H, cudaError_t e, const char* what) { return cuda_fail(H, e, what); }
 
 template <typename T>
@@ -457,10 +497,10 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
     if (in->graph_chunk < 0 || (in->graph_chunk % 2) != 0 || in->graph_chunk > 4096)
         return fail(H, TF_LBM_ERR_ARG, "graph_chunk must be 0 or an even number <= 4096");
     if (in->pipeline != kPipeTma && in->pipeline != kPipeLdg && in->pipeline != kPipeAsync &&
-        in->pipeline != kPipePair)
+        in->pipeline != kPipePair && in->pipeline != kPipeTile)
         return fail(H, TF_LBM_ERR_ARG,
-                    "pipeline must be 0 (bulk copies), 1 (per-thread loads), 2 (per-thread async copies) "
-                    "or 3 (two columns per thread)");
+                    "pipeline must be 0 (bulk copies), 1 (per-thread loads), 2 (per-thread async copies), "
+                    "3 (two columns per thread) or 4 (tiles)");
     if (in->pipeline == kPipePair && !pair_pipeline_ok(H->G.nx, H->desc.store))
         return fail(H, TF_LBM_ERR_ARG, "the two-column pipeline needs nx even and an FP32 compute type");
     if (in->pipeline == kPipeAsync && H->msize != H->esize)
@@ -472,6 +512,7 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
     H->shape.block_x = bx;
     H->shape.rows = in->rows;
     H->shape.bands = 0;
+    H->shape.tile = in->pipeline == kPipeTile ? bx : 0;
     H->graph_chunk = in->graph_chunk;
     return TF_LBM_OK;
 }

@@ -19,6 +19,13 @@ constexpr int kPipeTma = 0;
 constexpr int kPipeLdg = 1;
 constexpr int kPipeAsync = 2;  // per-thread cp.async staging (full-width storage only)
 constexpr int kPipePair = 3;   // two columns per thread (FP32 compute type, nx even)
+constexpr int kPipeTile = 4;   // one tile per CTA (any size)
+// Tile of the tile kernel for a block_x: half its nodes (one thread per two
+// nodes with an FP32 compute type).
+struct TileShape {
+    int tx, ty;
+};
+constexpr TileShape tile_of(int block_x) { return block_x == 64 ? TileShape{16, 8} : TileShape{block_x / 8, 16}; }
 inline bool tma_pipeline_ok(int nx) { return nx % 8 == 0 && nx >= 16; }
 inline bool pair_pipeline_ok(int nx, int store) { return nx % 2 == 0 && store != 1 /* kStoreF64 */; }
 
@@ -84,8 +91,9 @@ struct Consts {
 struct Shape {
     int block_x;    // 64, 128, 256
     int rows;       // rows per CTA (band height)
-    int pipeline;   // kPipeTma, kPipeLdg, kPipeAsync or kPipePair
+    int pipeline;   // kPipeTma, kPipeLdg, kPipeAsync, kPipePair, or kPipeTile (then tile == block_x)
     int bands = 0;  // balanced bands per launch; 0: ny / rows rounded up
+    int tile = 0;   // run the tile kernel with this block_x (tile_of) instead of a march; 0: march
 };
 
 // Bands of one launch of a step kernel for a shape (at most 65535, the grid's
@@ -118,6 +126,9 @@ cudaError_t pair_step_f16(int block_x, const void* fin, void* fout, const void* 
                           const Consts<float>& C, int bands, cudaStream_t st);
 cudaError_t pair_step_bf16(int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
                            const Consts<float>& C, int bands, cudaStream_t st);
+// The tile step (tile_*.cu).
+cudaError_t launch_tile(int store, int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
+                        const Consts<float>* C32, const Consts<double>* C64, cudaStream_t st);
 int pair_blocks_per_sm_f32(int block_x, bool omega1, bool kfield);
 int pair_blocks_per_sm_f16(int block_x, bool omega1, bool kfield);
 int pair_blocks_per_sm_bf16(int block_x, bool omega1, bool kfield);

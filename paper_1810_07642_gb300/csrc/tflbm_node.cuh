@@ -1,0 +1,301 @@
+// Node arithmetic of the fused step in the storage units of
+// tflbm_step2.cuh: film pressure, force and collision (Section II of Zitz et
+// al., arXiv:1810.07642), written once for X = float2 (two nodes on
+// Blackwell's paired FP32 instructions) and X = double (one node).  The
+// two-column march (tflbm_step2.cuh) and the tile kernel (tflbm_tile.cuh) use
+// it; where a value comes from and where a result goes is theirs.
+#pragma once
+#include "tflbm_step.cuh"
+
+namespace tflbm {
+
+// ---- paired FP32 arithmetic (one instruction for both columns) ------------
+__device__ __forceinline__ float2 pk(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+__device__ __forceinline__ float2 pneg(float2 a) { return make_float2(-a.x, -a.y); }
+// 1 / a by CUDA's fast single-precision division (within 2 ulp)
+__device__ __forceinline__ float2 prcp(float2 a) { return make_float2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y)); }
+__device__ __forceinline__ float2 pfdisj(float2 r, int n, int m) { return make_float2(fdisj(r.x, n, m), fdisj(r.y, n, m)); }
+
+// the same names for one FP64 node
+__device__ __forceinline__ double padd(double a, double b) { return a + b; }
+__device__ __forceinline__ double psub(double a, double b) { return a - b; }
+__device__ __forceinline__ double pmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double pfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double pneg(double a) { return -a; }
+__device__ __forceinline__ double prcp(double a) { return 1.0 / a; }
+__device__ __forceinline__ double pfdisj(double r, int n, int m) { return fdisj(r, n, m); }
+__device__ __forceinline__ void ptwo_sum(double a, double b, double& s, double& e) { two_sum(a, b, s, e); }
+
+// X: the nodes of one thread; S: their scalar type
+template <typename X> struct Lanes;
+template <> struct Lanes<float2> {
+    using S = float;
+    static constexpr int N = 2;
+    static __device__ __forceinline__ float2 all(float a) { return make_float2(a, a); }
+};
+template <> struct Lanes<double> {
+    using S = double;
+    static constexpr int N = 1;
+    static __device__ __forceinline__ double all(double a) { return a; }
+};
+
+// Error-free TwoSum on both lanes: a + b = s + e exactly.
+__device__ __forceinline__ void ptwo_sum(float2 a, float2 b, float2& s, float2& e)
+{
+    s = padd(a, b);
+    const float2 bb = psub(s, a);
+    e = padd(psub(a, psub(s, bb)), psub(b, bb));
+}
+
+// ---- pair storage of the moving populations --------------------------------
+// V is one aligned pair of stored values; dec gives them as floats in storage
+// units (exact), enc rounds two floats to the storage type, dec1 converts one
+// stored element.
+template <typename SM> struct PairIO;
+template <> struct PairIO<float> {
+    using V = float2;
+    static __device__ __forceinline__ float2 dec(float2 q) { return q; }
+    static __device__ __forceinline__ float2 enc(float2 v) { return v; }
+    static __device__ __forceinline__ float dec1(float q) { return q; }
+};
+template <> struct PairIO<double> {
+    using V = double;
+    static __device__ __forceinline__ double dec(double q) { return q; }
+    static __device__ __forceinline__ double enc(double v) { return v; }
+    static __device__ __forceinline__ double dec1(double q) { return q; }
+};
+template <> struct PairIO<__half> {
+    using V = __half2;
+    static __device__ __forceinline__ float2 dec(__half2 q) { return __half22float2(q); }
+    static __device__ __forceinline__ __half2 enc(float2 v) { return __float22half2_rn(v); }
+    static __device__ __forceinline__ float dec1(__half q) { return __half2float(q); }
+};
+template <> struct PairIO<__nv_bfloat16> {
+    using V = __nv_bfloat162;
+    static __device__ __forceinline__ float2 dec(__nv_bfloat162 q) { return __bfloat1622float2(q); }
+    static __device__ __forceinline__ __nv_bfloat162 enc(float2 v) { return __float22bfloat162_rn(v); }
+    static __device__ __forceinline__ float dec1(__nv_bfloat16 q) { return __bfloat162float(q); }
+};
+
+template <typename V> __device__ __forceinline__ uint32_t bits(V v)
+{
+    static_assert(sizeof(V) == 4, "16-bit pairs only");
+    uint32_t u;
+    memcpy(&u, &v, 4);
+    return u;
+}
+template <typename V> __device__ __forceinline__ V from_bits(uint32_t u)
+{
+    V v;
+    memcpy(&v, &u, 4);
+    return v;
+}
+// acc += the two stored values of q, each added to its lane in FP32 by the
+// mixed-precision add of sm_100 and later (16-bit operand, FP32 sum, one
+// rounding)
+template <typename SM> __device__ __forceinline__ void mixed_add(float2& acc, typename PairIO<SM>::V q);
+template <> __device__ __forceinline__ void mixed_add<__half>(float2& acc, __half2 q)
+{
+    unsigned short lo, hi;
+    asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(bits(q)));
+    asm("add.rn.f32.f16 %0, %1, %0;" : "+f"(acc.x) : "h"(lo));
+    asm("add.rn.f32.f16 %0, %1, %0;" : "+f"(acc.y) : "h"(hi));
+}
+template <> __device__ __forceinline__ void mixed_add<__nv_bfloat16>(float2& acc, __nv_bfloat162 q)
+{
+    unsigned short lo, hi;
+    asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(bits(q)));
+    asm("add.rn.f32.bf16 %0, %1, %0;" : "+f"(acc.x) : "h"(lo));
+    asm("add.rn.f32.bf16 %0, %1, %0;" : "+f"(acc.y) : "h"(hi));
+}
+
+// A 3 x 3 stencil window: for each of the rows n (+y), c, s (-y) the values
+// at the thread's own columns and the ones to the left and right of them.
+template <typename X>
+struct Win {
+    X n0, nL, nR, c0, cL, cR, s0, sL, sR;
+};
+
+// ---------------------------------------------------------------------------
+// Node arithmetic.
+
+// Film pressure (Eq. pfilm with Eq. disjoiningP) from the h window; writes 1/h
+// to ih.
+template <typename X>
+__device__ __forceinline__ X node_pressure(const Win<X>& H, X kap, bool disj, const Consts<typename Lanes<X>::S>& C,
+                                           X& ih)
+{
+    using S = typename Lanes<X>::S;
+    auto pk = [](S a) { return Lanes<X>::all(a); };
+    // Eq. (n_laplace): axis neighbours left + right + up + down, diagonal the four corners
+    const X axis = padd(padd(H.cL, H.cR), padd(H.n0, H.s0));
+    const X diag = padd(padd(H.nL, H.nR), padd(H.sL, H.sR));
+    X lap = pmul(pfma(pk(S(4.0)), axis, pfma(pk(-S(20.0)), H.c0, diag)), pk(S(1.0 / 6.0)));
+    const X h = padd(H.c0, pk(C.href));
+    ih = prcp(h);
+    if (disj) {
+        const X r = pmul(pk(C.hstar), ih);
+        X fd;
+        if (C.n_exp == 3 && C.m_exp == 2) fd = pmul(pmul(r, r), psub(r, pk(S(1.0))));
+        else fd = pfdisj(r, C.n_exp, C.m_exp);
+        lap = pfma(pmul(pk(C.pi_sgn), kap), fd, lap);
+    }
+    return pmul(pk(-C.gamma), lap);
+}
+
+// Force and collision (the arithmetic of collide_store on every lane, in
+// storage units).  P: the p window (n = row o+1, s = row o-1); f: the pulled
+// moving populations in storage units, fstride apart (omega != 1 only).  The
+// post-collision populations go to store(f_0 - href, q[8]), q as stored.
+template <typename SM, bool OMEGA1, typename X, typename Store>
+__device__ __forceinline__ void node_collide(const Win<X>& P, X dh, X ih, X jx, X jy, X er, const X* f, int fstride,
+                                             const Consts<typename Lanes<X>::S>& C, Store store)
+{
+    using S = typename Lanes<X>::S;
+    auto pk = [](S a) { return Lanes<X>::all(a); };
+    using IO = PairIO<SM>;
+    using V = typename IO::V;
+    constexpr bool NARROW = sizeof(SM) == 2;
+    // storage scale (1 for full-width storage, a compile-time constant there)
+    const S ms = NARROW ? C.mscale : S(1);
+    // Eq. (derivative): grad p = 3 sum_l w_l c_l p(x + c_l)
+    const X gpx = pfma(psub(P.cR, P.cL), pk(S(1.0 / 3.0)),
+                       pmul(padd(psub(P.nR, P.nL), psub(P.sR, P.sL)), pk(S(1.0 / 12.0))));
+    const X gpy = pfma(psub(P.n0, P.s0), pk(S(1.0 / 3.0)),
+                       pmul(padd(psub(P.nR, P.sR), psub(P.nL, P.sL)), pk(S(1.0 / 12.0))));
+    const X h = padd(dh, pk(C.href));
+    // Eqs. (force), (forcefric), (alphafric): nu alpha u = 6 nu j / (2h^2 + 6 delta h + 3 delta^2)
+    const X den = pfma(h, pfma(pk(S(2.0)), h, pk(S(6.0) * C.delta)), pk(S(3.0) * C.delta * C.delta));
+    const X fr = pmul(pk(C.nu6), prcp(den));
+    // Eq. (LBE) as printed: u = j/h.  Second-order forcing (C.forcing):
+    // u (h + nu alpha/2) = j + F'/2 and the equilibria use h u for j (see
+    // collide_store)
+    X Fx, Fy, ux, uy, ex, ey;
+    if (C.forcing) {
+        const X fpx = pmul(h, psub(pk(C.gx), gpx)), fpy = pmul(h, psub(pk(C.gy), gpy));
+        const X d = pfma(pk(S(0.5)), fr, pk(S(1.0)));
+        const X q = pmul(ih, prcp(d));
+        ux = pmul(pfma(pk(S(0.5)), fpx, jx), q);
+        uy = pmul(pfma(pk(S(0.5)), fpy, jy), q);
+        ex = pmul(h, ux);
+        ey = pmul(h, uy);
+        Fx = psub(fpx, pmul(fr, ex));
+        Fy = psub(fpy, pmul(fr, ey));
+    } else {
+        Fx = psub(pmul(h, psub(pk(C.gx), gpx)), pmul(fr, jx));
+        Fy = psub(pmul(h, psub(pk(C.gy), gpy)), pmul(fr, jy));
+        ux = pmul(jx, ih);
+        uy = pmul(jy, ih);
+        ex = jx;
+        ey = jy;
+    }
+    // Eq. (equilibria) with e^2 = 1 as S +- D per opposite pair, source
+    // 3 w_l c_l . F; in storage units S' = (S - R_l) ms, D' = D ms.
+    // A6 = 6 A = h (g h - u^2).
+    const X A6 = pmul(h, psub(pmul(pk(C.g), h), pfma(ux, ux, pmul(uy, uy))));
+    const X Aa = NARROW ? pfma(A6, pk(ms * S(1.0 / 6.0)), pk(C.nr_axis)) : pmul(A6, pk(S(1.0 / 6.0)));
+    const X Ad = NARROW ? pfma(A6, pk(ms * S(1.0 / 24.0)), pk(C.nr_diag)) : pmul(A6, pk(S(1.0 / 24.0)));
+    X Sx = pfma(pmul(ex, pk(S(0.5) * ms)), ux, Aa);
+    X Sy = pfma(pmul(ey, pk(S(0.5) * ms)), uy, Aa);
+    const X a = padd(ux, uy), b = psub(uy, ux);
+    const X h8 = pmul(h, pk(S(0.125) * ms));
+    X Sa = pfma(pmul(h8, a), a, Ad);
+    X Sb = pfma(pmul(h8, b), b, Ad);
+    // second-order source: odd part scaled by (1 - omega/2), even part T
+    X Tx = pk(S(0.0)), Ty = pk(S(0.0)), Ta = pk(S(0.0)), Tb = pk(S(0.0));
+    if (C.forcing) {
+        const X ks = pk(S(1.0) - S(0.5) * C.omega);
+        Fx = pmul(Fx, ks);
+        Fy = pmul(Fy, ks);
+        const X uF3 = pmul(pfma(ux, Fx, pmul(uy, Fy)), pk(ms * S(1.0 / 3.0)));
+        Tx = pfma(pmul(ux, Fx), pk(ms), pneg(uF3));
+        Ty = pfma(pmul(uy, Fy), pk(ms), pneg(uF3));
+        Ta = pmul(pfma(pmul(a, padd(Fx, Fy)), pk(ms), pneg(uF3)), pk(S(0.25)));
+        Tb = pmul(pfma(pmul(b, psub(Fy, Fx)), pk(ms), pneg(uF3)), pk(S(0.25)));
+        if constexpr (OMEGA1) {
+            Sx = padd(Sx, Tx);
+            Sy = padd(Sy, Ty);
+            Sa = padd(Sa, Ta);
+            Sb = padd(Sb, Tb);
+        }
+    }
+    const X m3 = pk(ms * S(1.0 / 3.0)), m12 = pk(ms * S(1.0 / 12.0));
+    X o1, o2, o3, o4, o5, o6, o7, o8;
+    if constexpr (OMEGA1) {
+        const X Gx = padd(ex, Fx), Gy = padd(ey, Fy);
+        const X Dx = pmul(Gx, m3), Dy = pmul(Gy, m3);
+        const X Da = pmul(padd(Gx, Gy), m12), Db = pmul(psub(Gy, Gx), m12);
+        o1 = padd(Sx, Dx); o5 = psub(Sx, Dx);
+        o3 = padd(Sy, Dy); o7 = psub(Sy, Dy);
+        o2 = padd(Sa, Da); o6 = psub(Sa, Da);
+        o4 = padd(Sb, Db); o8 = psub(Sb, Db);
+    } else {
+        // (1 - omega)(f_l - R_l) + omega (f_eq_l - R_l) + source, in storage units
+        const X w = pk(C.omega), m = pk(S(1.0) - C.omega);
+        const X Dx = pmul(ex, m3), Dy = pmul(ey, m3);
+        const X Da = pmul(padd(ex, ey), m12), Db = pmul(psub(ey, ex), m12);
+        const X Qx = pmul(Fx, m3), Qy = pmul(Fy, m3);
+        const X Qa = pmul(padd(Fx, Fy), m12), Qb = pmul(psub(Fy, Fx), m12);
+        o1 = padd(pfma(m, f[0 * fstride], pmul(w, padd(Sx, Dx))), padd(Tx, Qx));
+        o5 = padd(pfma(m, f[4 * fstride], pmul(w, psub(Sx, Dx))), psub(Tx, Qx));
+        o3 = padd(pfma(m, f[2 * fstride], pmul(w, padd(Sy, Dy))), padd(Ty, Qy));
+        o7 = padd(pfma(m, f[6 * fstride], pmul(w, psub(Sy, Dy))), psub(Ty, Qy));
+        o2 = padd(pfma(m, f[1 * fstride], pmul(w, padd(Sa, Da))), padd(Ta, Qa));
+        o6 = padd(pfma(m, f[5 * fstride], pmul(w, psub(Sa, Da))), psub(Ta, Qa));
+        o4 = padd(pfma(m, f[3 * fstride], pmul(w, padd(Sb, Db))), padd(Tb, Qb));
+        o8 = padd(pfma(m, f[7 * fstride], pmul(w, psub(Sb, Db))), psub(Tb, Qb));
+    }
+    // stored rest population f*_0 - href = (h - href) - sum_{l>0} f*_l, with
+    // the exact residuals folded back as in collide_store
+    if constexpr (!NARROW) {
+        const X osum = padd(padd(padd(o1, o5), padd(o3, o7)), padd(padd(o2, o6), padd(o4, o8)));
+        X o0v, e2;
+        ptwo_sum(dh, pneg(osum), o0v, e2);
+        const X half_r = pmul(padd(er, e2), pk(S(0.5)));
+        o1 = padd(o1, half_r);
+        o5 = padd(o5, half_r);
+        const V q[8] = {o1, o2, o3, o4, o5, o6, o7, o8};
+        store(o0v, q);
+    } else {
+        const V q2 = IO::enc(o2), q3 = IO::enc(o3), q4 = IO::enc(o4), q5 = IO::enc(o5);
+        const V q6 = IO::enc(o6), q7 = IO::enc(o7), q8 = IO::enc(o8), q1r = IO::enc(o1);
+        // what the readers reconstruct of l = 2..8 (storage units; each
+        // stored value enters the FP32 sum by a mixed-precision add, which
+        // takes the 16-bit operand as it is: one instruction per value
+        // instead of a conversion and half a paired add)
+        float2 rest = IO::dec(q2);
+        mixed_add<SM>(rest, q3);
+        mixed_add<SM>(rest, q4);
+        mixed_add<SM>(rest, q5);
+        mixed_add<SM>(rest, q6);
+        mixed_add<SM>(rest, q7);
+        mixed_add<SM>(rest, q8);
+        float2 rest1 = rest;
+        mixed_add<SM>(rest1, q1r);
+        // the moving populations' total with f_1 unrounded and rounded
+        const float2 osum = pfma(padd(rest, o1), pk(C.minv), pk(C.r_sum));
+        const float2 osr = pfma(rest1, pk(C.minv), pk(C.r_sum));
+        // the last residual goes to the finer of the two roundings: the 16-bit
+        // one of f_1 - R or the FP32 one of f_0 - href (see collide_store)
+        constexpr float kRatio = std::is_same<SM, __half>::value ? 8192.0f : 65536.0f;
+        const float kr = kRatio * C.minv;  // |f_1 - R| = |o1| / ms
+        const bool lx = fabsf(o1.x) * kr < fabsf(dh.x - osum.x);
+        const bool ly = fabsf(o1.y) * kr < fabsf(dh.y - osum.y);
+        const float2 os = make_float2(lx ? osum.x : osr.x, ly ? osum.y : osr.y);
+        float2 o0v, e2, o0n, e3;
+        ptwo_sum(dh, make_float2(-os.x, -os.y), o0v, e2);
+        ptwo_sum(o0v, padd(er, e2), o0n, e3);
+        const V q1l = IO::enc(pfma(e3, pk(ms), o1));
+        const uint32_t mask = (lx ? 0x0000ffffu : 0u) | (ly ? 0xffff0000u : 0u);
+        const V q1 = from_bits<V>((bits(q1l) & mask) | (bits(q1r) & ~mask));
+        const V q[8] = {q1, q2, q3, q4, q5, q6, q7, q8};
+        store(o0n, q);
+    }
+}
+
+}  // namespace tflbm

@@ -42,280 +42,22 @@
 // (pairs never straddle the periodic seam); compute type FP32, storage FP32,
 // FP16 or BF16.
 #pragma once
-#include "tflbm_step.cuh"
+#include "tflbm_node.cuh"
 
 namespace tflbm {
 
-// ---- paired FP32 arithmetic (one instruction for both columns) ------------
-__device__ __forceinline__ float2 pk(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
-// Error-free TwoSum on both lanes: a + b = s + e exactly.
-__device__ __forceinline__ void ptwo_sum(float2 a, float2 b, float2& s, float2& e)
-{
-    s = padd(a, b);
-    const float2 bb = psub(s, a);
-    e = padd(psub(a, psub(s, bb)), psub(b, bb));
-}
-
-// ---- pair storage of the moving populations --------------------------------
-// V is one aligned pair of stored values; dec gives them as floats in storage
-// units (exact), enc rounds two floats to the storage type, dec1 converts one
-// stored element.
-template <typename SM> struct PairIO;
-template <> struct PairIO<float> {
-    using V = float2;
-    static __device__ __forceinline__ float2 dec(float2 q) { return q; }
-    static __device__ __forceinline__ float2 enc(float2 v) { return v; }
-    static __device__ __forceinline__ float dec1(float q) { return q; }
-};
-template <> struct PairIO<__half> {
-    using V = __half2;
-    static __device__ __forceinline__ float2 dec(__half2 q) { return __half22float2(q); }
-    static __device__ __forceinline__ __half2 enc(float2 v) { return __float22half2_rn(v); }
-    static __device__ __forceinline__ float dec1(__half q) { return __half2float(q); }
-};
-template <> struct PairIO<__nv_bfloat16> {
-    using V = __nv_bfloat162;
-    static __device__ __forceinline__ float2 dec(__nv_bfloat162 q) { return __bfloat1622float2(q); }
-    static __device__ __forceinline__ __nv_bfloat162 enc(float2 v) { return __float22bfloat162_rn(v); }
-    static __device__ __forceinline__ float dec1(__nv_bfloat16 q) { return __bfloat162float(q); }
-};
-
 template <typename V> __device__ __forceinline__ V ldpair(const V* p) { return __ldg(p); }
-template <typename V> __device__ __forceinline__ uint32_t bits(V v)
-{
-    static_assert(sizeof(V) == 4, "16-bit pairs only");
-    uint32_t u;
-    memcpy(&u, &v, 4);
-    return u;
-}
-template <typename V> __device__ __forceinline__ V from_bits(uint32_t u)
-{
-    V v;
-    memcpy(&v, &u, 4);
-    return v;
-}
 __device__ __forceinline__ float2 lds2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 
-// acc += the two stored values of q, each added to its lane in FP32 by the
-// mixed-precision add of sm_100 and later (16-bit operand, FP32 sum, one
-// rounding)
-template <typename SM> __device__ __forceinline__ void mixed_add(float2& acc, typename PairIO<SM>::V q);
-template <> __device__ __forceinline__ void mixed_add<__half>(float2& acc, __half2 q)
+// the window of an aligned column pair: rows n, c, s of a ring; j is the slot
+// of the pair's first column
+__device__ __forceinline__ Win<float2> load_win(const float* rn, const float* rc, const float* rs, int j)
 {
-    unsigned short lo, hi;
-    asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(bits(q)));
-    asm("add.rn.f32.f16 %0, %1, %0;" : "+f"(acc.x) : "h"(lo));
-    asm("add.rn.f32.f16 %0, %1, %0;" : "+f"(acc.y) : "h"(hi));
-}
-template <> __device__ __forceinline__ void mixed_add<__nv_bfloat16>(float2& acc, __nv_bfloat162 q)
-{
-    unsigned short lo, hi;
-    asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(bits(q)));
-    asm("add.rn.f32.bf16 %0, %1, %0;" : "+f"(acc.x) : "h"(lo));
-    asm("add.rn.f32.bf16 %0, %1, %0;" : "+f"(acc.y) : "h"(hi));
-}
-
-// The nine pairs of one 3 x 4 stencil window of a shared row triple: for
-// each of the rows n (+y), c, s (-y) the pair at the thread's own columns
-// (x, x+1) and the shifted pairs (x-1, x) and (x+1, x+2).
-struct Win {
-    float2 n0, nL, nR, c0, cL, cR, s0, sL, sR;
-};
-// rows n, c, s of a ring; j is the slot of the pair's first column
-__device__ __forceinline__ Win load_win(const float* rn, const float* rc, const float* rs, int j)
-{
-    Win w;
+    Win<float2> w;
     w.n0 = lds2(rn + j); w.nL = make_float2(rn[j - 1], w.n0.x); w.nR = make_float2(w.n0.y, rn[j + 2]);
     w.c0 = lds2(rc + j); w.cL = make_float2(rc[j - 1], w.c0.x); w.cR = make_float2(w.c0.y, rc[j + 2]);
     w.s0 = lds2(rs + j); w.sL = make_float2(rs[j - 1], w.s0.x); w.sR = make_float2(w.s0.y, rs[j + 2]);
     return w;
-}
-
-// ---------------------------------------------------------------------------
-// Node arithmetic.
-
-// Film pressure (Eq. pfilm with Eq. disjoiningP) of the two nodes from the h
-// window; writes 1/h to ih.
-__device__ __forceinline__ float2 pair_pressure(const Win& H, float2 kap, bool disj, const Consts<float>& C,
-                                                float2& ih)
-{
-    // Eq. (n_laplace): axis neighbours left + right + up + down, diagonal the four corners
-    const float2 axis = padd(padd(H.cL, H.cR), padd(H.n0, H.s0));
-    const float2 diag = padd(padd(H.nL, H.nR), padd(H.sL, H.sR));
-    float2 lap = pmul(pfma(pk(4.0f), axis, pfma(pk(-20.0f), H.c0, diag)), pk(1.0f / 6.0f));
-    const float2 h = padd(H.c0, pk(C.href));
-    ih = make_float2(__fdividef(1.0f, h.x), __fdividef(1.0f, h.y));
-    if (disj) {
-        const float2 r = pmul(pk(C.hstar), ih);
-        float2 fd;
-        if (C.n_exp == 3 && C.m_exp == 2) fd = pmul(pmul(r, r), psub(r, pk(1.0f)));
-        else fd = make_float2(fdisj(r.x, C.n_exp, C.m_exp), fdisj(r.y, C.n_exp, C.m_exp));
-        lap = pfma(pmul(pk(C.pi_sgn), kap), fd, lap);
-    }
-    return pmul(pk(-C.gamma), lap);
-}
-
-// Force, collision and store of the two nodes (the arithmetic of
-// collide_store on both lanes, in storage units).  P: the p window around
-// the pair (n = row o+1, s = row o-1); f: the pulled moving populations in
-// storage units (omega != 1 only); i: the storage offset of the pair's first
-// column.
-template <typename SM, bool OMEGA1>
-__device__ __forceinline__ void pair_collide_store(const Win& P, float2 dh, float2 ih, float2 jx, float2 jy,
-                                                   float2 er, const float2* f, int fstride,
-                                                   float* __restrict__ fout0, SM* __restrict__ foutm, int i,
-                                                   int plane, const Consts<float>& C)
-{
-    using IO = PairIO<SM>;
-    using V = typename IO::V;
-    constexpr bool NARROW = !std::is_same<SM, float>::value;
-    // storage scale (1 for FP32, a compile-time constant there)
-    const float ms = NARROW ? C.mscale : 1.0f;
-    // Eq. (derivative): grad p = 3 sum_l w_l c_l p(x + c_l)
-    const float2 gpx = pfma(psub(P.cR, P.cL), pk(1.0f / 3.0f),
-                            pmul(padd(psub(P.nR, P.nL), psub(P.sR, P.sL)), pk(1.0f / 12.0f)));
-    const float2 gpy = pfma(psub(P.n0, P.s0), pk(1.0f / 3.0f),
-                            pmul(padd(psub(P.nR, P.sR), psub(P.nL, P.sL)), pk(1.0f / 12.0f)));
-    const float2 h = padd(dh, pk(C.href));
-    // Eqs. (force), (forcefric), (alphafric): nu alpha u = 6 nu j / (2h^2 + 6 delta h + 3 delta^2)
-    const float2 den = pfma(h, pfma(pk(2.0f), h, pk(6.0f * C.delta)), pk(3.0f * C.delta * C.delta));
-    const float2 fr = pmul(pk(C.nu6), make_float2(__fdividef(1.0f, den.x), __fdividef(1.0f, den.y)));
-    // Eq. (LBE) as printed: u = j/h.  Second-order forcing (C.forcing):
-    // u (h + nu alpha/2) = j + F'/2 and the equilibria use h u for j (see
-    // collide_store)
-    float2 Fx, Fy, ux, uy, ex, ey;
-    if (C.forcing) {
-        const float2 fpx = pmul(h, psub(pk(C.gx), gpx)), fpy = pmul(h, psub(pk(C.gy), gpy));
-        const float2 d = pfma(pk(0.5f), fr, pk(1.0f));
-        const float2 q = make_float2(__fdividef(ih.x, d.x), __fdividef(ih.y, d.y));
-        ux = pmul(pfma(pk(0.5f), fpx, jx), q);
-        uy = pmul(pfma(pk(0.5f), fpy, jy), q);
-        ex = pmul(h, ux);
-        ey = pmul(h, uy);
-        Fx = psub(fpx, pmul(fr, ex));
-        Fy = psub(fpy, pmul(fr, ey));
-    } else {
-        Fx = psub(pmul(h, psub(pk(C.gx), gpx)), pmul(fr, jx));
-        Fy = psub(pmul(h, psub(pk(C.gy), gpy)), pmul(fr, jy));
-        ux = pmul(jx, ih);
-        uy = pmul(jy, ih);
-        ex = jx;
-        ey = jy;
-    }
-    // Eq. (equilibria) with e^2 = 1 as S +- D per opposite pair, source
-    // 3 w_l c_l . F; in storage units S' = (S - R_l) ms, D' = D ms.
-    // A6 = 6 A = h (g h - u^2).
-    const float2 A6 = pmul(h, psub(pmul(pk(C.g), h), pfma(ux, ux, pmul(uy, uy))));
-    const float2 Aa = NARROW ? pfma(A6, pk(ms * (1.0f / 6.0f)), pk(C.nr_axis)) : pmul(A6, pk(1.0f / 6.0f));
-    const float2 Ad = NARROW ? pfma(A6, pk(ms * (1.0f / 24.0f)), pk(C.nr_diag)) : pmul(A6, pk(1.0f / 24.0f));
-    float2 Sx = pfma(pmul(ex, pk(0.5f * ms)), ux, Aa);
-    float2 Sy = pfma(pmul(ey, pk(0.5f * ms)), uy, Aa);
-    const float2 a = padd(ux, uy), b = psub(uy, ux);
-    const float2 h8 = pmul(h, pk(0.125f * ms));
-    float2 Sa = pfma(pmul(h8, a), a, Ad);
-    float2 Sb = pfma(pmul(h8, b), b, Ad);
-    // second-order source: odd part scaled by (1 - omega/2), even part T
-    float2 Tx = pk(0.0f), Ty = pk(0.0f), Ta = pk(0.0f), Tb = pk(0.0f);
-    if (C.forcing) {
-        const float2 ks = pk(1.0f - 0.5f * C.omega);
-        Fx = pmul(Fx, ks);
-        Fy = pmul(Fy, ks);
-        const float2 uF3 = pmul(pfma(ux, Fx, pmul(uy, Fy)), pk(ms * (1.0f / 3.0f)));
-        Tx = pfma(pmul(ux, Fx), pk(ms), make_float2(-uF3.x, -uF3.y));
-        Ty = pfma(pmul(uy, Fy), pk(ms), make_float2(-uF3.x, -uF3.y));
-        Ta = pmul(pfma(pmul(a, padd(Fx, Fy)), pk(ms), make_float2(-uF3.x, -uF3.y)), pk(0.25f));
-        Tb = pmul(pfma(pmul(b, psub(Fy, Fx)), pk(ms), make_float2(-uF3.x, -uF3.y)), pk(0.25f));
-        if constexpr (OMEGA1) {
-            Sx = padd(Sx, Tx);
-            Sy = padd(Sy, Ty);
-            Sa = padd(Sa, Ta);
-            Sb = padd(Sb, Tb);
-        }
-    }
-    const float2 m3 = pk(ms * (1.0f / 3.0f)), m12 = pk(ms * (1.0f / 12.0f));
-    float2 o1, o2, o3, o4, o5, o6, o7, o8;
-    if constexpr (OMEGA1) {
-        const float2 Gx = padd(ex, Fx), Gy = padd(ey, Fy);
-        const float2 Dx = pmul(Gx, m3), Dy = pmul(Gy, m3);
-        const float2 Da = pmul(padd(Gx, Gy), m12), Db = pmul(psub(Gy, Gx), m12);
-        o1 = padd(Sx, Dx); o5 = psub(Sx, Dx);
-        o3 = padd(Sy, Dy); o7 = psub(Sy, Dy);
-        o2 = padd(Sa, Da); o6 = psub(Sa, Da);
-        o4 = padd(Sb, Db); o8 = psub(Sb, Db);
-    } else {
-        // (1 - omega)(f_l - R_l) + omega (f_eq_l - R_l) + source, in storage units
-        const float2 w = pk(C.omega), m = pk(1.0f - C.omega);
-        const float2 Dx = pmul(ex, m3), Dy = pmul(ey, m3);
-        const float2 Da = pmul(padd(ex, ey), m12), Db = pmul(psub(ey, ex), m12);
-        const float2 Qx = pmul(Fx, m3), Qy = pmul(Fy, m3);
-        const float2 Qa = pmul(padd(Fx, Fy), m12), Qb = pmul(psub(Fy, Fx), m12);
-        o1 = padd(pfma(m, f[0 * fstride], pmul(w, padd(Sx, Dx))), padd(Tx, Qx));
-        o5 = padd(pfma(m, f[4 * fstride], pmul(w, psub(Sx, Dx))), psub(Tx, Qx));
-        o3 = padd(pfma(m, f[2 * fstride], pmul(w, padd(Sy, Dy))), padd(Ty, Qy));
-        o7 = padd(pfma(m, f[6 * fstride], pmul(w, psub(Sy, Dy))), psub(Ty, Qy));
-        o2 = padd(pfma(m, f[1 * fstride], pmul(w, padd(Sa, Da))), padd(Ta, Qa));
-        o6 = padd(pfma(m, f[5 * fstride], pmul(w, psub(Sa, Da))), psub(Ta, Qa));
-        o4 = padd(pfma(m, f[3 * fstride], pmul(w, padd(Sb, Db))), padd(Tb, Qb));
-        o8 = padd(pfma(m, f[7 * fstride], pmul(w, psub(Sb, Db))), psub(Tb, Qb));
-    }
-    // stored rest population f*_0 - href = (h - href) - sum_{l>0} f*_l, with
-    // the exact residuals folded back as in collide_store
-    const int hp = plane >> 1;  // pairs per plane
-    // the pair (i, i+1) of plane 0 and of the eight moving planes
-    TFLBM_CHECK(i >= 0 && (i & 1) == 0 && i + 1 < plane, C.status);
-    const int ip = TFLBM_IDX(i >> 1, hp, C.status);
-    V* om = reinterpret_cast<V*>(foutm) + ip;
-    if constexpr (!NARROW) {
-        const float2 osum = padd(padd(padd(o1, o5), padd(o3, o7)), padd(padd(o2, o6), padd(o4, o8)));
-        float2 o0v, e2;
-        ptwo_sum(dh, make_float2(-osum.x, -osum.y), o0v, e2);
-        const float2 half_r = pmul(padd(er, e2), pk(0.5f));
-        o1 = padd(o1, half_r);
-        o5 = padd(o5, half_r);
-        reinterpret_cast<float2*>(fout0)[ip] = o0v;
-        om[0] = o1; om[hp] = o2; om[2 * hp] = o3; om[3 * hp] = o4;
-        om[4 * hp] = o5; om[5 * hp] = o6; om[6 * hp] = o7; om[7 * hp] = o8;
-    } else {
-        const V q2 = IO::enc(o2), q3 = IO::enc(o3), q4 = IO::enc(o4), q5 = IO::enc(o5);
-        const V q6 = IO::enc(o6), q7 = IO::enc(o7), q8 = IO::enc(o8), q1r = IO::enc(o1);
-        // what the readers reconstruct of l = 2..8 (storage units; each
-        // stored value enters the FP32 sum by a mixed-precision add, which
-        // takes the 16-bit operand as it is: one instruction per value
-        // instead of a conversion and half a paired add)
-        float2 rest = IO::dec(q2);
-        mixed_add<SM>(rest, q3);
-        mixed_add<SM>(rest, q4);
-        mixed_add<SM>(rest, q5);
-        mixed_add<SM>(rest, q6);
-        mixed_add<SM>(rest, q7);
-        mixed_add<SM>(rest, q8);
-        float2 rest1 = rest;
-        mixed_add<SM>(rest1, q1r);
-        // the moving populations' total with f_1 unrounded and rounded
-        const float2 osum = pfma(padd(rest, o1), pk(C.minv), pk(C.r_sum));
-        const float2 osr = pfma(rest1, pk(C.minv), pk(C.r_sum));
-        // the last residual goes to the finer of the two roundings: the 16-bit
-        // one of f_1 - R or the FP32 one of f_0 - href (see collide_store)
-        constexpr float kRatio = std::is_same<SM, __half>::value ? 8192.0f : 65536.0f;
-        const float kr = kRatio * C.minv;  // |f_1 - R| = |o1| / ms
-        const bool lx = fabsf(o1.x) * kr < fabsf(dh.x - osum.x);
-        const bool ly = fabsf(o1.y) * kr < fabsf(dh.y - osum.y);
-        const float2 os = make_float2(lx ? osum.x : osr.x, ly ? osum.y : osr.y);
-        float2 o0v, e2, o0n, e3;
-        ptwo_sum(dh, make_float2(-os.x, -os.y), o0v, e2);
-        ptwo_sum(o0v, padd(er, e2), o0n, e3);
-        const V q1l = IO::enc(pfma(e3, pk(ms), o1));
-        const uint32_t mask = (lx ? 0x0000ffffu : 0u) | (ly ? 0xffff0000u : 0u);
-        const V q1 = from_bits<V>((bits(q1l) & mask) | (bits(q1r) & ~mask));
-        reinterpret_cast<float2*>(fout0)[ip] = o0n;
-        om[0] = q1; om[hp] = q2; om[2 * hp] = q3; om[3 * hp] = q4;
-        om[4 * hp] = q5; om[5 * hp] = q6; om[6 * hp] = q7; om[7 * hp] = q8;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -537,8 +279,8 @@ __device__ __forceinline__ void step_band2(const float* __restrict__ fin0, const
             // the window reads slots j2 - 1 .. j2 + 2 of rings of RW
             TFLBM_CHECK(j2 >= 1 && j2 + 2 < RW, C.status);
             float2 ih;
-            const Win Hw = load_win(hsm[s], hsm[s1], hsm[s2], j2);
-            const float2 p = pair_pressure(Hw, kap, disj, C, ih);
+            const Win<float2> Hw = load_win(hsm[s], hsm[s1], hsm[s2], j2);
+            const float2 p = node_pressure(Hw, kap, disj, C, ih);
             rsi[s1][t] = ih;
             *reinterpret_cast<float2*>(&psm[s1][j2]) = p;
         }
@@ -548,13 +290,22 @@ __device__ __forceinline__ void step_band2(const float* __restrict__ fin0, const
             TFLBM_CHECK(j2 >= 1 && j2 + 2 < RW && o >= 0 && o < ny, C.status);
             // rows o+1 and o-1 of the p ring
             const int sn = dir > 0 ? s2 : s, ss = dir > 0 ? s : s2;
-            const Win Pw = load_win(psm[sn], psm[s3], psm[ss], j2);
+            const Win<float2> Pw = load_win(psm[sn], psm[s3], psm[ss], j2);
             const float2 dh = lds2(&hsm[s3][j2]);
             const float4 jj = rsj[s3][t];
             const float2* fp = nullptr;
             if constexpr (!OMEGA1) fp = &fsm[s3][0][t];
-            pair_collide_store<SM, OMEGA1>(Pw, dh, rsi[s3][t], make_float2(jj.x, jj.y), make_float2(jj.z, jj.w),
-                                           rse[s3][t], fp, BX, fout0, foutm, o * pitch + c, plane, C);
+            // the pair (i, i+1) of plane 0 and of the eight moving planes
+            const int i = o * pitch + c;
+            TFLBM_CHECK(i >= 0 && (i & 1) == 0 && i + 1 < plane, C.status);
+            const int ip = TFLBM_IDX(i >> 1, half, C.status);
+            node_collide<SM, OMEGA1>(Pw, dh, rsi[s3][t], make_float2(jj.x, jj.y), make_float2(jj.z, jj.w), rse[s3][t],
+                                     fp, BX, C, [&](float2 o0, const V(&q)[8]) {
+                                         reinterpret_cast<float2*>(fout0)[ip] = o0;
+                                         V* om = reinterpret_cast<V*>(foutm) + ip;
+#pragma unroll
+                                         for (int l = 0; l < 8; ++l) om[l * half] = q[l];
+                                     });
         }
         wm1 = w0;
         w0 = w1;

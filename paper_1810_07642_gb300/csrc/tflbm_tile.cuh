@@ -1,0 +1,266 @@
+// Tile form of the fused step (Section II of Zitz et al., arXiv:1810.07642),
+// for lattices that the L2 cache holds.
+//
+// Why: the marching kernels (tflbm_step.cuh, tflbm_step2.cuh) walk a band row
+// by row, each row waiting for loads of the row before; a band of 16 rows is a
+// chain of 21 L2 round trips and barriers, about 14 us whatever the lattice's
+// size, and a small lattice has too few bands to hide them.  Here a CTA owns a
+// tile of TX x TY nodes and runs the step's three phases over all of it: pull
+// and moments of the tile and a halo of 2 (every load of the tile in flight at
+// once), a barrier, the pressure of the tile and a halo of 1, a barrier, force
+// and collision: one round trip and two barriers a step.  The halo costs
+// repeated pulls (1.4 a node at 32 x 16), which come from L1/L2; on a lattice
+// much larger than L2 the march, which pulls each node about 1.3 times and
+// loads ahead, is the faster one.
+//
+// A thread owns X::N nodes of its tile (FP32 compute type: two, TY / 2 rows
+// apart, on the paired FP32 instructions; FP64: one) and keeps their momenta
+// (and, when omega != 1, their pulled populations) in registers between the
+// phases; halo nodes only leave h or p in shared memory.  Columns and rows are
+// wrapped per node, so any lattice down to one node works; nodes of a tile that
+// lie past the lattice's edge are computed as their periodic images and not
+// stored.  The node arithmetic is that of tflbm_node.cuh.
+#pragma once
+#include "tflbm_handle.h"
+#include "tflbm_node.cuh"
+
+namespace tflbm {
+
+// i on a ring of n (the modulo only runs outside the lattice)
+__device__ __forceinline__ int ring_index(int i, int n) { return (unsigned)i < (unsigned)n ? i : wrap_index(i, n); }
+
+template <typename S> struct TileX { using X = float2; };
+template <> struct TileX<double> { using X = double; };
+
+// lane k of x
+template <int K> __device__ __forceinline__ float& lane_of(float2& x)
+{
+    if constexpr (K == 0) return x.x;
+    else return x.y;
+}
+template <int K> __device__ __forceinline__ double& lane_of(double& x) { return x; }
+
+// Moments of pulled populations in storage units (the sums of step_band2).
+template <typename SM, typename X>
+__device__ __forceinline__ void node_moments(X f0, const X (&n)[8], const Consts<typename Lanes<X>::S>& C, X& dh, X& er,
+                                             X& jx, X& jy)
+{
+    const X Rs = padd(padd(n[0], n[1]), n[7]), Ls = padd(padd(n[4], n[3]), n[5]);
+    const X jyr = padd(psub(n[2], n[6]), padd(psub(n[1], n[7]), psub(n[3], n[5])));
+    const X tot = padd(padd(n[2], n[6]), padd(Rs, Ls));
+    if constexpr (sizeof(SM) == 2) {
+        const X minv = Lanes<X>::all(C.minv);
+        ptwo_sum(f0, pfma(tot, minv, Lanes<X>::all(C.r_sum)), dh, er);
+        jx = pmul(psub(Rs, Ls), minv);
+        jy = pmul(jyr, minv);
+    } else {
+        ptwo_sum(f0, tot, dh, er);
+        jx = psub(Rs, Ls);
+        jy = jyr;
+    }
+}
+
+template <typename SM, typename S, int TX, int TY, bool OMEGA1, int RESIDENT>
+__global__ void __launch_bounds__(TX* TY / Lanes<typename TileX<S>::X>::N, RESIDENT / (TX * TY / Lanes<typename TileX<S>::X>::N))
+k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ fout0, SM* __restrict__ foutm,
+       const S* __restrict__ kappa, const Geom G, const Consts<S> C)
+{
+    using X = typename TileX<S>::X;
+    using IO = PairIO<SM>;
+    using V = typename IO::V;
+    constexpr int N = Lanes<X>::N, NT = TX * TY / N, HALF = TY / N;
+    constexpr int HW = TX + 4, PW = TX + 2;
+    // halo nodes of the h and p rings around the tile, and pairs of them
+    constexpr int HN = HW * (TY + 4) - TX * TY, PN = PW * (TY + 2) - TX * TY;
+    constexpr int HP = HN / N, PP = PN / N;
+    static_assert(HN % N == 0 && PN % N == 0 && TY % N == 0, "halo nodes come in whole groups");
+    __shared__ S hs[TY + 4][HW];  // h - href; tile node (c, r) at [r + 2][c + 2]
+    __shared__ S ps[TY + 2][PW];  // p; tile node (c, r) at [r + 1][c + 1]
+
+    dependent_launch_entry();
+    const int t = threadIdx.x, nx = G.nx, ny = G.ny, pitch = G.pitch, plane = (int)G.plane;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const int c = t % TX, r = t / TX;  // own nodes: (c, r + k HALF)
+    const bool disj = kappa != nullptr || C.kappa_u != S(0);
+
+    // the populations arriving at tile position (cc, rr), into lane K
+    auto pull = [&](auto k_c, int cc, int rr, X& f0, X (&n)[8]) {
+        constexpr int K = decltype(k_c)::value;
+        const int x = ring_index(x0 + cc, nx), y = ring_index(y0 + rr, ny);
+        const int xm = x == 0 ? nx - 1 : x - 1, xp = x + 1 == nx ? 0 : x + 1;
+        const int r0 = y * pitch, rm = (y == 0 ? ny - 1 : y - 1) * pitch, rp = (y + 1 == ny ? 0 : y + 1) * pitch;
+        const long long m8 = 8LL * plane;
+        int* st = C.status;
+        (void)m8;
+        (void)st;
+        lane_of<K>(f0) = ldro(fin0 + TFLBM_IDX(r0 + x, plane, st));
+        lane_of<K>(n[0]) = IO::dec1(ldro(finm + TFLBM_IDX(r0 + xm, m8, st)));
+        lane_of<K>(n[1]) = IO::dec1(ldro(finm + TFLBM_IDX(plane + rm + xm, m8, st)));
+        lane_of<K>(n[2]) = IO::dec1(ldro(finm + TFLBM_IDX(2 * plane + rm + x, m8, st)));
+        lane_of<K>(n[3]) = IO::dec1(ldro(finm + TFLBM_IDX(3 * plane + rm + xp, m8, st)));
+        lane_of<K>(n[4]) = IO::dec1(ldro(finm + TFLBM_IDX(4 * plane + r0 + xp, m8, st)));
+        lane_of<K>(n[5]) = IO::dec1(ldro(finm + TFLBM_IDX(5 * plane + rp + xp, m8, st)));
+        lane_of<K>(n[6]) = IO::dec1(ldro(finm + TFLBM_IDX(6 * plane + rp + x, m8, st)));
+        lane_of<K>(n[7]) = IO::dec1(ldro(finm + TFLBM_IDX(7 * plane + rp + xm, m8, st)));
+    };
+    auto kap_at = [&](int cc, int rr) -> S {
+        if (!kappa) return C.kappa_u;
+        const long long nk = (long long)nx * ny;
+        (void)nk;
+        return ldro(kappa + TFLBM_IDX(ring_index(y0 + rr, ny) * nx + ring_index(x0 + cc, nx), nk, C.status));
+    };
+    // position of node i of the halo of depth D (two rings: D rows above and
+    // below over the whole width, then the columns on both sides)
+    auto halo = [&](auto d_c, int i, int& cc, int& rr) {
+        constexpr int D = decltype(d_c)::value, FW = TX + 2 * D;
+        if (i < 2 * D * FW) {
+            const int k = i / FW;
+            cc = i % FW - D;
+            rr = k < D ? k - D : TY + k - D;
+        } else {
+            const int k = (i - 2 * D * FW) % (2 * D);
+            rr = (i - 2 * D * FW) / (2 * D);
+            cc = k < D ? k - D : TX + k - D;
+        }
+    };
+    auto lanes = [&](auto fn) {
+        fn(std::integral_constant<int, 0>{});
+        if constexpr (N == 2) fn(std::integral_constant<int, 1>{});
+    };
+    using D2 = std::integral_constant<int, 2>;
+    using D1 = std::integral_constant<int, 1>;
+
+    // ---- h and j of the tile, h of the halo of 2
+    X f0, n[8], dh, er, jx, jy, kap, ih;
+    lanes([&](auto k_c) {
+        constexpr int K = decltype(k_c)::value;
+        pull(k_c, c, r + K * HALF, f0, n);
+        lane_of<K>(kap) = kap_at(c, r + K * HALF);
+    });
+    for (int i = t; i < HP; i += NT) {
+        X g0, g[8], d, e, a, b;
+        int cc[N], rr[N];
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            halo(D2{}, i + K * HP, cc[K], rr[K]);
+            pull(k_c, cc[K], rr[K], g0, g);
+        });
+        node_moments<SM>(g0, g, C, d, e, a, b);
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            hs[rr[K] + 2][cc[K] + 2] = lane_of<K>(d);
+        });
+    }
+    node_moments<SM>(f0, n, C, dh, er, jx, jy);
+    lanes([&](auto k_c) {
+        constexpr int K = decltype(k_c)::value;
+        hs[r + K * HALF + 2][c + 2] = lane_of<K>(dh);
+    });
+    __syncthreads();
+
+    // ---- film pressure of the tile and the halo of 1
+    auto window = [&](auto k_c, const S* b, int w, Win<X>& W) {  // around element b of rows w wide
+        constexpr int K = decltype(k_c)::value;
+        lane_of<K>(W.nL) = b[w - 1]; lane_of<K>(W.n0) = b[w]; lane_of<K>(W.nR) = b[w + 1];
+        lane_of<K>(W.cL) = b[-1]; lane_of<K>(W.c0) = b[0]; lane_of<K>(W.cR) = b[1];
+        lane_of<K>(W.sL) = b[-w - 1]; lane_of<K>(W.s0) = b[-w]; lane_of<K>(W.sR) = b[-w + 1];
+    };
+    {
+        Win<X> W;
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            window(k_c, &hs[r + K * HALF + 2][c + 2], HW, W);
+        });
+        X p = node_pressure(W, kap, disj, C, ih);
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            ps[r + K * HALF + 1][c + 1] = lane_of<K>(p);
+        });
+    }
+    for (int i = t; i < PP; i += NT) {
+        Win<X> W;
+        X kh, q;
+        int cc[N], rr[N];
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            halo(D1{}, i + K * PP, cc[K], rr[K]);
+            lane_of<K>(kh) = kap_at(cc[K], rr[K]);
+            window(k_c, &hs[rr[K] + 2][cc[K] + 2], HW, W);
+        });
+        X p = node_pressure(W, kh, disj, C, q);
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            ps[rr[K] + 1][cc[K] + 1] = lane_of<K>(p);
+        });
+    }
+    __syncthreads();
+
+    // ---- force, collision and store of the tile
+    Win<X> W;
+    lanes([&](auto k_c) {
+        constexpr int K = decltype(k_c)::value;
+        window(k_c, &ps[r + K * HALF + 1][c + 1], PW, W);
+    });
+    node_collide<SM, OMEGA1>(W, dh, ih, jx, jy, er, n, 1, C, [&](X o0, const V(&q)[8]) {
+        const int x = x0 + c;
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            const int y = y0 + r + K * HALF;
+            if (x >= nx || y >= ny) return;
+            const int i = y * pitch + x;
+            const long long m8 = 8LL * plane;
+            (void)m8;
+            fout0[TFLBM_IDX(i, plane, C.status)] = lane_of<K>(o0);
+#pragma unroll
+            for (int l = 0; l < 8; ++l) {
+                SM v;
+                if constexpr (N == 1) v = q[l];
+                else if constexpr (K == 0) v = q[l].x;
+                else v = q[l].y;
+                foutm[TFLBM_IDX(l * plane + i, m8, C.status)] = v;
+            }
+        });
+    });
+}
+
+template <typename SM, typename S, int TX, int TY>
+cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, const Geom& G, const Consts<S>& C,
+                     cudaStream_t st)
+{
+    constexpr int NT = TX * TY / Lanes<typename TileX<S>::X>::N;
+    const dim3 grid((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY);
+    auto launch = [&](auto resident) {
+        constexpr int R = decltype(resident)::value;
+        if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, G, C);
+        return launch_dependent(k_tile<SM, S, TX, TY, false, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, G, C);
+    };
+    // Threads an SM holds.  512 leaves the registers that keep a thread's 18
+    // loads in flight (80); where 32 x 16 tiles outnumber the three an SM
+    // holds then, 64 registers and a fourth tile win (one box, tau = 1: 509 x
+    // 387 4.9 against 5.7 us a step, 512^2 6.4 against 5.3, 1024^2 17.8
+    // against 16.3).
+    if constexpr (TX == 32 && sizeof(S) == 4) {
+        if ((long long)grid.x * grid.y > 3LL * sm_count()) return launch(std::integral_constant<int, 1024>{});
+    }
+    return launch(std::integral_constant<int, 512>{});
+}
+
+// One step from fin to fout in the tiles that block_x names (tile_of).
+template <typename SM, typename S>
+cudaError_t tile_step(int block_x, const void* fin, void* fout, const void* kappa, const Geom& G, const Consts<S>& C,
+                      cudaStream_t st)
+{
+    const S* f0 = (const S*)fin;
+    const SM* fm = (const SM*)((const char*)fin + G.plane * sizeof(S));
+    S* g0 = (S*)fout;
+    SM* gm = (SM*)((char*)fout + G.plane * sizeof(S));
+    const S* k = (const S*)kappa;
+    switch (block_x) {
+        case 64: return tile_one<SM, S, 16, 8>(f0, fm, g0, gm, k, G, C, st);
+        case 128: return tile_one<SM, S, 16, 16>(f0, fm, g0, gm, k, G, C, st);
+        case 256: return tile_one<SM, S, 32, 16>(f0, fm, g0, gm, k, G, C, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace tflbm

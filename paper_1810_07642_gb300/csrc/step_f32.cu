@@ -31,7 +31,7 @@ cudaError_t launch_step(int store, const void* fin, void* fout, const void* kapp
                         const Consts<float>* C32, const Consts<double>* C64, const Shape& S,
                         cudaStream_t st)
 {
-    if (S.tile) return launch_tile(store, S.tile, fin, fout, kappa, G, C32, C64, st);
+    if (S.tile) return launch_tile(store, S.tile, fin, fout, kappa, nullptr, G, C32, C64, st);
     if (S.pipeline == kPipePair) {
         switch (store) {
             case kStoreF32: return pair_step_f32(S.block_x, fin, fout, kappa, G, *C32, launch_bands(S, G.ny), st);

@@ -17,17 +17,19 @@
 //   a_l(x,t) = aH + c_l . aJ + (1 - omega) mu_l            moments^T
 // with r = h_*/h, fr = 6 nu / (2h^2 + 6 delta h + 3 delta^2).
 //
-// The gradient tape runs the forward from the handle's state, keeping a copy
-// of the state every K steps (K ~ sqrt(T)); the backward pass restores each
-// checkpoint in reverse order, recomputes the K states of that segment and
-// runs the adjoint steps through them (sqrt(T) checkpoint-recompute).
+// The gradient tape runs the forward from the handle's state in tile steps
+// that record h and j of every state they start from (all that the adjoint
+// needs of f, see tflbm_adjoint_tile.cuh).  Where the records of all steps fit
+// in kTapeBytes it keeps them; else it keeps a copy of the state every K steps
+// (K ~ sqrt(T)) and the backward pass recomputes each segment's records from
+// its copy, in reverse order of the segments.
 #include <cuda_runtime.h>
 #include <math.h>
 
 #include <algorithm>
 #include <vector>
 
-#include "tflbm_adjoint_march.cuh"
+#include "tflbm_adjoint_tile.cuh"
 #include "tflbm_handle.h"
 
 namespace tflbm {
@@ -207,31 +209,43 @@ __global__ void k_adj_out(const T* __restrict__ aH, const T* __restrict__ alap, 
     }
 }
 
-// dL/dh0 = sum_l a_l(0) dE_l(h0, 0)/dh0; dL/dtheta = dL/dkappa sin(theta) c
+// dL/dh0 = sum_l a_l(0) dE_l(h0, 0)/dh0, which with a_l = aH + c_l . aJ (three
+// fields, omega = 1) is aH; dL/dtheta = dL/dkappa sin(theta) c
 template <typename T>
 __global__ void k_adj_init(const T* __restrict__ h0, const T* __restrict__ a0, T* gh0, const T* __restrict__ gk,
-                           const T* __restrict__ theta, T* gth, Dims D, Consts<T> C, T kc, T theta_u)
+                           const T* __restrict__ theta, T* gth, Dims D, Consts<T> C, T kc, T theta_u, bool three)
 {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= D.n) return;
     if (gh0) {
-        const T hh = h0[i];
-        T s = a0[i] * (T(1) - T(5) * C.g * hh / T(3));
+        T s = a0[i];
+        if (!three) {
+            const T hh = h0[i];
+            s *= T(1) - T(5) * C.g * hh / T(3);
 #pragma unroll
-        for (int l = 1; l < 9; ++l) s += a0[l * D.n + i] * C.g * hh * ((l & 1) ? T(1.0 / 3.0) : T(1.0 / 12.0));
+            for (int l = 1; l < 9; ++l) s += a0[l * D.n + i] * C.g * hh * ((l & 1) ? T(1.0 / 3.0) : T(1.0 / 12.0));
+        }
         gh0[i] = s;
     }
     if (gth) gth[i] = gk[i] * sin(theta ? theta[i] : theta_u) * kc;
 }
 
+// a(T) = dL/df(T): h = sum_l f_l, so aH = dL/dh, aJ = 0; dL/dkappa starts at 0
 template <typename T>
-__global__ void k_seed(const T* __restrict__ gh, T* a, Dims D)
+__global__ void k_seed(const T* __restrict__ gh, T* a, T* gk, Dims D, bool three)
 {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= D.n) return;
     const T v = gh[i];
+    gk[i] = T(0);
+    a[i] = v;
+    if (three) {
+        a[D.n + i] = T(0);
+        a[2 * D.n + i] = T(0);
+    } else {
 #pragma unroll
-    for (int l = 0; l < 9; ++l) a[l * D.n + i] = v;  // h = sum_l f_l
+        for (int l = 1; l < 9; ++l) a[l * D.n + i] = v;
+    }
 }
 
 inline dim3 g2(const Dims& D) { return dim3((D.nx + 127) / 128, D.ny); }
@@ -268,73 +282,57 @@ cudaError_t adjoint_step_dispatch(tf_lbm_handle* H, const void* f, const void* a
 
 namespace {
 
-template <typename SM, typename T, int BX>
-cudaError_t march_t(tf_lbm_handle* H, const void* fin, const void* an, void* a, void* gk, int rows,
-                    cudaStream_t st)
+template <typename S>
+cudaError_t adjoint_tile_t(tf_lbm_handle* H, const void* mom, const void* an, void* a, void* gk, cudaStream_t st)
 {
-    const Geom& G = H->G;
-    const T* f0 = (const T*)fin;
-    const SM* fm = (const SM*)((const char*)fin + G.plane * sizeof(T));
-    int bands = (G.ny + rows - 1) / rows;
-    if (bands > 65535) bands = 65535;
-    const dim3 grid((G.nx + BX - 9) / (BX - 8), bands);
-    k_adjoint_march<SM, T, BX><<<grid, BX, 0, st>>>(f0, fm, (const T*)an, (T*)a, (T*)gk, (const T*)H->kappa, G,
-                                                    make_consts<T>(H));
-    return cudaGetLastError();
+    const Consts<S> C = make_consts<S>(H);
+    const S *m = (const S*)mom, *n = (const S*)an, *k = (const S*)H->kappa;
+    switch (tile_block_x(H->dbl ? kStoreF64 : kStoreF32, H->G.nx, H->G.ny, H->sms)) {
+        case 64: return adjoint_tile_one<S, 16, 8>(m, n, (S*)a, (S*)gk, k, H->G, C, st);
+        case 128: return adjoint_tile_one<S, 16, 16>(m, n, (S*)a, (S*)gk, k, H->G, C, st);
+        default: return adjoint_tile_one<S, 32, 16>(m, n, (S*)a, (S*)gk, k, H->G, C, st);
+    }
 }
 
-template <typename SM, typename T, int BX>
-int march_rows(const tf_lbm_handle* H)
+// One adjoint step from the record of its state.
+cudaError_t adjoint_tile_step(tf_lbm_handle* H, const void* mom, const void* an, void* a, void* gk, cudaStream_t st)
 {
-    int occ = 0, sms = sm_count();
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_adjoint_march<SM, T, BX>, BX, 0) != cudaSuccess) {
-        cudaGetLastError();
-        occ = 1;
-    }
-    const int strips = (H->G.nx + BX - 9) / (BX - 8);
-    const int bands = std::max(1, std::max(occ, 1) * sms / strips);
-    return std::max(4, (H->G.ny + bands - 1) / bands);
+    return H->dbl ? adjoint_tile_t<double>(H, mom, an, a, gk, st) : adjoint_tile_t<float>(H, mom, an, a, gk, st);
+}
+
+// omega == 1 in the compute type: three-field adjoint states
+bool three_fields(const tf_lbm_handle* H)
+{
+    return H->dbl ? make_consts<double>(H).omega == 1.0 : make_consts<float>(H).omega == 1.0f;
 }
 
 }  // namespace
-
-// Fused adjoint step from the raw buffer whose pull is f(t).
-cudaError_t adjoint_march_dispatch(tf_lbm_handle* H, const void* fin, const void* an, void* a, void* gk,
-                                   cudaStream_t st)
-{
-    switch (H->desc.store) {
-        case kStoreF32: return march_t<float, float, 128>(H, fin, an, a, gk, march_rows<float, float, 128>(H), st);
-        case kStoreF64: return march_t<double, double, 64>(H, fin, an, a, gk, march_rows<double, double, 64>(H), st);
-        case kStoreF16: return march_t<__half, float, 128>(H, fin, an, a, gk, march_rows<__half, float, 128>(H), st);
-        case kStoreBF16:
-            return march_t<__nv_bfloat16, float, 128>(H, fin, an, a, gk, march_rows<__nv_bfloat16, float, 128>(H), st);
-        default: return cudaErrorInvalidValue;
-    }
-}
 
 }  // namespace tflbm
 
 // ---------------------------------------------------------------- the tape
 
+// Largest set of step records a tape keeps in place of state copies and
+// recomputation: 3 % of the device's memory.  A 512^2 step costs 5.2 us to
+// recompute and 3 MB to keep, and allocating and freeing that takes 1.2 us, so
+// more would still pay in time, but a tape is not the only tenant.
+constexpr size_t kTapeBytes = (size_t)8 << 30;
+
 struct tf_lbm_tape {
     tf_lbm_handle* H = nullptr;
     int64_t nsteps = 0;
-    int every = 1;
-    int nck = 0;                   // checkpoints: states at 0, K, 2K, ...
+    int every = 1;                 // records kept at a time: all steps, or one segment
+    int nseg = 0;                  // segments of `every` steps (the last may be shorter)
     size_t state_bytes = 0;        // one raw population buffer
-    void* ck = nullptr;            // nck raw buffers, then the final state
-    void* seg = nullptr;           // every raw population buffers: the states of one segment
+    size_t rec_bytes = 0;          // one record: h - href, j_x, j_y
+    size_t a_bytes = 0;            // one adjoint state
+    void* ck = nullptr;            // states at 0, K, 2K, ... (nseg > 1), then two buffers to recompute in
+    void* rec = nullptr;           // `every` records
     void* abuf = nullptr;          // 2 adjoint states
     void* gk = nullptr;            // dL/dkappa
     void* h0 = nullptr;            // copy of h0 (compute type)
     void* theta = nullptr;         // copy of theta or null (uniform)
-    int64_t t0 = 0;                // handle time when the forward started
     bool forwarded = false;
-    // CUDA graphs of one full segment: recompute and the adjoint chain (by
-    // starting adjoint buffer)
-    cudaGraphExec_t g_rec[2] = {nullptr, nullptr};  // only [0] is used
-    cudaGraphExec_t g_adj[2] = {nullptr, nullptr};
-    cudaStream_t cap = nullptr;
 };
 
 namespace {
@@ -347,54 +345,24 @@ int tape_fail(tf_lbm_tape* tp, int code, const char* msg) { return handle_fail(t
         if (e_ != cudaSuccess) return handle_cuda_fail((tp)->H, e_, what);      \
     } while (0)
 
-// Recompute the len states of a segment: seg slot 0 holds the checkpoint;
-// each step writes the next slot, so no state is exported or copied.
-cudaError_t recompute(tf_lbm_tape* tp, int64_t len, cudaStream_t st)
+int64_t segment_steps(const tf_lbm_tape* tp, int c)
 {
-    char* seg = (char*)tp->seg;
-    for (int64_t i = 0; i + 1 < len; ++i) {
-        cudaError_t e = launch_step_between(tp->H, seg + i * tp->state_bytes, seg + (i + 1) * tp->state_bytes, st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return std::min<int64_t>(tp->every, tp->nsteps - (int64_t)c * tp->every);
 }
 
-// Fused adjoint steps backwards through a segment of len states, starting
-// from the adjoint state in abuf slot `from`.
-cudaError_t adjoint_chain(tf_lbm_tape* tp, int from, int64_t len, cudaStream_t st)
+// Write the records of a segment of len steps that starts at the copy c.
+cudaError_t recompute(tf_lbm_tape* tp, int c, int64_t len, cudaStream_t st)
 {
-    tf_lbm_handle* H = tp->H;
-    const size_t abytes = 9ull * H->G.nx * H->G.ny * H->esize;
-    char* seg = (char*)tp->seg;
-    char* ab = (char*)tp->abuf;
-    int cur = from;
-    for (int64_t i = len - 1; i >= 0; --i) {
-        cudaError_t e = adjoint_march_dispatch(H, seg + i * tp->state_bytes, ab + cur * abytes,
-                                               ab + (cur ^ 1) * abytes, tp->gk, st);
+    char* ck = (char*)tp->ck;
+    char* work = ck + tp->nseg * tp->state_bytes;
+    const char* from = ck + c * tp->state_bytes;
+    for (int64_t i = 0; i < len; ++i) {
+        char* to = work + (i & 1) * tp->state_bytes;
+        const cudaError_t e = launch_recorded_step(tp->H, from, to, (char*)tp->rec + i * tp->rec_bytes, st);
         if (e != cudaSuccess) return e;
-        cur ^= 1;
+        from = to;
     }
     return cudaSuccess;
-}
-
-// Capture fn into an executable graph (on the tape's own capture stream).
-template <typename Fn>
-cudaError_t capture(tf_lbm_tape* tp, cudaGraphExec_t* out, Fn fn)
-{
-    cudaError_t e;
-    if (!tp->cap && (e = cudaStreamCreateWithFlags(&tp->cap, cudaStreamNonBlocking)) != cudaSuccess) return e;
-    if ((e = cudaStreamBeginCapture(tp->cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
-    cudaError_t fe = fn(tp->cap);
-    cudaGraph_t g = nullptr;
-    e = cudaStreamEndCapture(tp->cap, &g);
-    if (fe != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return fe;
-    }
-    if (e != cudaSuccess) return e;
-    e = cudaGraphInstantiate(out, g, 0);
-    cudaGraphDestroy(g);
-    return e;
 }
 
 }  // namespace
@@ -425,24 +393,34 @@ int tf_lbm_tape_create(tf_lbm_handle* H, const void* h0, const void* theta, int6
     if (nsteps < 1) return handle_fail(H, TF_LBM_ERR_ARG, "nsteps must be >= 1");
     if (H->p.forcing != 0)
         return handle_fail(H, TF_LBM_ERR_UNSUPPORTED, "the adjoint differentiates Eq. (LBE) as printed (forcing = 0)");
-    if (every <= 0) every = (int32_t)ceil(sqrt((double)nsteps));
-    if (every > nsteps) every = (int32_t)nsteps;
+    const long long n = (long long)H->G.nx * H->G.ny;
     tf_lbm_tape* tp = new tf_lbm_tape();
     tp->H = H;
     tp->nsteps = nsteps;
-    tp->every = every;
-    tp->nck = (int)((nsteps + every - 1) / every);
     tp->state_bytes = (size_t)H->G.plane * (H->esize + 8 * H->msize);
-    const long long n = (long long)H->G.nx * H->G.ny;
+    tp->rec_bytes = 3ull * n * H->esize;
+    tp->a_bytes = (three_fields(H) ? 3ull : 9ull) * n * H->esize;
     cudaError_t e;
     auto bail = [&](cudaError_t err, const char* what) {
         int rc = handle_cuda_fail(H, err, what);
         tf_lbm_tape_destroy(tp);
         return rc;
     };
-    if ((e = cudaMalloc(&tp->ck, tp->state_bytes * (tp->nck + 1))) != cudaSuccess) return bail(e, "cudaMalloc checkpoints");
-    if ((e = cudaMalloc(&tp->seg, tp->state_bytes * every)) != cudaSuccess) return bail(e, "cudaMalloc segment");
-    if ((e = cudaMalloc(&tp->abuf, 18ull * n * H->esize)) != cudaSuccess) return bail(e, "cudaMalloc adjoint");
+    // all records where they fit (every <= 0 leaves the choice here; an
+    // explicit `every` asks for segments of that length), else segments
+    if (every <= 0 && (size_t)nsteps <= kTapeBytes / tp->rec_bytes && nsteps <= INT32_MAX &&
+        cudaMalloc(&tp->rec, tp->rec_bytes * nsteps) == cudaSuccess) {
+        tp->every = (int)nsteps;
+    } else {
+        cudaGetLastError();
+        if (every <= 0) every = (int32_t)ceil(sqrt((double)nsteps));
+        tp->every = (int)std::min<int64_t>(every, nsteps);
+        if ((e = cudaMalloc(&tp->rec, tp->rec_bytes * tp->every)) != cudaSuccess) return bail(e, "cudaMalloc records");
+    }
+    tp->nseg = (int)((nsteps + tp->every - 1) / tp->every);
+    if (tp->nseg > 1 && (e = cudaMalloc(&tp->ck, tp->state_bytes * (tp->nseg + 2))) != cudaSuccess)
+        return bail(e, "cudaMalloc checkpoints");
+    if ((e = cudaMalloc(&tp->abuf, 2 * tp->a_bytes)) != cudaSuccess) return bail(e, "cudaMalloc adjoint");
     if ((e = cudaMalloc(&tp->gk, n * H->esize)) != cudaSuccess) return bail(e, "cudaMalloc grad kappa");
     if ((e = cudaMalloc(&tp->h0, n * H->esize)) != cudaSuccess) return bail(e, "cudaMalloc h0");
     if ((e = cudaMemcpy(tp->h0, h0, n * H->esize, cudaMemcpyDeviceToDevice)) != cudaSuccess) return bail(e, "copy h0");
@@ -460,17 +438,18 @@ int tf_lbm_tape_forward(tf_lbm_tape* tp, void* stream)
     if (!tp) return handle_fail(nullptr, TF_LBM_ERR_ARG, "tape is NULL");
     tf_lbm_handle* H = tp->H;
     cudaStream_t st = (cudaStream_t)stream;
-    tp->t0 = H->time;
-    char* ck = (char*)tp->ck;
-    for (int c = 0; c < tp->nck; ++c) {
-        TK(tp, cudaMemcpyAsync(ck + c * tp->state_bytes, H->buf[H->cur], tp->state_bytes, cudaMemcpyDeviceToDevice, st),
-           "checkpoint copy");
-        const int64_t len = (c + 1 == tp->nck) ? tp->nsteps - (int64_t)c * tp->every : tp->every;
-        const int rc = tf_lbm_step(H, len, stream);
-        if (rc) return rc;
+    for (int c = 0; c < tp->nseg; ++c) {
+        if (tp->nseg > 1)
+            TK(tp, cudaMemcpyAsync((char*)tp->ck + c * tp->state_bytes, H->buf[H->cur], tp->state_bytes,
+                                   cudaMemcpyDeviceToDevice, st), "checkpoint copy");
+        const int64_t len = segment_steps(tp, c);
+        for (int64_t i = 0; i < len; ++i) {
+            TK(tp, launch_recorded_step(H, H->buf[H->cur], H->buf[H->cur ^ 1], (char*)tp->rec + i * tp->rec_bytes, st),
+               "step kernel");
+            H->cur ^= 1;
+            ++H->time;
+        }
     }
-    TK(tp, cudaMemcpyAsync(ck + tp->nck * tp->state_bytes, H->buf[H->cur], tp->state_bytes, cudaMemcpyDeviceToDevice, st),
-       "final state copy");
     tp->forwarded = true;
     return TF_LBM_OK;
 }
@@ -483,50 +462,35 @@ int tf_lbm_tape_backward(tf_lbm_tape* tp, const void* grad_h, void* grad_theta, 
     if (!grad_h) return tape_fail(tp, TF_LBM_ERR_ARG, "grad_h must not be NULL");
     cudaStream_t st = (cudaStream_t)stream;
     const long long n = (long long)H->G.nx * H->G.ny;
-    const size_t sbytes = 9ull * n * H->esize;
-    char* seg = (char*)tp->seg;
     char* ab = (char*)tp->abuf;
-    char* ck = (char*)tp->ck;
+    const bool three = three_fields(H);
     Dims D{H->G.nx, H->G.ny, n};
-    int cur = 0;  // adjoint state in ab + cur * sbytes
-    if (H->dbl) k_seed<double><<<g1(D), 256, 0, st>>>((const double*)grad_h, (double*)ab, D);
-    else k_seed<float><<<g1(D), 256, 0, st>>>((const float*)grad_h, (float*)ab, D);
+    int cur = 0;  // adjoint state in ab + cur * a_bytes
+    if (H->dbl) k_seed<double><<<g1(D), 256, 0, st>>>((const double*)grad_h, (double*)ab, (double*)tp->gk, D, three);
+    else k_seed<float><<<g1(D), 256, 0, st>>>((const float*)grad_h, (float*)ab, (float*)tp->gk, D, three);
     TK(tp, cudaGetLastError(), "seed kernel");
-    TK(tp, cudaMemsetAsync(tp->gk, 0, n * H->esize, st), "cudaMemsetAsync");
-    for (int c = tp->nck - 1; c >= 0; --c) {
-        const int64_t len = (c + 1 == tp->nck) ? tp->nsteps - (int64_t)c * tp->every : tp->every;
-        // the checkpoint starts the segment; recompute its states, then run
-        // the adjoint back through them; full segments replay captured graphs
-        TK(tp, cudaMemcpyAsync(seg, ck + c * tp->state_bytes, tp->state_bytes, cudaMemcpyDeviceToDevice, st),
-           "checkpoint restore");
-        if (len == tp->every && len > 1) {
-            const int afrom = cur;
-            if (!tp->g_rec[0])
-                TK(tp, capture(tp, &tp->g_rec[0], [&](cudaStream_t cs) { return recompute(tp, len, cs); }),
-                   "recompute graph");
-            if (!tp->g_adj[afrom])
-                TK(tp, capture(tp, &tp->g_adj[afrom], [&](cudaStream_t cs) { return adjoint_chain(tp, afrom, len, cs); }),
-                   "adjoint graph");
-            TK(tp, cudaGraphLaunch(tp->g_rec[0], st), "cudaGraphLaunch");
-            TK(tp, cudaGraphLaunch(tp->g_adj[afrom], st), "cudaGraphLaunch");
-        } else {
-            TK(tp, recompute(tp, len, st), "recompute");
-            TK(tp, adjoint_chain(tp, cur, len, st), "adjoint chain");
+    for (int c = tp->nseg - 1; c >= 0; --c) {
+        const int64_t len = segment_steps(tp, c);
+        if (tp->nseg > 1) TK(tp, recompute(tp, c, len, st), "recompute");
+        for (int64_t i = len - 1; i >= 0; --i) {
+            TK(tp, adjoint_tile_step(H, (char*)tp->rec + i * tp->rec_bytes, ab + cur * tp->a_bytes,
+                                     ab + (cur ^ 1) * tp->a_bytes, tp->gk, st), "adjoint step");
+            cur ^= 1;
         }
-        cur ^= (int)(len & 1);
     }
     if (grad_h0 || grad_theta) {
         const double kc = (double)(H->p.n_exp - 1) * (H->p.m_exp - 1) / ((double)(H->p.n_exp - H->p.m_exp) * H->p.hstar);
+        const void* a0 = ab + cur * tp->a_bytes;
         if (H->dbl)
-            k_adj_init<double><<<g1(D), 256, 0, st>>>((const double*)tp->h0, (const double*)(ab + cur * sbytes),
-                                                      (double*)grad_h0, (const double*)tp->gk, (const double*)tp->theta,
+            k_adj_init<double><<<g1(D), 256, 0, st>>>((const double*)tp->h0, (const double*)a0, (double*)grad_h0,
+                                                      (const double*)tp->gk, (const double*)tp->theta,
                                                       (double*)grad_theta, D, make_consts<double>(H), kc,
-                                                      H->p.theta_uniform);
+                                                      H->p.theta_uniform, three);
         else
-            k_adj_init<float><<<g1(D), 256, 0, st>>>((const float*)tp->h0, (const float*)(ab + cur * sbytes),
-                                                     (float*)grad_h0, (const float*)tp->gk, (const float*)tp->theta,
+            k_adj_init<float><<<g1(D), 256, 0, st>>>((const float*)tp->h0, (const float*)a0, (float*)grad_h0,
+                                                     (const float*)tp->gk, (const float*)tp->theta,
                                                      (float*)grad_theta, D, make_consts<float>(H), (float)kc,
-                                                     (float)H->p.theta_uniform);
+                                                     (float)H->p.theta_uniform, three);
         TK(tp, cudaGetLastError(), "init adjoint kernel");
     }
     return TF_LBM_OK;
@@ -536,13 +500,8 @@ void tf_lbm_tape_destroy(tf_lbm_tape* tp)
 {
     if (!tp) return;
     cudaDeviceSynchronize();
-    for (void* p : {tp->ck, tp->seg, tp->abuf, tp->gk, tp->h0, tp->theta})
+    for (void* p : {tp->ck, tp->rec, tp->abuf, tp->gk, tp->h0, tp->theta})
         if (p) cudaFree(p);
-    for (auto& g : tp->g_rec)
-        if (g) cudaGraphExecDestroy(g);
-    for (auto& g : tp->g_adj)
-        if (g) cudaGraphExecDestroy(g);
-    if (tp->cap) cudaStreamDestroy(tp->cap);
     delete tp;
 }
 

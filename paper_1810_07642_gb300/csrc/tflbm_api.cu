@@ -21,6 +21,35 @@ int sm_count()
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms;
 }
+
+// The tile kernel's block_x for a lattice (tile_of): the shape with the least
+// work on the busiest SM, counting a node's pull as 0.45 of its cost and its
+// pressure as 0.2 (the halos repeat those) and 60 nodes' worth of fixed
+// latency a tile.  In FP64 the arithmetic units are the bound and halo work
+// counts in full, so tiles are as large as keeps every SM busy.  Measured, one
+// box, us a step with block_x 64 / 128 / 256: FP32 128^2 2.9 / 3.1 / 3.3, 384^2
+// 5.0 / 4.9 / 4.3, 512^2 6.6 / 6.5 / 5.1, 1024^2 19.2 / 19.0 / 15.8; FP64 64^2 7.5 / 11.5 / 20.2, 250 x
+// 190 38 / 20.7 / 38, 768^2 158 / 156 / 151.
+int tile_block_x(int store, int nx, int ny, int sms)
+{
+    auto tiles = [&](int bx) {
+        const TileShape t = tile_of(bx);
+        return (long long)((nx + t.tx - 1) / t.tx) * ((ny + t.ty - 1) / t.ty);
+    };
+    if (store == kStoreF64) return tiles(64) <= sms ? 64 : (tiles(256) >= 7LL * sms ? 256 : 128);
+    int best = 64;
+    double least = 0;
+    for (int bx : {64, 128, 256}) {
+        const TileShape t = tile_of(bx);
+        const double work = 60 + 0.35 * t.tx * t.ty + 0.45 * (t.tx + 4) * (t.ty + 4) + 0.2 * (t.tx + 2) * (t.ty + 2);
+        const double cost = (double)((tiles(bx) + sms - 1) / sms) * work;
+        if (bx == 64 || cost < least) {
+            best = bx;
+            least = cost;
+        }
+    }
+    return best;
+}
 }  // namespace tflbm
 
 namespace {
@@ -115,35 +144,6 @@ int store_of(int dtype)
     }
 }
 
-// The tile kernel's block_x for a lattice (tile_of): the shape with the least
-// work on the busiest SM, counting a node's pull as a third of its cost and its
-// pressure as a fifth (the halos repeat those) and 40 nodes' worth of fixed
-// latency a tile.  In FP64 the arithmetic units are the bound and halo work
-// counts in full, so tiles are as large as keeps every SM busy.  Measured, one
-// box, us a step with block_x 64 / 128 / 256: FP32 128^2 3.0 / 3.1 / 3.5, 384^2
-// 5.2 / 5.1 / 4.4, 1024^2 19.4 / 19.3 / 16.3; FP64 64^2 7.5 / 11.5 / 20.2, 250 x
-// 190 38 / 20.7 / 38, 768^2 158 / 156 / 151.
-int tile_block_x(int store, int nx, int ny, int sms)
-{
-    auto tiles = [&](int bx) {
-        const TileShape t = tile_of(bx);
-        return (long long)((nx + t.tx - 1) / t.tx) * ((ny + t.ty - 1) / t.ty);
-    };
-    if (store == kStoreF64) return tiles(64) <= sms ? 64 : (tiles(256) >= 7LL * sms ? 256 : 128);
-    int best = 64;
-    double least = 0;
-    for (int bx : {64, 128, 256}) {
-        const TileShape t = tile_of(bx);
-        const double work = 40 + 0.45 * t.tx * t.ty + 0.35 * (t.tx + 4) * (t.ty + 4) + 0.2 * (t.tx + 2) * (t.ty + 2);
-        const double cost = (double)((tiles(bx) + sms - 1) / sms) * work;
-        if (bx == 64 || cost < least) {
-            best = bx;
-            least = cost;
-        }
-    }
-    return best;
-}
-
 // Lattices up to this many nodes run the tile kernel with an FP32 compute type
 // (FP64: all).  Above it the marches win: they pull a node 1.3 times, not 1.4,
 // and prefetch from HBM.  One box, us a step, tile against march: 1024^2 FP32
@@ -168,14 +168,13 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     // bound; 16-bit storage uses it at 64 columns per CTA (one warp), FP32 at
     // 128.  At tau != 1 the one-column kernel is faster in every storage type
     // (the two-column kernel's pulled-population ring costs resident warps)
-    const int store = store_of(p.dtype);
+    const int store = store_of(p.dtype), sms = sm_count();
     const bool om1 = p.tau == 1.0;
-    if (store == kStoreF64 || (long long)G.nx * G.ny <= kTileNodes) s.tile = tile_block_x(store, G.nx, G.ny, sm_count());
+    if (store == kStoreF64 || (long long)G.nx * G.ny <= kTileNodes) s.tile = tile_block_x(store, G.nx, G.ny, sms);
     const bool narrow = store == kStoreF16 || store == kStoreBF16;
     const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     s.block_x = pair ? (narrow ? 64 : 128) : (G.nx >= 1024 ? 128 : 64);
     const int strips = (G.nx + s.block_x - 5) / (s.block_x - 4);  // CTAs overlap by 4 columns
-    const int sms = sm_count();
     // otherwise per-thread loads: measured faster than the bulk-copy pipeline
     // on GB300 once loads are prefetched a row ahead
     s.pipeline = pair ? kPipePair : kPipeLdg;
@@ -246,11 +245,12 @@ cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st)
                        H->shape, st);
 }
 
-cudaError_t launch_step_between(tf_lbm_handle* H, const void* fin, void* fout, cudaStream_t st)
+cudaError_t launch_recorded_step(tf_lbm_handle* H, const void* fin, void* fout, void* mom, cudaStream_t st)
 {
     const Consts<float> c32 = make_consts<float>(H);
     const Consts<double> c64 = make_consts<double>(H);
-    return launch_step(H->desc.store, fin, fout, H->kappa, H->G, &c32, &c64, H->shape, st);
+    const int bx = tile_block_x(H->desc.store, H->G.nx, H->G.ny, H->sms);
+    return launch_tile(H->desc.store, bx, fin, fout, H->kappa, mom, H->G, &c32, &c64, st);
 }
 
 template Consts<float> make_consts<float>(const tf_lbm_handle*);
@@ -297,6 +297,7 @@ int tf_lbm_init(tf_lbm_handle** out, const tf_lbm_params* params, const void* h0
         return fail(nullptr, TF_LBM_ERR_UNSUPPORTED,
                     "lattice too large: 9 * ny * pitch must stay below 2^31 elements");
     }
+    H->sms = sm_count();
     H->shape = default_shape(*params, H->G, theta != nullptr);
     H->graph_chunk = ((long long)params->nx * params->ny <= (1LL << 20)) ? 64 : 0;
 

@@ -126,9 +126,9 @@ cudaError_t pair_step_f16(int block_x, const void* fin, void* fout, const void* 
                           const Consts<float>& C, int bands, cudaStream_t st);
 cudaError_t pair_step_bf16(int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
                            const Consts<float>& C, int bands, cudaStream_t st);
-// The tile step (tile_*.cu).
-cudaError_t launch_tile(int store, int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
-                        const Consts<float>* C32, const Consts<double>* C64, cudaStream_t st);
+// The tile step (tile_*.cu); mom: see tile_step, or null.
+cudaError_t launch_tile(int store, int block_x, const void* fin, void* fout, const void* kappa, void* mom,
+                        const Geom& G, const Consts<float>* C32, const Consts<double>* C64, cudaStream_t st);
 int pair_blocks_per_sm_f32(int block_x, bool omega1, bool kfield);
 int pair_blocks_per_sm_f16(int block_x, bool omega1, bool kfield);
 int pair_blocks_per_sm_bf16(int block_x, bool omega1, bool kfield);

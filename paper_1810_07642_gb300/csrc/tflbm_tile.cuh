@@ -40,6 +40,32 @@ template <int K> __device__ __forceinline__ float& lane_of(float2& x)
 }
 template <int K> __device__ __forceinline__ double& lane_of(double& x) { return x; }
 
+// Position of node i of the halo of depth D around a TX x TY tile: D rows
+// below and above over the whole width, then the columns on both sides.
+template <int TX, int TY, int D>
+__device__ __forceinline__ void tile_halo(int i, int& c, int& r)
+{
+    constexpr int W = TX + 2 * D;
+    if (i < 2 * D * W) {
+        const int k = i / W;
+        c = i % W - D;
+        r = k < D ? k - D : TY + k - D;
+    } else {
+        const int k = (i - 2 * D * W) % (2 * D);
+        r = (i - 2 * D * W) / (2 * D);
+        c = k < D ? k - D : TX + k - D;
+    }
+}
+
+// Lane K of the window around element b of rows w wide.
+template <int K, typename S, typename X>
+__device__ __forceinline__ void tile_window(const S* b, int w, Win<X>& W)
+{
+    lane_of<K>(W.nL) = b[w - 1]; lane_of<K>(W.n0) = b[w]; lane_of<K>(W.nR) = b[w + 1];
+    lane_of<K>(W.cL) = b[-1]; lane_of<K>(W.c0) = b[0]; lane_of<K>(W.cR) = b[1];
+    lane_of<K>(W.sL) = b[-w - 1]; lane_of<K>(W.s0) = b[-w]; lane_of<K>(W.sR) = b[-w + 1];
+}
+
 // Moments of pulled populations in storage units (the sums of step_band2).
 template <typename SM, typename X>
 __device__ __forceinline__ void node_moments(X f0, const X (&n)[8], const Consts<typename Lanes<X>::S>& C, X& dh, X& er,
@@ -63,7 +89,7 @@ __device__ __forceinline__ void node_moments(X f0, const X (&n)[8], const Consts
 template <typename SM, typename S, int TX, int TY, bool OMEGA1, int RESIDENT>
 __global__ void __launch_bounds__(TX* TY / Lanes<typename TileX<S>::X>::N, RESIDENT / (TX * TY / Lanes<typename TileX<S>::X>::N))
 k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ fout0, SM* __restrict__ foutm,
-       const S* __restrict__ kappa, const Geom G, const Consts<S> C)
+       const S* __restrict__ kappa, S* __restrict__ mom, const Geom G, const Consts<S> C)
 {
     using X = typename TileX<S>::X;
     using IO = PairIO<SM>;
@@ -74,6 +100,7 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     constexpr int HN = HW * (TY + 4) - TX * TY, PN = PW * (TY + 2) - TX * TY;
     constexpr int HP = HN / N, PP = PN / N;
     static_assert(HN % N == 0 && PN % N == 0 && TY % N == 0, "halo nodes come in whole groups");
+    static_assert(HP <= NT && PP <= NT, "one group of halo nodes a thread");
     __shared__ S hs[TY + 4][HW];  // h - href; tile node (c, r) at [r + 2][c + 2]
     __shared__ S ps[TY + 2][PW];  // p; tile node (c, r) at [r + 1][c + 1]
 
@@ -109,26 +136,10 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
         (void)nk;
         return ldro(kappa + TFLBM_IDX(ring_index(y0 + rr, ny) * nx + ring_index(x0 + cc, nx), nk, C.status));
     };
-    // position of node i of the halo of depth D (two rings: D rows above and
-    // below over the whole width, then the columns on both sides)
-    auto halo = [&](auto d_c, int i, int& cc, int& rr) {
-        constexpr int D = decltype(d_c)::value, FW = TX + 2 * D;
-        if (i < 2 * D * FW) {
-            const int k = i / FW;
-            cc = i % FW - D;
-            rr = k < D ? k - D : TY + k - D;
-        } else {
-            const int k = (i - 2 * D * FW) % (2 * D);
-            rr = (i - 2 * D * FW) / (2 * D);
-            cc = k < D ? k - D : TX + k - D;
-        }
-    };
     auto lanes = [&](auto fn) {
         fn(std::integral_constant<int, 0>{});
         if constexpr (N == 2) fn(std::integral_constant<int, 1>{});
     };
-    using D2 = std::integral_constant<int, 2>;
-    using D1 = std::integral_constant<int, 1>;
 
     // ---- h and j of the tile, h of the halo of 2
     X f0, n[8], dh, er, jx, jy, kap, ih;
@@ -137,12 +148,22 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
         pull(k_c, c, r + K * HALF, f0, n);
         lane_of<K>(kap) = kap_at(c, r + K * HALF);
     });
-    for (int i = t; i < HP; i += NT) {
+    // kappa of the halo of 1, requested here so that phase 2 waits for no load
+    X kh;
+    int pc[N], pr[N];
+    if (t < PP) {
+        lanes([&](auto k_c) {
+            constexpr int K = decltype(k_c)::value;
+            tile_halo<TX, TY, 1>(t + K * PP, pc[K], pr[K]);
+            lane_of<K>(kh) = kap_at(pc[K], pr[K]);
+        });
+    }
+    if (t < HP) {
         X g0, g[8], d, e, a, b;
         int cc[N], rr[N];
         lanes([&](auto k_c) {
             constexpr int K = decltype(k_c)::value;
-            halo(D2{}, i + K * HP, cc[K], rr[K]);
+            tile_halo<TX, TY, 2>(t + K * HP, cc[K], rr[K]);
             pull(k_c, cc[K], rr[K], g0, g);
         });
         node_moments<SM>(g0, g, C, d, e, a, b);
@@ -155,21 +176,23 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     lanes([&](auto k_c) {
         constexpr int K = decltype(k_c)::value;
         hs[r + K * HALF + 2][c + 2] = lane_of<K>(dh);
+        const int x = x0 + c, y = y0 + r + K * HALF;
+        if (mom && x < nx && y < ny) {
+            const long long nn = (long long)nx * ny;
+            S* m = mom + (y * nx + x);
+            m[0] = lane_of<K>(dh);
+            m[nn] = lane_of<K>(jx);
+            m[2 * nn] = lane_of<K>(jy);
+        }
     });
     __syncthreads();
 
     // ---- film pressure of the tile and the halo of 1
-    auto window = [&](auto k_c, const S* b, int w, Win<X>& W) {  // around element b of rows w wide
-        constexpr int K = decltype(k_c)::value;
-        lane_of<K>(W.nL) = b[w - 1]; lane_of<K>(W.n0) = b[w]; lane_of<K>(W.nR) = b[w + 1];
-        lane_of<K>(W.cL) = b[-1]; lane_of<K>(W.c0) = b[0]; lane_of<K>(W.cR) = b[1];
-        lane_of<K>(W.sL) = b[-w - 1]; lane_of<K>(W.s0) = b[-w]; lane_of<K>(W.sR) = b[-w + 1];
-    };
     {
         Win<X> W;
         lanes([&](auto k_c) {
             constexpr int K = decltype(k_c)::value;
-            window(k_c, &hs[r + K * HALF + 2][c + 2], HW, W);
+            tile_window<K>(&hs[r + K * HALF + 2][c + 2], HW, W);
         });
         X p = node_pressure(W, kap, disj, C, ih);
         lanes([&](auto k_c) {
@@ -177,20 +200,17 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
             ps[r + K * HALF + 1][c + 1] = lane_of<K>(p);
         });
     }
-    for (int i = t; i < PP; i += NT) {
+    if (t < PP) {
         Win<X> W;
-        X kh, q;
-        int cc[N], rr[N];
+        X q;
         lanes([&](auto k_c) {
             constexpr int K = decltype(k_c)::value;
-            halo(D1{}, i + K * PP, cc[K], rr[K]);
-            lane_of<K>(kh) = kap_at(cc[K], rr[K]);
-            window(k_c, &hs[rr[K] + 2][cc[K] + 2], HW, W);
+            tile_window<K>(&hs[pr[K] + 2][pc[K] + 2], HW, W);
         });
         X p = node_pressure(W, kh, disj, C, q);
         lanes([&](auto k_c) {
             constexpr int K = decltype(k_c)::value;
-            ps[rr[K] + 1][cc[K] + 1] = lane_of<K>(p);
+            ps[pr[K] + 1][pc[K] + 1] = lane_of<K>(p);
         });
     }
     __syncthreads();
@@ -199,7 +219,7 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     Win<X> W;
     lanes([&](auto k_c) {
         constexpr int K = decltype(k_c)::value;
-        window(k_c, &ps[r + K * HALF + 1][c + 1], PW, W);
+        tile_window<K>(&ps[r + K * HALF + 1][c + 1], PW, W);
     });
     node_collide<SM, OMEGA1>(W, dh, ih, jx, jy, er, n, 1, C, [&](X o0, const V(&q)[8]) {
         const int x = x0 + c;
@@ -224,15 +244,15 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
 }
 
 template <typename SM, typename S, int TX, int TY>
-cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, const Geom& G, const Consts<S>& C,
-                     cudaStream_t st)
+cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S* mom, const Geom& G,
+                     const Consts<S>& C, cudaStream_t st)
 {
     constexpr int NT = TX * TY / Lanes<typename TileX<S>::X>::N;
     const dim3 grid((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY);
     auto launch = [&](auto resident) {
         constexpr int R = decltype(resident)::value;
-        if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, G, C);
-        return launch_dependent(k_tile<SM, S, TX, TY, false, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, G, C);
+        if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, G, C);
+        return launch_dependent(k_tile<SM, S, TX, TY, false, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, G, C);
     };
     // Threads an SM holds.  512 leaves the registers that keep a thread's 18
     // loads in flight (80); where 32 x 16 tiles outnumber the three an SM
@@ -245,20 +265,23 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, c
     return launch(std::integral_constant<int, 512>{});
 }
 
-// One step from fin to fout in the tiles that block_x names (tile_of).
+// One step from fin to fout in the tiles that block_x names (tile_of); mom, if
+// not null, receives (h - href, j_x, j_y) of the state that fin pulls to,
+// [3][ny][nx] (the gradient tape's record of the step).
 template <typename SM, typename S>
-cudaError_t tile_step(int block_x, const void* fin, void* fout, const void* kappa, const Geom& G, const Consts<S>& C,
-                      cudaStream_t st)
+cudaError_t tile_step(int block_x, const void* fin, void* fout, const void* kappa, void* mom, const Geom& G,
+                      const Consts<S>& C, cudaStream_t st)
 {
     const S* f0 = (const S*)fin;
     const SM* fm = (const SM*)((const char*)fin + G.plane * sizeof(S));
     S* g0 = (S*)fout;
     SM* gm = (SM*)((char*)fout + G.plane * sizeof(S));
     const S* k = (const S*)kappa;
+    S* m = (S*)mom;
     switch (block_x) {
-        case 64: return tile_one<SM, S, 16, 8>(f0, fm, g0, gm, k, G, C, st);
-        case 128: return tile_one<SM, S, 16, 16>(f0, fm, g0, gm, k, G, C, st);
-        case 256: return tile_one<SM, S, 32, 16>(f0, fm, g0, gm, k, G, C, st);
+        case 64: return tile_one<SM, S, 16, 8>(f0, fm, g0, gm, k, m, G, C, st);
+        case 128: return tile_one<SM, S, 16, 16>(f0, fm, g0, gm, k, m, G, C, st);
+        case 256: return tile_one<SM, S, 32, 16>(f0, fm, g0, gm, k, m, G, C, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -3,16 +3,16 @@
 
 namespace tflbm {
 
-cudaError_t tile_step_narrow(int store, int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
+cudaError_t tile_step_narrow(int store, int block_x, const void* fin, void* fout, const void* kappa, void* mom, const Geom& G,
                              const Consts<float>& C, cudaStream_t st);
 
-cudaError_t launch_tile(int store, int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
-                        const Consts<float>* C32, const Consts<double>* C64, cudaStream_t st)
+cudaError_t launch_tile(int store, int block_x, const void* fin, void* fout, const void* kappa, void* mom,
+                        const Geom& G, const Consts<float>* C32, const Consts<double>* C64, cudaStream_t st)
 {
     switch (store) {
-        case kStoreF32: return tile_step<float, float>(block_x, fin, fout, kappa, G, *C32, st);
-        case kStoreF64: return tile_step<double, double>(block_x, fin, fout, kappa, G, *C64, st);
-        default: return tile_step_narrow(store, block_x, fin, fout, kappa, G, *C32, st);
+        case kStoreF32: return tile_step<float, float>(block_x, fin, fout, kappa, mom, G, *C32, st);
+        case kStoreF64: return tile_step<double, double>(block_x, fin, fout, kappa, mom, G, *C64, st);
+        default: return tile_step_narrow(store, block_x, fin, fout, kappa, mom, G, *C32, st);
     }
 }
 

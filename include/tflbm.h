@@ -145,10 +145,14 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            asynchronous copies, two rows ahead (TF_LBM_F32 and TF_LBM_F64
  *            only); 0 = row segments streamed into shared memory by bulk
  *            copies four rows ahead (needs nx a multiple of 8, >= 16).
- * On lattices of up to 1.5 x 2^20 nodes, and for TF_LBM_F64 on all, the shape
- * chosen by tf_lbm_init runs tiles in place of the bands that its fields
- * describe, and so does the one chosen by tf_lbm_tune where tiles were the
- * fastest; passing the fields to tf_lbm_set_launch gives the bands.
+ * The shape chosen by tf_lbm_init runs other kernels in place of the one that
+ * its fields describe: tiles on lattices of up to 2^20 nodes (1.5 x 2^20 where
+ * the next one does not apply; for TF_LBM_F64 on all); above that, at tau = 1
+ * with forcing = 0, a march of four columns per thread, which between the
+ * steps of one call keeps moments in place of FP32 populations (16-bit storage:
+ * where nx is a multiple of 4).  So does the shape chosen by tf_lbm_tune where
+ * one of them was the fastest.  Passing the fields to tf_lbm_set_launch gives
+ * what they describe.
  * Results do not depend on rows or graph_chunk; the pipelines agree to
  * rounding. */
 typedef struct tf_lbm_launch {
@@ -259,8 +263,8 @@ void tf_lbm_tape_destroy(tf_lbm_tape* tape);
  * `stream`.  Candidates: block_x in {64, 128, 256}, every pipeline that
  * applies, and band counts of one, two and three waves of resident CTAs
  * (both balanced bands filling the waves exactly and their rounded-up band
- * heights) and band heights of 2 to 256 rows, then tiles of every block_x in
- * place of the fastest of these.  The state is copied aside first (one population
+ * heights) and band heights of 2 to 256 rows, then tiles of every block_x and
+ * the four-column march in place of the fastest of these.  The state is copied aside first (one population
  * buffer of device memory, freed before return) and put back after, so f
  * and tf_lbm_time are as before the call.  The graph chunk is kept.
  * Synchronises `stream`.  best (host, may be NULL) receives the shape now in
@@ -336,7 +340,8 @@ typedef struct tf_lbm_batch tf_lbm_batch;
  *   pipeline: 1 = one column per thread; 3 = two columns per thread, as in
  *            tf_lbm_launch (every domain's nx even, not TF_LBM_F64).  The
  *            default is 3 where it applies and every tau is 1 (as for a
- *            single handle), else 1.  Both run the node arithmetic of the
+ *            single handle), else 1; a default or tuned batch of pipeline 3
+ *            may run the four-column march in its place, see tf_lbm_launch.  Both run the node arithmetic of the
  *            single-handle kernel of the same pipeline. */
 typedef struct tf_lbm_batch_launch {
     int32_t block_x;

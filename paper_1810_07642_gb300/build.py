@@ -22,8 +22,8 @@ LIB = os.path.join(BUILD, f"libtflbm_{platform.machine()}.so")
 # kernels is checked; a bad one sets TF_LBM_STATUS_BOUNDS instead of trapping
 LIB_CHECKED = os.path.join(BUILD, f"libtflbm_checked_{platform.machine()}.so")
 SOURCES = ["tflbm_api.cu", "tflbm_aux.cu", "step_f32.cu", "step_f16.cu", "step2_f32.cu", "step2_f16.cu",
-           "step2_bf16.cu", "tile_f32.cu", "tile_f16.cu", "tflbm_adjoint.cu", "tflbm_noalloc.cu", "tflbm_batch.cu"]
-HEADERS = ["tflbm_internal.h", "tflbm_step.cuh", "tflbm_node.cuh", "tflbm_step2.cuh", "tflbm_tile.cuh", "tflbm_adjoint_tile.cuh", "tflbm_handle.h"]
+           "step2_bf16.cu", "tile_f32.cu", "tile_f16.cu", "step4.cu", "tflbm_adjoint.cu", "tflbm_noalloc.cu", "tflbm_batch.cu"]
+HEADERS = ["tflbm_internal.h", "tflbm_step.cuh", "tflbm_node.cuh", "tflbm_step2.cuh", "tflbm_tile.cuh", "tflbm_step4.cuh", "tflbm_adjoint_tile.cuh", "tflbm_handle.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          f"-I{os.path.join(ROOT, 'include')}"]

@@ -144,16 +144,16 @@ int store_of(int dtype)
     }
 }
 
-// Lattices up to this many nodes run the tile kernel with an FP32 compute type
-// (FP64: all).  Above it the marches win: they pull a node 1.3 times, not 1.4,
-// and prefetch from HBM.  One box, us a step, tile against march: 1024^2 FP32
-// 16.3 / 34.1 (18.5 with 4-row bands), FP16 18.4 / 32.2; 1448^2 FP32 36.7 /
-// 38.7, FP16 40.0 / 36.1, FP32 at tau = 0.8 39.8 / 37.1; 2048^2 FP32 65 / 52.7;
-// FP64 2048^2 1014 / 1101.
-constexpr long long kTileNodes = 3LL << 19;
+// Lattices up to this many nodes run the tile kernel (FP64: all of them).  Above
+// it the marches win: they pull a node 1.25 times, not 1.4, and load ahead.  One
+// box, us a step, tile against the four-column march: 900^2 FP32 12.5 / 12.2,
+// 1024^2 15.9 / 16.4, 1300 x 1100 25.4 / 17.5, 1448^2 36.3 / 21.6; FP16 1024^2
+// 16.1 / 16.4, 1448^2 34.3 / 21.4; against the one-column march at tau = 0.8:
+// 1024^2 18.4 / 24.9, 1448^2 39.8 / 37.1, 2048^2 73 / 63; FP64 2048^2 1014 / 1101.
+constexpr long long kTileNodes = 1LL << 20, kTileNodesOneColumn = 3LL << 19;
 
-// Default launch shape: tiles on lattices that L2 holds.  The other fields
-// describe the march that a larger lattice would run, and that the caller gets
+// Default launch shape: tiles on lattices that L2 holds, the four-column march
+// on larger ones at tau = 1.  The other fields describe the march that a larger lattice would run, and that the caller gets
 // back by setting them: the two-column kernel at tau = 1 where it applies
 // (CTAs 64 columns wide for 16-bit storage, 128 for FP32), else the one-column kernel
 // with CTAs 128 columns wide (64 on lattices narrower than 1024), and
@@ -170,7 +170,11 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     // (the two-column kernel's pulled-population ring costs resident warps)
     const int store = store_of(p.dtype), sms = sm_count();
     const bool om1 = p.tau == 1.0;
-    if (store == kStoreF64 || (long long)G.nx * G.ny <= kTileNodes) s.tile = tile_block_x(store, G.nx, G.ny, sms);
+    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G);
+    if (store == kStoreF64 || (long long)G.nx * G.ny <= (wide ? kTileNodes : kTileNodesOneColumn))
+        s.tile = tile_block_x(store, G.nx, G.ny, sms);
+    else if (wide)
+        s.wide = wide_bands(G, wide_slots(store, G.nx % 4 == 0, sms));
     const bool narrow = store == kStoreF16 || store == kStoreBF16;
     const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     s.block_x = pair ? (narrow ? 64 : 128) : (G.nx >= 1024 ? 128 : 64);
@@ -236,11 +240,21 @@ Consts<T> make_consts(const tf_lbm_handle* H)
     return C;
 }
 
-cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st)
+cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st, bool first, bool last)
 {
     Consts<float> c32 = make_consts<float>(H);
     Consts<double> c64 = make_consts<double>(H);
     c32.flip = c64.flip = from & 1;
+    if (H->shape.wide) {
+        const bool f32 = H->desc.store == kStoreF32;
+        if (!(f32 && first && last))
+            return launch_wide(H->desc.store, f32 && !first, f32 && !last, H->buf[from], H->buf[from ^ 1], H->kappa, H->G,
+                               c32, H->shape.wide, st);
+        // A run of one FP32 step has no moments to keep: the two-column march
+        // (2048^2: 53 against 56 us), or tiles where nx is odd; same bits.
+        if (!pair_pipeline_ok(H->G.nx, kStoreF32))
+            return launch_tile(H->desc.store, 256, H->buf[from], H->buf[from ^ 1], H->kappa, nullptr, H->G, &c32, &c64, st);
+    }
     return launch_step(H->desc.store, H->buf[from], H->buf[from ^ 1], H->kappa, H->G, &c32, &c64,
                        H->shape, st);
 }
@@ -375,7 +389,8 @@ int tf_lbm_step(tf_lbm_handle* H, int64_t nsteps, void* stream)
                 if (!H->cap) CK(H, cudaStreamCreateWithFlags(&H->cap, cudaStreamNonBlocking), "cudaStreamCreate");
                 CK(H, cudaStreamBeginCapture(H->cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
                 cudaError_t le = cudaSuccess;
-                for (int i = 0; i < chunk && le == cudaSuccess; ++i) le = launch_one_step(H, H->cur ^ (i & 1), H->cap);
+                for (int i = 0; i < chunk && le == cudaSuccess; ++i)
+                    le = launch_one_step(H, H->cur ^ (i & 1), H->cap, i == 0, i == chunk - 1);
                 cudaGraph_t g = nullptr;
                 cudaError_t ce = cudaStreamEndCapture(H->cap, &g);
                 if (le != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(H, le, "step kernel (capture)"); }
@@ -388,10 +403,12 @@ int tf_lbm_step(tf_lbm_handle* H, int64_t nsteps, void* stream)
             nsteps -= chunk;
             H->time += chunk;
         } else {
-            CK(H, launch_one_step(H, H->cur, st), "step kernel");
-            H->cur ^= 1;
-            --nsteps;
-            ++H->time;
+            // one run of all the steps that no graph takes
+            for (const int64_t n = nsteps; nsteps > 0; --nsteps) {
+                CK(H, launch_one_step(H, H->cur, st, nsteps == n, nsteps == 1), "step kernel");
+                H->cur ^= 1;
+                ++H->time;
+            }
         }
     }
     return TF_LBM_OK;
@@ -514,6 +531,7 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
     H->shape.rows = in->rows;
     H->shape.bands = 0;
     H->shape.tile = in->pipeline == kPipeTile ? bx : 0;
+    H->shape.wide = 0;
     H->graph_chunk = in->graph_chunk;
     return TF_LBM_OK;
 }

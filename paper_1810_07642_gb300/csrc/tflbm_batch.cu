@@ -46,6 +46,11 @@ struct tf_lbm_batch {
     int* queue = nullptr;  // item counter and finished-CTA counter (zero between launches)
     int grid = 0;
     tf_lbm_batch_launch L{64, 64, 0, 0, kPipeLdg};
+    // the four-column march in place of L's kernel (omega == 1 and forcing == 0
+    // everywhere, every nx even): its items, and whether it is in use
+    bool wide_ok = false, wide_quad = false, wide = false;
+    BatchItem* witems = nullptr;
+    int nwide = 0;
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     double* dpart = nullptr;  // diagnostics partials
@@ -210,8 +215,48 @@ int write_items(tf_lbm_batch* B, const tf_lbm_batch_launch& L, cudaStream_t st)
     return TF_LBM_OK;
 }
 
-cudaError_t launch_batch(tf_lbm_batch* B, int parity, cudaStream_t st)
+// Build the work items of the four-column march: the smallest band height
+// whose items fit in the GPU's slots.
+int write_wide_items(tf_lbm_batch* B, cudaStream_t st)
 {
+    const int slots = wide_slots(B->store, B->wide_quad, sm_count());
+    auto count = [&](int rows) {
+        long long n = 0;
+        for (auto* H : B->hs) n += (long long)wide_strips(H->G.nx) * bands_of(H->G.ny, rows);
+        return n;
+    };
+    int ymax = 8;
+    for (auto* H : B->hs) ymax = std::max(ymax, H->G.ny);
+    int lo = 8, hi = ymax;  // count decreases as rows grows
+    while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (count(mid) <= slots) hi = mid;
+        else lo = mid + 1;
+    }
+    const long long n = count(lo);
+    if (n > (1LL << 30)) return bfail(B, TF_LBM_ERR_ARG, "too many work items");
+    std::vector<BatchItem> host;
+    host.reserve((size_t)n);
+    for (int d = 0; d < (int)B->hs.size(); ++d) {
+        const Geom& G = B->hs[d]->G;
+        const int ns = wide_strips(G.nx), nb = bands_of(G.ny, lo);
+        for (int b = 0; b < nb; ++b)
+            for (int s = 0; s < ns; ++s) host.push_back(BatchItem{d, s, b, nb});
+    }
+    BCK(B, cudaMalloc(&B->witems, n * sizeof(BatchItem)), "cudaMalloc items");
+    BCK(B, cudaMemcpyAsync(B->witems, host.data(), n * sizeof(BatchItem), cudaMemcpyHostToDevice, st),
+        "cudaMemcpyAsync items");
+    B->nwide = (int)n;
+    return TF_LBM_OK;
+}
+
+// One step of a run; first, last: see launch_one_step.
+cudaError_t launch_batch(tf_lbm_batch* B, int parity, cudaStream_t st, bool first, bool last)
+{
+    const bool f32 = B->store == kStoreF32;
+    if (B->wide && !(f32 && first && last))
+        return launch_wide_batch(B->store, f32 && !first, f32 && !last, B->wide_quad, B->witems, B->nwide, B->doms,
+                                 parity, st);
     BatchLaunch q{};
     q.block_x = B->L.block_x;
     q.pair = B->L.pipeline == kPipePair;
@@ -256,9 +301,10 @@ int apply_launch(tf_lbm_batch* B, const tf_lbm_batch_launch& L, cudaStream_t st)
 int time_batch(tf_lbm_batch* B, int steps, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, float* ms)
 {
     int parity = B->phase;
-    for (int i = 0; i < 2; ++i, parity ^= 1) BCK(B, launch_batch(B, parity, st), "batched step (tuning)");
+    for (int i = 0; i < 2; ++i, parity ^= 1) BCK(B, launch_batch(B, parity, st, i == 0, false), "batched step (tuning)");
     BCK(B, cudaEventRecord(e0, st), "cudaEventRecord");
-    for (int i = 0; i < steps; ++i, parity ^= 1) BCK(B, launch_batch(B, parity, st), "batched step (tuning)");
+    for (int i = 1; i <= steps; ++i, parity ^= 1)
+        BCK(B, launch_batch(B, parity, st, false, i == steps), "batched step (tuning)");
     BCK(B, cudaEventRecord(e1, st), "cudaEventRecord");
     BCK(B, cudaEventSynchronize(e1), "cudaEventSynchronize");
     BCK(B, cudaEventElapsedTime(ms, e0, e1), "cudaEventElapsedTime");
@@ -367,21 +413,26 @@ int tf_lbm_tune(tf_lbm_handle* H, int32_t trial_steps, tf_lbm_launch* best, void
         H->shape = s;
         int from = H->cur;
         cudaError_t r = cudaSuccess;
-        for (int i = 0; i < 2 && r == cudaSuccess; ++i, from ^= 1) r = launch_one_step(H, from, st);
+        for (int i = 0; i < 2 && r == cudaSuccess; ++i, from ^= 1) r = launch_one_step(H, from, st, i == 0, false);
         if (r == cudaSuccess) r = cudaEventRecord(e0, st);
-        for (int i = 0; i < steps && r == cudaSuccess; ++i, from ^= 1) r = launch_one_step(H, from, st);
+        for (int i = 1; i <= steps && r == cudaSuccess; ++i, from ^= 1) r = launch_one_step(H, from, st, false, i == steps);
         if (r == cudaSuccess) r = cudaEventRecord(e1, st);
         if (r == cudaSuccess) r = cudaEventSynchronize(e1);
         if (r == cudaSuccess) r = cudaEventElapsedTime(ms, e0, e1);
         return r == cudaSuccess ? TF_LBM_OK : handle_cuda_fail(H, r, "step kernel (tuning)");
     };
-    // the fastest march, then tiles in its place if they beat it
+    // the fastest of these, then tiles or the four-column march in its place
+    // if they beat it
     const int k = pick_fastest(cands, time_one, &rc);
     std::vector<Shape> tiles;
     for (int bx : {0, 64, 128, 256}) {
         if (rc) break;
         tiles.push_back(cands[k]);
         tiles.back().tile = bx;
+    }
+    if (!rc && om1 && H->p.forcing == 0 && wide_applies(H->desc.store, H->G)) {
+        tiles.push_back(cands[k]);
+        tiles.back().wide = wide_bands(H->G, wide_slots(H->desc.store, H->G.nx % 4 == 0, sms));
     }
     const int kt = rc ? -1 : pick_fastest(tiles, time_one, &rc);
     if (rc) {
@@ -390,7 +441,7 @@ int tf_lbm_tune(tf_lbm_handle* H, int32_t trial_steps, tf_lbm_launch* best, void
     }
     H->shape = tiles[kt];
     if (H->shape.block_x != old.block_x || H->shape.rows != old.rows || H->shape.pipeline != old.pipeline ||
-        H->shape.bands != old.bands || H->shape.tile != old.tile)
+        H->shape.bands != old.bands || H->shape.tile != old.tile || H->shape.wide != old.wide)
         handle_drop_graphs(H);
     if (best) {
         best->block_x = H->shape.block_x;
@@ -485,6 +536,7 @@ void tf_lbm_batch_destroy(tf_lbm_batch* B)
         if (p) cudaFree(p);
     if (B->doms) cudaFree(B->doms);
     if (B->items) cudaFree(B->items);
+    if (B->witems) cudaFree(B->witems);
     if (B->queue) cudaFree(B->queue);
     if (B->dpart) cudaFree(B->dpart);
     if (B->dtrig) cudaFree(B->dtrig);
@@ -513,11 +565,15 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     B->kfill.assign(count, nullptr);
     B->om1 = true;
     B->pair_ok = !B->dbl;
+    B->wide_ok = B->wide_quad = true;
     for (auto* H : B->hs) {
         B->kf |= H->kappa != nullptr;
         B->om1 &= B->dbl ? make_consts<double>(H).omega == 1.0 : make_consts<float>(H).omega == 1.0f;
         B->pair_ok &= pair_pipeline_ok(H->G.nx, B->store);
+        B->wide_ok &= H->p.forcing == 0 && wide_applies(B->store, H->G);
+        B->wide_quad &= H->G.nx % 4 == 0;
     }
+    B->wide_ok = B->wide_ok && B->pair_ok && B->om1;
     auto bail = [&](int code) {
         set_thread_error(B->err);
         tf_lbm_batch_destroy(B);
@@ -571,11 +627,13 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     L.graph_chunk = nodes <= (1LL << 20) ? 64 : 0;
     L.queue = 0;
     if ((rc = apply_launch(B, L, st))) return bail(rc);
+    if (B->wide_ok && (rc = write_wide_items(B, st))) return bail(rc);
+    B->wide = B->wide_ok;
     *out = B;
     return TF_LBM_OK;
 }
 
-int32_t tf_lbm_batch_items(const tf_lbm_batch* B) { return B ? B->nitems : -1; }
+int32_t tf_lbm_batch_items(const tf_lbm_batch* B) { return B ? (B->wide ? B->nwide : B->nitems) : -1; }
 
 int tf_lbm_batch_get_launch(const tf_lbm_batch* B, tf_lbm_batch_launch* out)
 {
@@ -591,6 +649,7 @@ int tf_lbm_batch_set_launch(tf_lbm_batch* B, const tf_lbm_batch_launch* in)
     if (rc) return rc;
     // the work-item table is rewritten in place: let launches that read it finish
     BCK(B, cudaDeviceSynchronize(), "cudaDeviceSynchronize");
+    B->wide = false;
     return apply_launch(B, *in, nullptr);
 }
 
@@ -609,7 +668,8 @@ int tf_lbm_batch_step(tf_lbm_batch* B, int64_t nsteps, void* stream)
                 if (!B->cap) BCK(B, cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking), "cudaStreamCreate");
                 BCK(B, cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
                 cudaError_t le = cudaSuccess;
-                for (int i = 0; i < chunk && le == cudaSuccess; ++i) le = launch_batch(B, B->phase ^ (i & 1), B->cap);
+                for (int i = 0; i < chunk && le == cudaSuccess; ++i)
+                    le = launch_batch(B, B->phase ^ (i & 1), B->cap, i == 0, i == chunk - 1);
                 cudaGraph_t g = nullptr;
                 cudaError_t ce = cudaStreamEndCapture(B->cap, &g);
                 if (le != cudaSuccess) {
@@ -628,13 +688,15 @@ int tf_lbm_batch_step(tf_lbm_batch* B, int64_t nsteps, void* stream)
             for (auto* H : B->hs) H->time += chunk;  // chunk is even: buffer indices unchanged
             nsteps -= chunk;
         } else {
-            BCK(B, launch_batch(B, B->phase, st), "batched step");
-            B->phase ^= 1;
-            for (auto* H : B->hs) {
-                H->cur ^= 1;
-                ++H->time;
+            // one run of all the steps that no graph takes
+            for (const int64_t n = nsteps; nsteps > 0; --nsteps) {
+                BCK(B, launch_batch(B, B->phase, st, nsteps == n, nsteps == 1), "batched step");
+                B->phase ^= 1;
+                for (auto* H : B->hs) {
+                    H->cur ^= 1;
+                    ++H->time;
+                }
             }
-            --nsteps;
         }
     }
     return TF_LBM_OK;
@@ -703,14 +765,25 @@ int tf_lbm_batch_tune(tf_lbm_batch* B, int32_t trial_steps, tf_lbm_batch_launch*
         (e = cudaEventCreate(&e1)) != cudaSuccess)
         return finish(bcuda(B, e, "tuning setup"));
 
+    const bool old_wide = B->wide;
     auto time_one = [&](const tf_lbm_batch_launch& c, float* ms) -> int {
         int r = apply_launch(B, c, st);
         if (r) return r;
         return time_batch(B, steps, st, e0, e1, ms);
     };
+    B->wide = false;
     const int k = pick_fastest(cands, time_one, &rc);
     const tf_lbm_batch_launch chosen = k >= 0 ? cands[k] : old;
     const int rc2 = apply_launch(B, rc ? old : chosen, st);
+    // the four-column march in its place if it beats it
+    std::vector<int> both{0};
+    if (B->wide_ok && !rc && !rc2) both.push_back(1);
+    const int kw = rc || rc2 ? -1 : pick_fastest(both, [&](int w, float* ms) -> int {
+        B->wide = w != 0;
+        return time_batch(B, steps, st, e0, e1, ms);
+    }, &rc);
+    B->wide = kw >= 0 ? both[kw] != 0 : old_wide;
+    drop_batch_graphs(B);
     if (rc) return finish(rc);
     if (rc2) return finish(rc2);
     if (best) *best = B->L;

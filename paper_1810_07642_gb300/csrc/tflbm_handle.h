@@ -47,8 +47,10 @@ namespace tflbm {
 // Per-run step constants of a handle, in the compute type T.
 template <typename T>
 Consts<T> make_consts(const tf_lbm_handle* H);
-// Launch one fused step from buf[from] into buf[from ^ 1].
-cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st);
+// Launch one fused step from buf[from] into buf[from ^ 1].  A run of steps marks
+// its first and last one: between two steps of a run the buffer may hold
+// moments instead of populations (Shape::wide).
+cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st, bool first = true, bool last = true);
 // One tile step between two population buffers of the handle's layout that
 // also records the moments of the state it starts from (tflbm_tile.cuh).
 cudaError_t launch_recorded_step(tf_lbm_handle* H, const void* fin, void* fout, void* mom, cudaStream_t st);

@@ -94,6 +94,7 @@ struct Shape {
     int pipeline;   // kPipeTma, kPipeLdg, kPipeAsync, kPipePair, or kPipeTile (then tile == block_x)
     int bands = 0;  // balanced bands per launch; 0: ny / rows rounded up
     int tile = 0;   // run the tile kernel with this block_x (tile_of) instead of a march; 0: march
+    int wide = 0;   // run the four-column march in this many bands instead; 0: no
 };
 
 // Bands of one launch of a step kernel for a shape (at most 65535, the grid's
@@ -126,6 +127,21 @@ cudaError_t pair_step_f16(int block_x, const void* fin, void* fout, const void* 
                           const Consts<float>& C, int bands, cudaStream_t st);
 cudaError_t pair_step_bf16(int block_x, const void* fin, void* fout, const void* kappa, const Geom& G,
                            const Consts<float>& C, int bands, cudaStream_t st);
+// The four-column march (step4.cu): omega = 1, forcing = 0, FP32 compute type.
+// mom_in, mom_out: the source / destination holds moments (kStoreF32 only, see
+// tflbm_step4.cuh).  wide_applies: whether the kernel takes the lattice (16-bit
+// storage: nx a multiple of 4).  wide_slots: CTAs (strip, band) the GPU holds.
+cudaError_t launch_wide(int store, bool mom_in, bool mom_out, const void* fin, void* fout, const void* kappa,
+                        const Geom& G, const Consts<float>& C, int bands, cudaStream_t st);
+bool wide_applies(int store, const Geom& G);
+int wide_strips(int nx);
+int wide_slots(int store, bool quad, int sms);
+// Bands of a lattice that fill `slots` once, none shorter than 8 rows.
+inline int wide_bands(const Geom& G, int slots)
+{
+    const int b = slots / wide_strips(G.nx), most = G.ny / 8;
+    return b > most ? (most < 1 ? 1 : most) : (b < 1 ? 1 : b);
+}
 // The tile step (tile_*.cu); mom: see tile_step, or null.
 cudaError_t launch_tile(int store, int block_x, const void* fin, void* fout, const void* kappa, void* mom,
                         const Geom& G, const Consts<float>* C32, const Consts<double>* C64, cudaStream_t st);
@@ -163,6 +179,9 @@ struct BatchLaunch {
     int* query_occupancy;
 };
 cudaError_t launch_step_batch(int store, const BatchLaunch& L, cudaStream_t st);
+// The batched four-column march; quad: every domain's nx is a multiple of 4.
+cudaError_t launch_wide_batch(int store, bool mom_in, bool mom_out, bool quad, const BatchItem* items, int nitems,
+                              const void* doms, int parity, cudaStream_t st);
 // The batched two-column step per storage type (step2_*.cu).
 cudaError_t pair_step_batch_f32(const BatchLaunch& L, cudaStream_t st);
 cudaError_t pair_step_batch_f16(const BatchLaunch& L, cudaStream_t st);

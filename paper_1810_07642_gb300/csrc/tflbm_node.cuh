@@ -17,8 +17,7 @@ __device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 __device__ __forceinline__ float2 pneg(float2 a) { return make_float2(-a.x, -a.y); }
-// 1 / a by CUDA's fast single-precision division (within 2 ulp)
-__device__ __forceinline__ float2 prcp(float2 a) { return make_float2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y)); }
+__device__ __forceinline__ float2 prcp(float2 a) { return make_float2(rcp1(a.x), rcp1(a.y)); }
 __device__ __forceinline__ float2 pfdisj(float2 r, int n, int m) { return make_float2(fdisj(r.x, n, m), fdisj(r.y, n, m)); }
 
 // the same names for one FP64 node
@@ -148,34 +147,26 @@ __device__ __forceinline__ X node_pressure(const Win<X>& H, X kap, bool disj, co
     return pmul(pk(-C.gamma), lap);
 }
 
-// Force and collision (the arithmetic of collide_store on every lane, in
-// storage units).  P: the p window (n = row o+1, s = row o-1); f: the pulled
-// moving populations in storage units, fstride apart (omega != 1 only).  The
-// post-collision populations go to store(f_0 - href, q[8]), q as stored.
-template <typename SM, bool OMEGA1, typename X, typename Store>
-__device__ __forceinline__ void node_collide(const Win<X>& P, X dh, X ih, X jx, X jy, X er, const X* f, int fstride,
-                                             const Consts<typename Lanes<X>::S>& C, Store store)
+// The total force at a node, the velocity u and the momentum e of the
+// equilibria (Eqs. force, forcefric, alphafric).  P: the p window (n = row o+1,
+// s = row o-1).
+template <typename X>
+__device__ __forceinline__ void node_force(const Win<X>& P, X h, X ih, X jx, X jy, const Consts<typename Lanes<X>::S>& C,
+                                           X& ux, X& uy, X& ex, X& ey, X& Fx, X& Fy)
 {
     using S = typename Lanes<X>::S;
     auto pk = [](S a) { return Lanes<X>::all(a); };
-    using IO = PairIO<SM>;
-    using V = typename IO::V;
-    constexpr bool NARROW = sizeof(SM) == 2;
-    // storage scale (1 for full-width storage, a compile-time constant there)
-    const S ms = NARROW ? C.mscale : S(1);
     // Eq. (derivative): grad p = 3 sum_l w_l c_l p(x + c_l)
     const X gpx = pfma(psub(P.cR, P.cL), pk(S(1.0 / 3.0)),
                        pmul(padd(psub(P.nR, P.nL), psub(P.sR, P.sL)), pk(S(1.0 / 12.0))));
     const X gpy = pfma(psub(P.n0, P.s0), pk(S(1.0 / 3.0)),
                        pmul(padd(psub(P.nR, P.sR), psub(P.nL, P.sL)), pk(S(1.0 / 12.0))));
-    const X h = padd(dh, pk(C.href));
-    // Eqs. (force), (forcefric), (alphafric): nu alpha u = 6 nu j / (2h^2 + 6 delta h + 3 delta^2)
+    // nu alpha u = 6 nu j / (2h^2 + 6 delta h + 3 delta^2)
     const X den = pfma(h, pfma(pk(S(2.0)), h, pk(S(6.0) * C.delta)), pk(S(3.0) * C.delta * C.delta));
     const X fr = pmul(pk(C.nu6), prcp(den));
     // Eq. (LBE) as printed: u = j/h.  Second-order forcing (C.forcing):
     // u (h + nu alpha/2) = j + F'/2 and the equilibria use h u for j (see
     // collide_store)
-    X Fx, Fy, ux, uy, ex, ey;
     if (C.forcing) {
         const X fpx = pmul(h, psub(pk(C.gx), gpx)), fpy = pmul(h, psub(pk(C.gy), gpy));
         const X d = pfma(pk(S(0.5)), fr, pk(S(1.0)));
@@ -194,22 +185,124 @@ __device__ __forceinline__ void node_collide(const Win<X>& P, X dh, X ih, X jx, 
         ex = jx;
         ey = jy;
     }
-    // Eq. (equilibria) with e^2 = 1 as S +- D per opposite pair, source
-    // 3 w_l c_l . F; in storage units S' = (S - R_l) ms, D' = D ms.
-    // A6 = 6 A = h (g h - u^2).
+}
+
+// Eq. (equilibria) with e^2 = 1 as S +- D per opposite pair; the even parts S in
+// storage units, (S - R_l) ms.
+template <typename SM, typename X>
+__device__ __forceinline__ void node_even(X h, X ux, X uy, X ex, X ey, const Consts<typename Lanes<X>::S>& C, X& Sx,
+                                          X& Sy, X& Sa, X& Sb)
+{
+    using S = typename Lanes<X>::S;
+    auto pk = [](S a) { return Lanes<X>::all(a); };
+    constexpr bool NARROW = sizeof(SM) == 2;
+    // storage scale (1 for full-width storage, a compile-time constant there)
+    const S ms = NARROW ? C.mscale : S(1);
+    // A6 = 6 A = h (g h - u^2)
     const X A6 = pmul(h, psub(pmul(pk(C.g), h), pfma(ux, ux, pmul(uy, uy))));
     const X Aa = NARROW ? pfma(A6, pk(ms * S(1.0 / 6.0)), pk(C.nr_axis)) : pmul(A6, pk(S(1.0 / 6.0)));
     const X Ad = NARROW ? pfma(A6, pk(ms * S(1.0 / 24.0)), pk(C.nr_diag)) : pmul(A6, pk(S(1.0 / 24.0)));
-    X Sx = pfma(pmul(ex, pk(S(0.5) * ms)), ux, Aa);
-    X Sy = pfma(pmul(ey, pk(S(0.5) * ms)), uy, Aa);
+    Sx = pfma(pmul(ex, pk(S(0.5) * ms)), ux, Aa);
+    Sy = pfma(pmul(ey, pk(S(0.5) * ms)), uy, Aa);
     const X a = padd(ux, uy), b = psub(uy, ux);
     const X h8 = pmul(h, pk(S(0.125) * ms));
-    X Sa = pfma(pmul(h8, a), a, Ad);
-    X Sb = pfma(pmul(h8, b), b, Ad);
+    Sa = pfma(pmul(h8, a), a, Ad);
+    Sb = pfma(pmul(h8, b), b, Ad);
+}
+
+// Post-collision moving populations at omega = 1: the even parts and the odd
+// parts of G = e + F (source 3 w_l c_l . F), in storage units; o[l - 1].
+template <typename SM, typename X>
+__device__ __forceinline__ void node_odd(X Sx, X Sy, X Sa, X Sb, X Gx, X Gy, const Consts<typename Lanes<X>::S>& C,
+                                         X (&o)[8])
+{
+    using S = typename Lanes<X>::S;
+    const S ms = sizeof(SM) == 2 ? C.mscale : S(1);
+    const X m3 = Lanes<X>::all(ms * S(1.0 / 3.0)), m12 = Lanes<X>::all(ms * S(1.0 / 12.0));
+    const X Dx = pmul(Gx, m3), Dy = pmul(Gy, m3);
+    const X Da = pmul(padd(Gx, Gy), m12), Db = pmul(psub(Gy, Gx), m12);
+    o[0] = padd(Sx, Dx); o[4] = psub(Sx, Dx);
+    o[2] = padd(Sy, Dy); o[6] = psub(Sy, Dy);
+    o[1] = padd(Sa, Da); o[5] = psub(Sa, Da);
+    o[3] = padd(Sb, Db); o[7] = psub(Sb, Db);
+}
+
+// Stored rest population f*_0 - href = (h - href) - sum_{l>0} f*_l, with the
+// exact residuals (er: of the pull sum) folded back into f_1 and f_5 as in
+// collide_store; full-width storage.
+template <typename X>
+__device__ __forceinline__ X node_fold(X dh, X er, X (&o)[8])
+{
+    const X osum = padd(padd(padd(o[0], o[4]), padd(o[2], o[6])), padd(padd(o[1], o[5]), padd(o[3], o[7])));
+    X o0, e2;
+    ptwo_sum(dh, pneg(osum), o0, e2);
+    const X half_r = pmul(padd(er, e2), Lanes<X>::all(typename Lanes<X>::S(0.5)));
+    o[0] = padd(o[0], half_r);
+    o[4] = padd(o[4], half_r);
+    return o0;
+}
+
+// The same for 16-bit storage: q receives the stored values.
+template <typename SM>
+__device__ __forceinline__ float2 node_fold_narrow(float2 dh, float2 er, const float2 (&o)[8], const Consts<float>& C,
+                                                   typename PairIO<SM>::V (&q)[8])
+{
+    using IO = PairIO<SM>;
+    using V = typename IO::V;
+    const V q1r = IO::enc(o[0]);
+#pragma unroll
+    for (int l = 1; l < 8; ++l) q[l] = IO::enc(o[l]);
+    // what the readers reconstruct of l = 2..8 (storage units; each stored
+    // value enters the FP32 sum by a mixed-precision add, which takes the
+    // 16-bit operand as it is), summed so that exchanging +y and -y (a march
+    // the other way) gives the same bits
+    float2 r28 = IO::dec(q[1]), r37 = IO::dec(q[2]), r46 = IO::dec(q[3]);
+    mixed_add<SM>(r28, q[7]);
+    mixed_add<SM>(r37, q[6]);
+    mixed_add<SM>(r46, q[5]);
+    float2 rest = padd(padd(r28, r46), r37);
+    mixed_add<SM>(rest, q[4]);
+    float2 rest1 = rest;
+    mixed_add<SM>(rest1, q1r);
+    // the moving populations' total with f_1 unrounded and rounded
+    const float2 osum = pfma(padd(rest, o[0]), pk(C.minv), pk(C.r_sum));
+    const float2 osr = pfma(rest1, pk(C.minv), pk(C.r_sum));
+    // the last residual goes to the finer of the two roundings: the 16-bit
+    // one of f_1 - R or the FP32 one of f_0 - href (see collide_store)
+    constexpr float kRatio = std::is_same<SM, __half>::value ? 8192.0f : 65536.0f;
+    const float kr = kRatio * C.minv;  // |f_1 - R| = |o1| / ms
+    const bool lx = fabsf(o[0].x) * kr < fabsf(dh.x - osum.x);
+    const bool ly = fabsf(o[0].y) * kr < fabsf(dh.y - osum.y);
+    const float2 os = make_float2(lx ? osum.x : osr.x, ly ? osum.y : osr.y);
+    float2 o0v, e2, o0n, e3;
+    ptwo_sum(dh, pneg(os), o0v, e2);
+    ptwo_sum(o0v, padd(er, e2), o0n, e3);
+    const V q1l = IO::enc(pfma(e3, pk(C.mscale), o[0]));
+    const uint32_t mask = (lx ? 0x0000ffffu : 0u) | (ly ? 0xffff0000u : 0u);
+    q[0] = from_bits<V>((bits(q1l) & mask) | (bits(q1r) & ~mask));
+    return o0n;
+}
+
+// Force and collision (the arithmetic of collide_store on every lane, in
+// storage units).  f: the pulled moving populations in storage units, fstride
+// apart (omega != 1 only).  The post-collision populations go to
+// store(f_0 - href, q[8]), q as stored.
+template <typename SM, bool OMEGA1, typename X, typename Store>
+__device__ __forceinline__ void node_collide(const Win<X>& P, X dh, X ih, X jx, X jy, X er, const X* f, int fstride,
+                                             const Consts<typename Lanes<X>::S>& C, Store store)
+{
+    using S = typename Lanes<X>::S;
+    auto pk = [](S a) { return Lanes<X>::all(a); };
+    constexpr bool NARROW = sizeof(SM) == 2;
+    const S ms = NARROW ? C.mscale : S(1);
+    const X h = padd(dh, pk(C.href));
+    X ux, uy, ex, ey, Fx, Fy, Sx, Sy, Sa, Sb;
+    node_force(P, h, ih, jx, jy, C, ux, uy, ex, ey, Fx, Fy);
+    node_even<SM>(h, ux, uy, ex, ey, C, Sx, Sy, Sa, Sb);
     // second-order source: odd part scaled by (1 - omega/2), even part T
     X Tx = pk(S(0.0)), Ty = pk(S(0.0)), Ta = pk(S(0.0)), Tb = pk(S(0.0));
     if (C.forcing) {
-        const X ks = pk(S(1.0) - S(0.5) * C.omega);
+        const X ks = pk(S(1.0) - S(0.5) * C.omega), a = padd(ux, uy), b = psub(uy, ux);
         Fx = pmul(Fx, ks);
         Fy = pmul(Fy, ks);
         const X uF3 = pmul(pfma(ux, Fx, pmul(uy, Fy)), pk(ms * S(1.0 / 3.0)));
@@ -224,77 +317,54 @@ __device__ __forceinline__ void node_collide(const Win<X>& P, X dh, X ih, X jx, 
             Sb = padd(Sb, Tb);
         }
     }
-    const X m3 = pk(ms * S(1.0 / 3.0)), m12 = pk(ms * S(1.0 / 12.0));
-    X o1, o2, o3, o4, o5, o6, o7, o8;
+    X o[8];
     if constexpr (OMEGA1) {
-        const X Gx = padd(ex, Fx), Gy = padd(ey, Fy);
-        const X Dx = pmul(Gx, m3), Dy = pmul(Gy, m3);
-        const X Da = pmul(padd(Gx, Gy), m12), Db = pmul(psub(Gy, Gx), m12);
-        o1 = padd(Sx, Dx); o5 = psub(Sx, Dx);
-        o3 = padd(Sy, Dy); o7 = psub(Sy, Dy);
-        o2 = padd(Sa, Da); o6 = psub(Sa, Da);
-        o4 = padd(Sb, Db); o8 = psub(Sb, Db);
+        node_odd<SM>(Sx, Sy, Sa, Sb, padd(ex, Fx), padd(ey, Fy), C, o);
     } else {
         // (1 - omega)(f_l - R_l) + omega (f_eq_l - R_l) + source, in storage units
         const X w = pk(C.omega), m = pk(S(1.0) - C.omega);
+        const X m3 = pk(ms * S(1.0 / 3.0)), m12 = pk(ms * S(1.0 / 12.0));
         const X Dx = pmul(ex, m3), Dy = pmul(ey, m3);
         const X Da = pmul(padd(ex, ey), m12), Db = pmul(psub(ey, ex), m12);
         const X Qx = pmul(Fx, m3), Qy = pmul(Fy, m3);
         const X Qa = pmul(padd(Fx, Fy), m12), Qb = pmul(psub(Fy, Fx), m12);
-        o1 = padd(pfma(m, f[0 * fstride], pmul(w, padd(Sx, Dx))), padd(Tx, Qx));
-        o5 = padd(pfma(m, f[4 * fstride], pmul(w, psub(Sx, Dx))), psub(Tx, Qx));
-        o3 = padd(pfma(m, f[2 * fstride], pmul(w, padd(Sy, Dy))), padd(Ty, Qy));
-        o7 = padd(pfma(m, f[6 * fstride], pmul(w, psub(Sy, Dy))), psub(Ty, Qy));
-        o2 = padd(pfma(m, f[1 * fstride], pmul(w, padd(Sa, Da))), padd(Ta, Qa));
-        o6 = padd(pfma(m, f[5 * fstride], pmul(w, psub(Sa, Da))), psub(Ta, Qa));
-        o4 = padd(pfma(m, f[3 * fstride], pmul(w, padd(Sb, Db))), padd(Tb, Qb));
-        o8 = padd(pfma(m, f[7 * fstride], pmul(w, psub(Sb, Db))), psub(Tb, Qb));
+        o[0] = padd(pfma(m, f[0 * fstride], pmul(w, padd(Sx, Dx))), padd(Tx, Qx));
+        o[4] = padd(pfma(m, f[4 * fstride], pmul(w, psub(Sx, Dx))), psub(Tx, Qx));
+        o[2] = padd(pfma(m, f[2 * fstride], pmul(w, padd(Sy, Dy))), padd(Ty, Qy));
+        o[6] = padd(pfma(m, f[6 * fstride], pmul(w, psub(Sy, Dy))), psub(Ty, Qy));
+        o[1] = padd(pfma(m, f[1 * fstride], pmul(w, padd(Sa, Da))), padd(Ta, Qa));
+        o[5] = padd(pfma(m, f[5 * fstride], pmul(w, psub(Sa, Da))), psub(Ta, Qa));
+        o[3] = padd(pfma(m, f[3 * fstride], pmul(w, padd(Sb, Db))), padd(Tb, Qb));
+        o[7] = padd(pfma(m, f[7 * fstride], pmul(w, psub(Sb, Db))), psub(Tb, Qb));
     }
-    // stored rest population f*_0 - href = (h - href) - sum_{l>0} f*_l, with
-    // the exact residuals folded back as in collide_store
     if constexpr (!NARROW) {
-        const X osum = padd(padd(padd(o1, o5), padd(o3, o7)), padd(padd(o2, o6), padd(o4, o8)));
-        X o0v, e2;
-        ptwo_sum(dh, pneg(osum), o0v, e2);
-        const X half_r = pmul(padd(er, e2), pk(S(0.5)));
-        o1 = padd(o1, half_r);
-        o5 = padd(o5, half_r);
-        const V q[8] = {o1, o2, o3, o4, o5, o6, o7, o8};
-        store(o0v, q);
+        const X o0 = node_fold(dh, er, o);
+        store(o0, o);
     } else {
-        const V q2 = IO::enc(o2), q3 = IO::enc(o3), q4 = IO::enc(o4), q5 = IO::enc(o5);
-        const V q6 = IO::enc(o6), q7 = IO::enc(o7), q8 = IO::enc(o8), q1r = IO::enc(o1);
-        // what the readers reconstruct of l = 2..8 (storage units; each
-        // stored value enters the FP32 sum by a mixed-precision add, which
-        // takes the 16-bit operand as it is: one instruction per value
-        // instead of a conversion and half a paired add)
-        float2 rest = IO::dec(q2);
-        mixed_add<SM>(rest, q3);
-        mixed_add<SM>(rest, q4);
-        mixed_add<SM>(rest, q5);
-        mixed_add<SM>(rest, q6);
-        mixed_add<SM>(rest, q7);
-        mixed_add<SM>(rest, q8);
-        float2 rest1 = rest;
-        mixed_add<SM>(rest1, q1r);
-        // the moving populations' total with f_1 unrounded and rounded
-        const float2 osum = pfma(padd(rest, o1), pk(C.minv), pk(C.r_sum));
-        const float2 osr = pfma(rest1, pk(C.minv), pk(C.r_sum));
-        // the last residual goes to the finer of the two roundings: the 16-bit
-        // one of f_1 - R or the FP32 one of f_0 - href (see collide_store)
-        constexpr float kRatio = std::is_same<SM, __half>::value ? 8192.0f : 65536.0f;
-        const float kr = kRatio * C.minv;  // |f_1 - R| = |o1| / ms
-        const bool lx = fabsf(o1.x) * kr < fabsf(dh.x - osum.x);
-        const bool ly = fabsf(o1.y) * kr < fabsf(dh.y - osum.y);
-        const float2 os = make_float2(lx ? osum.x : osr.x, ly ? osum.y : osr.y);
-        float2 o0v, e2, o0n, e3;
-        ptwo_sum(dh, make_float2(-os.x, -os.y), o0v, e2);
-        ptwo_sum(o0v, padd(er, e2), o0n, e3);
-        const V q1l = IO::enc(pfma(e3, pk(ms), o1));
-        const uint32_t mask = (lx ? 0x0000ffffu : 0u) | (ly ? 0xffff0000u : 0u);
-        const V q1 = from_bits<V>((bits(q1l) & mask) | (bits(q1r) & ~mask));
-        const V q[8] = {q1, q2, q3, q4, q5, q6, q7, q8};
-        store(o0n, q);
+        typename PairIO<SM>::V q[8];
+        const X o0 = node_fold_narrow<SM>(dh, er, o, C, q);
+        store(o0, q);
+    }
+}
+
+// Moments from the sums of pulled populations in storage units: f0 - href;
+// Rs, Ls the populations arriving from the left (l = 1, 2, 8) and the right (l
+// = 5, 4, 6), s26 those along y (l = 3, 7), jyr their y momentum.  dh = h -
+// href: the moving total is small, the last addition is error-free (see sum9).
+template <typename SM, typename X>
+__device__ __forceinline__ void node_moments(X f0, X Rs, X Ls, X s26, X jyr, const Consts<typename Lanes<X>::S>& C,
+                                             X& dh, X& er, X& jx, X& jy)
+{
+    const X tot = padd(s26, padd(Rs, Ls));
+    if constexpr (sizeof(SM) == 2) {
+        const X minv = Lanes<X>::all(C.minv);
+        ptwo_sum(f0, pfma(tot, minv, Lanes<X>::all(C.r_sum)), dh, er);
+        jx = pmul(psub(Rs, Ls), minv);
+        jy = pmul(jyr, minv);
+    } else {
+        ptwo_sum(f0, tot, dh, er);
+        jx = psub(Rs, Ls);
+        jy = jyr;
     }
 }
 

@@ -44,9 +44,17 @@ __device__ __forceinline__ int wrap_index(int i, int n)
     return i < 0 ? i + n : i;
 }
 
-// a / b: CUDA's fast single-precision division (within 2 ulp) in FP32, the
-// IEEE division in FP64.
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
+// 1 / a by the approximate reciprocal (rcp.approx, 1 ulp): one instruction where
+// the fast division adds the handling of denominators that a film height never
+// takes.
+__device__ __forceinline__ float rcp1(float a)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+// a / b: by that reciprocal (2 ulp) in FP32, the IEEE division in FP64.
+__device__ __forceinline__ float fdiv(float a, float b) { return a * rcp1(b); }
 __device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
 
 // r^n for 0 <= n < 64 by binary powering over a fixed number of bits (no

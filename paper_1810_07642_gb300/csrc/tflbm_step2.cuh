@@ -213,14 +213,15 @@ __device__ __forceinline__ void step_band2(const float* __restrict__ fin0, const
                 kap_n = reinterpret_cast<const float2*>(kappa)[TFLBM_IDX(((long long)w0 * nx + c) >> 1, npair,
                                                                           C.status)];
             // Rs, Ls: sums of the populations arriving from the left (l = 1,
-            // 2, 8) and from the right (l = 4, 5, 6) at the two nodes; tot:
-            // all eight; jyr: their y momentum (storage units)
-            float2 Rs, Ls, tot, jyr;
+            // 2, 8) and from the right (l = 4, 5, 6) at the two nodes; s26:
+            // l = 3, 7; jyr: their y momentum (storage units)
+            float2 Rs, Ls, s26, jyr;
             if constexpr (OMEGA1) {
-                const float2 Pc = padd(padd(v[0], v[1]), v[7]), Py = psub(v[1], v[7]);
-                const float2 Qc = padd(padd(v[4], v[3]), v[5]), Qy = psub(v[3], v[5]);
-                const float2 s26 = padd(v[2], v[6]), d26 = psub(v[2], v[6]);
-                const float es = (ea + eb) + ed, ey = eb - ed;
+                const float2 Pc = padd(v[0], padd(v[1], v[7])), Py = psub(v[1], v[7]);
+                const float2 Qc = padd(v[4], padd(v[3], v[5])), Qy = psub(v[3], v[5]);
+                const float2 d26 = psub(v[2], v[6]);
+                s26 = padd(v[2], v[6]);
+                const float es = ea + (eb + ed), ey = eb - ed;
                 if constexpr (!EARLY) issue_next();
                 float pl = __shfl_up_sync(0xffffffffu, Pc.y, 1), pyl = __shfl_up_sync(0xffffffffu, Py.y, 1);
                 float qr = __shfl_down_sync(0xffffffffu, Qc.x, 1), qyr = __shfl_down_sync(0xffffffffu, Qy.x, 1);
@@ -229,7 +230,6 @@ __device__ __forceinline__ void step_band2(const float* __restrict__ fin0, const
                 Rs = make_float2(pl, Pc.x);
                 Ls = make_float2(Qc.y, qr);
                 jyr = padd(d26, padd(make_float2(pyl, Py.x), make_float2(Qy.y, qyr)));
-                tot = padd(s26, padd(Rs, Ls));
             } else {
                 // the single arriving values, kept for the relaxation
                 float u1 = __shfl_up_sync(0xffffffffu, v[0].y, 1);
@@ -249,25 +249,15 @@ __device__ __forceinline__ void step_band2(const float* __restrict__ fin0, const
                 n[5] = make_float2(v[5].y, d6);
                 n[6] = v[6];
                 n[7] = make_float2(u8, v[7].x);
-                Rs = padd(padd(n[0], n[1]), n[7]);
-                Ls = padd(padd(n[4], n[3]), n[5]);
-                jyr = padd(padd(psub(n[2], n[6]), psub(n[1], n[7])), psub(n[3], n[5]));
-                tot = padd(padd(n[2], n[6]), padd(Rs, Ls));
+                Rs = padd(n[0], padd(n[1], n[7]));
+                Ls = padd(n[4], padd(n[3], n[5]));
+                jyr = padd(psub(n[2], n[6]), padd(psub(n[1], n[7]), psub(n[3], n[5])));
+                s26 = padd(n[2], n[6]);
 #pragma unroll
                 for (int l = 0; l < 8; ++l) fsm[s][l][t] = n[l];
             }
-            // h - href: the moving total is small, the last addition is
-            // error-free (see sum9)
             float2 dh, er, jx, jy;
-            if constexpr (NARROW) {
-                ptwo_sum(f0, pfma(tot, pk(C.minv), pk(C.r_sum)), dh, er);
-                jx = pmul(psub(Rs, Ls), pk(C.minv));
-                jy = pmul(jyr, pk(C.minv));
-            } else {
-                ptwo_sum(f0, tot, dh, er);
-                jx = psub(Rs, Ls);
-                jy = jyr;
-            }
+            node_moments<SM>(f0, Rs, Ls, s26, jyr, C, dh, er, jx, jy);
             TFLBM_CHECK(j2 >= OFF && j2 + 1 < RW, C.status);
             *reinterpret_cast<float2*>(&hsm[s][j2]) = dh;
             rsj[s][t] = make_float4(jx.x, jx.y, jy.x, jy.y);

@@ -66,24 +66,14 @@ __device__ __forceinline__ void tile_window(const S* b, int w, Win<X>& W)
     lane_of<K>(W.sL) = b[-w - 1]; lane_of<K>(W.s0) = b[-w]; lane_of<K>(W.sR) = b[-w + 1];
 }
 
-// Moments of pulled populations in storage units (the sums of step_band2).
+// Moments of the nine pulled populations n (storage units).
 template <typename SM, typename X>
 __device__ __forceinline__ void node_moments(X f0, const X (&n)[8], const Consts<typename Lanes<X>::S>& C, X& dh, X& er,
                                              X& jx, X& jy)
 {
-    const X Rs = padd(padd(n[0], n[1]), n[7]), Ls = padd(padd(n[4], n[3]), n[5]);
+    const X Rs = padd(n[0], padd(n[1], n[7])), Ls = padd(n[4], padd(n[3], n[5]));
     const X jyr = padd(psub(n[2], n[6]), padd(psub(n[1], n[7]), psub(n[3], n[5])));
-    const X tot = padd(padd(n[2], n[6]), padd(Rs, Ls));
-    if constexpr (sizeof(SM) == 2) {
-        const X minv = Lanes<X>::all(C.minv);
-        ptwo_sum(f0, pfma(tot, minv, Lanes<X>::all(C.r_sum)), dh, er);
-        jx = pmul(psub(Rs, Ls), minv);
-        jy = pmul(jyr, minv);
-    } else {
-        ptwo_sum(f0, tot, dh, er);
-        jx = psub(Rs, Ls);
-        jy = jyr;
-    }
+    node_moments<SM>(f0, Rs, Ls, padd(n[2], n[6]), jyr, C, dh, er, jx, jy);
 }
 
 template <typename SM, typename S, int TX, int TY, bool OMEGA1, int RESIDENT>

@@ -147,7 +147,8 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            copies four rows ahead (needs nx a multiple of 8, >= 16).
  * The shape chosen by tf_lbm_init runs other kernels in place of the one that
  * its fields describe: tiles on lattices of up to 2^20 nodes (1.5 x 2^20 where
- * the next one does not apply; for TF_LBM_F64 on all); above that, at tau = 1
+ * the next one does not apply; any size for TF_LBM_F64, and for 16-bit storage
+ * where the fields describe pipeline 1); above that, at tau = 1
  * with forcing = 0, a march of four columns per thread, which between the
  * steps of one call keeps moments in place of FP32 populations (16-bit storage:
  * where nx is a multiple of 4).  So does the shape chosen by tf_lbm_tune where

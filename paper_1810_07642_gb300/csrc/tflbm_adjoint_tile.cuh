@@ -54,7 +54,7 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
     __shared__ S ps[TY + 2][PW], ls[TY + 2][PW];    // p and -gamma ap; tile node at [r + 1][c + 1]
     __shared__ S as[OMEGA1 ? 3 : 1][OMEGA1 ? TY + 6 : 1][OMEGA1 ? AW : 1];  // a(t+1); tile node at [r + 3][c + 3]
 
-    dependent_launch_entry();
+    dependent_launch_wait();
     const int t = threadIdx.x, nx = G.nx, ny = G.ny;
     const long long n = (long long)nx * ny;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
@@ -258,6 +258,7 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
     }
     __syncthreads();
 
+    dependent_launch_next();  // as in k_tile
     // ---- 4
     Win<X> P, L;
     lanes([&](auto k_c) {

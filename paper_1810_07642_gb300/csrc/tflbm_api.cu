@@ -144,12 +144,15 @@ int store_of(int dtype)
     }
 }
 
-// Lattices up to this many nodes run the tile kernel (FP64: all of them).  Above
-// it the marches win: they pull a node 1.25 times, not 1.4, and load ahead.  One
-// box, us a step, tile against the four-column march: 900^2 FP32 12.5 / 12.2,
-// 1024^2 15.9 / 16.4, 1300 x 1100 25.4 / 17.5, 1448^2 36.3 / 21.6; FP16 1024^2
-// 16.1 / 16.4, 1448^2 34.3 / 21.4; against the one-column march at tau = 0.8:
-// 1024^2 18.4 / 24.9, 1448^2 39.8 / 37.1, 2048^2 73 / 63; FP64 2048^2 1014 / 1101.
+// Lattices up to this many nodes run the tile kernel where the four-column
+// march, or (tau != 1, forcing, an odd nx) the one-column march, would take
+// larger ones; FP64, and 16-bit storage where the one-column march is what is
+// left, run tiles at any size.  Above the limits the marches win: they pull a
+// node 1.25 times, not 1.4, and load ahead.  One box, us a step, tile against
+// the four-column march: 900^2 FP32 12.5 / 12.2, 1024^2 15.2 / 16.4, 1300 x 1100
+// 25.4 / 17.5, 1448^2 36.3 / 21.6; FP16 1024^2 16.1 / 16.4, 1448^2 34.3 / 21.4;
+// against the one-column march at tau = 0.8: FP32 1448^2 37.2 / 36.7, 2048^2 69
+// / 63, FP16 1448^2 32.3 / 41.7, 2048^2 59.8 / 69.2; FP64 2048^2 1014 / 1101.
 constexpr long long kTileNodes = 1LL << 20, kTileNodesOneColumn = 3LL << 19;
 
 // Default launch shape: tiles on lattices that L2 holds, the four-column march
@@ -171,12 +174,13 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     const int store = store_of(p.dtype), sms = sm_count();
     const bool om1 = p.tau == 1.0;
     const bool wide = om1 && p.forcing == 0 && wide_applies(store, G);
-    if (store == kStoreF64 || (long long)G.nx * G.ny <= (wide ? kTileNodes : kTileNodesOneColumn))
+    const bool pair = pair_pipeline_ok(G.nx, store) && om1;
+    const bool narrow = store == kStoreF16 || store == kStoreBF16;
+    if (store == kStoreF64 || (narrow && !wide && !pair) ||
+        (long long)G.nx * G.ny <= (wide ? kTileNodes : kTileNodesOneColumn))
         s.tile = tile_block_x(store, G.nx, G.ny, sms);
     else if (wide)
         s.wide = wide_bands(G, wide_slots(store, G.nx % 4 == 0, sms));
-    const bool narrow = store == kStoreF16 || store == kStoreBF16;
-    const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     s.block_x = pair ? (narrow ? 64 : 128) : (G.nx >= 1024 ? 128 : 64);
     const int strips = (G.nx + s.block_x - 5) / (s.block_x - 4);  // CTAs overlap by 4 columns
     // otherwise per-thread loads: measured faster than the bulk-copy pipeline

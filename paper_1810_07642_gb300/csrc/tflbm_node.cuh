@@ -321,21 +321,21 @@ __device__ __forceinline__ void node_collide(const Win<X>& P, X dh, X ih, X jx, 
     if constexpr (OMEGA1) {
         node_odd<SM>(Sx, Sy, Sa, Sb, padd(ex, Fx), padd(ey, Fy), C, o);
     } else {
-        // (1 - omega)(f_l - R_l) + omega (f_eq_l - R_l) + source, in storage units
+        // (1 - omega)(f_l - R_l) + omega (f_eq_l - R_l) + source, in storage
+        // units: (1 - omega) f_l + V +- E per opposite pair, V = omega S + T, E
+        // the odd parts of omega e + F
         const X w = pk(C.omega), m = pk(S(1.0) - C.omega);
         const X m3 = pk(ms * S(1.0 / 3.0)), m12 = pk(ms * S(1.0 / 12.0));
-        const X Dx = pmul(ex, m3), Dy = pmul(ey, m3);
-        const X Da = pmul(padd(ex, ey), m12), Db = pmul(psub(ey, ex), m12);
-        const X Qx = pmul(Fx, m3), Qy = pmul(Fy, m3);
-        const X Qa = pmul(padd(Fx, Fy), m12), Qb = pmul(psub(Fy, Fx), m12);
-        o[0] = padd(pfma(m, f[0 * fstride], pmul(w, padd(Sx, Dx))), padd(Tx, Qx));
-        o[4] = padd(pfma(m, f[4 * fstride], pmul(w, psub(Sx, Dx))), psub(Tx, Qx));
-        o[2] = padd(pfma(m, f[2 * fstride], pmul(w, padd(Sy, Dy))), padd(Ty, Qy));
-        o[6] = padd(pfma(m, f[6 * fstride], pmul(w, psub(Sy, Dy))), psub(Ty, Qy));
-        o[1] = padd(pfma(m, f[1 * fstride], pmul(w, padd(Sa, Da))), padd(Ta, Qa));
-        o[5] = padd(pfma(m, f[5 * fstride], pmul(w, psub(Sa, Da))), psub(Ta, Qa));
-        o[3] = padd(pfma(m, f[3 * fstride], pmul(w, padd(Sb, Db))), padd(Tb, Qb));
-        o[7] = padd(pfma(m, f[7 * fstride], pmul(w, psub(Sb, Db))), psub(Tb, Qb));
+        const X Gx = pfma(w, ex, Fx), Gy = pfma(w, ey, Fy);
+        auto opposite = [&](X s, X t, X e, int l) {  // populations l + 1 and l + 5
+            const X v = pfma(w, s, t);
+            o[l] = pfma(m, f[l * fstride], padd(v, e));
+            o[l + 4] = pfma(m, f[(l + 4) * fstride], psub(v, e));
+        };
+        opposite(Sx, Tx, pmul(Gx, m3), 0);
+        opposite(Sa, Ta, pmul(padd(Gx, Gy), m12), 1);
+        opposite(Sy, Ty, pmul(Gy, m3), 2);
+        opposite(Sb, Tb, pmul(psub(Gy, Gx), m12), 3);
     }
     if constexpr (!NARROW) {
         const X o0 = node_fold(dh, er, o);

@@ -88,10 +88,12 @@ template <typename S> __device__ __forceinline__ S ldro(const S* p) { return __l
 // complete, with its writes visible, before it touches global memory.  Both
 // are hardware dependencies (no polling); without the launch attribute the
 // wait returns at once.
+__device__ __forceinline__ void dependent_launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependent_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependent_launch_entry()
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    dependent_launch_next();
+    dependent_launch_wait();
 }
 
 // Launch `kern` with the programmatic-stream-serialization attribute (see
@@ -290,19 +292,21 @@ __device__ __forceinline__ void collide_store(const T* pn, const T* pc, const T*
         o2 = Sa + Da; o6 = Sa - Da;
         o4 = Sb + Db; o8 = Sb - Db;
     } else {
+        // (1 - omega) f_l + V +- E per opposite pair, V = omega S + T, E the
+        // odd parts of omega e + F
         const T w = C.omega, m = T(1) - C.omega;
-        const T Dx = ex * third, Dy = ey * third;
-        const T Da = (ex + ey) * twelfth, Db = (ey - ex) * twelfth;
-        const T Qx = Fx * third, Qy = Fy * third;
-        const T Qa = (Fx + Fy) * twelfth, Qb = (Fy - Fx) * twelfth;
-        o1 = m * f[1] + w * (Sx + Dx) + (Tx + Qx);
-        o5 = m * f[5] + w * (Sx - Dx) + (Tx - Qx);
-        o3 = m * f[3] + w * (Sy + Dy) + (Ty + Qy);
-        o7 = m * f[7] + w * (Sy - Dy) + (Ty - Qy);
-        o2 = m * f[2] + w * (Sa + Da) + (Ta + Qa);
-        o6 = m * f[6] + w * (Sa - Da) + (Ta - Qa);
-        o4 = m * f[4] + w * (Sb + Db) + (Tb + Qb);
-        o8 = m * f[8] + w * (Sb - Db) + (Tb - Qb);
+        const T Gx = w * ex + Fx, Gy = w * ey + Fy;
+        const T Ex = Gx * third, Ey = Gy * third;
+        const T Ea = (Gx + Gy) * twelfth, Eb = (Gy - Gx) * twelfth;
+        const T Vx = w * Sx + Tx, Vy = w * Sy + Ty, Va = w * Sa + Ta, Vb = w * Sb + Tb;
+        o1 = m * f[1] + (Vx + Ex);
+        o5 = m * f[5] + (Vx - Ex);
+        o3 = m * f[3] + (Vy + Ey);
+        o7 = m * f[7] + (Vy - Ey);
+        o2 = m * f[2] + (Va + Ea);
+        o6 = m * f[6] + (Va - Ea);
+        o4 = m * f[4] + (Vb + Eb);
+        o8 = m * f[8] + (Vb - Eb);
     }
     // In 16-bit storage, round the moving populations to what the readers
     // will reconstruct before the rest population is formed (f_1 possibly

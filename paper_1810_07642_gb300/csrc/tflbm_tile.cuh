@@ -94,31 +94,38 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     __shared__ S hs[TY + 4][HW];  // h - href; tile node (c, r) at [r + 2][c + 2]
     __shared__ S ps[TY + 2][PW];  // p; tile node (c, r) at [r + 1][c + 1]
 
-    dependent_launch_entry();
     const int t = threadIdx.x, nx = G.nx, ny = G.ny, pitch = G.pitch, plane = (int)G.plane;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int c = t % TX, r = t / TX;  // own nodes: (c, r + k HALF)
     const bool disj = kappa != nullptr || C.kappa_u != S(0);
 
-    // the populations arriving at tile position (cc, rr), into lane K
-    auto pull = [&](auto k_c, int cc, int rr, X& f0, X (&n)[8]) {
-        constexpr int K = decltype(k_c)::value;
+    // where the populations arriving at a node lie: its columns x - 1, x, x + 1
+    // and the offsets of its rows y - 1, y, y + 1
+    struct Spot {
+        uint32_t xm, x, xp, rm, r0, rp;
+    };
+    auto spot = [&](int cc, int rr) -> Spot {
         const int x = ring_index(x0 + cc, nx), y = ring_index(y0 + rr, ny);
-        const int xm = x == 0 ? nx - 1 : x - 1, xp = x + 1 == nx ? 0 : x + 1;
-        const int r0 = y * pitch, rm = (y == 0 ? ny - 1 : y - 1) * pitch, rp = (y + 1 == ny ? 0 : y + 1) * pitch;
-        const long long m8 = 8LL * plane;
+        return {(uint32_t)(x == 0 ? nx - 1 : x - 1), (uint32_t)x, (uint32_t)(x + 1 == nx ? 0 : x + 1),
+                (uint32_t)((y == 0 ? ny - 1 : y - 1) * pitch), (uint32_t)(y * pitch),
+                (uint32_t)((y + 1 == ny ? 0 : y + 1) * pitch)};
+    };
+    // load them into lane K: a uniform plane and a 32-bit offset within it, one
+    // register an access
+    auto pull = [&](auto k_c, const Spot& p, X& f0, X (&n)[8]) {
+        constexpr int K = decltype(k_c)::value;
         int* st = C.status;
-        (void)m8;
         (void)st;
-        lane_of<K>(f0) = ldro(fin0 + TFLBM_IDX(r0 + x, plane, st));
-        lane_of<K>(n[0]) = IO::dec1(ldro(finm + TFLBM_IDX(r0 + xm, m8, st)));
-        lane_of<K>(n[1]) = IO::dec1(ldro(finm + TFLBM_IDX(plane + rm + xm, m8, st)));
-        lane_of<K>(n[2]) = IO::dec1(ldro(finm + TFLBM_IDX(2 * plane + rm + x, m8, st)));
-        lane_of<K>(n[3]) = IO::dec1(ldro(finm + TFLBM_IDX(3 * plane + rm + xp, m8, st)));
-        lane_of<K>(n[4]) = IO::dec1(ldro(finm + TFLBM_IDX(4 * plane + r0 + xp, m8, st)));
-        lane_of<K>(n[5]) = IO::dec1(ldro(finm + TFLBM_IDX(5 * plane + rp + xp, m8, st)));
-        lane_of<K>(n[6]) = IO::dec1(ldro(finm + TFLBM_IDX(6 * plane + rp + x, m8, st)));
-        lane_of<K>(n[7]) = IO::dec1(ldro(finm + TFLBM_IDX(7 * plane + rp + xm, m8, st)));
+        auto at = [&](int l, uint32_t i) { return IO::dec1(ldro(finm + l * plane + TFLBM_IDX(i, plane, st))); };
+        lane_of<K>(f0) = ldro(fin0 + TFLBM_IDX(p.r0 + p.x, plane, st));
+        lane_of<K>(n[0]) = at(0, p.r0 + p.xm);
+        lane_of<K>(n[1]) = at(1, p.rm + p.xm);
+        lane_of<K>(n[2]) = at(2, p.rm + p.x);
+        lane_of<K>(n[3]) = at(3, p.rm + p.xp);
+        lane_of<K>(n[4]) = at(4, p.r0 + p.xp);
+        lane_of<K>(n[5]) = at(5, p.rp + p.xp);
+        lane_of<K>(n[6]) = at(6, p.rp + p.x);
+        lane_of<K>(n[7]) = at(7, p.rp + p.xm);
     };
     auto kap_at = [&](int cc, int rr) -> S {
         if (!kappa) return C.kappa_u;
@@ -131,35 +138,34 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
         if constexpr (N == 2) fn(std::integral_constant<int, 1>{});
     };
 
-    // ---- h and j of the tile, h of the halo of 2
-    X f0, n[8], dh, er, jx, jy, kap, ih;
+    // ---- before the previous step has ended: places, and kappa (which it does
+    // not write)
+    X f0, n[8], dh, er, jx, jy, kap, kh, ih;
+    Spot own[N], beside[N];
+    int hc[N], hr[N], pc[N], pr[N];
     lanes([&](auto k_c) {
         constexpr int K = decltype(k_c)::value;
-        pull(k_c, c, r + K * HALF, f0, n);
+        own[K] = spot(c, r + K * HALF);
         lane_of<K>(kap) = kap_at(c, r + K * HALF);
-    });
-    // kappa of the halo of 1, requested here so that phase 2 waits for no load
-    X kh;
-    int pc[N], pr[N];
-    if (t < PP) {
-        lanes([&](auto k_c) {
-            constexpr int K = decltype(k_c)::value;
+        if (t < HP) {
+            tile_halo<TX, TY, 2>(t + K * HP, hc[K], hr[K]);
+            beside[K] = spot(hc[K], hr[K]);
+        }
+        if (t < PP) {
             tile_halo<TX, TY, 1>(t + K * PP, pc[K], pr[K]);
             lane_of<K>(kh) = kap_at(pc[K], pr[K]);
-        });
-    }
+        }
+    });
+    dependent_launch_wait();
+    // ---- h and j of the tile, h of the halo of 2
+    lanes([&](auto k_c) { pull(k_c, own[decltype(k_c)::value], f0, n); });
     if (t < HP) {
         X g0, g[8], d, e, a, b;
-        int cc[N], rr[N];
-        lanes([&](auto k_c) {
-            constexpr int K = decltype(k_c)::value;
-            tile_halo<TX, TY, 2>(t + K * HP, cc[K], rr[K]);
-            pull(k_c, cc[K], rr[K], g0, g);
-        });
+        lanes([&](auto k_c) { pull(k_c, beside[decltype(k_c)::value], g0, g); });
         node_moments<SM>(g0, g, C, d, e, a, b);
         lanes([&](auto k_c) {
             constexpr int K = decltype(k_c)::value;
-            hs[rr[K] + 2][cc[K] + 2] = lane_of<K>(d);
+            hs[hr[K] + 2][hc[K] + 2] = lane_of<K>(d);
         });
     }
     node_moments<SM>(f0, n, C, dh, er, jx, jy);
@@ -205,6 +211,12 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     }
     __syncthreads();
 
+    // Let the next step's CTAs be placed now, when every tile of this step is on
+    // an SM and near its end.  Placed as soon as this step starts, they went to
+    // the SMs that had room then, two or three to one and none to another (one
+    // box, us a step: FP64 tau = 0.8 128^2 25.3 / 8.5, 250 x 190 25.2 / 20.1; FP32
+    // 256^2 3.6 / 3.1).
+    dependent_launch_next();
     // ---- force, collision and store of the tile
     Win<X> W;
     lanes([&](auto k_c) {
@@ -217,17 +229,15 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
             constexpr int K = decltype(k_c)::value;
             const int y = y0 + r + K * HALF;
             if (x >= nx || y >= ny) return;
-            const int i = y * pitch + x;
-            const long long m8 = 8LL * plane;
-            (void)m8;
-            fout0[TFLBM_IDX(i, plane, C.status)] = lane_of<K>(o0);
+            const uint32_t i = TFLBM_IDX((uint32_t)(y * pitch + x), plane, C.status);
+            fout0[i] = lane_of<K>(o0);
 #pragma unroll
             for (int l = 0; l < 8; ++l) {
                 SM v;
                 if constexpr (N == 1) v = q[l];
                 else if constexpr (K == 0) v = q[l].x;
                 else v = q[l].y;
-                foutm[TFLBM_IDX(l * plane + i, m8, C.status)] = v;
+                (foutm + l * plane)[i] = v;
             }
         });
     });
@@ -244,7 +254,7 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
         if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, G, C);
         return launch_dependent(k_tile<SM, S, TX, TY, false, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, G, C);
     };
-    // Threads an SM holds.  512 leaves the registers that keep a thread's 18
+    // Threads an SM holds.  768 leaves the registers that keep a thread's 18
     // loads in flight (80); where 32 x 16 tiles outnumber the three an SM
     // holds then, 64 registers and a fourth tile win (one box, tau = 1: 509 x
     // 387 4.9 against 5.7 us a step, 512^2 6.4 against 5.3, 1024^2 17.8
@@ -252,7 +262,7 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
     if constexpr (TX == 32 && sizeof(S) == 4) {
         if ((long long)grid.x * grid.y > 3LL * sm_count()) return launch(std::integral_constant<int, 1024>{});
     }
-    return launch(std::integral_constant<int, 512>{});
+    return launch(std::integral_constant<int, sizeof(S) == 4 ? 768 : 512>{});
 }
 
 // One step from fin to fout in the tiles that block_x names (tile_of); mom, if

@@ -326,6 +326,7 @@ struct tf_lbm_tape {
     size_t state_bytes = 0;        // one raw population buffer
     size_t rec_bytes = 0;          // one record: h - href, j_x, j_y
     size_t a_bytes = 0;            // one adjoint state
+    void* block = nullptr;         // one allocation for what follows
     void* ck = nullptr;            // states at 0, K, 2K, ... (nseg > 1), then two buffers to recompute in
     void* rec = nullptr;           // `every` records
     void* abuf = nullptr;          // 2 adjoint states
@@ -406,29 +407,41 @@ int tf_lbm_tape_create(tf_lbm_handle* H, const void* h0, const void* theta, int6
         tf_lbm_tape_destroy(tp);
         return rc;
     };
-    // all records where they fit (every <= 0 leaves the choice here; an
-    // explicit `every` asks for segments of that length), else segments
+    // One allocation.  All records where they fit (every <= 0 leaves the choice
+    // here; an explicit `every` asks for segments of that length), else segments
+    const size_t field = n * H->esize;
+    auto allocate = [&](int64_t kept) {
+        tp->every = (int)kept;
+        tp->nseg = (int)((nsteps + kept - 1) / kept);
+        Carver cut;
+        const size_t at_a = cut.take(2 * tp->a_bytes), at_gk = cut.take(field), at_h0 = cut.take(field);
+        const size_t at_theta = cut.take(theta ? field : 0);
+        const size_t at_ck = cut.take(tp->nseg > 1 ? tp->state_bytes * (tp->nseg + 2) : 0);
+        const size_t at_rec = cut.take(tp->rec_bytes * kept);
+        const cudaError_t err = cudaMalloc(&tp->block, cut.total);
+        if (err != cudaSuccess) {
+            tp->block = nullptr;
+            return err;
+        }
+        char* block = (char*)tp->block;
+        tp->abuf = block + at_a;
+        tp->gk = block + at_gk;
+        tp->h0 = block + at_h0;
+        tp->theta = theta ? block + at_theta : nullptr;
+        tp->ck = block + at_ck;
+        tp->rec = block + at_rec;
+        return cudaSuccess;
+    };
     if (every <= 0 && (size_t)nsteps <= kTapeBytes / tp->rec_bytes && nsteps <= INT32_MAX &&
-        cudaMalloc(&tp->rec, tp->rec_bytes * nsteps) == cudaSuccess) {
-        tp->every = (int)nsteps;
-    } else {
+        allocate(nsteps) != cudaSuccess)
         cudaGetLastError();
+    if (!tp->block) {
         if (every <= 0) every = (int32_t)ceil(sqrt((double)nsteps));
-        tp->every = (int)std::min<int64_t>(every, nsteps);
-        if ((e = cudaMalloc(&tp->rec, tp->rec_bytes * tp->every)) != cudaSuccess) return bail(e, "cudaMalloc records");
+        if ((e = allocate(std::min<int64_t>(every, nsteps))) != cudaSuccess) return bail(e, "cudaMalloc tape");
     }
-    tp->nseg = (int)((nsteps + tp->every - 1) / tp->every);
-    if (tp->nseg > 1 && (e = cudaMalloc(&tp->ck, tp->state_bytes * (tp->nseg + 2))) != cudaSuccess)
-        return bail(e, "cudaMalloc checkpoints");
-    if ((e = cudaMalloc(&tp->abuf, 2 * tp->a_bytes)) != cudaSuccess) return bail(e, "cudaMalloc adjoint");
-    if ((e = cudaMalloc(&tp->gk, n * H->esize)) != cudaSuccess) return bail(e, "cudaMalloc grad kappa");
-    if ((e = cudaMalloc(&tp->h0, n * H->esize)) != cudaSuccess) return bail(e, "cudaMalloc h0");
-    if ((e = cudaMemcpy(tp->h0, h0, n * H->esize, cudaMemcpyDeviceToDevice)) != cudaSuccess) return bail(e, "copy h0");
-    if (theta) {
-        if ((e = cudaMalloc(&tp->theta, n * H->esize)) != cudaSuccess) return bail(e, "cudaMalloc theta");
-        if ((e = cudaMemcpy(tp->theta, theta, n * H->esize, cudaMemcpyDeviceToDevice)) != cudaSuccess)
-            return bail(e, "copy theta");
-    }
+    if ((e = cudaMemcpy(tp->h0, h0, field, cudaMemcpyDeviceToDevice)) != cudaSuccess) return bail(e, "copy h0");
+    if (theta && (e = cudaMemcpy(tp->theta, theta, field, cudaMemcpyDeviceToDevice)) != cudaSuccess)
+        return bail(e, "copy theta");
     *out = tp;
     return TF_LBM_OK;
 }
@@ -500,8 +513,7 @@ void tf_lbm_tape_destroy(tf_lbm_tape* tp)
 {
     if (!tp) return;
     cudaDeviceSynchronize();
-    for (void* p : {tp->ck, tp->rec, tp->abuf, tp->gk, tp->h0, tp->theta})
-        if (p) cudaFree(p);
+    if (tp->block) cudaFree(tp->block);
     delete tp;
 }
 

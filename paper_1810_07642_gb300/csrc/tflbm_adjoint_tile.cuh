@@ -95,20 +95,32 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
         });
     }
     if constexpr (OMEGA1) {
-        constexpr int AN = AW * (TY + 6), PASSES = (AN + NT - 1) / NT;
-        S v[PASSES][3];
+        // the tile's columns, NT / TX rows a pass, then the three on either side
+        constexpr int RP = NT / TX, PASSES = (TY + 6 + RP - 1) / RP, SIDES = (6 * (TY + 6) + NT - 1) / NT;
+        S v[PASSES + SIDES][3];
+        const uint32_t xc = ring_index(x0 + c, nx);
 #pragma unroll
         for (int p = 0; p < PASSES; ++p) {
-            const int i = t + p * NT, k = node(i % AW - 3, i / AW - 3);
+            const int rr = r + p * RP;
+            const uint32_t k = ring_index(y0 + rr - 3, ny) * nx + xc;
 #pragma unroll
-            for (int f = 0; f < 3; ++f) v[p][f] = i < AN ? ldro(an + f * n + k) : S(0);
+            for (int f = 0; f < 3; ++f) v[p][f] = rr < TY + 6 ? ldro(an + f * n + k) : S(0);
         }
 #pragma unroll
-        for (int p = 0; p < PASSES; ++p) {
-            const int i = t + p * NT;
-            if (i < AN) {
+        for (int p = 0; p < SIDES; ++p) {
+            const int i = t + p * NT, rr = i / 6, cc = i % 6 < 3 ? i % 6 - 3 : TX + i % 6 - 3;
+            const uint32_t k = node(cc, rr - 3);
 #pragma unroll
-                for (int f = 0; f < 3; ++f) (&as[f][0][0])[i] = v[p][f];
+            for (int f = 0; f < 3; ++f) v[PASSES + p][f] = rr < TY + 6 ? ldro(an + f * n + k) : S(0);
+        }
+#pragma unroll
+        for (int p = 0; p < PASSES + SIDES; ++p) {
+            const int i = t + (p - PASSES) * NT;
+            const int rr = p < PASSES ? r + p * RP : i / 6;
+            const int cc = p < PASSES ? c : (i % 6 < 3 ? i % 6 - 3 : TX + i % 6 - 3);
+            if (rr < TY + 6) {
+#pragma unroll
+                for (int f = 0; f < 3; ++f) as[f][rr][cc + 3] = v[p][f];
             }
         }
     }

@@ -324,26 +324,32 @@ int tf_lbm_init(tf_lbm_handle** out, const tf_lbm_params* params, const void* h0
         tf_lbm_destroy(H);
         return code;
     };
+    // one allocation (35 to 80 us each to make and to free, of which a gradient's
+    // handle and tape took sixteen): populations and flag, which start at zero,
+    // then kappa and the reduction scratch
     const size_t bytes = (size_t)H->G.plane * (H->esize + 8 * H->msize);
-    cudaError_t e;
-    for (int b = 0; b < 2; ++b) {
-        if ((e = cudaMalloc(&H->buf[b], bytes)) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMalloc populations"));
-        if ((e = cudaMemsetAsync(H->buf[b], 0, bytes, st)) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMemsetAsync"));
-    }
+    const long long n = (long long)params->nx * params->ny;
     H->nmass = mass_blocks(H->G);
     if (H->nmass < kSumBlocks) H->nmass = kSumBlocks;
-    if ((e = cudaMalloc(&H->partials, sizeof(double) * 2 * H->nmass + sizeof(double))) != cudaSuccess)
-        return bail(cuda_fail(H, e, "cudaMalloc scratch"));
-    H->result = H->partials + 2 * H->nmass;
-    if ((e = cudaMalloc(&H->flag, 2 * sizeof(int))) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMalloc flag"));
+    Carver cut;
+    const size_t at0 = cut.take(bytes), at1 = cut.take(bytes), at_flag = cut.take(2 * sizeof(int)), zeros = cut.total;
+    const size_t at_kappa = cut.take(theta ? n * H->esize : 0);
+    const size_t at_partials = cut.take(sizeof(double) * 2 * H->nmass + sizeof(double));
+    cudaError_t e;
+    if ((e = cudaMalloc(&H->block, cut.total)) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMalloc populations"));
+    char* block = (char*)H->block;
+    H->buf[0] = block + at0;
+    H->buf[1] = block + at1;
+    H->flag = (int*)(block + at_flag);
     H->status = H->flag + 1;
-    if ((e = cudaMemsetAsync(H->flag, 0, 2 * sizeof(int), st)) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMemsetAsync"));
+    H->partials = (double*)(block + at_partials);
+    H->result = H->partials + 2 * H->nmass;
+    if ((e = cudaMemsetAsync(H->block, 0, zeros, st)) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMemsetAsync"));
 
     const double kscale = (double)(params->n_exp - 1) * (params->m_exp - 1) /
                           ((double)(params->n_exp - params->m_exp) * params->hstar);
-    const long long n = (long long)params->nx * params->ny;
     if (theta) {
-        if ((e = cudaMalloc(&H->kappa, n * H->esize)) != cudaSuccess) return bail(cuda_fail(H, e, "cudaMalloc kappa"));
+        H->kappa = block + at_kappa;
         e = aux_kappa(H->dbl, H->kappa, theta, params->nx, params->ny, params->n_exp, params->m_exp,
                       params->hstar, st);
         if (e != cudaSuccess) return bail(cuda_fail(H, e, "kappa kernel"));
@@ -554,11 +560,7 @@ void tf_lbm_destroy(tf_lbm_handle* H)
     cudaDeviceSynchronize();
     drop_graphs(H);
     if (H->cap) cudaStreamDestroy(H->cap);
-    for (auto& b : H->buf)
-        if (b) cudaFree(b);
-    if (H->kappa) cudaFree(H->kappa);
-    if (H->partials) cudaFree(H->partials);
-    if (H->flag) cudaFree(H->flag);
+    if (H->block) cudaFree(H->block);
     if (H->adj) cudaFree(H->adj);
     if (H->dscr) cudaFree(H->dscr);
     if (H->tscr) cudaFree(H->tscr);

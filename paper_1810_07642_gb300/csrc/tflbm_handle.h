@@ -20,6 +20,7 @@ struct tf_lbm_handle {
     bool dbl = false;          // compute type is double
     StoreDesc desc{};          // storage encoding (for the auxiliary kernels)
     Geom G{};
+    void* block = nullptr;     // one allocation for everything below that is not lazy
     void* buf[2] = {nullptr, nullptr};
     int cur = 0;               // buf[cur] holds the post-collision populations of step t-1
     void* kappa = nullptr;     // [ny][nx] or null (uniform)
@@ -44,6 +45,16 @@ struct tf_lbm_handle {
 
 
 namespace tflbm {
+// Offsets of several arrays in one allocation, each on a 256-byte boundary.
+struct Carver {
+    size_t total = 0;
+    size_t take(size_t bytes)
+    {
+        const size_t at = total;
+        total += (bytes + 255) / 256 * 256;
+        return at;
+    }
+};
 // Per-run step constants of a handle, in the compute type T.
 template <typename T>
 Consts<T> make_consts(const tf_lbm_handle* H);

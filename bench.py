@@ -35,21 +35,32 @@ sys.path.insert(0, ROOT)
 
 METRIC = "MLUPS (D2Q9 thin-film step) and % of HBM roofline; adjoint/forward cost ratio"
 N_SIDE = 2048
-BYTES_PER_LU = 76  # FP32: 9 populations read + 9 written + kappa(x)
+# FP32 populations: 9 read + 9 written + kappa(x).  Between the steps of one call
+# the default kernel keeps six moments a node instead (24 B, see step_bytes).
+BYTES_PER_LU = 76
 _CSRC = "paper_1810_07642_gb300/csrc/"
 # committed ncu summary of the default step kernel of each storage form and
 # the sources that kernel is compiled from (the summary's kernel_hash)
 PROFILES = {
-    "f32": ("k_step2_f32_patterned_2048.txt",
-            [_CSRC + "tflbm_step.cuh", _CSRC + "tflbm_step2.cuh", _CSRC + "step2_f32.cu",
-             _CSRC + "tflbm_internal.h"]),
-    "f16": ("k_step2_f16_patterned_2048.txt",
-            [_CSRC + "tflbm_step.cuh", _CSRC + "tflbm_step2.cuh", _CSRC + "step2_f16.cu",
-             _CSRC + "tflbm_internal.h"]),
+    s: (f"k_step4_{s}_patterned_2048.txt",
+        [_CSRC + f for f in ("tflbm_step.cuh", "tflbm_node.cuh", "tflbm_tile.cuh", "tflbm_step4.cuh", "step4.cu",
+                             "tflbm_internal.h")])
+    for s in ("f32", "f16")
 }
 WORKLOAD = ("chemically patterned dewetting, 2048x2048 periodic D2Q9 thin film, FP32 "
             "populations; h0=1+U(-1e-2,1e-2); theta stripes period 256 (10/40 deg) + 32 "
             "seeded discs (10 deg); gamma=0.01, h*=0.07, (n,m)=(3,2), tau=1, delta=1, g=0")
+
+
+def step_bytes(storage: str, steps: int, moments: bool, kappa: int = 4) -> float:
+    """Bytes per node and step of a run of `steps` steps: FP32 populations (36 B)
+    or, between two steps of a call of the four-column march, moments (24 B); 16-bit
+    populations 20 B; plus kappa."""
+    if storage != "f32":
+        return 40 + kappa
+    if not moments or steps < 2:
+        return 72 + kappa
+    return (2 * 36 + (2 * steps - 2) * 24) / steps + kappa
 
 
 def kernel_hash(storage: str = "f32") -> str:
@@ -250,7 +261,7 @@ def storage_variants(steps: int = 2000, check_steps: int = 1000):
     from paper_1810_07642_gb300.film import ThinFilm
     out = {}
     h0, th, p = inputs.patterned_dewetting(N_SIDE, seed=0)
-    for dt, bpl in (("f32", 76), ("f16", 44), ("bf16", 44), ("f64", 152)):
+    for dt, bpl in (("f32", step_bytes("f32", steps, True)), ("f16", 44), ("bf16", 44), ("f64", 152)):
         sim = ThinFilm(p, h0, th, dtype=dt)
         sim.step(50)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -281,11 +292,20 @@ def storage_variants(steps: int = 2000, check_steps: int = 1000):
     return out
 
 
+def tape_form(n: int, steps: int):
+    """What the gradient tape does for an n^2 FP32 lattice: its description and
+    its kernel launches a gradient (records of 12 B a node and step, kept while
+    they fit in 8 GiB; else recomputed in segments of ceil(sqrt(steps)))."""
+    if steps * 12 * n * n <= 8 << 30:
+        return "all step records kept", 2 * steps
+    return f"checkpoints every {int(math.ceil(math.sqrt(steps)))} steps", 3 * steps
+
+
 def adjoint_cost(n: int = 512, nsteps: int = 20000, repeats: int = 3):
     """Cost of one gradient of the inverse-design loss (checkpointed forward +
     backward with the hand-written adjoint) in units of a plain forward run,
-    FP32, on the inverse-design workload (n^2, T = nsteps, sqrt(T)
-    checkpoints).  Both are timed with CUDA events on the current stream,
+    FP32, on the inverse-design workload (n^2, T = nsteps; at the default
+    T sqrt(T) checkpoints).  Both are timed with CUDA events on the current stream,
     `repeats` times each; the median and the spread (max/min - 1) are
     reported."""
     import torch
@@ -322,8 +342,7 @@ def adjoint_cost(n: int = 512, nsteps: int = 20000, repeats: int = 3):
     t_fwd = sorted(timed(forward) for _ in range(repeats))
     t_grad = sorted(timed(gradient) for _ in range(repeats))
     med = lambda v: v[len(v) // 2]
-    return {"workload": f"inverse design {n}x{n}, T={nsteps}, checkpoints every "
-                        f"{int(math.ceil(math.sqrt(nsteps)))} steps, FP32",
+    return {"workload": f"inverse design {n}x{n}, T={nsteps}, {tape_form(n, nsteps)[0]}, FP32",
             "timing": f"CUDA events, {repeats} runs each, median",
             "forward_s": med(t_fwd), "gradient_s": med(t_grad),
             "forward_spread": t_fwd[-1] / t_fwd[0] - 1, "gradient_spread": t_grad[-1] / t_grad[0] - 1,
@@ -687,7 +706,8 @@ def run_tflbm(args):
     # dominant kernel: the fused step, one launch per step, launches back to
     # back, so its average duration is the timed region over K
     kern_s = t_local / args.steps
-    bpl = BYTES_PER_LU if args.storage == "f32" else 44  # 16-bit: 2 x (4 + 8 x 2) + 4
+    moments = not args.launch  # the default shape runs the four-column march
+    bpl = step_bytes(args.storage, args.steps, moments)
     achieved = bpl * nodes / kern_s / 1e9
     peak, peak_kind = measured_peaks()
     traffic, prof = profiled_traffic(args.storage)
@@ -703,7 +723,8 @@ def run_tflbm(args):
         hd = h_host.to("cuda", non_blocking=True)
         thd = th_host.to("cuda", non_blocking=True)
         sim2 = ThinFilm(p, hd, thd, dtype=args.storage, stream=stream)
-        sim2.set_launch(**launch)
+        if args.launch:
+            sim2.set_launch(**launch)
         sim2.step(args.steps)
         hres = sim2.moments(("h",))["h"]
         out_host.copy_(hres, non_blocking=True)
@@ -739,7 +760,7 @@ def run_tflbm(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_kind": f"{peak_kind} copy bandwidth",
-                     "kernel": ("k_step2<" if launch["pipeline"] == 3 else "k_step<") +
+                     "kernel": ("k_step4<" if moments else "k_step2<" if launch["pipeline"] == 3 else "k_step<") +
                                {"f32": "float", "f16": "__half", "bf16": "__nv_bfloat16"}[args.storage] + ",...>",
                      "kernel_ms": kern_s * 1e3},
         "cpu_baseline": cpu,
@@ -804,7 +825,7 @@ def run_sweep(args):
     t_local = ev0.elapsed_time(ev1) / 1e3
     t_max = max_over_ranks(t_local, dist, "cuda")
     value = aggregate_mlups(nodes, args.steps, world, t_max)
-    bpl = 72  # FP32, uniform theta: 9 populations read + 9 written
+    bpl = step_bytes("f32", args.steps, not args.batch_launch, kappa=0)  # uniform theta
     achieved = bpl * nodes / (t_local / args.steps) / 1e9
     peak, peak_kind = measured_peaks()
     if rank == 0:
@@ -820,7 +841,7 @@ def run_sweep(args):
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                              "frac": achieved / peak, "traffic": None,
                              "peak_kind": f"{peak_kind} copy bandwidth",
-                             "kernel": "k_step_batch<float,float,...>"},
+                             "kernel": "k_step4_batch<float,...>" if not args.batch_launch else "k_step2_batch<float,...>"},
                 "gpu_launches": args.steps, "clocks": clk.summary()}
         print(json.dumps(line), flush=True)
     B.close()
@@ -882,8 +903,6 @@ def run_adjoint(args):
         torch.cuda.synchronize()
         t_local = time.perf_counter() - t0
     t_max = max_over_ranks(t_local, dist, "cuda")
-    every = int(math.ceil(math.sqrt(T)))
-    nck = (T + every - 1) // every
     if rank == 0:
         line = {"metric": METRIC, "value": aggregate_mlups(n * n, T * args.steps, world, t_max),
                 "unit": "MLUPS", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -891,14 +910,13 @@ def run_adjoint(args):
                 "vs_baseline": None, "dtype": "f32", "data": "synthetic",
                 "config": {"workload": f"inverse design gradient: {n}x{n} periodic, FP32, flat film "
                                        f"with 1e-2 noise, theta 30 deg + 5 deg noise, 8-drop target, L2 "
-                                       f"loss, T={T}, checkpoints every {int(math.ceil(math.sqrt(T)))} "
-                                       f"steps", "l2": "L2-resident lattice (20 MB); timed on the host "
+                                       f"loss, T={T}, {tape_form(n, T)[0]}", "l2": "L2-resident lattice (20 MB); timed on the host "
                                        "clock around whole gradients"},
                 "adjoint_forward_cost_ratio": t_local / args.steps / t_fwd,
                 "forward_s": t_fwd,
-                # per gradient: T forward steps, T - nck recomputed steps, T adjoint
-                # steps, the seed, the initial-state adjoint and the final moments
-                "gpu_launches": args.steps * (3 * T - nck + 3), "clocks": clk.summary()}
+                # per gradient: the tape's steps, the seed, the initial-state
+                # adjoint and the final moments
+                "gpu_launches": args.steps * (tape_form(n, T)[1] + 3), "clocks": clk.summary()}
         print(json.dumps(line), flush=True)
     if dist:
         dist.destroy_process_group()

@@ -241,18 +241,21 @@ int tf_lbm_set_wait_limit(tf_lbm_handle* H, int32_t polls);
 int tf_lbm_adjoint_step(tf_lbm_handle* H, const void* f_t, const void* a_next, void* a_t,
                         void* grad_kappa, void* stream);
 
-/* Gradient tape over nsteps steps with checkpoint-recompute: a copy of the
- * state every `every` steps (<= 0: ceil(sqrt(nsteps))).  h0 and theta
+/* Gradient tape over nsteps steps.  It keeps a record of every step (h and j,
+ * 3 elements a node; what the adjoint reads of a state).  every > 0: records of
+ * `every` steps at a time, recomputed from copies of the state that many steps
+ * apart.  every <= 0: the records of all steps while these take 8 GiB or less
+ * and can be allocated, else as every = ceil(sqrt(nsteps)).  h0 and theta
  * (device [ny][nx], theta NULL = params->theta_uniform) must be the ones the
  * handle was created from; they are copied. */
 typedef struct tf_lbm_tape tf_lbm_tape;
 int tf_lbm_tape_create(tf_lbm_handle* H, const void* h0, const void* theta, int64_t nsteps,
                        int32_t every, tf_lbm_tape** out);
-/* Advance the handle by nsteps, storing the checkpoints. */
+/* Advance the handle by nsteps, storing the records and the state copies. */
 int tf_lbm_tape_forward(tf_lbm_tape* tape, void* stream);
 /* Given grad_h = dL/dh at the final time ([ny][nx]), write dL/dtheta and
  * dL/dh0 (each [ny][nx], or NULL to skip).  Recomputes each segment from its
- * checkpoint; the handle ends at the final state again. */
+ * state copy where not all records are kept; the handle ends at the final state again. */
 int tf_lbm_tape_backward(tf_lbm_tape* tape, const void* grad_h, void* grad_theta, void* grad_h0,
                          void* stream);
 void tf_lbm_tape_destroy(tf_lbm_tape* tape);

@@ -130,10 +130,7 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            tf_lbm_set_launch gives ceil(ny / rows) bands;
  *   graph_chunk: steps per captured CUDA graph in tf_lbm_step (0 = none,
  *            otherwise an even number >= 2);
- *   pipeline: 4 = every CTA owns one tile (16 x 8 nodes for block_x 64, 16 x
- *            16 for 128, 32 x 16 for 256; rows is not used) and runs the
- *            step's phases over all of it (any nx, ny and dtype);
- *            3 = every thread owns two adjacent columns, loads aligned
+ *   pipeline: 3 = every thread owns two adjacent columns, loads aligned
  *            pairs one (FP32) or two (16-bit) rows ahead, takes the values
  *            that cross a pair boundary from the neighbouring lane and
  *            computes both nodes with paired FP32 instructions (nx even, not
@@ -146,7 +143,9 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            only); 0 = row segments streamed into shared memory by bulk
  *            copies four rows ahead (needs nx a multiple of 8, >= 16).
  * The shape chosen by tf_lbm_init runs other kernels in place of the one that
- * its fields describe: tiles on lattices of up to 2^20 nodes (1.5 x 2^20 where
+ * its fields describe: tiles (a CTA
+ * owns 16 x 8, 16 x 16 or 32 x 16 nodes and runs the step's phases over all of
+ * them; any nx, ny and dtype) on lattices of up to 2^20 nodes (1.5 x 2^20 where
  * the next one does not apply; any size for TF_LBM_F64, and for 16-bit storage
  * where the fields describe pipeline 1); above that, at tau = 1
  * with forcing = 0, a march of four columns per thread, which between the

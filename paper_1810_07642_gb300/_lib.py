@@ -197,6 +197,13 @@ def tf_lbm_set_launch(handle: int, block_x: int, rows: int, graph_chunk: int,
     _check(lib().tf_lbm_set_launch(_VP(handle), ctypes.byref(L)), _VP(handle))
 
 
+def use_tiles(handle: int, block_x: int, graph_chunk: int = 0) -> None:
+    """For tests, not part of the interface: run the tile kernel of this
+    block_x whatever the lattice's size."""
+    if lib().tflbm_use_tiles(_VP(handle), block_x, graph_chunk):
+        raise ValueError("block_x or graph_chunk")
+
+
 def tf_lbm_set_wait_limit(handle: int, polls: int) -> None:
     _check(lib().tf_lbm_set_wait_limit(_VP(handle), int(polls)), _VP(handle))
 

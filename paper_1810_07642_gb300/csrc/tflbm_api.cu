@@ -525,10 +525,10 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
     if (in->graph_chunk < 0 || (in->graph_chunk % 2) != 0 || in->graph_chunk > 4096)
         return fail(H, TF_LBM_ERR_ARG, "graph_chunk must be 0 or an even number <= 4096");
     if (in->pipeline != kPipeTma && in->pipeline != kPipeLdg && in->pipeline != kPipeAsync &&
-        in->pipeline != kPipePair && in->pipeline != kPipeTile)
+        in->pipeline != kPipePair)
         return fail(H, TF_LBM_ERR_ARG,
-                    "pipeline must be 0 (bulk copies), 1 (per-thread loads), 2 (per-thread async copies), "
-                    "3 (two columns per thread) or 4 (tiles)");
+                    "pipeline must be 0 (bulk copies), 1 (per-thread loads), 2 (per-thread async copies) "
+                    "or 3 (two columns per thread)");
     if (in->pipeline == kPipePair && !pair_pipeline_ok(H->G.nx, H->desc.store))
         return fail(H, TF_LBM_ERR_ARG, "the two-column pipeline needs nx even and an FP32 compute type");
     if (in->pipeline == kPipeAsync && H->msize != H->esize)
@@ -540,9 +540,22 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
     H->shape.block_x = bx;
     H->shape.rows = in->rows;
     H->shape.bands = 0;
-    H->shape.tile = in->pipeline == kPipeTile ? bx : 0;
+    H->shape.tile = 0;
     H->shape.wide = 0;
     H->graph_chunk = in->graph_chunk;
+    return TF_LBM_OK;
+}
+
+// Not part of the interface: run the tiles that block_x names (tile_of) on any
+// lattice, for the tests of tile edges.
+int tflbm_use_tiles(tf_lbm_handle* H, int32_t block_x, int32_t graph_chunk)
+{
+    if (!H || (block_x != 64 && block_x != 128 && block_x != 256) || graph_chunk < 0 || graph_chunk % 2 != 0)
+        return TF_LBM_ERR_ARG;
+    drop_graphs(H);
+    H->shape.tile = block_x;
+    H->shape.wide = 0;
+    H->graph_chunk = graph_chunk;
     return TF_LBM_OK;
 }
 

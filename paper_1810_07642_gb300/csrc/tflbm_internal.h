@@ -19,7 +19,6 @@ constexpr int kPipeTma = 0;
 constexpr int kPipeLdg = 1;
 constexpr int kPipeAsync = 2;  // per-thread cp.async staging (full-width storage only)
 constexpr int kPipePair = 3;   // two columns per thread (FP32 compute type, nx even)
-constexpr int kPipeTile = 4;   // one tile per CTA (any size)
 // Tile of the tile kernel for a block_x: half its nodes (one thread per two
 // nodes with an FP32 compute type).
 struct TileShape {
@@ -91,7 +90,7 @@ struct Consts {
 struct Shape {
     int block_x;    // 64, 128, 256
     int rows;       // rows per CTA (band height)
-    int pipeline;   // kPipeTma, kPipeLdg, kPipeAsync, kPipePair, or kPipeTile (then tile == block_x)
+    int pipeline;   // kPipeTma, kPipeLdg, kPipeAsync or kPipePair
     int bands = 0;  // balanced bands per launch; 0: ny / rows rounded up
     int tile = 0;   // run the tile kernel with this block_x (tile_of) instead of a march; 0: march
     int wide = 0;   // run the four-column march in this many bands instead; 0: no

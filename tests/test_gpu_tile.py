@@ -1,4 +1,4 @@
-"""The tile kernel (pipeline 4) at the edges of its tiles against the oracle.
+"""The tile kernel at the edges of its tiles against the oracle.
 
 Tolerances: those of the parity tests (relative L-infinity on h, 60 steps):
 FP32 1e-5, FP64 1e-11, 16-bit storage 1e-3; relative mass drift 1e-6.
@@ -14,7 +14,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 import oracle as O
-from paper_1810_07642_gb300 import inputs
+from paper_1810_07642_gb300 import _lib, inputs
 from paper_1810_07642_gb300.film import ThinFilm
 
 pytestmark = pytest.mark.gpu
@@ -34,7 +34,7 @@ def compare(nx, ny, dtype, tau, forcing, theta_field):
         p["theta_uniform"] = math.radians(20.0)
     for block_x in (64, 128, 256):
         sim = ThinFilm(p, h0, th if theta_field else None, dtype=dtype)
-        sim.set_launch(pipeline=4, block_x=block_x, rows=16, graph_chunk=4)
+        _lib.use_tiles(sim.handle, block_x, graph_chunk=4)
         m0 = sim.mass()
         sim.step(60)
         h = sim.h().double().cpu().numpy()
@@ -61,9 +61,11 @@ def test_tiles_give_the_two_column_march_bit_for_bit(dtype):
         h0, th, p = inputs.small_random(nx, ny, seed=5, amp=0.05)
         p.update(g=2e-4, gx_body=1e-5)
         states = []
-        for shape in (None, dict(pipeline=4, block_x=256), dict(pipeline=4, block_x=64), dict(pipeline=3, block_x=128, rows=16)):
+        for shape in (None, 256, 64, dict(pipeline=3, block_x=128, rows=16)):
             sim = ThinFilm(p, h0, th, dtype=dtype)
-            if shape:
+            if isinstance(shape, int):
+                _lib.use_tiles(sim.handle, shape)
+            elif shape:
                 sim.set_launch(**shape)
             sim.step(50)
             states.append(sim.get_state())
@@ -76,8 +78,8 @@ def test_tile_launch_reporting():
     h0, th, p = inputs.small_random(200, 120, seed=4)
     sim = ThinFilm(p, h0, th)
     assert sim.launch["pipeline"] == 3  # the march that the fields describe
-    sim.set_launch(pipeline=4, block_x=128)
-    assert sim.launch["pipeline"] == 4 and sim.launch["block_x"] == 128
+    with pytest.raises(Exception):
+        sim.set_launch(pipeline=4, block_x=128)
     sim.step(3)
     sim.set_launch(**dict(sim.launch, pipeline=1))
     assert sim.launch["pipeline"] == 1
@@ -92,7 +94,7 @@ def test_tile_indices_stay_in_bounds():
     lib = build.build(checked=True)
     code = """
 import sys
-from paper_1810_07642_gb300 import inputs
+from paper_1810_07642_gb300 import _lib, inputs
 from paper_1810_07642_gb300.film import ThinFilm
 bad = []
 for nx, ny in %r:
@@ -100,7 +102,7 @@ for nx, ny in %r:
         for bx in (64, 128, 256):
             h0, th, p = inputs.small_random(nx, ny, seed=1, amp=0.05)
             sim = ThinFilm(dict(p, tau=0.9), h0, th, dtype=dtype)
-            sim.set_launch(pipeline=4, block_x=bx, rows=16)
+            _lib.use_tiles(sim.handle, bx)
             sim.step(5)
             if sim.check():
                 bad.append((nx, ny, dtype, bx, sim.check()))

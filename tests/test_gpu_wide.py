@@ -15,7 +15,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 import oracle as O
-from paper_1810_07642_gb300 import inputs
+from paper_1810_07642_gb300 import _lib, inputs
 from paper_1810_07642_gb300.film import FilmBatch, ThinFilm
 
 pytestmark = pytest.mark.gpu
@@ -67,7 +67,7 @@ def test_large_lattice_splits_and_bits(dtype, nx, ny):
         sim = ThinFilm(p, h0, th, dtype=dtype)
         m0 = sim.mass()
         if split is None:
-            sim.set_launch(pipeline=4, block_x=256)  # tiles run the same node arithmetic
+            _lib.use_tiles(sim.handle, 256)  # tiles run the same node arithmetic
             sim.step(12)
         else:
             for n in split:

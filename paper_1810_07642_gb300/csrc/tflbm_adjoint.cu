@@ -283,21 +283,24 @@ cudaError_t adjoint_step_dispatch(tf_lbm_handle* H, const void* f, const void* a
 namespace {
 
 template <typename S>
-cudaError_t adjoint_tile_t(tf_lbm_handle* H, const void* mom, const void* an, void* a, void* gk, cudaStream_t st)
+cudaError_t adjoint_tile_t(tf_lbm_handle* H, const void* mom, bool fresh, const void* an, void* a, void* gk, cudaStream_t st)
 {
     const Consts<S> C = make_consts<S>(H);
     const S *m = (const S*)mom, *n = (const S*)an, *k = (const S*)H->kappa;
     switch (tile_block_x(H->dbl ? kStoreF64 : kStoreF32, H->G.nx, H->G.ny, H->sms)) {
-        case 64: return adjoint_tile_one<S, 16, 8>(m, n, (S*)a, (S*)gk, k, H->G, C, st);
-        case 128: return adjoint_tile_one<S, 16, 16>(m, n, (S*)a, (S*)gk, k, H->G, C, st);
-        default: return adjoint_tile_one<S, 32, 16>(m, n, (S*)a, (S*)gk, k, H->G, C, st);
+        case 64: return adjoint_tile_one<S, 16, 8>(m, fresh, n, (S*)a, (S*)gk, k, H->G, C, st);
+        case 128: return adjoint_tile_one<S, 16, 16>(m, fresh, n, (S*)a, (S*)gk, k, H->G, C, st);
+        default: return adjoint_tile_one<S, 32, 16>(m, fresh, n, (S*)a, (S*)gk, k, H->G, C, st);
     }
 }
 
-// One adjoint step from the record of its state.
-cudaError_t adjoint_tile_step(tf_lbm_handle* H, const void* mom, const void* an, void* a, void* gk, cudaStream_t st)
+// One adjoint step from the record of its state.  fresh: the launch before this
+// one may have written it.
+cudaError_t adjoint_tile_step(tf_lbm_handle* H, const void* mom, bool fresh, const void* an, void* a,
+                              void* gk, cudaStream_t st)
 {
-    return H->dbl ? adjoint_tile_t<double>(H, mom, an, a, gk, st) : adjoint_tile_t<float>(H, mom, an, a, gk, st);
+    return H->dbl ? adjoint_tile_t<double>(H, mom, fresh, an, a, gk, st)
+                  : adjoint_tile_t<float>(H, mom, fresh, an, a, gk, st);
 }
 
 // omega == 1 in the compute type: three-field adjoint states
@@ -486,7 +489,7 @@ int tf_lbm_tape_backward(tf_lbm_tape* tp, const void* grad_h, void* grad_theta, 
         const int64_t len = segment_steps(tp, c);
         if (tp->nseg > 1) TK(tp, recompute(tp, c, len, st), "recompute");
         for (int64_t i = len - 1; i >= 0; --i) {
-            TK(tp, adjoint_tile_step(H, (char*)tp->rec + i * tp->rec_bytes, ab + cur * tp->a_bytes,
+            TK(tp, adjoint_tile_step(H, (char*)tp->rec + i * tp->rec_bytes, i == len - 1, ab + cur * tp->a_bytes,
                                      ab + (cur ^ 1) * tp->a_bytes, tp->gk, st), "adjoint step");
             cur ^= 1;
         }

@@ -22,7 +22,7 @@
 //      tile the disjoining-pressure adjoint and dL/dkappa
 //   4  on the tile grad p, the force adjoint, the Laplacian of -gamma ap, a(t)
 // 512^2 FP32, a gradient of 400 steps: 23.8 ms as marches of populations, 6.4 now,
-// of which an adjoint step takes 27 us before, 9 now (911 instructions for two
+// of which an adjoint step took 27 us, 8 now (911 instructions for two
 // nodes, half of the issue slots; 512 tiles on 152 SMs); threads, lanes, tiles and the
 // treatment of the edges are those of tflbm_tile.cuh.
 #pragma once
@@ -36,12 +36,14 @@ __device__ __forceinline__ float2 operator*(float2 a, float2 b) { return pmul(a,
 __device__ __forceinline__ float2 pipow(float2 r, int n) { return make_float2(ipow(r.x, n), ipow(r.y, n)); }
 __device__ __forceinline__ double pipow(double r, int n) { return ipow(r, n); }
 
-// mom: (h - href, j_x, j_y) of the state f(t), [3][ny][nx]; an, a: a(t+1) and
+// mom: (h - href, j_x, j_y) of the state f(t), [3][ny][nx], and whether the
+// launch before this one may still be writing it (fresh); early: let the next
+// step's CTAs in a phase earlier; an, a: a(t+1) and
 // a(t), [3][ny][nx] at omega = 1, else [9][ny][nx]; gk += dL/dkappa.
 template <typename S, int TX, int TY, bool OMEGA1, int RESIDENT>
 __global__ void __launch_bounds__(TX* TY / Lanes<typename TileX<S>::X>::N, RESIDENT / (TX * TY / Lanes<typename TileX<S>::X>::N))
-k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restrict__ a, S* __restrict__ gk,
-               const S* __restrict__ kappa, const Geom G, const Consts<S> C)
+k_adjoint_tile(const S* __restrict__ mom, bool fresh, bool early, const S* __restrict__ an, S* __restrict__ a,
+               S* __restrict__ gk, const S* __restrict__ kappa, const Geom G, const Consts<S> C)
 {
     using X = typename TileX<S>::X;
     constexpr int N = Lanes<X>::N, NT = TX * TY / N, HALF = TY / N;
@@ -55,7 +57,6 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
     __shared__ S ps[TY + 2][PW], ls[TY + 2][PW];    // p and -gamma ap; tile node at [r + 1][c + 1]
     __shared__ S as[OMEGA1 ? 3 : 1][OMEGA1 ? TY + 6 : 1][OMEGA1 ? AW : 1];  // a(t+1); tile node at [r + 3][c + 3]
 
-    dependent_launch_wait();
     const int t = threadIdx.x, nx = G.nx, ny = G.ny;
     const long long n = (long long)nx * ny;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
@@ -68,7 +69,9 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
         if constexpr (N == 2) fn(std::integral_constant<int, 1>{});
     };
 
-    // ---- 1: every load of the step is requested before any is waited for
+    // ---- 1: every load of the step is requested before any is waited for; the
+    // record and kappa, which no adjoint step writes, before the step at t + 1 ends
+    if (fresh) dependent_launch_wait();
     X dh, jx, jy, kap, gold, kh;
     lanes([&](auto k_c) {
         constexpr int K = decltype(k_c)::value;
@@ -77,7 +80,6 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
         lane_of<K>(jx) = ldro(mom + n + i);
         lane_of<K>(jy) = ldro(mom + 2 * n + i);
         lane_of<K>(kap) = kappa ? ldro(kappa + i) : C.kappa_u;
-        lane_of<K>(gold) = gk[i];
     });
     X hh;  // halo nodes of h: h - href, then h
     int hc[N], hr[N], pc[N], pr[N];
@@ -95,6 +97,11 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
             lane_of<K>(kh) = kappa ? ldro(kappa + node(pc[K], pr[K])) : C.kappa_u;
         });
     }
+    dependent_launch_wait();
+    lanes([&](auto k_c) {
+        constexpr int K = decltype(k_c)::value;
+        lane_of<K>(gold) = gk[node(c, r + K * HALF)];
+    });
     if constexpr (OMEGA1) {
         // the tile's columns, NT / TX rows a pass, then the three on either side
         constexpr int RP = NT / TX, PASSES = (TY + 6 + RP - 1) / RP, SIDES = (6 * (TY + 6) + NT - 1) / NT;
@@ -210,6 +217,7 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
     }
     __syncthreads();
 
+    if (RESIDENT != 1024 && early) dependent_launch_next();
     // ---- 3
     // p and -gamma ap from the h and ag windows; ap(x) = sum_l 3 w_l c_l . ag(x - c_l)
     auto both = [&](const Win<X>& H, const Win<X>& gx, const Win<X>& gy, X k, X& p, X& l, X& ih) {
@@ -271,7 +279,7 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
     }
     __syncthreads();
 
-    dependent_launch_next();  // as in k_tile
+    if (RESIDENT == 1024 || !early) dependent_launch_next();
     // ---- 4
     Win<X> P, L;
     lanes([&](auto k_c) {
@@ -318,20 +326,28 @@ k_adjoint_tile(const S* __restrict__ mom, const S* __restrict__ an, S* __restric
 }
 
 template <typename S, int TX, int TY>
-cudaError_t adjoint_tile_one(const S* mom, const S* an, S* a, S* gk, const S* kappa, const Geom& G, const Consts<S>& C,
+cudaError_t adjoint_tile_one(const S* mom, bool fresh, const S* an, S* a, S* gk, const S* kappa, const Geom& G, const Consts<S>& C,
                              cudaStream_t st)
 {
     constexpr int NT = TX * TY / Lanes<typename TileX<S>::X>::N;
     const dim3 grid((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY);
-    if (C.omega != S(1)) return launch_dependent(k_adjoint_tile<S, TX, TY, false, 512>, grid, NT, 0, st, mom, an, a, gk, kappa, G, C);
+    // When the next step's CTAs may be placed (see tile_one): after ag where tiles
+    // number at most one an SM or fill nearly all slots once, else after p (us a
+    // backward step, after p / after ag: 128^2 4.8 / 4.3, 300 x 200 5.8 / 5.1,
+    // 384^2 6.8 / 6.5; 320^2 6.8 / 7.2, 400^2 9.7 / 10.1, 512^2 9.6 / 9.8, 1024^2
+    // 32.2 / 32.8; with the record fetched after the wait, after p: 128^2 4.8, 300
+    // x 200 5.6, 512^2 10.2, 1024^2 33.0).
+    const long long tiles = (long long)grid.x * grid.y, sms = sm_count(), slots = 512 / NT * sms;
+    const bool early = tiles <= sms || (tiles <= slots && 6 * tiles >= 5 * slots);
+    if (C.omega != S(1)) return launch_dependent(k_adjoint_tile<S, TX, TY, false, 512>, grid, NT, 0, st, mom, fresh, early, an, a, gk, kappa, G, C);
     // threads an SM holds, as for the forward tiles (one box, omega = 1, us a
     // backward step, 512 / 1024: 300 x 200 6.9 / 9.0, 512^2 11.8 / 11.1, 1024^2
     // 39.7 / 36.1)
     if constexpr (TX == 32 && sizeof(S) == 4) {
-        if ((long long)grid.x * grid.y > 3LL * sm_count())
-            return launch_dependent(k_adjoint_tile<S, TX, TY, true, 1024>, grid, NT, 0, st, mom, an, a, gk, kappa, G, C);
+        if (tiles > 3 * sms)
+            return launch_dependent(k_adjoint_tile<S, TX, TY, true, 1024>, grid, NT, 0, st, mom, fresh, early, an, a, gk, kappa, G, C);
     }
-    return launch_dependent(k_adjoint_tile<S, TX, TY, true, 512>, grid, NT, 0, st, mom, an, a, gk, kappa, G, C);
+    return launch_dependent(k_adjoint_tile<S, TX, TY, true, 512>, grid, NT, 0, st, mom, fresh, early, an, a, gk, kappa, G, C);
 }
 
 }  // namespace tflbm

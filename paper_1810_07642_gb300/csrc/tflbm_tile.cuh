@@ -79,7 +79,7 @@ __device__ __forceinline__ void node_moments(X f0, const X (&n)[8], const Consts
 template <typename SM, typename S, int TX, int TY, bool OMEGA1, int RESIDENT>
 __global__ void __launch_bounds__(TX* TY / Lanes<typename TileX<S>::X>::N, RESIDENT / (TX * TY / Lanes<typename TileX<S>::X>::N))
 k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ fout0, SM* __restrict__ foutm,
-       const S* __restrict__ kappa, S* __restrict__ mom, const Geom G, const Consts<S> C)
+       const S* __restrict__ kappa, S* __restrict__ mom, bool early, const Geom G, const Consts<S> C)
 {
     using X = typename TileX<S>::X;
     using IO = PairIO<SM>;
@@ -183,6 +183,7 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     });
     __syncthreads();
 
+    if (early) dependent_launch_next();
     // ---- film pressure of the tile and the halo of 1
     {
         Win<X> W;
@@ -211,12 +212,7 @@ k_tile(const S* __restrict__ fin0, const SM* __restrict__ finm, S* __restrict__ 
     }
     __syncthreads();
 
-    // Let the next step's CTAs be placed now, when every tile of this step is on
-    // an SM and near its end.  Placed as soon as this step starts, they went to
-    // the SMs that had room then, two or three to one and none to another (one
-    // box, us a step: FP64 tau = 0.8 128^2 25.3 / 8.5, 250 x 190 25.2 / 20.1; FP32
-    // 256^2 3.6 / 3.1).
-    dependent_launch_next();
+    if (!early) dependent_launch_next();
     // ---- force, collision and store of the tile
     Win<X> W;
     lanes([&](auto k_c) {
@@ -249,10 +245,25 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
 {
     constexpr int NT = TX * TY / Lanes<typename TileX<S>::X>::N;
     const dim3 grid((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY);
+    // When the next step's CTAs may be placed.  As soon as this step starts, they
+    // go to the SMs that have room then, two or three to one and none to another
+    // (us a step against after the pressure: FP64 tau = 0.8 128^2 25.3 / 8.5, 250
+    // x 190 25.2 / 20.1).  After the pressure, every tile is on an SM and near
+    // its end; after h already, another phase of the next step's preamble and
+    // launch is hidden, but the placement is uneven again unless half of the SMs
+    // are empty, small tiles number at most one an SM, or the slots (768 threads
+    // an SM, or 1024) are nearly full.  FP32, us a step, after the pressure / after
+    // h: 64^2 2.61 / 2.45, 128^2 2.77 / 2.55, 200 x 150 (130 tiles of 16 x 16) 3.22
+    // / 2.90; 256^2 (128 of 32 x 16) 3.03 / 3.18, 320^2 (400 of 16 x 16) 3.41 /
+    // 3.67, 384^2 (288 of 32 x 16) 3.54 / 3.83; 509 x 387 (400) 4.58 / 4.23, 512^2
+    // (512) 4.70 / 4.58, 1024^2 14.95 / 14.80.  With records 512^2 loses 0.08.
+    const long long tiles = (long long)grid.x * grid.y, sms = sm_count();
+    const bool early = 2 * tiles <= sms || (TX * TY <= 256 && tiles <= sms) ||
+                       (TX == 32 && sizeof(S) == 4 && !mom && 2 * tiles >= 5 * sms && (tiles <= 3 * sms || 3 * tiles >= 10 * sms));
     auto launch = [&](auto resident) {
         constexpr int R = decltype(resident)::value;
-        if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, G, C);
-        return launch_dependent(k_tile<SM, S, TX, TY, false, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, G, C);
+        if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, early, G, C);
+        return launch_dependent(k_tile<SM, S, TX, TY, false, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, early, G, C);
     };
     // Threads an SM holds.  768 leaves the registers that keep a thread's 18
     // loads in flight (80); where 32 x 16 tiles outnumber the three an SM
@@ -260,7 +271,7 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
     // 387 4.9 against 5.7 us a step, 512^2 6.4 against 5.3, 1024^2 17.8
     // against 16.3).
     if constexpr (TX == 32 && sizeof(S) == 4) {
-        if ((long long)grid.x * grid.y > 3LL * sm_count()) return launch(std::integral_constant<int, 1024>{});
+        if (tiles > 3 * sms) return launch(std::integral_constant<int, 1024>{});
     }
     return launch(std::integral_constant<int, sizeof(S) == 4 ? 768 : 512>{});
 }

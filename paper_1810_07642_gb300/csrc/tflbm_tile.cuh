@@ -257,9 +257,12 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
     // / 2.90; 256^2 (128 of 32 x 16) 3.03 / 3.18, 320^2 (400 of 16 x 16) 3.41 /
     // 3.67, 384^2 (288 of 32 x 16) 3.54 / 3.83; 509 x 387 (400) 4.58 / 4.23, 512^2
     // (512) 4.70 / 4.58, 1024^2 14.95 / 14.80.  With records 512^2 loses 0.08.
+    // Without a kappa field the preamble is too short to hide anything (one kappa,
+    // 128^2 2.32 / 2.51, 512^2 4.45 / 4.51).
     const long long tiles = (long long)grid.x * grid.y, sms = sm_count();
-    const bool early = 2 * tiles <= sms || (TX * TY <= 256 && tiles <= sms) ||
+    const bool spread = 2 * tiles <= sms || (TX * TY <= 256 && tiles <= sms) ||
                        (TX == 32 && sizeof(S) == 4 && !mom && 2 * tiles >= 5 * sms && (tiles <= 3 * sms || 3 * tiles >= 10 * sms));
+    const bool early = kappa && spread;
     auto launch = [&](auto resident) {
         constexpr int R = decltype(resident)::value;
         if (C.omega == S(1)) return launch_dependent(k_tile<SM, S, TX, TY, true, R>, grid, NT, 0, st, f0, fm, g0, gm, kappa, mom, early, G, C);

@@ -21,9 +21,9 @@
 //   3  p and -gamma ap (transposed gradient of ag) on the halo of 1; on the
 //      tile the disjoining-pressure adjoint and dL/dkappa
 //   4  on the tile grad p, the force adjoint, the Laplacian of -gamma ap, a(t)
-// 512^2 FP32, a gradient of 400 steps: 23.8 ms as marches of populations, 6.4 now,
-// of which an adjoint step took 27 us, 8 now (911 instructions for two
-// nodes, half of the issue slots; 512 tiles on 152 SMs); threads, lanes, tiles and the
+// 512^2 FP32, a gradient of 400 steps: 23.8 ms as marches of populations, 6.1 now,
+// of which an adjoint step took 27 us, 8 now (820 instructions a warp,
+// half of the issue slots; 512 tiles on 152 SMs); threads, lanes, tiles and the
 // treatment of the edges are those of tflbm_tile.cuh.
 #pragma once
 #include "tflbm_tile.cuh"

@@ -204,6 +204,13 @@ def use_tiles(handle: int, block_x: int, graph_chunk: int = 0) -> None:
         raise ValueError("block_x or graph_chunk")
 
 
+def use_wide(handle: int = 0, batch: int = 0) -> None:
+    """For tests, not part of the interface: put the four-column march over the
+    shape of a handle or a batch."""
+    if lib().tflbm_use_wide(_VP(handle)) if handle else lib().tflbm_batch_use_wide(_VP(batch)):
+        raise ValueError("the four-column march does not apply")
+
+
 def tf_lbm_set_wait_limit(handle: int, polls: int) -> None:
     _check(lib().tf_lbm_set_wait_limit(_VP(handle), int(polls)), _VP(handle))
 

@@ -155,14 +155,27 @@ int store_of(int dtype)
 // / 63, FP16 1448^2 32.3 / 41.7, 2048^2 59.8 / 69.2; FP64 2048^2 1014 / 1101.
 constexpr long long kTileNodes = 1LL << 20, kTileNodesOneColumn = 3LL << 19;
 
+// A march filled with balanced bands: as many as fill the resident slots once
+// (all bands do the same work, so a partial second wave would idle most SMs),
+// but none shorter than 16 rows: each band spends 5 warm-up rows.
+void fill_bands(Shape& s, int store, const Geom& G, bool om1, bool kfield, int sms)
+{
+    const int strips = (G.nx + s.block_x - 5) / (s.block_x - 4);  // CTAs overlap by 4 columns
+    int occ = step_blocks_per_sm(store, s.pipeline, s.block_x, om1, kfield);
+    if (occ < 1) occ = 4;
+    int bands = occ * sms / strips;
+    if (bands > G.ny / 16) bands = G.ny / 16;
+    if (bands < 1) bands = 1;
+    if (bands > 65535) bands = 65535;
+    s.bands = bands;
+    s.rows = (G.ny + bands - 1) / bands;
+}
+
 // Default launch shape: tiles on lattices that L2 holds, the four-column march
 // on larger ones at tau = 1.  The other fields describe the march that a larger lattice would run, and that the caller gets
 // back by setting them: the two-column kernel at tau = 1 where it applies
 // (CTAs 64 columns wide for 16-bit storage, 128 for FP32), else the one-column kernel
-// with CTAs 128 columns wide (64 on lattices narrower than 1024), and
-// a band height that makes the grid one full wave of
-// resident CTAs (all bands do the same work, so a partial second wave would
-// idle most SMs), but no shorter than 16 rows: each band spends 5 warm-up rows.
+// with CTAs 128 columns wide (64 on lattices narrower than 1024).
 Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
 {
     Shape s;
@@ -182,20 +195,10 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     else if (wide)
         s.wide = wide_bands(G, wide_slots(store, G.nx % 4 == 0, sms));
     s.block_x = pair ? (narrow ? 64 : 128) : (G.nx >= 1024 ? 128 : 64);
-    const int strips = (G.nx + s.block_x - 5) / (s.block_x - 4);  // CTAs overlap by 4 columns
     // otherwise per-thread loads: measured faster than the bulk-copy pipeline
     // on GB300 once loads are prefetched a row ahead
     s.pipeline = pair ? kPipePair : kPipeLdg;
-    int occ = step_blocks_per_sm(store_of(p.dtype), s.pipeline, s.block_x, om1, kfield);
-    if (occ < 1) occ = 4;
-    // bands of balanced height (the kernels spread ny rows over them), as
-    // many as fill the resident slots once, but none shorter than 16 rows
-    int bands = occ * sms / strips;
-    if (bands > G.ny / 16) bands = G.ny / 16;
-    if (bands < 1) bands = 1;
-    if (bands > 65535) bands = 65535;
-    s.bands = bands;
-    s.rows = (G.ny + bands - 1) / bands;
+    fill_bands(s, store, G, om1, kfield, sms);
     return s;
 }
 
@@ -255,9 +258,11 @@ cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st, bool fi
             return launch_wide(H->desc.store, f32 && !first, f32 && !last, H->buf[from], H->buf[from ^ 1], H->kappa, H->G,
                                c32, H->shape.wide, st);
         // A run of one FP32 step has no moments to keep: the two-column march
-        // (2048^2: 53 against 56 us), or tiles where nx is odd; same bits.
+        // (2048^2: 53 against 56 us), or tiles where nx is odd; same bits,
+        // whatever march the shape was put in place of.
         if (!pair_pipeline_ok(H->G.nx, kStoreF32))
             return launch_tile(H->desc.store, 256, H->buf[from], H->buf[from ^ 1], H->kappa, nullptr, H->G, &c32, &c64, st);
+        return launch_step(H->desc.store, H->buf[from], H->buf[from ^ 1], H->kappa, H->G, &c32, &c64, H->one, st);
     }
     return launch_step(H->desc.store, H->buf[from], H->buf[from ^ 1], H->kappa, H->G, &c32, &c64,
                        H->shape, st);
@@ -317,6 +322,8 @@ int tf_lbm_init(tf_lbm_handle** out, const tf_lbm_params* params, const void* h0
     }
     H->sms = sm_count();
     H->shape = default_shape(*params, H->G, theta != nullptr);
+    if (H->desc.store == kStoreF32 && pair_pipeline_ok(H->G.nx, kStoreF32))
+        fill_bands(H->one, kStoreF32, H->G, true, theta != nullptr, H->sms);
     H->graph_chunk = ((long long)params->nx * params->ny <= (1LL << 20)) ? 64 : 0;
 
     auto bail = [&](int code) {
@@ -556,6 +563,17 @@ int tflbm_use_tiles(tf_lbm_handle* H, int32_t block_x, int32_t graph_chunk)
     H->shape.tile = block_x;
     H->shape.wide = 0;
     H->graph_chunk = graph_chunk;
+    return TF_LBM_OK;
+}
+
+// The same for the four-column march, over whatever march the shape describes.
+int tflbm_use_wide(tf_lbm_handle* H)
+{
+    if (!H || H->dbl || H->p.forcing != 0 || make_consts<float>(H).omega != 1.0f || !wide_applies(H->desc.store, H->G))
+        return TF_LBM_ERR_ARG;
+    drop_graphs(H);
+    H->shape.tile = 0;
+    H->shape.wide = wide_bands(H->G, wide_slots(H->desc.store, H->G.nx % 4 == 0, H->sms));
     return TF_LBM_OK;
 }
 

@@ -51,6 +51,10 @@ struct tf_lbm_batch {
     bool wide_ok = false, wide_quad = false, wide = false;
     BatchItem* witems = nullptr;
     int nwide = 0;
+    // a run of one FP32 step of it: the two-column kernel in its default shape
+    // (the same bits, whatever kernel L names), and its items behind witems
+    tf_lbm_batch_launch one{};
+    int none = 0;
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     double* dpart = nullptr;  // diagnostics partials
@@ -181,20 +185,26 @@ int sync_table(tf_lbm_batch* B, cudaStream_t st)
     return TF_LBM_OK;
 }
 
-// Build the work items of a launch shape: domains in order, bands of a
-// domain in order, strips fastest (as the single-domain grid orders them).
+// The work items of a launch shape: domains in order, bands of a domain in
+// order, strips fastest (as the single-domain grid orders them).
+template <typename Strips>
+void add_items(const tf_lbm_batch* B, int rows, Strips strips, std::vector<BatchItem>& out)
+{
+    for (int d = 0; d < (int)B->hs.size(); ++d) {
+        const Geom& G = B->hs[d]->G;
+        const int ns = strips(G.nx), nb = bands_of(G.ny, rows);
+        for (int b = 0; b < nb; ++b)
+            for (int s = 0; s < ns; ++s) out.push_back(BatchItem{d, s, b, nb});
+    }
+}
+
 int write_items(tf_lbm_batch* B, const tf_lbm_batch_launch& L, cudaStream_t st)
 {
     const long long n = count_items(B, L.block_x, L.rows);
     if (n > (1LL << 30)) return bfail(B, TF_LBM_ERR_ARG, "too many work items: raise rows");
     std::vector<BatchItem> host;
     host.reserve((size_t)n);
-    for (int d = 0; d < (int)B->hs.size(); ++d) {
-        const Geom& G = B->hs[d]->G;
-        const int ns = strips_of(G.nx, L.block_x), nb = bands_of(G.ny, L.rows);
-        for (int b = 0; b < nb; ++b)
-            for (int s = 0; s < ns; ++s) host.push_back(BatchItem{d, s, b, nb});
-    }
+    add_items(B, L.rows, [&](int nx) { return strips_of(nx, L.block_x); }, host);
     if ((int)n > B->item_cap) {
         if (B->items) cudaFree(B->items);
         B->items = nullptr;
@@ -216,7 +226,8 @@ int write_items(tf_lbm_batch* B, const tf_lbm_batch_launch& L, cudaStream_t st)
 }
 
 // Build the work items of the four-column march: the smallest band height
-// whose items fit in the GPU's slots.
+// whose items fit in the GPU's slots; and those of its one-step runs, which
+// take the shape L (the default one, two-column).
 int write_wide_items(tf_lbm_batch* B, cudaStream_t st)
 {
     const int slots = wide_slots(B->store, B->wide_quad, sm_count());
@@ -236,17 +247,14 @@ int write_wide_items(tf_lbm_batch* B, cudaStream_t st)
     const long long n = count(lo);
     if (n > (1LL << 30)) return bfail(B, TF_LBM_ERR_ARG, "too many work items");
     std::vector<BatchItem> host;
-    host.reserve((size_t)n);
-    for (int d = 0; d < (int)B->hs.size(); ++d) {
-        const Geom& G = B->hs[d]->G;
-        const int ns = wide_strips(G.nx), nb = bands_of(G.ny, lo);
-        for (int b = 0; b < nb; ++b)
-            for (int s = 0; s < ns; ++s) host.push_back(BatchItem{d, s, b, nb});
-    }
-    BCK(B, cudaMalloc(&B->witems, n * sizeof(BatchItem)), "cudaMalloc items");
-    BCK(B, cudaMemcpyAsync(B->witems, host.data(), n * sizeof(BatchItem), cudaMemcpyHostToDevice, st),
+    add_items(B, lo, wide_strips, host);
+    B->nwide = (int)host.size();
+    B->one = B->L;
+    if (B->store == kStoreF32) add_items(B, B->one.rows, [&](int nx) { return strips_of(nx, B->one.block_x); }, host);
+    B->none = (int)host.size() - B->nwide;
+    BCK(B, cudaMalloc(&B->witems, host.size() * sizeof(BatchItem)), "cudaMalloc items");
+    BCK(B, cudaMemcpyAsync(B->witems, host.data(), host.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, st),
         "cudaMemcpyAsync items");
-    B->nwide = (int)n;
     return TF_LBM_OK;
 }
 
@@ -257,17 +265,18 @@ cudaError_t launch_batch(tf_lbm_batch* B, int parity, cudaStream_t st, bool firs
     if (B->wide && !(f32 && first && last))
         return launch_wide_batch(B->store, f32 && !first, f32 && !last, B->wide_quad, B->witems, B->nwide, B->doms,
                                  parity, st);
+    const tf_lbm_batch_launch& L = B->wide ? B->one : B->L;
     BatchLaunch q{};
-    q.block_x = B->L.block_x;
-    q.pair = B->L.pipeline == kPipePair;
+    q.block_x = L.block_x;
+    q.pair = L.pipeline == kPipePair;
     q.omega1 = B->om1;
     q.kfield = B->kf;
-    q.items = B->items;
-    q.nitems = B->nitems;
+    q.items = B->wide ? B->witems + B->nwide : B->items;
+    q.nitems = B->wide ? B->none : B->nitems;
     q.doms = B->doms;
     q.parity = parity;
-    q.queue = B->L.queue ? B->queue : nullptr;
-    q.grid = B->grid;
+    q.queue = L.queue ? B->queue : nullptr;
+    q.grid = B->wide ? B->none : B->grid;
     return launch_step_batch(B->store, q, st);
 }
 
@@ -651,6 +660,16 @@ int tf_lbm_batch_set_launch(tf_lbm_batch* B, const tf_lbm_batch_launch* in)
     BCK(B, cudaDeviceSynchronize(), "cudaDeviceSynchronize");
     B->wide = false;
     return apply_launch(B, *in, nullptr);
+}
+
+// Not part of the interface, for tests: the four-column march over whatever
+// kernel the shape names.
+int tflbm_batch_use_wide(tf_lbm_batch* B)
+{
+    if (!B || !B->wide_ok) return TF_LBM_ERR_ARG;
+    drop_batch_graphs(B);
+    B->wide = true;
+    return TF_LBM_OK;
 }
 
 int tf_lbm_batch_step(tf_lbm_batch* B, int64_t nsteps, void* stream)

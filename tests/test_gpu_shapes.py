@@ -1,0 +1,53 @@
+"""Launch shapes: what a run gives may not depend on how it is split into calls
+or on which march the four-column march was put in place of.
+
+The four-column, two-column and tile kernels run the same node arithmetic with
+paired FP32 instructions, which leave the compiler no contraction: states agree
+bit for bit (tolerance 0).
+"""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1810_07642_gb300 import _lib, inputs
+from paper_1810_07642_gb300.film import FilmBatch, ThinFilm
+
+pytestmark = pytest.mark.gpu
+
+
+def film(nx, ny, dtype="f32", tau=1.0, field=True):
+    h0, th, p = inputs.small_random(nx, ny, seed=nx + 3 * ny, amp=0.05)
+    p.update(tau=tau, g=2e-4, gx_body=1e-5, gy_body=-2e-5, theta_uniform=0.3)
+    return ThinFilm(p, h0, th if field else None, dtype=dtype)
+
+
+# ragged and whole groups of four columns; the one-column march beneath
+@pytest.mark.parametrize("nx,ny", [(244, 100), (242, 51), (121, 60)])
+@pytest.mark.parametrize("base", [dict(pipeline=1, block_x=64, rows=16), dict(pipeline=2, block_x=128, rows=30)])
+def test_one_step_runs_of_the_four_column_march_keep_its_bits(nx, ny, base):
+    states = []
+    for split in ((9,), (1,) * 9, (1, 2, 1, 5)):
+        sim = film(nx, ny)
+        sim.set_launch(graph_chunk=0, **base)
+        _lib.use_wide(sim.handle)
+        for n in split:
+            sim.step(n)
+        states.append(sim.get_state())
+        sim.close()
+    assert torch.equal(states[0], states[1]) and torch.equal(states[0], states[2])
+
+
+@pytest.mark.parametrize("sizes", [[(244, 100), (120, 33)], [(242, 51), (118, 17), (10, 9)]])
+def test_one_step_runs_of_a_batch_keep_its_bits(sizes):
+    states = []
+    for split in ((9,), (1,) * 9, (1, 2, 1, 5)):
+        films = [film(nx, ny) for nx, ny in sizes]
+        with FilmBatch(films) as batch:
+            batch.set_launch(pipeline=1, block_x=64, rows=16, graph_chunk=0)
+            _lib.use_wide(batch=batch.batch)
+            for n in split:
+                batch.step(n)
+            states.append([f.get_state() for f in films])
+        [f.close() for f in films]
+    for s in states[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(states[0], s))

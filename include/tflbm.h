@@ -126,8 +126,7 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  *            tf_lbm_init (and bands-exact candidates of tf_lbm_tune) instead
  *            uses the number of bands that fills the GPU's resident CTA
  *            slots once, so its bands need not all have `rows` rows; rows
- *            then reports the tallest band, and passing it back to
- *            tf_lbm_set_launch gives ceil(ny / rows) bands;
+ *            then reports the tallest band;
  *   graph_chunk: steps per captured CUDA graph in tf_lbm_step (0 = none,
  *            otherwise an even number >= 2);
  *   pipeline: 3 = every thread owns two adjacent columns, loads aligned
@@ -151,10 +150,14 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  * with forcing = 0, a march of four columns per thread, which between the
  * steps of one call keeps moments in place of FP32 populations (16-bit storage:
  * where nx is a multiple of 4).  So does the shape chosen by tf_lbm_tune where
- * one of them was the fastest.  Passing the fields to tf_lbm_set_launch gives
- * what they describe.
- * Results do not depend on rows or graph_chunk; the pipelines agree to
- * rounding. */
+ * one of them was the fastest (reported by the fields that
+ * tf_lbm_init chose).  Passing block_x, rows and pipeline as tf_lbm_init or the
+ * last tf_lbm_tune reported them to tf_lbm_set_launch gives all of that shape
+ * back, its balanced bands and its tiles or four columns among it, whatever
+ * graph_chunk; other fields give the march that they describe.
+ * Results do not depend on rows or graph_chunk as long as the kernel is the
+ * same; the kernels agree to rounding (those with two or more nodes per thread
+ * and an FP32 compute type bit for bit at tau = 1). */
 typedef struct tf_lbm_launch {
     int32_t block_x;
     int32_t rows;
@@ -344,7 +347,9 @@ typedef struct tf_lbm_batch tf_lbm_batch;
  *            tf_lbm_launch (every domain's nx even, not TF_LBM_F64).  The
  *            default is 3 where it applies and every tau is 1 (as for a
  *            single handle), else 1; a default or tuned batch of pipeline 3
- *            may run the four-column march in its place, see tf_lbm_launch.  Both run the node arithmetic of the
+ *            may run the four-column march in its place, and setting its
+ *            block_x, rows and pipeline with queue = 0 keeps that, see
+ *            tf_lbm_launch.  Both run the node arithmetic of the
  *            single-handle kernel of the same pipeline. */
 typedef struct tf_lbm_batch_launch {
     int32_t block_x;

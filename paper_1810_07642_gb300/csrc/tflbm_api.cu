@@ -321,7 +321,7 @@ int tf_lbm_init(tf_lbm_handle** out, const tf_lbm_params* params, const void* h0
                     "lattice too large: 9 * ny * pitch must stay below 2^31 elements");
     }
     H->sms = sm_count();
-    H->shape = default_shape(*params, H->G, theta != nullptr);
+    H->shape = H->def = H->own = default_shape(*params, H->G, theta != nullptr);
     if (H->desc.store == kStoreF32 && pair_pipeline_ok(H->G.nx, kStoreF32))
         fill_bands(H->one, kStoreF32, H->G, true, theta != nullptr, H->sms);
     H->graph_chunk = ((long long)params->nx * params->ny <= (1LL << 20)) ? 64 : 0;
@@ -543,12 +543,10 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
     if (in->pipeline == kPipeTma && !tma_pipeline_ok(H->G.nx))
         return fail(H, TF_LBM_ERR_ARG, "the bulk-copy pipeline needs nx to be a multiple of 8 and >= 16");
     drop_graphs(H);
-    H->shape.pipeline = in->pipeline;
-    H->shape.block_x = bx;
-    H->shape.rows = in->rows;
-    H->shape.bands = 0;
-    H->shape.tile = 0;
-    H->shape.wide = 0;
+    // the fields of the shape that init or tuning chose stand for all of it:
+    // its balanced bands, and the tiles or the four-column march it runs
+    if (bx == H->own.block_x && in->rows == H->own.rows && in->pipeline == H->own.pipeline) H->shape = H->own;
+    else H->shape = Shape{bx, in->rows, in->pipeline};
     H->graph_chunk = in->graph_chunk;
     return TF_LBM_OK;
 }

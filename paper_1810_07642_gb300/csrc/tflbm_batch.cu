@@ -55,6 +55,9 @@ struct tf_lbm_batch {
     // (the same bits, whatever kernel L names), and its items behind witems
     tf_lbm_batch_launch one{};
     int none = 0;
+    // what creation or tuning chose (see tf_lbm_batch_set_launch)
+    tf_lbm_batch_launch own{};
+    bool own_wide = false;
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     double* dpart = nullptr;  // diagnostics partials
@@ -430,25 +433,28 @@ int tf_lbm_tune(tf_lbm_handle* H, int32_t trial_steps, tf_lbm_launch* best, void
         if (r == cudaSuccess) r = cudaEventElapsedTime(ms, e0, e1);
         return r == cudaSuccess ? TF_LBM_OK : handle_cuda_fail(H, r, "step kernel (tuning)");
     };
-    // the fastest of these, then tiles or the four-column march in its place
-    // if they beat it
+    // the fastest of these, or tiles or the four-column march if they beat it;
+    // those are put on the default shape, whose fields then stand for them on
+    // other handles too
     const int k = pick_fastest(cands, time_one, &rc);
-    std::vector<Shape> tiles;
-    for (int bx : {0, 64, 128, 256}) {
-        if (rc) break;
-        tiles.push_back(cands[k]);
-        tiles.back().tile = bx;
+    std::vector<Shape> last;
+    if (!rc) last.push_back(cands[k]);
+    for (int bx : {64, 128, 256}) {
+        last.push_back(H->def);
+        last.back().wide = 0;
+        last.back().tile = bx;
     }
-    if (!rc && om1 && H->p.forcing == 0 && wide_applies(H->desc.store, H->G)) {
-        tiles.push_back(cands[k]);
-        tiles.back().wide = wide_bands(H->G, wide_slots(H->desc.store, H->G.nx % 4 == 0, sms));
+    if (om1 && H->p.forcing == 0 && wide_applies(H->desc.store, H->G)) {
+        last.push_back(H->def);
+        last.back().tile = 0;
+        last.back().wide = wide_bands(H->G, wide_slots(H->desc.store, H->G.nx % 4 == 0, sms));
     }
-    const int kt = rc ? -1 : pick_fastest(tiles, time_one, &rc);
+    const int kt = rc ? -1 : pick_fastest(last, time_one, &rc);
     if (rc) {
         H->shape = old;
         return finish(rc);
     }
-    H->shape = tiles[kt];
+    H->shape = H->own = last[kt];
     if (H->shape.block_x != old.block_x || H->shape.rows != old.rows || H->shape.pipeline != old.pipeline ||
         H->shape.bands != old.bands || H->shape.tile != old.tile || H->shape.wide != old.wide)
         handle_drop_graphs(H);
@@ -637,7 +643,8 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     L.queue = 0;
     if ((rc = apply_launch(B, L, st))) return bail(rc);
     if (B->wide_ok && (rc = write_wide_items(B, st))) return bail(rc);
-    B->wide = B->wide_ok;
+    B->own = B->L;
+    B->own_wide = B->wide = B->wide_ok;
     *out = B;
     return TF_LBM_OK;
 }
@@ -658,8 +665,13 @@ int tf_lbm_batch_set_launch(tf_lbm_batch* B, const tf_lbm_batch_launch* in)
     if (rc) return rc;
     // the work-item table is rewritten in place: let launches that read it finish
     BCK(B, cudaDeviceSynchronize(), "cudaDeviceSynchronize");
-    B->wide = false;
-    return apply_launch(B, *in, nullptr);
+    // the fields that creation or tuning chose stand for the four-column march
+    // where it chose that (the queue is one of the other kernels)
+    const bool wide = B->own_wide && in->queue == 0 && in->block_x == B->own.block_x && in->rows == B->own.rows &&
+                      in->pipeline == B->own.pipeline;
+    if ((rc = apply_launch(B, *in, nullptr))) return rc;
+    B->wide = wide;
+    return TF_LBM_OK;
 }
 
 // Not part of the interface, for tests: the four-column march over whatever
@@ -793,7 +805,7 @@ int tf_lbm_batch_tune(tf_lbm_batch* B, int32_t trial_steps, tf_lbm_batch_launch*
     B->wide = false;
     const int k = pick_fastest(cands, time_one, &rc);
     const tf_lbm_batch_launch chosen = k >= 0 ? cands[k] : old;
-    const int rc2 = apply_launch(B, rc ? old : chosen, st);
+    int rc2 = apply_launch(B, rc ? old : chosen, st);
     // the four-column march in its place if it beats it
     std::vector<int> both{0};
     if (B->wide_ok && !rc && !rc2) both.push_back(1);
@@ -803,8 +815,15 @@ int tf_lbm_batch_tune(tf_lbm_batch* B, int32_t trial_steps, tf_lbm_batch_launch*
     }, &rc);
     B->wide = kw >= 0 ? both[kw] != 0 : old_wide;
     drop_batch_graphs(B);
+    if (kw >= 0 && B->wide) {  // reported as the default shape, which stands for it on other batches too
+        tf_lbm_batch_launch L = B->one;
+        L.graph_chunk = chosen.graph_chunk;
+        rc2 = apply_launch(B, L, st);
+    }
     if (rc) return finish(rc);
     if (rc2) return finish(rc2);
+    B->own = B->L;
+    B->own_wide = B->wide;
     if (best) *best = B->L;
     return finish(TF_LBM_OK);
 }

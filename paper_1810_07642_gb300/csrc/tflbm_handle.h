@@ -34,6 +34,8 @@ struct tf_lbm_handle {
     int wait_limit = kWaitLimit;  // polls of one mbarrier before a bulk-copy kernel gives up
     int64_t time = 0;
     Shape shape{128, 64, kPipeLdg};  // replaced by the occupancy-derived default in tf_lbm_init
+    Shape def{128, 64, kPipeLdg};    // the default: what tuning puts tiles and the four-column march on
+    Shape own{128, 64, kPipeLdg};    // what init or tuning chose: setting its fields gives it back whole
     Shape one{128, 64, kPipePair};   // the two-column march that takes a run of one FP32 step of a wide shape
     int graph_chunk = 0;
     cudaStream_t cap = nullptr;

@@ -1,5 +1,6 @@
 """Launch shapes: what a run gives may not depend on how it is split into calls
-or on which march the four-column march was put in place of.
+or on which march the four-column march was put in place of, and a shape that
+the library chose is kept by reading it and setting it again.
 
 The four-column, two-column and tile kernels run the same node arithmetic with
 paired FP32 instructions, which leave the compiler no contraction: states agree
@@ -51,3 +52,51 @@ def test_one_step_runs_of_a_batch_keep_its_bits(sizes):
         [f.close() for f in films]
     for s in states[1:]:
         assert all(torch.equal(a, b) for a, b in zip(states[0], s))
+
+
+@pytest.mark.parametrize("dtype,tau", [("f32", 0.8), ("f64", 1.0), ("bf16", 1.3)])
+def test_setting_what_was_read_keeps_the_kernel(dtype, tau):
+    """Off tau = 1, and in FP64, tiles and the march that the fields describe
+    differ in the last bits, which shows the kernel; default and tuned shape,
+    set as they are, with another graph_chunk, and after other shapes."""
+    sim = film(300, 200, dtype, tau)
+    s0 = sim.get_state()
+
+    def after(steps=40):
+        sim.set_state(s0)
+        sim.step(steps)
+        return sim.get_state()
+
+    for tuned in (False, True):
+        shape, want = sim.launch, after()
+        sim.set_launch(**shape)
+        assert torch.equal(after(), want)
+        sim.set_launch(graph_chunk=8)
+        assert torch.equal(after(), want) and sim.launch == dict(shape, graph_chunk=8)
+        sim.set_launch(block_x=128, rows=23, pipeline=1)
+        assert tuned or not torch.equal(after(), want)
+        sim.set_launch(**shape)
+        assert torch.equal(after(), want)
+        sim.set_state(s0)
+        assert sim.tune(4) == sim.launch
+    sim.close()
+
+
+def test_setting_what_was_read_keeps_the_kernel_of_a_batch():
+    """The number of work items shows the kernel."""
+    films = [film(nx, ny) for nx, ny in [(512, 256)] * 6 + [(1024, 512)]]
+    with FilmBatch(films) as batch:
+        for _ in range(2):
+            shape, items = batch.launch, batch.items
+            batch.set_launch(**shape)
+            assert batch.items == items
+            batch.set_launch(graph_chunk=4, queue=0)
+            if not shape["queue"]:
+                assert batch.items == items
+            batch.set_launch(block_x=64, rows=1, pipeline=1)
+            assert batch.items > items
+            batch.set_launch(**shape)
+            assert batch.items == items and batch.launch == shape
+            batch.step(3)
+            assert batch.tune(4) == batch.launch
+    [f.close() for f in films]

@@ -441,47 +441,110 @@ __device__ __forceinline__ Pops<T, SM> pops_of(const BatchDomain<T>& D, int pari
     return P;
 }
 
-// Running sums of the diagnostics, two at a time.  With an FP32 compute type a
-// sum is an error-free FP32 pair (Knuth's TwoSum per addend, products split by
-// fma), which resolves it to about 2^-48, and both sums share Blackwell's
-// paired FP32 instructions; FP64 state sums in compensated doubles.  GB300
-// retires 2 FP64 operations a clock and SM: the same sums in doubles, with a
-// double sincospi per node, were what bounded this pass (32 domains: 2130 us),
-// and per-unit merges in doubles still took half of it (155 us).
+// One entry of a domain's trigonometric table: cos and sin of 2 pi i / n, with
+// an FP32 compute type as the sum of three floats, which holds all bits of the
+// double.  Entries 0 .. nx-1 are the columns, nx .. nx+ny-1 the rows.  A
+// Fourier phase 2 pi m x / n is entry m x mod n, so the table does not depend
+// on the mode.
+template <typename T> struct Trig;
+template <> struct __align__(16) Trig<float> {
+    float2 hi, lo, lo2, pad;  // (cos, sin)
+    __device__ __forceinline__ void set(double c, double s)
+    {
+        hi = make_float2((float)c, (float)s);
+        const double cr = c - (double)hi.x, sr = s - (double)hi.y;
+        lo = make_float2((float)cr, (float)sr);
+        lo2 = make_float2((float)(cr - (double)lo.x), (float)(sr - (double)lo.y));
+        pad = make_float2(0.0f, 0.0f);
+    }
+    // the factors (-sin, cos)
+    __device__ __forceinline__ Trig turned() const
+    {
+        return {make_float2(-hi.y, hi.x), make_float2(-lo.y, lo.x), make_float2(-lo2.y, lo2.x), pad};
+    }
+};
+template <> struct __align__(16) Trig<double> {
+    double2 hi;
+    __device__ __forceinline__ void set(double c, double s) { hi = make_double2(c, s); }
+    __device__ __forceinline__ Trig turned() const { return {make_double2(-hi.y, hi.x)}; }
+};
+static_assert(sizeof(Trig<float>) == diag_trig_bytes(false) && sizeof(Trig<double>) == diag_trig_bytes(true),
+              "table entry size");
+
+// Running sums of the diagnostics, two at a time.  The reference is sums in
+// compensated doubles, whose error is the rounding of the result; but GB300
+// retires 2 FP64 operations a clock and SM, and such sums, with a double
+// sincospi per node, took 2130 us for 32 domains.  With an FP32 compute type a
+// sum is therefore three floats: Knuth's TwoSum of the sum and each addend, of
+// its errors and theirs, and a plain sum of the errors of that (as good as a sum
+// in three times the precision, rounded once: an error of about n 2^-72 of the
+// sum of |addends|, n addends); products are split by fma.  Both sums share
+// Blackwell's paired FP32 instructions.  A sum of two floats, without the third,
+// loses with its length: 2^-48 of the sum for 16 addends, 2^-44 for 128, 2^-38
+// for 8192.  Addends are scaled by kSumScale, so that no sum of a lattice
+// overflows where its addends do not.  FP64 state sums in compensated doubles.
+constexpr double kSumScale = 1.0 / 4294967296.0;  // 2^-32; fewer than 2^31 nodes
 // a - b in one instruction (the paired add takes no negated operand)
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+// s += v; returns the rounding error
+__device__ __forceinline__ float2 two_sum2(float2& s, float2 v)
+{
+    const float2 t = __fadd2_rn(s, v), b = sub2(t, s);
+    const float2 e = __fadd2_rn(sub2(s, sub2(t, b)), sub2(v, b));
+    s = t;
+    return e;
+}
 template <typename T> struct Acc2;
 template <> struct Acc2<float> {
     using V = float2;
-    V s = {0.0f, 0.0f}, c = {0.0f, 0.0f};
-    __device__ __forceinline__ void add(V v)
+    static constexpr double kScale = kSumScale;
+    V s = {0.0f, 0.0f}, c = {0.0f, 0.0f}, d = {0.0f, 0.0f};
+    __device__ __forceinline__ void add(V v) { d = __fadd2_rn(d, two_sum2(c, two_sum2(s, v))); }
+    // += v * w
+    __device__ __forceinline__ void add_product(V v, const Trig<float>& w)
     {
-        const V t = __fadd2_rn(s, v), b = sub2(t, s);
-        c = __fadd2_rn(c, __fadd2_rn(sub2(s, sub2(t, b)), sub2(v, b)));
-        s = t;
+        // the rounding error of a product, v hi - q, is exact in one fma
+        const V q = __fmul2_rn(v, w.hi), r = __fmul2_rn(v, w.lo);
+        const V e = two_sum2(c, two_sum2(s, q)), f = two_sum2(c, __ffma2_rn(v, w.hi, V{-q.x, -q.y}));
+        const V g = two_sum2(c, r), l = __ffma2_rn(v, w.lo2, __ffma2_rn(v, w.lo, V{-r.x, -r.y}));
+        d = __fadd2_rn(d, __fadd2_rn(__fadd2_rn(e, f), __fadd2_rn(g, l)));
     }
-    // += v * (hi + lo)
-    __device__ __forceinline__ void add_product(V v, V hi, V lo)
-    {
-        const V q = __fmul2_rn(v, hi);
-        // the product's rounding error v hi - q is exact in one fma
-        c = __fadd2_rn(c, __ffma2_rn(v, lo, __ffma2_rn(v, hi, V{-q.x, -q.y})));
-        add(q);
-    }
-    // += (s_ + c_) * (hi + lo)
-    __device__ __forceinline__ void add_product(float s_, float c_, V hi, V lo)
-    {
-        add_product(V{s_, s_}, hi, lo);
-        c = __ffma2_rn(V{c_, c_}, hi, c);
-    }
+    // += the first or second sum of a * w
+    __device__ __forceinline__ void add_first(const Acc2& a, const Trig<float>& w) { add_sum(a.s.x, a.c.x, a.d.x, w); }
+    __device__ __forceinline__ void add_second(const Acc2& a, const Trig<float>& w) { add_sum(a.s.y, a.c.y, a.d.y, w); }
     __device__ __forceinline__ void merge(const Acc2& a)
     {
-        add(a.s);
-        c = __fadd2_rn(c, a.c);
+        const V e = two_sum2(c, two_sum2(s, a.s));
+        d = __fadd2_rn(d, __fadd2_rn(__fadd2_rn(e, two_sum2(c, a.c)), a.d));
+    }
+    __device__ __forceinline__ Acc2 down(int o) const  // of the lane o above
+    {
+        auto at = [&](V v) { return V{__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o)}; };
+        Acc2 a;
+        a.s = at(s);
+        a.c = at(c);
+        a.d = at(d);
+        return a;
+    }
+    __device__ __forceinline__ void store(double* out) const  // first and second sum, each as (sum, compensation)
+    {
+        out[0] = (double)s.x / kScale;
+        out[1] = ((double)c.x + (double)d.x) / kScale;
+        out[2] = (double)s.y / kScale;
+        out[3] = ((double)c.y + (double)d.y) / kScale;
+    }
+
+private:
+    __device__ __forceinline__ void add_sum(float s_, float c_, float d_, const Trig<float>& w)
+    {
+        add_product(V{s_, s_}, w);
+        add_product(V{c_, c_}, w);
+        d = __ffma2_rn(V{d_, d_}, w.hi, d);
     }
 };
 template <> struct Acc2<double> {
     using V = double2;
+    static constexpr double kScale = 1.0;
     V s = {0.0, 0.0}, c = {0.0, 0.0};
     __device__ __forceinline__ void add(V v)
     {
@@ -491,54 +554,47 @@ template <> struct Acc2<double> {
         s = V{a.s, b.s};
         c = V{a.c, b.c};
     }
-    __device__ __forceinline__ void add_product(V v, V hi, V) { add(V{v.x * hi.x, v.y * hi.y}); }
-    __device__ __forceinline__ void add_product(double s_, double c_, V hi, V)
-    {
-        add(V{s_ * hi.x, s_ * hi.y});
-        c.x += c_ * hi.x;
-        c.y += c_ * hi.y;
-    }
+    __device__ __forceinline__ void add_product(V v, const Trig<double>& w) { add(V{v.x * w.hi.x, v.y * w.hi.y}); }
+    __device__ __forceinline__ void add_first(const Acc2& a, const Trig<double>& w) { add_sum(a.s.x, a.c.x, w); }
+    __device__ __forceinline__ void add_second(const Acc2& a, const Trig<double>& w) { add_sum(a.s.y, a.c.y, w); }
     __device__ __forceinline__ void merge(const Acc2& a)
     {
         add(a.s);
         c.x += a.c.x;
         c.y += a.c.y;
     }
+    __device__ __forceinline__ Acc2 down(int o) const
+    {
+        auto at = [&](V v) { return V{__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o)}; };
+        Acc2 a;
+        a.s = at(s);
+        a.c = at(c);
+        return a;
+    }
+    __device__ __forceinline__ void store(double* out) const
+    {
+        out[0] = s.x;
+        out[1] = c.x;
+        out[2] = s.y;
+        out[3] = c.y;
+    }
+
+private:
+    __device__ __forceinline__ void add_sum(double s_, double c_, const Trig<double>& w)
+    {
+        const V q{s_ * w.hi.x, s_ * w.hi.y};
+        add(q);
+        c.x += fma(c_, w.hi.x, fma(s_, w.hi.x, -q.x));
+        c.y += fma(c_, w.hi.y, fma(s_, w.hi.y, -q.y));
+    }
 };
 template <typename T>
 __device__ __forceinline__ Acc2<T> warp_total(Acc2<T> a)
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        Acc2<T> b;
-        b.s.x = __shfl_down_sync(0xffffffffu, a.s.x, o);
-        b.s.y = __shfl_down_sync(0xffffffffu, a.s.y, o);
-        b.c.x = __shfl_down_sync(0xffffffffu, a.c.x, o);
-        b.c.y = __shfl_down_sync(0xffffffffu, a.c.y, o);
-        a.merge(b);
-    }
+    for (int o = 16; o > 0; o >>= 1) a.merge(a.down(o));
     return a;
 }
-
-// One entry of a domain's trigonometric table: cos and sin of 2 pi i / n as
-// hi + lo (FP64 state: lo = 0).  Entries 0 .. nx-1 are the columns, nx ..
-// nx+ny-1 the rows.  A Fourier phase 2 pi m x / n is entry m x mod n, so the
-// table does not depend on the mode and is written once.
-template <typename T> struct Trig;
-template <> struct __align__(16) Trig<float> {
-    float2 hi, lo;  // (cos, sin)
-    __device__ __forceinline__ void set(double c, double s)
-    {
-        hi = make_float2((float)c, (float)s);
-        lo = make_float2((float)(c - (double)hi.x), (float)(s - (double)hi.y));
-    }
-};
-template <> struct __align__(16) Trig<double> {
-    double2 hi;
-    static constexpr double2 lo{0.0, 0.0};
-    __device__ __forceinline__ void set(double c, double s) { hi = make_double2(c, s); }
-};
-static_assert(sizeof(Trig<float>) == kDiagTrigBytes && sizeof(Trig<double>) == kDiagTrigBytes, "table entry size");
 
 template <typename T>
 __global__ void k_diag_table(const BatchDomain<T>* __restrict__ doms, Trig<T>* table, int stride)
@@ -563,14 +619,16 @@ __global__ void k_diag_table(const BatchDomain<T>* __restrict__ doms, Trig<T>* t
 //
 // A warp takes units of 32 columns x `rows` rows; a lane sums its own column
 // down the rows, so the column's trigonometric factors multiply one sum per
-// unit and the mode's phase splits into a row factor per node and a column
-// factor per unit (cos(a + b) from the two angles).  The unit height gives
-// every warp of the launch one unit where it can, but at least kDiagRows rows
-// (a unit's products and its reduction over the warp cost about five rows),
-// and the sums of a unit leave the registers at its end, which are then eight
-// sums and two rows of loads.
-// Bound by HBM: 36 B a node in FP32.  32 domains, 7.6 M nodes: 2150 -> 90 us
-// with the final kernel.
+// unit and the mode's phase splits into a row factor per node (none where the
+// mode has no wave along y) and a column factor per unit (cos(a + b) from the
+// two angles).  The unit height gives every warp of the launch one unit where it
+// can, but at least kDiagRows rows (a unit's products and its reduction over the
+// warp cost about ten rows).
+// Bound by the chains of TwoSums (60 paired operations a node, 90 with a row
+// phase) and the latency of a row's nine loads: 32 warps an SM hide them better
+// than 24 with the next row's loads in flight (32 domains, 7.6 M nodes, with the
+// final kernel and the launches: 117 against 129 us; 40 warps spill: 138).  In
+// doubles 2150 us.
 constexpr int kDiagPartial = 2 * kDiagSums + 1;
 constexpr int kDiagRows = 16;
 template <typename T, typename SM>
@@ -629,21 +687,19 @@ k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T
                 ra = r0;
                 r0 = rb;
             };
-            T v[9], n[9];
-            pull(y0, n);
             for (int y = y0; y < y1; ++y) {
-#pragma unroll
-                for (int l = 0; l < 9; ++l) v[l] = n[l];
-                if (y + 1 < y1) pull(y + 1, n);
+                T v[9];
+                pull(y, v);
                 T hh, jx, jy;
                 moments9(v, hh, jx, jy);
                 const bool wet = hh > wet_above;
                 const T hw = wet ? hh : T(0);
-                const Trig<T> m = ty[iy], w = ty[y];
-                ah.add(V{hh, hw});
-                aj.add(V{wet ? jx : T(0), wet ? jy : T(0)});
-                ar.add_product(V{hw, hw}, w.hi, w.lo);
-                am.add_product(V{hh, hh}, m.hi, m.lo);
+                const Trig<T> w = ty[y];
+                const T k = T(Acc2<T>::kScale), hs = hh * k, ws = hw * k;
+                ah.add(V{hs, ws});
+                aj.add(V{wet ? jx * k : T(0), wet ? jy * k : T(0)});
+                ar.add_product(V{ws, ws}, w);
+                if (ky != 0) am.add_product(V{hs, hs}, ty[iy]);
                 count += wet;
                 iy += ky;
                 if (iy >= G.ny) iy -= G.ny;
@@ -653,9 +709,13 @@ k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T
         const int xc = min(x, G.nx - 1);  // a lane past the lattice holds zeros
         const Trig<T> w = tx[xc], m = tx[(long long)kx * xc % G.nx];
         Acc2<T> ac, ap;  // the column angle; the mode: cos(a + b), sin(a + b)
-        ac.add_product(ah.s.y, ah.c.y, w.hi, w.lo);
-        ap.add_product(am.s.x, am.c.x, m.hi, m.lo);
-        ap.add_product(am.s.y, am.c.y, V{-m.hi.y, m.hi.x}, V{-m.lo.y, m.lo.x});
+        ac.add_second(ah, w);
+        if (ky == 0) {  // the rows' phase is 0: (1, 0) times the sum of h
+            ap.add_first(ah, m);
+        } else {
+            ap.add_first(am, m);
+            ap.add_second(am, m.turned());
+        }
         auto total = [&](int k, const Acc2<T>& a) {
             const Acc2<T> q = warp_total(a);
             if (lane == 0) sm[k][wid].merge(q);
@@ -680,10 +740,7 @@ k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T
         Acc2<T> b = sm[k][0];
         for (int w = 1; w < NW; ++w) b.merge(sm[k][w]);
         const int q = 2 * (k < 2 ? 2 * k : 2 * k + 1);  // sums (0, 1), (2, 3), (5, 6), (7, 8), (9, 10)
-        out[q] = b.s.x;
-        out[q + 1] = b.c.x;
-        out[q + 2] = b.s.y;
-        out[q + 3] = b.c.y;
+        b.store(out + q);
     } else if (k == 5) {
         long long b = 0;
         for (int w = 0; w < NW; ++w) b += scount[w];

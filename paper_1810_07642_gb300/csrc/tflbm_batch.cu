@@ -485,7 +485,7 @@ int tf_lbm_diagnostics(tf_lbm_handle* H, double h_wet, int32_t mode_x, int32_t m
     const int stride = H->G.nx + H->G.ny;
     const bool first = !H->dscr;
     if (first) {
-        cudaError_t e = cudaMalloc(&H->dscr, trig + kDiagTrigBytes * stride);
+        cudaError_t e = cudaMalloc(&H->dscr, trig + diag_trig_bytes(H->dbl) * stride);
         if (e != cudaSuccess) {
             H->dscr = nullptr;
             return handle_cuda_fail(H, e, "cudaMalloc diagnostics scratch");
@@ -614,7 +614,7 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     const size_t dp = diag_partials(count, kDiagBlocksPerDomain);
     if ((e = cudaMalloc(&B->dpart, dp * sizeof(double))) != cudaSuccess) return bail(bcuda(B, e, "cudaMalloc diagnostics"));
     for (auto* H : B->hs) B->dstride = std::max(B->dstride, H->G.nx + H->G.ny);
-    if ((e = cudaMalloc(&B->dtrig, kDiagTrigBytes * B->dstride * count)) != cudaSuccess)
+    if ((e = cudaMalloc(&B->dtrig, diag_trig_bytes(B->dbl) * B->dstride * count)) != cudaSuccess)
         return bail(bcuda(B, e, "cudaMalloc diagnostics table"));
     int rc = write_table(B, st);
     if (rc) return bail(rc);

@@ -223,7 +223,7 @@ cudaError_t aux_set_state(const StoreDesc& D, void* f, const double* in, const G
 constexpr int kDiagSums = 11;
 constexpr int kDiagOut = kDiagSums + 1;
 inline size_t diag_partials(int ndom, int nb) { return (size_t)ndom * nb * (2 * kDiagSums + 1); }
-constexpr size_t kDiagTrigBytes = 16;  // one table entry
+constexpr size_t diag_trig_bytes(bool dbl) { return dbl ? 16 : 32; }  // one table entry
 cudaError_t aux_diag_table(bool dbl, const void* doms, int ndom, int stride, void* table, cudaStream_t st);
 cudaError_t aux_diag(int store, const void* doms, int ndom, int parity, const void* table, int stride, double h_wet,
                      int mx, int my, double* partials, int nb, double* out, cudaStream_t st);

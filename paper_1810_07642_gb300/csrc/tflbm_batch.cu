@@ -483,24 +483,32 @@ int tf_lbm_diagnostics(tf_lbm_handle* H, double h_wet, int32_t mode_x, int32_t m
     static_assert(sizeof(BatchDomain<double>) <= 256, "diagnostics record too large");
     const size_t trig = (tab + sizeof(double) * diag_partials(1, kSumBlocks) + 255) / 256 * 256;
     const int stride = H->G.nx + H->G.ny;
-    const bool first = !H->dscr;
-    if (first) {
-        cudaError_t e = cudaMalloc(&H->dscr, trig + diag_trig_bytes(H->dbl) * stride);
-        if (e != cudaSuccess) {
-            H->dscr = nullptr;
-            return handle_cuda_fail(H, e, "cudaMalloc diagnostics scratch");
-        }
-    }
     BatchDomain<double> d64;
     BatchDomain<float> d32;
     const void* rec = H->dbl ? (const void*)&d64 : (const void*)&d32;
     if (H->dbl) d64 = domain_of<double>(H, H->cur, H->kappa);
     else d32 = domain_of<float>(H, H->cur, H->kappa);
-    cudaError_t e = cudaMemcpyAsync(H->dscr, rec, domain_bytes(H->dbl), cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaSuccess;
+    if (!H->dscr) {
+        // The first call writes the trigonometric table and waits for it, on a
+        // stream of the handle's own: later calls may come on any stream, and
+        // this one's stream may be capturing.
+        char* scr = nullptr;
+        if ((e = cudaMalloc(&scr, trig + diag_trig_bytes(H->dbl) * stride)) != cudaSuccess)
+            return handle_cuda_fail(H, e, "cudaMalloc diagnostics scratch");
+        if (!H->cap) e = cudaStreamCreateWithFlags(&H->cap, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(scr, rec, domain_bytes(H->dbl), cudaMemcpyHostToDevice, H->cap);
+        if (e == cudaSuccess) e = aux_diag_table(H->dbl, scr, 1, stride, scr + trig, H->cap);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(H->cap);
+        if (e != cudaSuccess) {
+            cudaFree(scr);
+            return handle_cuda_fail(H, e, "diagnostics table");
+        }
+        H->dscr = scr;
+    }
+    e = cudaMemcpyAsync(H->dscr, rec, domain_bytes(H->dbl), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return handle_cuda_fail(H, e, "cudaMemcpyAsync diagnostics record");
-    char* table = (char*)H->dscr + trig;
-    if (first && (e = aux_diag_table(H->dbl, H->dscr, 1, stride, table, st)) != cudaSuccess)
-        return handle_cuda_fail(H, e, "diagnostics table kernel");
+    const char* table = (const char*)H->dscr + trig;
     e = aux_diag(H->desc.store, H->dscr, 1, 0, table, stride, h_wet, mode_x, mode_y,
                  (double*)((char*)H->dscr + tab), nb, (double*)out, st);
     if (e != cudaSuccess) return handle_cuda_fail(H, e, "diagnostics kernels");

@@ -295,8 +295,8 @@ def storage_variants(steps: int = 2000, check_steps: int = 1000):
 def tape_form(n: int, steps: int):
     """What the gradient tape does for an n^2 FP32 lattice: its description and
     its kernel launches a gradient (records of 12 B a node and step, kept while
-    they fit in 8 GiB; else recomputed in segments of ceil(sqrt(steps)))."""
-    if steps * 12 * n * n <= 8 << 30:
+    they fit in 4 GiB; else recomputed in segments of ceil(sqrt(steps)))."""
+    if steps * 12 * n * n <= 4 << 30:
         return "all step records kept", 2 * steps
     return f"checkpoints every {int(math.ceil(math.sqrt(steps)))} steps", 3 * steps
 

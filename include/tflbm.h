@@ -246,8 +246,9 @@ int tf_lbm_adjoint_step(tf_lbm_handle* H, const void* f_t, const void* a_next, v
 /* Gradient tape over nsteps steps.  It keeps a record of every step (h and j,
  * 3 elements a node; what the adjoint reads of a state).  every > 0: records of
  * `every` steps at a time, recomputed from copies of the state that many steps
- * apart.  every <= 0: the records of all steps while these take 8 GiB or less
- * and can be allocated, else as every = ceil(sqrt(nsteps)).  h0 and theta
+ * apart.  every <= 0: the records of all steps where these take no more memory
+ * than every = ceil(sqrt(nsteps)) would, or at most 4 GiB and 1/64 of the device
+ * memory that is free at the call; else as every = ceil(sqrt(nsteps)).  h0 and theta
  * (device [ny][nx], theta NULL = params->theta_uniform) must be the ones the
  * handle was created from; they are copied. */
 typedef struct tf_lbm_tape tf_lbm_tape;

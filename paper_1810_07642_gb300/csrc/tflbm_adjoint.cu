@@ -316,10 +316,13 @@ bool three_fields(const tf_lbm_handle* H)
 // ---------------------------------------------------------------- the tape
 
 // Largest set of step records a tape keeps in place of state copies and
-// recomputation: 3 % of the device's memory.  A 512^2 step costs 5.2 us to
-// recompute and 3 MB to keep, and allocating and freeing that takes 1.2 us, so
-// more would still pay in time, but a tape is not the only tenant.
-constexpr size_t kTapeBytes = (size_t)8 << 30;
+// recomputation where these take less: 4 GiB, and 1/64 of the memory that is
+// free when the tape is made.  Keeping all pays in time at any size (512^2: a step
+// costs 5.2 us to recompute and its 3 MB 2 us to allocate and free), but a tape
+// is not the only tenant: the caller's own allocations come after it, and many
+// tapes may live at a time, each of which leaves 63/64 of what it found.
+constexpr size_t kTapeBytes = (size_t)4 << 30;
+constexpr size_t kTapeShare = 64;
 
 struct tf_lbm_tape {
     tf_lbm_handle* H = nullptr;
@@ -410,9 +413,20 @@ int tf_lbm_tape_create(tf_lbm_handle* H, const void* h0, const void* theta, int6
         tf_lbm_tape_destroy(tp);
         return rc;
     };
-    // One allocation.  All records where they fit (every <= 0 leaves the choice
-    // here; an explicit `every` asks for segments of that length), else segments
+    // One allocation.  All records where they may be kept (every <= 0 leaves the
+    // choice here; an explicit `every` asks for segments of that length), else
+    // segments
     const size_t field = n * H->esize;
+    const int64_t root = (int64_t)ceil(sqrt((double)nsteps));
+    auto may_keep_all = [&]() {
+        const size_t most = kTapeBytes / tp->rec_bytes;
+        if (nsteps > INT32_MAX) return false;
+        const size_t segments = tp->state_bytes * ((nsteps + root - 1) / root + 2) + tp->rec_bytes * root;
+        if ((size_t)nsteps <= segments / tp->rec_bytes) return true;  // no more than segments would take
+        size_t left = 0, total = 0;
+        if ((size_t)nsteps > most || cudaMemGetInfo(&left, &total) != cudaSuccess) return false;
+        return (size_t)nsteps <= left / kTapeShare / tp->rec_bytes;
+    };
     auto allocate = [&](int64_t kept) {
         tp->every = (int)kept;
         tp->nseg = (int)((nsteps + kept - 1) / kept);
@@ -435,11 +449,9 @@ int tf_lbm_tape_create(tf_lbm_handle* H, const void* h0, const void* theta, int6
         tp->rec = block + at_rec;
         return cudaSuccess;
     };
-    if (every <= 0 && (size_t)nsteps <= kTapeBytes / tp->rec_bytes && nsteps <= INT32_MAX &&
-        allocate(nsteps) != cudaSuccess)
-        cudaGetLastError();
+    if (every <= 0 && may_keep_all() && allocate(nsteps) != cudaSuccess) cudaGetLastError();
     if (!tp->block) {
-        if (every <= 0) every = (int32_t)ceil(sqrt((double)nsteps));
+        if (every <= 0) every = (int32_t)root;
         if ((e = allocate(std::min<int64_t>(every, nsteps))) != cudaSuccess) return bail(e, "cudaMalloc tape");
     }
     if ((e = cudaMemcpy(tp->h0, h0, field, cudaMemcpyDeviceToDevice)) != cudaSuccess) return bail(e, "copy h0");

@@ -28,10 +28,10 @@ cudaError_t wide_variant(int store, bool mom_in, bool mom_out, bool quad, Fn fn)
 
 }  // namespace
 
-bool wide_applies(int store, const Geom& G)
+bool wide_applies(int store, const Geom& G, bool quad)
 {
     if (store == kStoreF64) return false;
-    if (G.nx % 4 == 0) return true;
+    if (quad) return G.nx % 4 == 0;
     return store == kStoreF32 && G.nx >= 8 && 6LL * mom_pitch(G.nx) * G.ny + 128 <= 9LL * G.plane;
 }
 

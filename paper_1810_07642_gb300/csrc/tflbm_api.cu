@@ -186,7 +186,7 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     // (the two-column kernel's pulled-population ring costs resident warps)
     const int store = store_of(p.dtype), sms = sm_count();
     const bool om1 = p.tau == 1.0;
-    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G);
+    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G, G.nx % 4 == 0);
     const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     const bool narrow = store == kStoreF16 || store == kStoreBF16;
     if (store == kStoreF64 || (narrow && !wide && !pair) ||
@@ -567,7 +567,7 @@ int tflbm_use_tiles(tf_lbm_handle* H, int32_t block_x, int32_t graph_chunk)
 // The same for the four-column march, over whatever march the shape describes.
 int tflbm_use_wide(tf_lbm_handle* H)
 {
-    if (!H || H->dbl || H->p.forcing != 0 || make_consts<float>(H).omega != 1.0f || !wide_applies(H->desc.store, H->G))
+    if (!H || H->dbl || H->p.forcing != 0 || make_consts<float>(H).omega != 1.0f || !wide_applies(H->desc.store, H->G, H->G.nx % 4 == 0))
         return TF_LBM_ERR_ARG;
     drop_graphs(H);
     H->shape.tile = 0;

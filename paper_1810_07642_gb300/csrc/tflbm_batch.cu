@@ -444,7 +444,7 @@ int tf_lbm_tune(tf_lbm_handle* H, int32_t trial_steps, tf_lbm_launch* best, void
         last.back().wide = 0;
         last.back().tile = bx;
     }
-    if (om1 && H->p.forcing == 0 && wide_applies(H->desc.store, H->G)) {
+    if (om1 && H->p.forcing == 0 && wide_applies(H->desc.store, H->G, H->G.nx % 4 == 0)) {
         last.push_back(H->def);
         last.back().tile = 0;
         last.back().wide = wide_bands(H->G, wide_slots(H->desc.store, H->G.nx % 4 == 0, sms));
@@ -593,9 +593,11 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
         B->kf |= H->kappa != nullptr;
         B->om1 &= B->dbl ? make_consts<double>(H).omega == 1.0 : make_consts<float>(H).omega == 1.0f;
         B->pair_ok &= pair_pipeline_ok(H->G.nx, B->store);
-        B->wide_ok &= H->p.forcing == 0 && wide_applies(B->store, H->G);
         B->wide_quad &= H->G.nx % 4 == 0;
     }
+    // one layout for all domains: a width that is no multiple of 4 makes it the
+    // ragged one for those that are, too
+    for (auto* H : B->hs) B->wide_ok &= H->p.forcing == 0 && wide_applies(B->store, H->G, B->wide_quad);
     B->wide_ok = B->wide_ok && B->pair_ok && B->om1;
     auto bail = [&](int code) {
         set_thread_error(B->err);

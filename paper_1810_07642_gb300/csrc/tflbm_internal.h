@@ -128,11 +128,12 @@ cudaError_t pair_step_bf16(int block_x, const void* fin, void* fout, const void*
                            const Consts<float>& C, int bands, cudaStream_t st);
 // The four-column march (step4.cu): omega = 1, forcing = 0, FP32 compute type.
 // mom_in, mom_out: the source / destination holds moments (kStoreF32 only, see
-// tflbm_step4.cuh).  wide_applies: whether the kernel takes the lattice (16-bit
-// storage: nx a multiple of 4).  wide_slots: CTAs (strip, band) the GPU holds.
+// tflbm_step4.cuh).  wide_applies: whether the kernel takes the lattice in the
+// layout for nx a multiple of 4 (quad) or in the ragged one (FP32 only, where the
+// moment rows fit).  wide_slots: CTAs (strip, band) the GPU holds.
 cudaError_t launch_wide(int store, bool mom_in, bool mom_out, const void* fin, void* fout, const void* kappa,
                         const Geom& G, const Consts<float>& C, int bands, cudaStream_t st);
-bool wide_applies(int store, const Geom& G);
+bool wide_applies(int store, const Geom& G, bool quad);
 int wide_strips(int nx);
 int wide_slots(int store, bool quad, int sms);
 // Bands of a lattice that fill `slots` once, none shorter than 8 rows.

@@ -100,3 +100,29 @@ def test_setting_what_was_read_keeps_the_kernel_of_a_batch():
             batch.step(3)
             assert batch.tune(4) == batch.launch
     [f.close() for f in films]
+
+
+# widths that are multiples of 4 beside one that is not: all run the ragged
+# layout, whose moment rows (padded to 8 more columns, read 124 past their end)
+# have to fit; 32 x 1 and 32 x 2 do not, and 4 is narrower than the layout takes
+@pytest.mark.parametrize("sizes,fits", [([(240, 64), (242, 100), (64, 33), (122, 9)], True),
+                                        ([(32, 3), (242, 20), (8, 40)], True),
+                                        ([(32, 2), (242, 20)], False), ([(32, 1), (122, 7)], False),
+                                        ([(4, 9), (242, 20)], False)])
+def test_batches_that_mix_layouts(sizes, fits):
+    films = [film(nx, ny) for nx, ny in sizes]
+    with FilmBatch(films) as batch:
+        if fits:
+            _lib.use_wide(batch=batch.batch)
+        else:
+            with pytest.raises(ValueError):
+                _lib.use_wide(batch=batch.batch)
+        for n in (1, 2, 3, 17):
+            batch.step(n)
+    for f, (nx, ny) in zip(films, sizes):
+        ref = film(nx, ny)
+        ref.set_launch(pipeline=3, block_x=64, rows=7)
+        ref.step(23)
+        assert f.check() == 0 and torch.equal(f.get_state(), ref.get_state()), (nx, ny)
+        ref.close()
+        f.close()

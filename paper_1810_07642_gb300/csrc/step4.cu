@@ -46,13 +46,12 @@ cudaError_t launch_wide(int store, bool mom_in, bool mom_out, const void* fin, v
     });
 }
 
-cudaError_t launch_wide_batch(int store, bool mom_in, bool mom_out, bool quad, const BatchItem* items, int nitems,
+cudaError_t launch_wide_batch(int store, bool mom_in, bool mom_out, const BatchItem* items, int nitems,
                               const void* doms, int parity, cudaStream_t st)
 {
-    return wide_variant(store, mom_in, mom_out, quad, [&](auto sm, auto mi, auto mo, auto q) {
-        return launch_dependent(
-            k_step4_batch<decltype(sm), decltype(mi)::value, decltype(mo)::value, decltype(q)::value>, dim3(nitems), 32,
-            0, st, items, (const BatchDomain<float>*)doms, parity);
+    return wide_variant(store, mom_in, mom_out, true, [&](auto sm, auto mi, auto mo, auto) {
+        return launch_dependent(k_step4_batch<decltype(sm), decltype(mi)::value, decltype(mo)::value>, dim3(nitems), 32,
+                                0, st, items, (const BatchDomain<float>*)doms, parity);
     });
 }
 

@@ -47,8 +47,8 @@ struct tf_lbm_batch {
     int grid = 0;
     tf_lbm_batch_launch L{64, 64, 0, 0, kPipeLdg};
     // the four-column march in place of L's kernel (omega == 1 and forcing == 0
-    // everywhere, every nx even): its items, and whether it is in use
-    bool wide_ok = false, wide_quad = false, wide = false;
+    // everywhere, every nx a multiple of 4): its items, and whether it is in use
+    bool wide_ok = false, wide = false;
     BatchItem* witems = nullptr;
     int nwide = 0;
     // a run of one FP32 step of it: the two-column kernel in its default shape
@@ -233,7 +233,7 @@ int write_items(tf_lbm_batch* B, const tf_lbm_batch_launch& L, cudaStream_t st)
 // take the shape L (the default one, two-column).
 int write_wide_items(tf_lbm_batch* B, cudaStream_t st)
 {
-    const int slots = wide_slots(B->store, B->wide_quad, sm_count());
+    const int slots = wide_slots(B->store, true, sm_count());
     auto count = [&](int rows) {
         long long n = 0;
         for (auto* H : B->hs) n += (long long)wide_strips(H->G.nx) * bands_of(H->G.ny, rows);
@@ -266,7 +266,7 @@ cudaError_t launch_batch(tf_lbm_batch* B, int parity, cudaStream_t st, bool firs
 {
     const bool f32 = B->store == kStoreF32;
     if (B->wide && !(f32 && first && last))
-        return launch_wide_batch(B->store, f32 && !first, f32 && !last, B->wide_quad, B->witems, B->nwide, B->doms,
+        return launch_wide_batch(B->store, f32 && !first, f32 && !last, B->witems, B->nwide, B->doms,
                                  parity, st);
     const tf_lbm_batch_launch& L = B->wide ? B->one : B->L;
     BatchLaunch q{};
@@ -588,16 +588,15 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     B->kfill.assign(count, nullptr);
     B->om1 = true;
     B->pair_ok = !B->dbl;
-    B->wide_ok = B->wide_quad = true;
+    B->wide_ok = true;
+    WideCover cover;
     for (auto* H : B->hs) {
         B->kf |= H->kappa != nullptr;
         B->om1 &= B->dbl ? make_consts<double>(H).omega == 1.0 : make_consts<float>(H).omega == 1.0f;
         B->pair_ok &= pair_pipeline_ok(H->G.nx, B->store);
-        B->wide_quad &= H->G.nx % 4 == 0;
+        B->wide_ok &= H->p.forcing == 0 && wide_applies(B->store, H->G, true);
+        cover.add(H->G.nx, H->G.ny);
     }
-    // one layout for all domains: a width that is no multiple of 4 makes it the
-    // ragged one for those that are, too
-    for (auto* H : B->hs) B->wide_ok &= H->p.forcing == 0 && wide_applies(B->store, H->G, B->wide_quad);
     B->wide_ok = B->wide_ok && B->pair_ok && B->om1;
     auto bail = [&](int code) {
         set_thread_error(B->err);
@@ -654,7 +653,7 @@ int tf_lbm_batch_create(tf_lbm_batch** out, tf_lbm_handle* const* handles, int32
     if ((rc = apply_launch(B, L, st))) return bail(rc);
     if (B->wide_ok && (rc = write_wide_items(B, st))) return bail(rc);
     B->own = B->L;
-    B->own_wide = B->wide = B->wide_ok;
+    B->own_wide = B->wide = B->wide_ok && cover.pays(B->store);
     *out = B;
     return TF_LBM_OK;
 }

@@ -135,6 +135,24 @@ cudaError_t launch_wide(int store, bool mom_in, bool mom_out, const void* fin, v
                         const Geom& G, const Consts<float>& C, int bands, cudaStream_t st);
 bool wide_applies(int store, const Geom& G, bool quad);
 int wide_strips(int nx);
+// Nodes that a 16-bit lattice's four-column march, 120 columns a strip, and its
+// two-column march, 60, walk, those past the lattice's last column among them,
+// and whether the first is the faster one: where it walks at most half as much
+// again, or few enough that both are a chain of row latencies.  FP16, us a step,
+// two-column / four-column (walked nodes of the latter): 60 x 18333 29.2 / 20.5
+// (2.2 M), 40 x 27500 26.6 / 27.4 (3.3 M), 60 x 50000 39.9 / 47.1 (6 M, twice the
+// other), 64 x 46875 55.1 / 41.8 (5.6 M, as many), twelve of 8 x 3000 34.0 / 39.3
+// (4.3 M, twice).  FP32 is faster by moments between steps at any width: 20 x
+// 65535 73 / 50.
+struct WideCover {
+    long long four = 0, two = 0;
+    void add(int nx, int ny)
+    {
+        four += (long long)wide_strips(nx) * 120 * ny;
+        two += (nx + 59LL) / 60 * 60 * ny;
+    }
+    bool pays(int store) const { return store == 0 /* kStoreF32 */ || four <= 3LL << 20 || 2 * four <= 3 * two; }
+};
 int wide_slots(int store, bool quad, int sms);
 // Bands of a lattice that fill `slots` once, none shorter than 8 rows.
 inline int wide_bands(const Geom& G, int slots)
@@ -179,8 +197,8 @@ struct BatchLaunch {
     int* query_occupancy;
 };
 cudaError_t launch_step_batch(int store, const BatchLaunch& L, cudaStream_t st);
-// The batched four-column march; quad: every domain's nx is a multiple of 4.
-cudaError_t launch_wide_batch(int store, bool mom_in, bool mom_out, bool quad, const BatchItem* items, int nitems,
+// The batched four-column march, every domain's nx a multiple of 4.
+cudaError_t launch_wide_batch(int store, bool mom_in, bool mom_out, const BatchItem* items, int nitems,
                               const void* doms, int parity, cudaStream_t st);
 // The batched two-column step per storage type (step2_*.cu).
 cudaError_t pair_step_batch_f32(const BatchLaunch& L, cudaStream_t st);

@@ -431,8 +431,10 @@ k_step4(const void* __restrict__ fin, void* __restrict__ fout, const float* __re
 }
 
 // Batched form: CTA i takes work item i, a band of a strip (of kWideCols
-// columns) of one domain.
-template <typename SM, bool MOM_IN, bool MOM_OUT, bool QUAD>
+// columns) of one domain.  QUAD only: the ragged layout lost to the two-column
+// march in batches of every size (us a step: 4 domains of 122 x 61 15.3 / 23.1, 64
+// of 250 x 125 36 / 62, 16 of 1018 x 509 102 / 155).
+template <typename SM, bool MOM_IN, bool MOM_OUT>
 __global__ void __launch_bounds__(32, 12)
 k_step4_batch(const BatchItem* __restrict__ items, const BatchDomain<float>* __restrict__ doms, int parity)
 {
@@ -442,7 +444,7 @@ k_step4_batch(const BatchItem* __restrict__ items, const BatchDomain<float>* __r
     const Geom G = D.G;
     Consts<float> C = D.C;
     C.flip = parity;
-    step_band4<SM, MOM_IN, MOM_OUT, QUAD>(D.buf[parity], D.buf[parity ^ 1], D.kappa, G, C, it.strip, it.band, it.nbands);
+    step_band4<SM, MOM_IN, MOM_OUT, true>(D.buf[parity], D.buf[parity ^ 1], D.kappa, G, C, it.strip, it.band, it.nbands);
 }
 
 }  // namespace tflbm

@@ -38,7 +38,7 @@ def test_one_step_runs_of_the_four_column_march_keep_its_bits(nx, ny, base):
     assert torch.equal(states[0], states[1]) and torch.equal(states[0], states[2])
 
 
-@pytest.mark.parametrize("sizes", [[(244, 100), (120, 33)], [(242, 51), (118, 17), (10, 9)]])
+@pytest.mark.parametrize("sizes", [[(244, 100), (120, 33)], [(240, 51), (116, 17), (12, 9)]])
 def test_one_step_runs_of_a_batch_keep_its_bits(sizes):
     states = []
     for split in ((9,), (1,) * 9, (1, 2, 1, 5)):
@@ -102,21 +102,15 @@ def test_setting_what_was_read_keeps_the_kernel_of_a_batch():
     [f.close() for f in films]
 
 
-# widths that are multiples of 4 beside one that is not: all run the ragged
-# layout, whose moment rows (padded to 8 more columns, read 124 past their end)
-# have to fit; 32 x 1 and 32 x 2 do not, and 4 is narrower than the layout takes
-@pytest.mark.parametrize("sizes,fits", [([(240, 64), (242, 100), (64, 33), (122, 9)], True),
-                                        ([(32, 3), (242, 20), (8, 40)], True),
-                                        ([(32, 2), (242, 20)], False), ([(32, 1), (122, 7)], False),
-                                        ([(4, 9), (242, 20)], False)])
-def test_batches_that_mix_layouts(sizes, fits):
+# widths that are multiples of 4 beside one that is not, down to lattices whose
+# moment rows would not fit a population buffer: no four-column march
+@pytest.mark.parametrize("sizes", [[(240, 64), (242, 100), (64, 33), (122, 9)], [(32, 3), (242, 20), (8, 40)],
+                                   [(32, 2), (242, 20)], [(32, 1), (122, 7)], [(4, 9), (242, 20)]])
+def test_batches_that_mix_layouts(sizes):
     films = [film(nx, ny) for nx, ny in sizes]
     with FilmBatch(films) as batch:
-        if fits:
+        with pytest.raises(ValueError):
             _lib.use_wide(batch=batch.batch)
-        else:
-            with pytest.raises(ValueError):
-                _lib.use_wide(batch=batch.batch)
         for n in (1, 2, 3, 17):
             batch.step(n)
     for f, (nx, ny) in zip(films, sizes):
@@ -126,3 +120,18 @@ def test_batches_that_mix_layouts(sizes, fits):
         assert f.check() == 0 and torch.equal(f.get_state(), ref.get_state()), (nx, ny)
         ref.close()
         f.close()
+
+
+# 16-bit domains whose strips are mostly empty: two columns where there are many,
+# four where there are few; items = strips x bands of the march in use
+@pytest.mark.parametrize("nx,ny,count,four", [(8, 3000, 12, False), (8, 700, 3, True), (64, 3000, 12, True)])
+def test_narrow_16_bit_batches(nx, ny, count, four):
+    films = [film(nx, ny, "f16", field=False) for _ in range(count)]
+    with FilmBatch(films) as batch:
+        default = batch.items
+        batch.set_launch(queue=1)
+        two = batch.items
+        assert (default != two) == four
+        batch.step(2)
+        assert all(f.check() == 0 for f in films)
+    [f.close() for f in films]

@@ -22,33 +22,60 @@ int sm_count()
     return sms;
 }
 
-// The tile kernel's block_x for a lattice (tile_of): the shape with the least
-// work on the busiest SM, counting a node's pull as 0.45 of its cost and its
-// pressure as 0.2 (the halos repeat those) and 60 nodes' worth of fixed
-// latency a tile.  In FP64 the arithmetic units are the bound and halo work
-// counts in full, so tiles are as large as keeps every SM busy.  Measured, one
-// box, us a step with block_x 64 / 128 / 256: FP32 128^2 2.9 / 3.1 / 3.3, 384^2
-// 5.0 / 4.9 / 4.3, 512^2 6.6 / 6.5 / 5.1, 1024^2 19.2 / 19.0 / 15.8; FP64 64^2 7.5 / 11.5 / 20.2, 250 x
-// 190 38 / 20.7 / 38, 768^2 158 / 156 / 151.
-int tile_block_x(int store, int nx, int ny, int sms)
+static int rows_covered(int bx, int ny) { return (ny + tile_of(bx).ty - 1) / tile_of(bx).ty * tile_of(bx).ty; }
+static long long tiles_of(int bx, int nx, int ny)
 {
-    auto tiles = [&](int bx) {
-        const TileShape t = tile_of(bx);
-        return (long long)((nx + t.tx - 1) / t.tx) * ((ny + t.ty - 1) / t.ty);
-    };
-    if (store == kStoreF64) return tiles(64) <= sms ? 64 : (tiles(256) >= 7LL * sms ? 256 : 128);
+    const TileShape t = tile_of(bx);
+    return (long long)((nx + t.tx - 1) / t.tx) * ((ny + t.ty - 1) / t.ty);
+}
+
+// The FP32 shape with the least work on the busiest SM, counting a node's pull
+// as 0.45 of its cost and its pressure as 0.2 (the halos repeat those) and 60
+// nodes' worth of fixed latency a tile.  Measured, one box, us a step with block_x
+// 64 / 128 / 256: 128^2 2.9 / 3.1 / 3.3, 384^2 5.0 / 4.9 / 4.3, 512^2 6.6 / 6.5 / 5.1 (an
+// earlier form of the kernel), 1500 x 700 20.9 / 20.4 / 17.1.
+static int tile_block_f32(int nx, int ny, int sms)
+{
     int best = 64;
     double least = 0;
     for (int bx : {64, 128, 256}) {
         const TileShape t = tile_of(bx);
         const double work = 60 + 0.35 * t.tx * t.ty + 0.45 * (t.tx + 4) * (t.ty + 4) + 0.2 * (t.tx + 2) * (t.ty + 2);
-        const double cost = (double)((tiles(bx) + sms - 1) / sms) * work;
+        const double cost = (double)((tiles_of(bx, nx, ny) + sms - 1) / sms) * work;
         if (bx == 64 || cost < least) {
             best = bx;
             least = cost;
         }
     }
     return best;
+}
+
+// The tile kernel's block_x for a lattice (tile_of).  FP32: as above, but 16 x 8
+// tiles on long lattices of a few rows, of which 16-row tiles would cover over 1.2
+// times as many (block_x 64 / 256: 60000 x 20 28.3 / 30.9, 20000 x 24 10.9 / 11.2, 30000
+// x 33, 1.2 times, 22.9 / 21.8).  FP64 is bound by its arithmetic units: the least
+// tiles times the cost of one, of which the halos are a smaller part the larger it
+// is, but the small ones, which spread best over the SMs, up to six an SM.  Us a
+// step with block_x 64 / 128 / 256: 100^2 8.2 / 12.8 / 22.2, 250 x 190 18.3 / 23.0 /
+// 22.4, 400 x 300 40.1 / 43.9 / 43.7, 512^2 78 / 76 / 85, 2048^2 1175 / 1135 / 1179, 60000 x
+// 20 409 / 525 / 549; omega = 1: 512^2 - / 70 / 77, 3000 x 500 396 / 389 / 378.
+int tile_block_x(int store, int nx, int ny, int sms, bool omega1)
+{
+    if (store != kStoreF64) {
+        if ((long long)nx * rows_covered(256, ny) >= 1LL << 19 && 5 * rows_covered(256, ny) > 6 * rows_covered(64, ny))
+            return 64;
+        return tile_block_f32(nx, ny, sms);
+    }
+    const double small = (double)tiles_of(64, nx, ny), mid = 1.93 * tiles_of(128, nx, ny),
+                 large = (omega1 ? 3.76 : 4.0) * tiles_of(256, nx, ny);
+    if (small <= 6.0 * sms || (small <= mid && small <= large)) return 64;
+    return mid <= large || tiles_of(256, nx, ny) < 7LL * sms ? 128 : 256;
+}
+// The adjoint's tiles, whose halos are one node deeper.
+int adjoint_block_x(bool dbl, int nx, int ny, int sms)
+{
+    if (!dbl) return tile_block_f32(nx, ny, sms);
+    return tiles_of(64, nx, ny) <= sms ? 64 : (tiles_of(256, nx, ny) >= 7LL * sms ? 256 : 128);
 }
 }  // namespace tflbm
 
@@ -155,6 +182,21 @@ int store_of(int dtype)
 // / 63, FP16 1448^2 32.3 / 41.7, 2048^2 59.8 / 69.2; FP64 2048^2 1014 / 1101.
 constexpr long long kTileNodes = 1LL << 20, kTileNodesOneColumn = 3LL << 19;
 
+// Long lattices of a few rows, of which tiles cover too many: they cost more than
+// the latency of a march's few rows (us a step, tile of the best shape against
+// march; nodes covered, thousands, of those in the lattice): FP64 65000 x 17 408 /
+// 338 (1560 of 1105), 40000 x 9 165 / 141 (640 of 360), 20000 x 9 88 / 118 (320 of
+// 180), 30000 x 3 73 / 46 (240 of 90), 60000 x 20 378 / 394 (1440 of 1200); FP32 100000
+// x 3 15.0 / 11.5 (800 of 300), 30000 x 3 6.7 / 6.2 (240 of 90), 40000 x 9 10.7 / 14.7,
+// 65000 x 17 31 / 29, 30000 x 33 21.9 / 28.8 (1440 of 990), 60000 x 20 28 / 36 in long
+// runs, 30.6 / 25.8 in runs of two.
+bool tiles_wasted(int store, long long covered, long long nodes)
+{
+    if (3 * covered <= 4 * nodes) return false;
+    if (store == kStoreF64) return covered - nodes > 9LL << 14;
+    return covered > 1500000 || (covered > 2 * nodes && covered - nodes > 1LL << 17);
+}
+
 // A march filled with balanced bands: as many as fill the resident slots once
 // (all bands do the same work, so a partial second wave would idle most SMs),
 // but none shorter than 16 rows: each band spends 5 warm-up rows.
@@ -172,8 +214,8 @@ void fill_bands(Shape& s, int store, const Geom& G, bool om1, bool kfield, int s
 }
 
 // Default launch shape: tiles on lattices that L2 holds, the four-column march
-// on larger ones at tau = 1.  The other fields describe the march that a larger lattice would run, and that the caller gets
-// back by setting them: the two-column kernel at tau = 1 where it applies
+// on larger ones at tau = 1, by the rules above.  The other fields describe the
+// march that is left: the two-column kernel at tau = 1 where it applies
 // (CTAs 64 columns wide for 16-bit storage, 128 for FP32), else the one-column kernel
 // with CTAs 128 columns wide (64 on lattices narrower than 1024).
 Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
@@ -186,14 +228,18 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     // (the two-column kernel's pulled-population ring costs resident warps)
     const int store = store_of(p.dtype), sms = sm_count();
     const bool om1 = p.tau == 1.0;
-    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G, G.nx % 4 == 0);
+    const bool quad = G.nx % 4 == 0;
+    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G, quad);
     const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     const bool narrow = store == kStoreF16 || store == kStoreBF16;
-    if (store == kStoreF64 || (narrow && !wide && !pair) ||
-        (long long)G.nx * G.ny <= (wide ? kTileNodes : kTileNodesOneColumn))
-        s.tile = tile_block_x(store, G.nx, G.ny, sms);
+    const int bx = tile_block_x(store, G.nx, G.ny, sms, om1);
+    const long long covered = (long long)G.nx * rows_covered(bx, G.ny);
+    const long long limit = wide ? kTileNodes : kTileNodesOneColumn;
+    if ((store == kStoreF64 || (narrow && !wide && !pair) || covered <= limit) &&
+        !tiles_wasted(store, covered, (long long)G.nx * G.ny))
+        s.tile = bx;
     else if (wide)
-        s.wide = wide_bands(G, wide_slots(store, G.nx % 4 == 0, sms));
+        s.wide = wide_bands(G, wide_slots(store, quad, sms));
     s.block_x = pair ? (narrow ? 64 : 128) : (G.nx >= 1024 ? 128 : 64);
     // otherwise per-thread loads: measured faster than the bulk-copy pipeline
     // on GB300 once loads are prefetched a row ahead
@@ -272,7 +318,8 @@ cudaError_t launch_recorded_step(tf_lbm_handle* H, const void* fin, void* fout, 
 {
     const Consts<float> c32 = make_consts<float>(H);
     const Consts<double> c64 = make_consts<double>(H);
-    const int bx = tile_block_x(H->desc.store, H->G.nx, H->G.ny, H->sms);
+    const bool om1 = H->dbl ? c64.omega == 1.0 : c32.omega == 1.0f;
+    const int bx = tile_block_x(H->desc.store, H->G.nx, H->G.ny, H->sms, om1);
     return launch_tile(H->desc.store, bx, fin, fout, H->kappa, mom, H->G, &c32, &c64, st);
 }
 

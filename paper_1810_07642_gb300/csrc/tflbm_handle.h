@@ -68,8 +68,9 @@ cudaError_t launch_one_step(tf_lbm_handle* H, int from, cudaStream_t st, bool fi
 // One tile step between two population buffers of the handle's layout that
 // also records the moments of the state it starts from (tflbm_tile.cuh).
 cudaError_t launch_recorded_step(tf_lbm_handle* H, const void* fin, void* fout, void* mom, cudaStream_t st);
-// block_x of the tile kernel for a lattice (see tile_of).
-int tile_block_x(int store, int nx, int ny, int sms);
+// block_x of the tile kernel for a lattice (see tile_of), forward and adjoint.
+int tile_block_x(int store, int nx, int ny, int sms, bool omega1);
+int adjoint_block_x(bool dbl, int nx, int ny, int sms);
 // Record an error message on H (or for the calling thread when H is null).
 int handle_fail(tf_lbm_handle* H, int code, const std::string& msg);
 int handle_cuda_fail(tf_lbm_handle* H, cudaError_t e, const char* what);

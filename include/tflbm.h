@@ -144,13 +144,13 @@ typedef struct tf_lbm_handle tf_lbm_handle;
  * The shape chosen by tf_lbm_init runs other kernels in place of the one that
  * its fields describe: tiles (a CTA
  * owns 16 x 8, 16 x 16 or 32 x 16 nodes and runs the step's phases over all of
- * them; any nx, ny and dtype) on lattices of up to 2^20 nodes (1.5 x 2^20
- * where the next one does not apply; any size for TF_LBM_F64, and for 16-bit storage
+ * them; any nx, ny and dtype) on lattices of up to about 10^6 nodes (1.5 x 2^20
+ * where the next one does not run; any size for TF_LBM_F64, and for 16-bit storage
  * where the fields describe pipeline 1; not on long lattices of a few rows or
  * columns, which tiles would mostly overhang); above that, at tau = 1
  * with forcing = 0, a march of four columns per thread, which between the
  * steps of one call keeps moments in place of FP32 populations (16-bit storage:
- * where nx is a multiple of 4).  So does the shape chosen by tf_lbm_tune where
+ * where nx is a multiple of 4; not on narrow lattices).  So does the shape chosen by tf_lbm_tune where
  * one of them was the fastest (reported by the fields that
  * tf_lbm_init chose).  Passing block_x, rows and pipeline as tf_lbm_init or the
  * last tf_lbm_tune reported them to tf_lbm_set_launch gives all of that shape

@@ -161,6 +161,17 @@ int validate(const tf_lbm_params* p)
     return TF_LBM_OK;
 }
 
+// Whether a run's steps go one by one to the two-column march, which has the
+// same bits: short runs of the four-column march in the ragged layout, whose first
+// and last step, from and to populations, cost more than the steps between them
+// save (us a step in runs of two, two-column / four-column: 362 x 11602 58.1 / 76.0, 602
+// x 6976 55.5 / 68.9, 1030 x 4077 55.9 / 61.3, 2046^2 52.7 / 54.3; in runs of eight the
+// two are even).
+bool one_by_one(const tf_lbm_handle* H, int64_t steps)
+{
+    return H->shape.wide && H->desc.store == kStoreF32 && H->G.nx % 4 == 2 && steps < 8;
+}
+
 int store_of(int dtype)
 {
     switch (dtype) {
@@ -171,16 +182,17 @@ int store_of(int dtype)
     }
 }
 
-// Lattices up to this many nodes run the tile kernel where the four-column
-// march, or (tau != 1, forcing, an odd nx) the one-column march, would take
-// larger ones; FP64, and 16-bit storage where the one-column march is what is
-// left, run tiles at any size.  Above the limits the marches win: they pull a
-// node 1.25 times, not 1.4, and load ahead.  One box, us a step, tile against
-// the four-column march: 900^2 FP32 12.5 / 12.2, 1024^2 15.2 / 16.4, 1300 x 1100
-// 25.4 / 17.5, 1448^2 36.3 / 21.6; FP16 1024^2 16.1 / 16.4, 1448^2 34.3 / 21.4;
-// against the one-column march at tau = 0.8: FP32 1448^2 37.2 / 36.7, 2048^2 69
-// / 63, FP16 1448^2 32.3 / 41.7, 2048^2 59.8 / 69.2; FP64 2048^2 1014 / 1101.
-constexpr long long kTileNodes = 1LL << 20, kTileNodesOneColumn = 3LL << 19;
+// The tile kernel runs where its rows cover at most this many nodes in place of:
+// the four-column march (nx a multiple of 4; ragged), the two-column march of
+// narrow 16-bit lattices, the other marches (tau != 1, forcing, narrow ragged
+// lattices).  FP64, and 16-bit storage where the one-column march is what is left,
+// run tiles at any size.  Above the limits the marches win: they pull a node 1.25
+// times, not 1.4, and load ahead.  Us a step, tile against march: FP32 four-column
+// 1024^2 14.9 / 16.4, 1200 x 1000 20 / 17.2, 1448^2 36.3 / 21.6; ragged 1030 x 1067 17.9 /
+// 21.4, 1205 x 1078 22.8 / 22.0, 1030 x 1262 23.1 / 22.2; FP16 1024^2 16.1 / 16.4, 1448^2
+// 34.3 / 21.4; against the one-column march at tau = 0.8: FP32 1448^2 37.2 / 36.7,
+// 2048^2 69 / 63, FP16 1448^2 32.3 / 41.7, 2048^2 59.8 / 69.2; FP64 2048^2 1135 / 1372.
+constexpr long long kTileQuad = 17LL << 16, kTileRagged = 5LL << 18, kTileMarch = 3LL << 19;
 
 // Long lattices of a few rows, of which tiles cover too many: they cost more than
 // the latency of a march's few rows (us a step, tile of the best shape against
@@ -195,6 +207,23 @@ bool tiles_wasted(int store, long long covered, long long nodes)
     if (3 * covered <= 4 * nodes) return false;
     if (store == kStoreF64) return covered - nodes > 9LL << 14;
     return covered > 1500000 || (covered > 2 * nodes && covered - nodes > 1LL << 17);
+}
+
+// Whether the four-column march beats the others on a lattice that it takes.
+// Ragged: its strips at either end of a row, which load and store by nodes, have
+// to be few beside the others (us a step in runs of 20, two-column / four-column:
+// 122 x 24590 44.9 / 57.8, 126 x 17460 43.3 / 45.0, 242 x 17355 58.0 / 61.5, 242 x 9090 39.9 /
+// 36.5, 362 x 11602 56.5 / 57.5, 362 x 6077 39.7 / 34.3, 482 x 8713 56.0 / 54.5, 1030 x 4077
+// 54.6 / 48.0; one-column, nx odd: 483 x 4554 36.4 / 32.5, 2047 x 2049 60 / 45, 243 x 9053
+// 38.7 / 36.3, but 40.6 / 47.8 in runs of two).  A run of one step, which tiles take
+// where nx is odd, costs more than the one-column march there: 2047 x 2049 74 / 65.
+bool wide_wins(int store, const Geom& G)
+{
+    WideCover cover;
+    cover.add(G.nx, G.ny);
+    if (G.nx % 4 == 0) return cover.pays(store);
+    const int strips = wide_strips(G.nx);
+    return strips >= 5 || (strips >= 3 && G.nx % 2 == 0 && (long long)G.nx * G.ny <= 3LL << 20);
 }
 
 // A march filled with balanced bands: as many as fill the resident slots once
@@ -229,12 +258,12 @@ Shape default_shape(const tf_lbm_params& p, const Geom& G, bool kfield)
     const int store = store_of(p.dtype), sms = sm_count();
     const bool om1 = p.tau == 1.0;
     const bool quad = G.nx % 4 == 0;
-    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G, quad);
+    const bool wide = om1 && p.forcing == 0 && wide_applies(store, G, quad) && wide_wins(store, G);
     const bool pair = pair_pipeline_ok(G.nx, store) && om1;
     const bool narrow = store == kStoreF16 || store == kStoreBF16;
     const int bx = tile_block_x(store, G.nx, G.ny, sms, om1);
     const long long covered = (long long)G.nx * rows_covered(bx, G.ny);
-    const long long limit = wide ? kTileNodes : kTileNodesOneColumn;
+    const long long limit = wide ? (quad ? kTileQuad : kTileRagged) : (narrow && pair && quad ? kTileQuad : kTileMarch);
     if ((store == kStoreF64 || (narrow && !wide && !pair) || covered <= limit) &&
         !tiles_wasted(store, covered, (long long)G.nx * G.ny))
         s.tile = bx;
@@ -453,8 +482,9 @@ int tf_lbm_step(tf_lbm_handle* H, int64_t nsteps, void* stream)
                 if (!H->cap) CK(H, cudaStreamCreateWithFlags(&H->cap, cudaStreamNonBlocking), "cudaStreamCreate");
                 CK(H, cudaStreamBeginCapture(H->cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
                 cudaError_t le = cudaSuccess;
+                const bool alone = one_by_one(H, chunk);
                 for (int i = 0; i < chunk && le == cudaSuccess; ++i)
-                    le = launch_one_step(H, H->cur ^ (i & 1), H->cap, i == 0, i == chunk - 1);
+                    le = launch_one_step(H, H->cur ^ (i & 1), H->cap, alone || i == 0, alone || i == chunk - 1);
                 cudaGraph_t g = nullptr;
                 cudaError_t ce = cudaStreamEndCapture(H->cap, &g);
                 if (le != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(H, le, "step kernel (capture)"); }
@@ -468,8 +498,9 @@ int tf_lbm_step(tf_lbm_handle* H, int64_t nsteps, void* stream)
             H->time += chunk;
         } else {
             // one run of all the steps that no graph takes
+            const bool alone = one_by_one(H, nsteps);
             for (const int64_t n = nsteps; nsteps > 0; --nsteps) {
-                CK(H, launch_one_step(H, H->cur, st, nsteps == n, nsteps == 1), "step kernel");
+                CK(H, launch_one_step(H, H->cur, st, alone || nsteps == n, alone || nsteps == 1), "step kernel");
                 H->cur ^= 1;
                 ++H->time;
             }

@@ -135,3 +135,22 @@ def test_narrow_16_bit_batches(nx, ny, count, four):
         batch.step(2)
         assert all(f.check() == 0 for f in films)
     [f.close() for f in films]
+
+
+# ragged lattices on either side of the rules: tiles, the four-column march with
+# runs of at least eight steps, the two-column march (two strips); odd: no two
+# columns.  FP32 at tau = 1: the same bits whatever the kernel.
+@pytest.mark.parametrize("nx,ny", [(1030, 1040), (1030, 1262), (126, 13000), (242, 9090), (1205, 1330), (362, 4000)])
+def test_ragged_runs_of_any_length_give_the_same_bits(nx, ny):
+    states = []
+    for split in ((17,), (3, 8, 1, 5), (7, 10), (2,) * 8 + (1,), None):
+        sim = film(nx, ny)
+        if split is None:
+            _lib.use_tiles(sim.handle, 256, graph_chunk=4)
+            split = (17,)
+        for n in split:
+            sim.step(n)
+        assert sim.check() == 0 and sim.time == 17
+        states.append(sim.get_state())
+        sim.close()
+    assert all(torch.equal(states[0], s) for s in states[1:])

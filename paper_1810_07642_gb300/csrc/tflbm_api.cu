@@ -75,6 +75,7 @@ int tile_block_x(int store, int nx, int ny, int sms, bool omega1)
 int adjoint_block_x(bool dbl, int nx, int ny, int sms)
 {
     if (!dbl) return tile_block_f32(nx, ny, sms);
+    if (5 * rows_covered(256, ny) > 6 * rows_covered(64, ny)) return 64;
     return tiles_of(64, nx, ny) <= sms ? 64 : (tiles_of(256, nx, ny) >= 7LL * sms ? 256 : 128);
 }
 }  // namespace tflbm

@@ -201,14 +201,17 @@ __device__ __forceinline__ int ringi(int i, int n)
 // from L1/L2; before, three kernels read the populations twice and moved h
 // and p through memory.  A CTA owns a tile of kPfX x kPfY nodes: h - href of
 // the tile and a halo of 2, the pressure of the tile and a halo of 1, then the
-// force; each thread keeps the momenta of its own four nodes.  64 x 16: rows
+// force; each thread keeps the momenta of its own nodes.  64 x 16: rows
 // long enough for coalesced pulls, 1.33 pulls a node.  2048^2 FP32 read-out
-// (k_moments and this): 250 -> 93 us.
-constexpr int kPfX = 64, kPfY = 16, kPfThreads = 256, kPfOwn = kPfX * kPfY / kPfThreads;
-template <typename T, typename SM>
+// (k_moments and this): 250 -> 93 us.  64 x 4 for FP64 state on lattices of fewer
+// 64 x 16 tiles than half the SMs, where a CTA's FP64 arithmetic is a chain on one
+// SM (128^2, with the launch: 28 us as three kernels, 38 in 16 rows, 25 in 4).
+constexpr int kPfX = 64, kPfThreads = 256;
+template <typename T, typename SM, int kPfY>
 __global__ void __launch_bounds__(kPfThreads) k_pf(Pops<T, SM> P, const T* __restrict__ kappa, T* p, T* fx, T* fy,
                                                    Geom G, Consts<T> C)
 {
+    constexpr int kPfOwn = kPfX * kPfY / kPfThreads;
     __shared__ T hs[kPfY + 4][kPfX + 4];
     __shared__ T ps[kPfY + 2][kPfX + 2];
     const int x0 = blockIdx.x * kPfX, y0 = blockIdx.y * kPfY;
@@ -1073,9 +1076,16 @@ template <typename T, typename SM>
 cudaError_t pf_t(const StoreDesc& D, const void* f, const void* kappa, void* p, void* fx, void* fy,
                  const Geom& G, const Consts<T>& C, cudaStream_t st)
 {
-    const dim3 grid((G.nx + kPfX - 1) / kPfX, (G.ny + kPfY - 1) / kPfY);
-    k_pf<T, SM><<<grid, kPfThreads, 0, st>>>(make_pops<T, SM>(f, G, D), (const T*)kappa, (T*)p, (T*)fx, (T*)fy, G, C);
-    return cudaGetLastError();
+    auto launch = [&](auto rows) {
+        constexpr int Y = decltype(rows)::value;
+        const dim3 grid((G.nx + kPfX - 1) / kPfX, (G.ny + Y - 1) / Y);
+        k_pf<T, SM, Y><<<grid, kPfThreads, 0, st>>>(make_pops<T, SM>(f, G, D), (const T*)kappa, (T*)p, (T*)fx, (T*)fy, G, C);
+        return cudaGetLastError();
+    };
+    if constexpr (sizeof(T) == 8) {
+        if (2LL * ((G.nx + kPfX - 1) / kPfX) * ((G.ny + 15) / 16) < sm_count()) return launch(std::integral_constant<int, 4>());
+    }
+    return launch(std::integral_constant<int, 16>());
 }
 
 template <typename T, typename SM>

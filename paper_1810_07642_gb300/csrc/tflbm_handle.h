@@ -78,8 +78,6 @@ int handle_cuda_fail(tf_lbm_handle* H, cudaError_t e, const char* what);
 int handle_check_dev_ptr(tf_lbm_handle* H, const void* ptr, const char* name, bool allow_null);
 // Forget the handle's captured step graphs (after a launch-shape change).
 void handle_drop_graphs(tf_lbm_handle* H);
-// Streaming multiprocessors of the current device.
-int sm_count();
 // Adjoint of one step (tflbm_adjoint.cu).
 cudaError_t adjoint_step_dispatch(tf_lbm_handle* H, const void* f, const void* a_next, void* a,
                                   void* grad_kappa, cudaStream_t st);

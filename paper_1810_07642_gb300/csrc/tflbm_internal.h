@@ -6,6 +6,9 @@
 
 namespace tflbm {
 
+// Streaming multiprocessors of the current device.
+int sm_count();
+
 // Geometry of the population buffers: 9 planes of ny rows of `pitch`
 // elements; only the first nx columns of a row are lattice nodes.
 struct Geom {

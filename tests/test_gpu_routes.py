@@ -44,3 +44,17 @@ def test_long_lattices(nx, ny, dtype, tau):
 @pytest.mark.parametrize("tau", [1.0, 0.8])
 def test_fp64_tile_shapes(nx, ny, tau):
     compare(nx, ny, "f64", tau)
+
+
+# 64 x 4 tiles on few of them, 64 x 16 from half the SMs on
+@pytest.mark.parametrize("nx,ny", [(64, 4), (65, 5), (63, 37), (321, 190), (321, 260), (257, 511)])
+def test_fp64_pressure_and_force_in_either_tile(nx, ny):
+    h0, th, p = inputs.small_random(nx, ny, seed=3, amp=0.05)
+    p.update(gx_body=1e-4, gy_body=-2e-4, g=1e-3)
+    sim = ThinFilm(p, h0, th, dtype="f64")
+    sim.step(3)
+    cfg = O.Config(**{k: v for k, v in p.items() if k in O.Config.__dataclass_fields__})
+    f = np.ascontiguousarray(sim.get_state().cpu().numpy())
+    got = sim.pressure_force()
+    for name, want in zip(("p", "fx", "fy"), O.pressure_force(cfg, O.kappa_field(cfg, th), f)):
+        assert np.abs(got[name].cpu().numpy() - want).max() <= 1e-11 * np.abs(want).max(), name

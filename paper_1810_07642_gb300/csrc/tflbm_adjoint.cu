@@ -287,7 +287,7 @@ cudaError_t adjoint_tile_t(tf_lbm_handle* H, const void* mom, bool fresh, const 
 {
     const Consts<S> C = make_consts<S>(H);
     const S *m = (const S*)mom, *n = (const S*)an, *k = (const S*)H->kappa;
-    switch (adjoint_block_x(H->dbl, H->G.nx, H->G.ny, H->sms)) {
+    switch (H->tape_tile ? H->tape_tile : adjoint_block_x(H->dbl, H->G.nx, H->G.ny, H->sms)) {
         case 64: return adjoint_tile_one<S, 16, 8>(m, fresh, n, (S*)a, (S*)gk, k, H->G, C, st);
         case 128: return adjoint_tile_one<S, 16, 16>(m, fresh, n, (S*)a, (S*)gk, k, H->G, C, st);
         default: return adjoint_tile_one<S, 32, 16>(m, fresh, n, (S*)a, (S*)gk, k, H->G, C, st);

@@ -349,7 +349,7 @@ cudaError_t launch_recorded_step(tf_lbm_handle* H, const void* fin, void* fout, 
     const Consts<float> c32 = make_consts<float>(H);
     const Consts<double> c64 = make_consts<double>(H);
     const bool om1 = H->dbl ? c64.omega == 1.0 : c32.omega == 1.0f;
-    const int bx = tile_block_x(H->desc.store, H->G.nx, H->G.ny, H->sms, om1);
+    const int bx = H->tape_tile ? H->tape_tile : tile_block_x(H->desc.store, H->G.nx, H->G.ny, H->sms, om1);
     return launch_tile(H->desc.store, bx, fin, fout, H->kappa, mom, H->G, &c32, &c64, st);
 }
 
@@ -631,13 +631,13 @@ int tf_lbm_set_launch(tf_lbm_handle* H, const tf_lbm_launch* in)
 }
 
 // Not part of the interface: run the tiles that block_x names (tile_of) on any
-// lattice, for the tests of tile edges.
+// lattice, in steps and in the handle's tapes, for the tests of tile edges.
 int tflbm_use_tiles(tf_lbm_handle* H, int32_t block_x, int32_t graph_chunk)
 {
     if (!H || (block_x != 64 && block_x != 128 && block_x != 256) || graph_chunk < 0 || graph_chunk % 2 != 0)
         return TF_LBM_ERR_ARG;
     drop_graphs(H);
-    H->shape.tile = block_x;
+    H->shape.tile = H->tape_tile = block_x;
     H->shape.wide = 0;
     H->graph_chunk = graph_chunk;
     return TF_LBM_OK;

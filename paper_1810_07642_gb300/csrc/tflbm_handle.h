@@ -37,6 +37,7 @@ struct tf_lbm_handle {
     Shape def{128, 64, kPipeLdg};    // the default: what tuning puts tiles and the four-column march on
     Shape own{128, 64, kPipeLdg};    // what init or tuning chose: setting its fields gives it back whole
     Shape one{128, 64, kPipePair};   // the two-column march that takes a run of one FP32 step of a wide shape
+    int tape_tile = 0;               // tests: block_x of a tape's tiles, forward and adjoint; 0: by the lattice
     int graph_chunk = 0;
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};

@@ -63,7 +63,11 @@ k_adjoint_tile(const S* __restrict__ mom, bool fresh, bool early, const S* __res
     const int c = t % TX, r = t / TX;  // own nodes: (c, r + k HALF)
     const bool disj = kappa != nullptr || C.kappa_u != S(0);
     auto pk = [](S v) { return Lanes<X>::all(v); };
-    auto node = [&](int cc, int rr) { return ring_index(y0 + rr, ny) * nx + ring_index(x0 + cc, nx); };
+    auto node = [&](int cc, int rr) {
+        return TFLBM_IDX(ring_index(y0 + rr, ny) * nx + ring_index(x0 + cc, nx), n, C.status);
+    };
+    // offset k within a plane of an or a
+    auto in_plane = [&](uint32_t k) { return TFLBM_IDX(k, n, C.status); };
     auto lanes = [&](auto fn) {
         fn(std::integral_constant<int, 0>{});
         if constexpr (N == 2) fn(std::integral_constant<int, 1>{});
@@ -110,7 +114,7 @@ k_adjoint_tile(const S* __restrict__ mom, bool fresh, bool early, const S* __res
 #pragma unroll
         for (int p = 0; p < PASSES; ++p) {
             const int rr = r + p * RP;
-            const uint32_t k = ring_index(y0 + rr - 3, ny) * nx + xc;
+            const uint32_t k = in_plane(ring_index(y0 + rr - 3, ny) * nx + xc);
 #pragma unroll
             for (int f = 0; f < 3; ++f) v[p][f] = rr < TY + 6 ? ldro(an + f * n + k) : S(0);
         }
@@ -157,15 +161,15 @@ k_adjoint_tile(const S* __restrict__ mom, bool fresh, bool early, const S* __res
             const int x = ring_index(x0 + cc, nx), y = ring_index(y0 + rr, ny);
             const int xm = x == 0 ? nx - 1 : x - 1, xp = x + 1 == nx ? 0 : x + 1;
             const int r0 = y * nx, rD = (y == 0 ? ny - 1 : y - 1) * nx, rU = (y + 1 == ny ? 0 : y + 1) * nx;
-            lane_of<K>(mu[0]) = ldro(an + (r0 + x));
-            lane_of<K>(mu[1]) = ldro(an + (n + r0 + xp));
-            lane_of<K>(mu[2]) = ldro(an + (2 * n + rU + xp));
-            lane_of<K>(mu[3]) = ldro(an + (3 * n + rU + x));
-            lane_of<K>(mu[4]) = ldro(an + (4 * n + rU + xm));
-            lane_of<K>(mu[5]) = ldro(an + (5 * n + r0 + xm));
-            lane_of<K>(mu[6]) = ldro(an + (6 * n + rD + xm));
-            lane_of<K>(mu[7]) = ldro(an + (7 * n + rD + x));
-            lane_of<K>(mu[8]) = ldro(an + (8 * n + rD + xp));
+            lane_of<K>(mu[0]) = ldro(an + in_plane(r0 + x));
+            lane_of<K>(mu[1]) = ldro(an + (n + in_plane(r0 + xp)));
+            lane_of<K>(mu[2]) = ldro(an + (2 * n + in_plane(rU + xp)));
+            lane_of<K>(mu[3]) = ldro(an + (3 * n + in_plane(rU + x)));
+            lane_of<K>(mu[4]) = ldro(an + (4 * n + in_plane(rU + xm)));
+            lane_of<K>(mu[5]) = ldro(an + (5 * n + in_plane(r0 + xm)));
+            lane_of<K>(mu[6]) = ldro(an + (6 * n + in_plane(rD + xm)));
+            lane_of<K>(mu[7]) = ldro(an + (7 * n + in_plane(rD + x)));
+            lane_of<K>(mu[8]) = ldro(an + (8 * n + in_plane(rD + xp)));
         }
     };
     const X third = pk(S(1.0 / 3.0)), twelfth = pk(S(1.0 / 12.0));
@@ -258,7 +262,7 @@ k_adjoint_tile(const S* __restrict__ mom, bool fresh, bool early, const S* __res
         lanes([&](auto k_c) {
             constexpr int K = decltype(k_c)::value;
             const int x = x0 + c, y = y0 + r + K * HALF;
-            if (x < nx && y < ny) gk[y * nx + x] = lane_of<K>(sum);
+            if (x < nx && y < ny) gk[in_plane(y * nx + x)] = lane_of<K>(sum);
         });
     }
     if (t < PP) {
@@ -319,7 +323,7 @@ k_adjoint_tile(const S* __restrict__ mom, bool fresh, bool early, const S* __res
         constexpr int K = decltype(k_c)::value;
         const int x = x0 + c, y = y0 + r + K * HALF;
         if (x >= nx || y >= ny) return;
-        S* out = a + (y * nx + x);
+        S* out = a + in_plane(y * nx + x);
 #pragma unroll
         for (int l = 0; l < (OMEGA1 ? 3 : 9); ++l) out[l * n] = lane_of<K>(o[l]);
     });

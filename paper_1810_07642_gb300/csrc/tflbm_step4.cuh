@@ -147,6 +147,11 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
     const int mpitch = QUAD ? pitch : mom_pitch(nx), mplane = ny * mpitch;
     const int xg = QUAD ? xw : xt, xm = QUAD ? xw : xt + 4;  // the group in a population and in a moments row
     (void)mplane;
+    // offsets within a moments plane at which the last plane's group still lies in
+    // the population buffer
+    const long long mroom = 9LL * plane - (kMomPlanes - 1LL) * mplane - 3;
+    (void)mroom;
+    TFLBM_CHECK(!whole || (xm >= 0 && xm + 3 < mpitch && xg >= 0 && xg + 3 < nx), C.status);
     const float* __restrict__ in0 = (const float*)fin;
     const SM* __restrict__ inm = (const SM*)(in0 + plane);
     float* __restrict__ out0 = (float*)fout;
@@ -172,6 +177,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
     // ends (only in strips with odd: one branch a row)
     const bool odd = !QUAD && (ends || weff % 4 != 0);
     auto store_odd = [&](auto* __restrict__ row, bool images, const auto (&v)[NP]) {  // row: at column 0
+        TFLBM_CHECK(!part || (xt >= 0 && xt < nx), C.status);
         if (part) {
             row[xt] = v[0].x;
             if (xt + 1 < nx) row[xt + 1] = v[0].y;
@@ -182,6 +188,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
             for (int i = 0; i < 4; ++i) {
                 const int x = xt + i;
                 const auto c = i == 0 ? v[0].x : (i == 1 ? v[0].y : (i == 2 ? v[1].x : v[1].y));
+                TFLBM_CHECK(x >= 0 && nx >= 4 && nx + 8 <= mpitch, C.status);
                 if (x < 4) row[nx + x] = c;
                 if (x >= nx - 4 && x < nx) row[x - nx] = c;
             }
@@ -196,7 +203,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
     auto copy = [&](auto* dst, const auto* __restrict__ row, bool groups) {  // dst: 4 elements; row: of a population plane
         using E = typename std::remove_reference<decltype(*dst)>::type;
         if (groups) {
-            cp_async4<E>(dst, row + xg);
+            cp_async4<E>(dst, row + TFLBM_IDX(xg, pitch - 3, C.status));
         } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -210,7 +217,8 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
     auto copy_row = [&](int st, int y) {
         TFLBM_CHECK(y >= 0 && y < ny, C.status);
         if constexpr (MOM_IN) {
-            const uint32_t off = (uint32_t)y * (uint32_t)mpitch + (uint32_t)xm;
+            // the window may run past its row (see mom_pitch), not past the buffer
+            const uint32_t off = TFLBM_IDX((uint32_t)y * (uint32_t)mpitch + (uint32_t)xm, mroom, C.status);
 #pragma unroll
             for (int f = 0; f < kMomPlanes; ++f) cp_async4<float>(&wide[st][f][4 * t], in0 + f * mplane + off);
         } else {
@@ -296,6 +304,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
         if (kappa) {
             const float* row = kappa + TFLBM_IDX(wk * nx, nk, C.status);
             if constexpr (QUAD) {
+                TFLBM_CHECK(xw >= 0 && xw + 3 < nx, C.status);
                 lds_pairs<NP>(row + xw, kap);
             } else {
                 const int x1 = xw + 1 == nx ? 0 : xw + 1, x2 = x1 + 1 == nx ? 0 : x1 + 1, x3 = x2 + 1 == nx ? 0 : x2 + 1;

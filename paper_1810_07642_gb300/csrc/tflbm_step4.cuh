@@ -58,8 +58,8 @@ enum { kMomH = 0, kMomE, kMomJx, kMomJy, kMomGx, kMomGy, kMomPlanes };
 // row; wide_applies says whether the planes, with that, fit a population buffer.
 __host__ __device__ inline int mom_pitch(int nx) { return (nx + 8 + 3) / 4 * 4; }
 
-// One row of h or p at the thread's columns and the two beside them.
-template <int NP>
+// One row of h or p at the thread's columns (NP pairs) and the two beside them.
+constexpr int NP = 2;
 struct WideRow {
     float2 c[NP];
     float l, r;
@@ -74,28 +74,20 @@ struct WideRow {
     __device__ __forceinline__ float2 right(int p) const { return make_float2(c[p].y, p == NP - 1 ? r : c[p + 1].x); }
 };
 // the window of the thread's pair p
-template <int NP>
-__device__ __forceinline__ Win<float2> wide_window(const WideRow<NP>& n, const WideRow<NP>& c, const WideRow<NP>& s, int p)
+__device__ __forceinline__ Win<float2> wide_window(const WideRow& n, const WideRow& c, const WideRow& s, int p)
 {
     return {n.c[p], n.left(p), n.right(p), c.c[p], c.left(p), c.right(p), s.c[p], s.left(p), s.right(p)};
 }
-// a thread's 2 NP consecutive values
-template <int NP>
+// a thread's four consecutive values
 __device__ __forceinline__ void lds_pairs(const float* p, float2 (&v)[NP])
 {
-    if constexpr (NP == 2) {
-        const float4 q = *reinterpret_cast<const float4*>(p);
-        v[0] = make_float2(q.x, q.y);
-        v[1] = make_float2(q.z, q.w);
-    } else {
-        v[0] = *reinterpret_cast<const float2*>(p);
-    }
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = make_float2(q.x, q.y);
+    v[1] = make_float2(q.z, q.w);
 }
-template <int NP>
 __device__ __forceinline__ void sts_pairs(float* p, const float2 (&v)[NP])
 {
-    if constexpr (NP == 2) *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-    else *reinterpret_cast<float2*>(p) = v[0];
+    *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
 }
 
 // Four elements, 16 (or, of a 16-bit type, 8) bytes; .cg: through L2 only.
@@ -114,13 +106,13 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
                                            const float* __restrict__ kappa, const Geom& G, const Consts<float>& C0,
                                            int strip, int band, int nbands)
 {
-    static_assert(!(MOM_IN || MOM_OUT) || sizeof(SM) == 4, "moments go with FP32 storage");
+    static_assert((!(MOM_IN || MOM_OUT) && QUAD) || sizeof(SM) == 4, "moments and ragged rows go with FP32 storage");
     using IO = PairIO<SM>;
     using V = typename IO::V;
     // rows on their way: full-width planes, and 8 moving planes of the storage type
     constexpr int kAhead = sizeof(SM) == 4 && !MOM_IN ? 1 : 2, kStagesW = kAhead + 1;
     constexpr int kFull = MOM_IN ? (int)kMomPlanes : 1;
-    constexpr int NP = 2, NC = 128;
+    constexpr int NC = 128;
     __shared__ __align__(16) float wide[kStagesW][kFull][NC];
     __shared__ __align__(16) SM moving[MOM_IN ? 1 : kStagesW][MOM_IN ? 1 : 8][MOM_IN ? 8 : NC];
     // the thread's j_x, j_y and sum residual of the last three rows
@@ -207,9 +199,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
         } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int x = wrap_index(xt + i, nx);
-                if constexpr (sizeof(E) == 4) cp_async<4>(dst + i, row + x);
-                else dst[i] = __ldg(row + x);
+                if constexpr (!QUAD) cp_async<sizeof(E)>(dst + i, row + wrap_index(xt + i, nx));
             }
         }
     };
@@ -234,7 +224,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
     };
     // populations l = 2, 3, 4 of the last two rows, f_0, l = 1 and 5 of the last
     float2 E1[3][NP], E2[3][NP], W[3][NP];
-    WideRow<NP> H[3], P[3];
+    WideRow H[3], P[3];
     float2 ih[3][NP], kap[NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
@@ -266,7 +256,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
         cp_async_wait<kAhead - 1>();
         float2 f0[NP], o[NP][8], m[kFull][NP];
 #pragma unroll
-        for (int f = 0; f < kFull; ++f) lds_pairs<NP>(&wide[st][f][2 * NP * t], m[f]);
+        for (int f = 0; f < kFull; ++f) lds_pairs(&wide[st][f][2 * NP * t], m[f]);
         if constexpr (!MOM_IN) {
 #pragma unroll
             for (int l = 0; l < 8; ++l) {
@@ -305,7 +295,7 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
             const float* row = kappa + TFLBM_IDX(wk * nx, nk, C.status);
             if constexpr (QUAD) {
                 TFLBM_CHECK(xw >= 0 && xw + 3 < nx, C.status);
-                lds_pairs<NP>(row + xw, kap);
+                lds_pairs(row + xw, kap);
             } else {
                 const int x1 = xw + 1 == nx ? 0 : xw + 1, x2 = x1 + 1 == nx ? 0 : x1 + 1, x3 = x2 + 1 == nx ? 0 : x2 + 1;
                 kap[0] = make_float2(__ldg(row + xw), __ldg(row + x1));
@@ -342,9 +332,9 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
             W[1][p] = o[p][0];
             W[2][p] = o[p][4];
         }
-        sts_pairs<NP>(&ring[s][0][2 * NP * t], jx);
-        sts_pairs<NP>(&ring[s][1][2 * NP * t], jy);
-        sts_pairs<NP>(&ring[s][2][2 * NP * t], er);
+        sts_pairs(&ring[s][0][2 * NP * t], jx);
+        sts_pairs(&ring[s][1][2 * NP * t], jy);
+        sts_pairs(&ring[s][2][2 * NP * t], er);
         H[s].sides();
         // ---- pressure of row r(k-2)
         if (k >= 4) {
@@ -359,9 +349,9 @@ __device__ __forceinline__ void step_band4(const void* __restrict__ fin, void* _
             TFLBM_CHECK(y >= 0 && y < ny, C.status);
             float2 kx[NP], ky[NP], e[NP], Gx[NP], Gy[NP], r0[NP], n[8][NP];
             V v[8][NP];
-            lds_pairs<NP>(&ring[spp][0][2 * NP * t], kx);
-            lds_pairs<NP>(&ring[spp][1][2 * NP * t], ky);
-            lds_pairs<NP>(&ring[spp][2][2 * NP * t], e);
+            lds_pairs(&ring[spp][0][2 * NP * t], kx);
+            lds_pairs(&ring[spp][1][2 * NP * t], ky);
+            lds_pairs(&ring[spp][2][2 * NP * t], e);
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
                 const float2 d = H[spp].c[p], h = padd(d, pk(C.href));

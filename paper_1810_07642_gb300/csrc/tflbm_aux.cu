@@ -520,21 +520,20 @@ template <> struct Acc2<float> {
         const V e = two_sum2(c, two_sum2(s, a.s));
         d = __fadd2_rn(d, __fadd2_rn(__fadd2_rn(e, two_sum2(c, a.c)), a.d));
     }
-    __device__ __forceinline__ Acc2 down(int o) const  // of the lane o above
+    // fn of the values of a and b, part by part
+    template <typename Fn>
+    static __device__ __forceinline__ Acc2 of(const Acc2& a, const Acc2& b, Fn fn)
     {
-        auto at = [&](V v) { return V{__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o)}; };
-        Acc2 a;
-        a.s = at(s);
-        a.c = at(c);
-        a.d = at(d);
-        return a;
+        Acc2 r;
+        r.s = fn(a.s, b.s);
+        r.c = fn(a.c, b.c);
+        r.d = fn(a.d, b.d);
+        return r;
     }
-    __device__ __forceinline__ void store(double* out) const  // first and second sum, each as (sum, compensation)
+    __device__ __forceinline__ void store_first(double* out) const  // as (sum, compensation)
     {
         out[0] = (double)s.x / kScale;
         out[1] = ((double)c.x + (double)d.x) / kScale;
-        out[2] = (double)s.y / kScale;
-        out[3] = ((double)c.y + (double)d.y) / kScale;
     }
 
 private:
@@ -566,20 +565,18 @@ template <> struct Acc2<double> {
         c.x += a.c.x;
         c.y += a.c.y;
     }
-    __device__ __forceinline__ Acc2 down(int o) const
+    template <typename Fn>
+    static __device__ __forceinline__ Acc2 of(const Acc2& a, const Acc2& b, Fn fn)
     {
-        auto at = [&](V v) { return V{__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o)}; };
-        Acc2 a;
-        a.s = at(s);
-        a.c = at(c);
-        return a;
+        Acc2 r;
+        r.s = fn(a.s, b.s);
+        r.c = fn(a.c, b.c);
+        return r;
     }
-    __device__ __forceinline__ void store(double* out) const
+    __device__ __forceinline__ void store_first(double* out) const
     {
         out[0] = s.x;
         out[1] = c.x;
-        out[2] = s.y;
-        out[3] = c.y;
     }
 
 private:
@@ -591,12 +588,47 @@ private:
         c.y += fma(c_, w.hi.y, fma(s_, w.hi.y, -q.y));
     }
 };
-template <typename T>
-__device__ __forceinline__ Acc2<T> warp_total(Acc2<T> a)
+// a lane's value v of the lane across bit o
+template <typename V>
+__device__ __forceinline__ V lane_across(V v, int o)
 {
+    return V{__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
+}
+// Half of a warp's 2 N sums to either of the lanes across bit o: the first sums
+// of the pairs where the bit is 0, the second ones where it is 1, packed in pairs
+// again.  A reduction by halves moves and merges each sum once a level over all
+// lanes: 36 shuffles and 8 merges for ten sums of three parts, not 150 and 25.
+template <typename T, int N>
+__device__ __forceinline__ void warp_halve(const Acc2<T> (&a)[N], Acc2<T> (&out)[(N + 1) / 2], int o)
+{
+    using V = typename Acc2<T>::V;
+    const bool upper = (threadIdx.x & o) != 0;
+    auto pack = [](const Acc2<T>& p, const Acc2<T>& q, bool second) {
+        return Acc2<T>::of(p, q, [&](V u, V v) { return V{second ? u.y : u.x, second ? v.y : v.x}; });
+    };
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a.merge(a.down(o));
-    return a;
+    for (int j = 0; j < (N + 1) / 2; ++j) {
+        const Acc2<T> q = 2 * j + 1 < N ? a[2 * j + 1 < N ? 2 * j + 1 : 0] : Acc2<T>();
+        const Acc2<T> give = pack(a[2 * j], q, !upper);
+        out[j] = pack(a[2 * j], q, upper);
+        out[j].merge(Acc2<T>::of(give, give, [&](V u, V) { return lane_across(u, o); }));
+    }
+}
+// The warp's totals of five pairs of sums: the first sum of the result is that
+// of pair `index` / 2, its second one where index is odd; index >= 10: nothing.
+template <typename T>
+__device__ __forceinline__ Acc2<T> warp_totals(const Acc2<T> (&a)[5], int& index)
+{
+    using V = typename Acc2<T>::V;
+    Acc2<T> b[3], c[2], d[1], e[1];
+    warp_halve(a, b, 16);
+    warp_halve(b, c, 8);
+    warp_halve(c, d, 4);
+    warp_halve(d, e, 2);
+    e[0].merge(Acc2<T>::of(e[0], e[0], [](V u, V) { return lane_across(u, 1); }));
+    const int l = threadIdx.x;
+    index = 2 * (2 * (2 * (l >> 1 & 1) + (l >> 2 & 1)) + (l >> 3 & 1)) + (l >> 4 & 1);
+    return e[0];
 }
 
 template <typename T>
@@ -626,12 +658,12 @@ __global__ void k_diag_table(const BatchDomain<T>* __restrict__ doms, Trig<T>* t
 // mode has no wave along y) and a column factor per unit (cos(a + b) from the
 // two angles).  The unit height gives every warp of the launch one unit where it
 // can, but at least kDiagRows rows (a unit's products and its reduction over the
-// warp cost about ten rows).
+// warp cost about five rows).
 // Bound by the chains of TwoSums (60 paired operations a node, 90 with a row
 // phase) and the latency of a row's nine loads: 32 warps an SM hide them better
 // than 24 with the next row's loads in flight (32 domains, 7.6 M nodes, with the
-// final kernel and the launches: 117 against 129 us; 40 warps spill: 138).  In
-// doubles 2150 us.
+// final kernel and the launches: 107 us; 24 warps 114; 40 spill: 124; skipping the
+// wetted sums of dry rows by a vote 128).  In doubles 2150 us.
 constexpr int kDiagPartial = 2 * kDiagSums + 1;
 constexpr int kDiagRows = 16;
 template <typename T, typename SM>
@@ -648,13 +680,13 @@ k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T
     using V = typename Acc2<T>::V;
     // per warp: (h, wetted h), (j_x, j_y), wetted h (cos, sin) of the column
     // and of the row angle, h (cos, sin) of the mode; wetted nodes; largest h
-    __shared__ Acc2<T> sm[5][NW];
+    __shared__ Acc2<T> sm[10][NW];  // first sums only
     __shared__ long long scount[NW];
     __shared__ T smax[NW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane < 5) sm[lane][wid] = Acc2<T>();
-    if (lane == 5) scount[wid] = 0;
-    if (lane == 6) smax[wid] = -INFINITY;
+    if (lane < 10) sm[lane][wid] = Acc2<T>();
+    if (lane == 10) scount[wid] = 0;
+    if (lane == 11) smax[wid] = -INFINITY;
     __syncwarp();
     // integer wave numbers reduced modulo the lattice, so phases stay exact
     const int kx = ((mx % G.nx) + G.nx) % G.nx, ky = ((my % G.ny) + G.ny) % G.ny;
@@ -719,15 +751,9 @@ k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T
             ap.add_first(am, m);
             ap.add_second(am, m.turned());
         }
-        auto total = [&](int k, const Acc2<T>& a) {
-            const Acc2<T> q = warp_total(a);
-            if (lane == 0) sm[k][wid].merge(q);
-        };
-        total(0, ah);
-        total(1, aj);
-        total(2, ac);
-        total(3, ar);
-        total(4, ap);
+        int k;
+        const Acc2<T> q = warp_totals<T>({ah, aj, ac, ar, ap}, k);
+        if (k < 10 && lane % 2 == 0) sm[k][wid].merge(q);
         count = __reduce_add_sync(0xffffffffu, count);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_down_sync(0xffffffffu, top, o));
@@ -739,17 +765,16 @@ k_diag_partial(const BatchDomain<T>* __restrict__ doms, int parity, const Trig<T
     __syncthreads();
     double* out = partials + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kDiagPartial;
     const int k = threadIdx.x;
-    if (k < 5) {
+    if (k < 10) {
         Acc2<T> b = sm[k][0];
         for (int w = 1; w < NW; ++w) b.merge(sm[k][w]);
-        const int q = 2 * (k < 2 ? 2 * k : 2 * k + 1);  // sums (0, 1), (2, 3), (5, 6), (7, 8), (9, 10)
-        b.store(out + q);
-    } else if (k == 5) {
+        b.store_first(out + 2 * (k < 4 ? k : k + 1));  // sums 0 .. 3, 5 .. 10
+    } else if (k == 10) {
         long long b = 0;
         for (int w = 0; w < NW; ++w) b += scount[w];
         out[8] = (double)b;  // exact below 2^53
         out[9] = 0.0;
-    } else if (k == 6) {
+    } else if (k == 11) {
         T b = smax[0];
         for (int w = 1; w < NW; ++w) b = fmax(b, smax[w]);
         out[2 * kDiagSums] = b;

@@ -65,7 +65,9 @@ class Evolve(torch.autograd.Function):
                        dtype=dtype, device=h0.device if h0.is_cuda else "cuda")
         wanted = tape and any(ctx.needs_input_grad[:2])
         if not wanted and int(nsteps) >= 1 and int(params.get("forcing", 0)) == 0:
-            # nothing to differentiate (the tape refuses other steps and forcings)
+            # nothing to differentiate (the tape refuses other steps and forcings);
+            # no graph, which this handle would replay once or twice
+            sim.set_launch(graph_chunk=0)
             sim.step(int(nsteps))
             h_t = sim.h()
             sim.close()

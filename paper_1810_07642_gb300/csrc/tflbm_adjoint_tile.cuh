@@ -22,7 +22,7 @@
 //      tile the disjoining-pressure adjoint and dL/dkappa
 //   4  on the tile grad p, the force adjoint, the Laplacian of -gamma ap, a(t)
 // 512^2 FP32, a gradient of 400 steps: 23.8 ms as marches of populations, 6.1 now,
-// of which an adjoint step took 27 us, 8 now (820 instructions a warp,
+// of which an adjoint step took 27 us, 9 now (820 instructions a warp,
 // half of the issue slots; 512 tiles on 152 SMs); threads, lanes, tiles and the
 // treatment of the edges are those of tflbm_tile.cuh.
 #pragma once
@@ -344,9 +344,9 @@ cudaError_t adjoint_tile_one(const S* mom, bool fresh, const S* an, S* a, S* gk,
     const long long tiles = (long long)grid.x * grid.y, sms = sm_count(), slots = 512 / NT * sms;
     const bool early = tiles <= sms || (tiles <= slots && 6 * tiles >= 5 * slots);
     if (C.omega != S(1)) return launch_dependent(k_adjoint_tile<S, TX, TY, false, 512>, grid, NT, 0, st, mom, fresh, early, an, a, gk, kappa, G, C);
-    // threads an SM holds, as for the forward tiles (one box, omega = 1, us a
-    // backward step, 512 / 1024: 300 x 200 6.9 / 9.0, 512^2 11.8 / 11.1, 1024^2
-    // 39.7 / 36.1)
+    // threads an SM holds, as for the forward tiles (one box, omega = 1, us of a
+    // gradient a step with neither rule / both: 512^2 16.3 / 13.8, 768^2 29.7 / 25.6,
+    // 1024^2 52.9 / 45.1; 384^2, below both, 9.1)
     if constexpr (TX == 32 && sizeof(S) == 4) {
         if (tiles > 3 * sms)
             return launch_dependent(k_adjoint_tile<S, TX, TY, true, 1024>, grid, NT, 0, st, mom, fresh, early, an, a, gk, kappa, G, C);

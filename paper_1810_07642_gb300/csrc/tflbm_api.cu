@@ -32,8 +32,9 @@ static long long tiles_of(int bx, int nx, int ny)
 // The FP32 shape with the least work on the busiest SM, counting a node's pull
 // as 0.45 of its cost and its pressure as 0.2 (the halos repeat those) and 60
 // nodes' worth of fixed latency a tile.  Measured, one box, us a step with block_x
-// 64 / 128 / 256: 128^2 2.9 / 3.1 / 3.3, 384^2 5.0 / 4.9 / 4.3, 512^2 6.6 / 6.5 / 5.1 (an
-// earlier form of the kernel), 1500 x 700 20.9 / 20.4 / 17.1.
+// 64 / 128 / 256: 64^2 2.34 / 2.40 / 2.46, 128^2 2.53 / 2.50 / 2.59, 200 x 150 3.16 / 2.90 /
+// 2.94, 384^2 3.94 / 3.77 / 3.51, 512^2 6.92 / 6.62 / 4.53, 1024^2 20.7 / 20.2 / 15.1 (where
+// 32 x 16 tiles run four an SM, see tile_one).
 static int tile_block_f32(int nx, int ny, int sms)
 {
     int best = 64;
@@ -189,10 +190,11 @@ int store_of(int dtype)
 // lattices).  FP64, and 16-bit storage where the one-column march is what is left,
 // run tiles at any size.  Above the limits the marches win: they pull a node 1.25
 // times, not 1.4, and load ahead.  Us a step, tile against march: FP32 four-column
-// 1024^2 14.9 / 16.4, 1200 x 1000 20 / 17.2, 1448^2 36.3 / 21.6; ragged 1030 x 1067 17.9 /
-// 21.4, 1205 x 1078 22.8 / 22.0, 1030 x 1262 23.1 / 22.2; FP16 1024^2 16.1 / 16.4, 1448^2
-// 34.3 / 21.4; against the one-column march at tau = 0.8: FP32 1448^2 37.2 / 36.7,
-// 2048^2 69 / 63, FP16 1448^2 32.3 / 41.7, 2048^2 59.8 / 69.2; FP64 2048^2 1135 / 1372.
+// 900^2 12.7 / 13.2, 1028^2 17.1 / 17.3, 1064^2 18.5 / 17.3, 1448^2 36.9 / 22.3; ragged 1030 x 1067 17.9 /
+// 21.4, 1205 x 1078 22.8 / 22.0, 1030 x 1262 23.1 / 22.2; FP16 1028^2 16.8 / 17.3, 1100^2
+// 18.3 / 17.6, 1448^2 31.8 / 21.6; against the one-column march at tau = 0.8: FP32 1228^2
+// 27.6 / 39.0, 1448^2 37.3 / 39.7, 1700^2 49.8 / 47.3, 2048^2 69 / 64, FP16 1448^2 32.7 /
+// 45.0, 2048^2 59.9 / 71.7; FP64 2048^2 1135 / 1372.
 constexpr long long kTileQuad = 17LL << 16, kTileRagged = 5LL << 18, kTileMarch = 3LL << 19;
 
 // Long lattices of a few rows, of which tiles cover too many: they cost more than

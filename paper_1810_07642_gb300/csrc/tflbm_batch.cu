@@ -2,9 +2,9 @@
 // the launch-shape autotuner and the on-device film diagnostics
 // (include/tflbm.h).
 //
-// A batched step is one launch of k_step_batch (one column per thread) or
-// k_step2_batch (two columns per thread, every nx even, FP32 compute type)
-// over a flat table of work items (domain, column strip, row band); a table
+// A batched step is one launch of k_step_batch (one column per thread),
+// k_step2_batch (two columns per thread, every nx even, FP32 compute type) or
+// k_step4_batch (four, tau = 1, every nx a multiple of 4) over a flat table of work items (domain, column strip, row band); a table
 // of per-domain records
 // (geometry, constants, the two population buffers, kappa) lives in device
 // memory next to it.  The records name the buffers in the order they had

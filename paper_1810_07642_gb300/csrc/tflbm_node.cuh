@@ -2,8 +2,9 @@
 // tflbm_step2.cuh: film pressure, force and collision (Section II of Zitz et
 // al., arXiv:1810.07642), written once for X = float2 (two nodes on
 // Blackwell's paired FP32 instructions) and X = double (one node).  The
-// two-column march (tflbm_step2.cuh) and the tile kernel (tflbm_tile.cuh) use
-// it; where a value comes from and where a result goes is theirs.
+// two- and four-column marches (tflbm_step2.cuh, tflbm_step4.cuh) and the tile
+// kernels (tflbm_tile.cuh, tflbm_adjoint_tile.cuh) use it; where a value comes
+// from and where a result goes is theirs.
 #pragma once
 #include "tflbm_step.cuh"
 

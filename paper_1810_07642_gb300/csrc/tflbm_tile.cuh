@@ -251,8 +251,9 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
     // x 190 25.2 / 20.1).  After the pressure, every tile is on an SM and near
     // its end; after h already, another phase of the next step's preamble and
     // launch is hidden, but the placement is uneven again unless half of the SMs
-    // are empty, small tiles number at most one an SM, or the slots (768 threads
-    // an SM, or 1024) are nearly full.  FP32, us a step, after the pressure / after
+    // are empty, small tiles number at most one an SM, or at least 5/6 of the
+    // slots are full (one wave, or several: the sizes measured have up to 13.5
+    // tiles an SM).  FP32, us a step, after the pressure / after
     // h: 64^2 2.61 / 2.45, 128^2 2.77 / 2.55, 200 x 150 (130 tiles of 16 x 16) 3.22
     // / 2.90; 256^2 (128 of 32 x 16) 3.03 / 3.18, 320^2 (400 of 16 x 16) 3.41 /
     // 3.67, 384^2 (288 of 32 x 16) 3.54 / 3.83; 509 x 387 (400) 4.58 / 4.23, 512^2
@@ -260,8 +261,9 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
     // Without a kappa field the preamble is too short to hide anything (one kappa,
     // 128^2 2.32 / 2.51, 512^2 4.45 / 4.51).
     const long long tiles = (long long)grid.x * grid.y, sms = sm_count();
+    const long long slots = (tiles > 3 * sms ? 4 : 3) * sms;  // of FP32 32 x 16 tiles, see below
     const bool spread = 2 * tiles <= sms || (TX * TY <= 256 && tiles <= sms) ||
-                       (TX == 32 && sizeof(S) == 4 && !mom && 2 * tiles >= 5 * sms && (tiles <= 3 * sms || 3 * tiles >= 10 * sms));
+                       (TX == 32 && sizeof(S) == 4 && !mom && 6 * tiles >= 5 * slots);
     const bool early = kappa && spread;
     auto launch = [&](auto resident) {
         constexpr int R = decltype(resident)::value;
@@ -270,9 +272,9 @@ cudaError_t tile_one(const S* f0, const SM* fm, S* g0, SM* gm, const S* kappa, S
     };
     // Threads an SM holds.  768 leaves the registers that keep a thread's 18
     // loads in flight (80); where 32 x 16 tiles outnumber the three an SM
-    // holds then, 64 registers and a fourth tile win (one box, tau = 1: 509 x
-    // 387 4.9 against 5.7 us a step, 512^2 6.4 against 5.3, 1024^2 17.8
-    // against 16.3).
+    // holds then, 64 registers and a fourth tile win (one box, tau = 1, us a step
+    // with 768 / 1024: 512^2 6.12 / 4.53, 640 x 480 6.36 / 4.57, 768^2 10.2 / 8.7, 1024^2
+    // 18.0 / 15.1; 509 x 387, 2.6 tiles an SM, 4.24 with 768).
     if constexpr (TX == 32 && sizeof(S) == 4) {
         if (tiles > 3 * sms) return launch(std::integral_constant<int, 1024>{});
     }

@@ -394,7 +394,8 @@ def batched_sweep(steps: int = 30000, timed: int = 400):
     out["mlups_batched_tuned"] = mlups(B.step, nodes, timed)
     out["speedup_batched_over_single_domain_launches"] = (out["mlups_batched_tuned"] /
                                                          out["mlups_single_domain_launches"])
-    # the persistent work queue and graph replay, beside the tuned shape
+    # graph replay of the tuned shape, and the persistent work queue, which is the
+    # two-column march's (asking for it leaves the four-column march)
     forms = {}
     for queue in (0, 1):
         for chunk in (0, 64):

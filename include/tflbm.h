@@ -259,7 +259,8 @@ int tf_lbm_tape_create(tf_lbm_handle* H, const void* h0, const void* theta, int6
 int tf_lbm_tape_forward(tf_lbm_tape* tape, void* stream);
 /* Given grad_h = dL/dh at the final time ([ny][nx]), write dL/dtheta and
  * dL/dh0 (each [ny][nx], or NULL to skip).  Recomputes each segment from its
- * state copy where not all records are kept; the handle ends at the final state again. */
+ * state copy where not all records are kept, in the tape's own buffers: the
+ * handle is left as it is (at the final state, unless it was stepped since). */
 int tf_lbm_tape_backward(tf_lbm_tape* tape, const void* grad_h, void* grad_theta, void* grad_h0,
                          void* stream);
 void tf_lbm_tape_destroy(tf_lbm_tape* tape);
@@ -272,7 +273,7 @@ void tf_lbm_tape_destroy(tf_lbm_tape* tape);
  * applies, and band counts of one, two and three waves of resident CTAs
  * (both balanced bands filling the waves exactly and their rounded-up band
  * heights) and band heights of 2 to 256 rows, then tiles of every block_x and
- * the four-column march in place of the fastest of these.  The state is copied aside first (one population
+ * the four-column march, which take the fields that tf_lbm_init chose.  The state is copied aside first (one population
  * buffer of device memory, freed before return) and put back after, so f
  * and tf_lbm_time are as before the call.  The graph chunk is kept.
  * Synchronises `stream`.  best (host, may be NULL) receives the shape now in

@@ -135,7 +135,10 @@ __device__ __forceinline__ X node_pressure(const Win<X>& H, X kap, bool disj, co
     // Eq. (n_laplace): axis neighbours left + right + up + down, diagonal the four corners
     const X axis = padd(padd(H.cL, H.cR), padd(H.n0, H.s0));
     const X diag = padd(padd(H.nL, H.nR), padd(H.sL, H.sR));
-    X lap = pmul(pfma(pk(S(4.0)), axis, pfma(pk(-S(20.0)), H.c0, diag)), pk(S(1.0 / 6.0)));
+    // the large terms cancel in the last fma, exactly but for the rounding of
+    // 4 axis + diag; with -20 c0 + diag rounded first, heights after 60 steps of a
+    // 700^2 drop were 1.15 times as far from FP64 (1.48e-7 against 1.29e-7)
+    X lap = pmul(pfma(pk(-S(20.0)), H.c0, pfma(pk(S(4.0)), axis, diag)), pk(S(1.0 / 6.0)));
     const X h = padd(H.c0, pk(C.href));
     ih = prcp(h);
     if (disj) {
